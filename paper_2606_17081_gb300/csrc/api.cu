@@ -580,10 +580,12 @@ static rs_status run_poa(rs_ctx* ctx, const rs_records& rec, std::vector<PoaProb
   CK(cudaMemcpyAsync(ctx->p_prob.p, probs.data(), np * sizeof(PoaProblem), cudaMemcpyHostToDevice,
                      ctx->st),
      "copy poa problems");
-  // last window of every problem (p_nwin serves as the span's output)
-  CK(launch_poa_span(P<PoaProblem>(ctx->p_prob), np, rec, ctx->cfg.poa_window,
-                     reinterpret_cast<long long*>(ctx->p_nwin.p), ctx->st),
-     "poa span launch");
+  // window of every row, last window of every problem (p_nwin takes the latter)
+  int64_t max_rows = 0;
+  for (const PoaProblem& p : probs) max_rows = std::max(max_rows, p.n);
+  CK(launch_poa_keys(P<PoaProblem>(ctx->p_prob), np, max_rows, rec, ctx->cfg.poa_window,
+                     P<int32_t>(ctx->p_wkey), reinterpret_cast<long long*>(ctx->p_nwin.p), ctx->st),
+     "poa keys launch");
   CK(cudaMemcpyAsync(ctx->pinned, ctx->p_nwin.p, (size_t)np * 8, cudaMemcpyDeviceToHost, ctx->st),
      "read poa spans");
   CK(cudaStreamSynchronize(ctx->st), "sync");

@@ -4,7 +4,7 @@
 // estimate: a serving process whose GPU memory is owned up front by another
 // allocator (so a cudaMalloc would fail or fragment it), or a latency-critical
 // path where cudaMalloc / cudaFree would synchronise the device.  This entry
-// point runs the same two PoA kernels as poa_estimate, but their scratch lives
+// point runs the same PoA kernels as poa_estimate, but their scratch lives
 // in one fixed array of static device memory (RS_NOALLOC_POA_BYTES bytes)
 // that every GPU loading the library holds until the process exits.  The
 // caller passes inputs and outputs in device memory; nothing is allocated and
@@ -163,7 +163,9 @@ extern "C" rs_status poa_estimate_noalloc(const rs_config* cfg, const rs_records
   b.wprob = nullptr;   // one problem: its windows stay on its own CTAs
   b.wnext = nullptr;
   b.nslots = 0;
-  if (launch_poa(dprob, 1, b, mc, st) != cudaSuccess) return RS_ERR_CUDA;
+  if (launch_poa_keys(dprob, 1, n, u, mc.poa_window, b.wkey, nullptr, st) != cudaSuccess ||
+      launch_poa(dprob, 1, b, mc, st) != cudaSuccess)
+    return RS_ERR_CUDA;
   k_noalloc_out<<<64, 256, 0, st>>>(b.wnum, b.wopt, b.wcnt, b.total, b.nwin, max_windows,
                                     numer_dev, opt_dev, count_dev, poa_total_dev, n_windows_dev);
   if (cudaGetLastError() != cudaSuccess) return RS_ERR_CUDA;

@@ -10,7 +10,7 @@
 namespace rs {
 
 constexpr int NT_SIM = 256;      // threads of a simulation / router CTA
-constexpr int NT_POA = 256;      // threads of a PoA CTA (8 warps, one window each)
+constexpr int NT_POA = 256;      // threads of a PoA key / total CTA
 constexpr int POA_WMAX = 16;     // workers of the per-warp PoA solver (wider: k_poa_solve_wide)
 constexpr int POA_WMAX_WIDE = 64;  // workers supported by the PoA estimate
 constexpr int WMAX = 64;         // workers supported by the simulation
@@ -159,10 +159,10 @@ struct PoaProblem {
 
 struct PoaBuffers {
   rs_records rec;
-  double* cost;             // [rows][W]
+  double* cost;             // [rows][W] by sorted row (a window past a capacity: fixed point)
   int32_t* order;           // [rows] row (relative) sorted by window, stable
   int32_t* asg;             // [rows]
-  int32_t* wkey;            // [rows] window of each row (-1 skipped)
+  int32_t* wkey;            // [rows] window of each row (-1 skipped); past the sort, scratch
   int64_t* wstart;          // [win slots + problems]
   int64_t* wfill;           // [win slots]
   double* wnum;             // [win slots]
@@ -188,9 +188,12 @@ cudaError_t launch_sweep_knee(const int32_t* worker, const double* ttft, const i
                               int n_sweeps, int pct, double theta, double* stat, double* d1,
                               double* d2, double* knee_load, int32_t* knee_index,
                               cudaStream_t st);
-// maxw[p] = last window index of problem p's routed rows (-1 if none).
-cudaError_t launch_poa_span(const PoaProblem* d_prob, int nprob, const rs_records& rec,
-                            double window, long long* maxw, cudaStream_t st);
+// wkey[scratch row] = window of every row; maxw[p] (nullable) = last window
+// index of problem p's routed rows (-1 if none).  max_rows: the largest problem.
+cudaError_t launch_poa_keys(const PoaProblem* d_prob, int nprob, int64_t max_rows,
+                            const rs_records& rec, double window, int32_t* wkey, long long* maxw,
+                            cudaStream_t st);
+// The sort, OPT and totals of problems whose keys are in b.wkey.
 cudaError_t launch_poa(const PoaProblem* d_prob, int nprob, const PoaBuffers& b,
                        const ModelConsts& mc, cudaStream_t st);
 

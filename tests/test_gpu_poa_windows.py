@@ -93,3 +93,39 @@ def test_windows_far_apart_and_empty_records():
     rec, keep = _to_device(o, 4, W)
     gn, go, gc, gt, nw = rs.poa_estimate(ctx.h, rec, 4, 4)
     assert nw == 0 and gt == 0.0
+
+
+def _random_records(rng, n, W, span, tied):
+    """Records whose cheapest workers exceed their capacity: worker 0 is cheap for every row;
+    `tied` makes many costs equal (few load levels, no prefixes)."""
+    nbt = rng.integers(1, 60, n).astype(np.int32)
+    nf = rng.integers(20, 23 if tied else 60, (n, W)).astype(np.uint16)
+    nf[:, 0] = rng.integers(1, 3 if tied else 20, n)
+    pre = np.zeros((n, W), np.uint16) if tied else \
+        (rng.integers(0, 2, (n, W)) * rng.integers(0, 60, (n, W)) % (nbt[:, None] + 1)).astype(np.uint16)
+    comp = rng.uniform(0.0, span, n)
+    comp[-1] = span - 1e-3
+    worker = rng.integers(-1, W, n).astype(np.int32)
+    worker[-1] = 0
+    return {"worker": worker, "completion": comp, "ttft": rng.uniform(0.01, 3.0, n), "nbt": nbt,
+            "n_frozen": nf, "prefix": pre}
+
+
+# windows up to the sort's table (11 264) and one past it; rows that end inside a warp's 32; solvers
+# for W = 3, 6, up to 16 and wider, at capacities that bind (rows per window > 64 on worker 0)
+@pytest.mark.parametrize("W,n,windows,tied", [
+    (2, 1, 1, False), (3, 331, 2, True), (6, 1537, 4, False), (6, 1000, 11264, False),
+    (6, 1000, 11265, False), (16, 900, 3, True), (17, 801, 2, False), (33, 700, 2, True),
+    (64, 1400, 2, False)])
+def test_sort_and_solvers_at_their_edges(W, n, windows, tied):
+    ctx = rs.Context(W=W, K=64)
+    o = _random_records(np.random.default_rng(W * n + windows), n, W, 5.0 * windows, tied)
+    num, opt, cnt, tot = O.poa(oracle_cfg(ctx), o)
+    assert num.size == windows
+    rec, keep = _to_device(o, n, W)
+    gn, go, gc, gt, nw = rs.poa_estimate(ctx.h, rec, n, windows)
+    assert nw == windows and np.array_equal(gc, cnt)
+    # sums of at most 1400 rows of one sign: n 2^-53 relative (1.6e-13); OPT's costs also carry
+    # 2^-52 of the window's largest cost each
+    assert np.allclose(gn, num, rtol=1e-12, atol=0) and np.allclose(go, opt, rtol=1e-12, atol=0)
+    assert abs(gt - tot) <= 1e-12 * tot
