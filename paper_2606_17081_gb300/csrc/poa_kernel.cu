@@ -39,8 +39,8 @@
 // below the 1e-12 below which a search on doubles must ignore gains.
 // Measured: poa_estimate on 20 000 records, W = 6 (81 windows): 4.22 -> 0.61 ms
 // a call (keys 97 -> 5 us, sort and costs 1480 -> 17 us, solver 2941 -> 578 us,
-// total 19 -> 6 us); the estimate of 16 replicas x 5000 requests at W = 64,
-// 126 -> 18 ms.
+// total 19 -> 6 us) with one warp per window, 0.43 ms with a CTA; the estimate
+// of 16 replicas x 5000 requests at W = 64, 126 -> 7 ms.
 //
 // k_poa_total (one warp per replica): the whole-run PoA, sum of observed
 // latency over sum of OPT across the replica's windows; and the static
@@ -67,12 +67,20 @@ __device__ __forceinline__ void fill_ftab(const ModelConsts& mc, double* ftab) {
   __syncthreads();
 }
 
-// c_ij of §6.4; a prefix of 0 leaves f(n) - w_c 0 = f(n) without the division.
+// c_ij of §6.4; a prefix of 0 leaves f(n) - w_c 0 without the division (and,
+// w_c being finite, f(n) itself).
 __device__ __forceinline__ double frozen_cost(const ModelConsts& mc, const double* ftab, int nft,
-                                              int nf, int m, int nbt) {
+                                              bool wc_finite, int nf, int m, int nbt) {
   const double f = nf < nft ? ftab[nf] : frozen_f(mc, nf);
-  if (m == 0 || nbt <= 0) return __dsub_rn(f, __dmul_rn(mc.w_c, 0.0));
+  if (m == 0 || nbt <= 0) return wc_finite ? f : __dsub_rn(f, __dmul_rn(mc.w_c, 0.0));
   return __dsub_rn(f, __dmul_rn(mc.w_c, __ddiv_rn((double)m, (double)nbt)));
+}
+
+// Order-preserving map of a double onto int64 (not NaN; -0 below +0): the
+// comparisons run on the integer units.
+__device__ __forceinline__ long long okey(double x) {
+  const long long u = __double_as_longlong(x);
+  return u ^ ((u >> 63) & 0x7FFFFFFFFFFFFFFFll);
 }
 
 // Window of each row into wkey: -1 for a row that was not routed, KEY_BAD for
@@ -329,12 +337,18 @@ __device__ __forceinline__ int warp_argmin(long long v, bool in, long long* best
   return who ? __ffs(who) - 1 : -1;
 }
 
-constexpr int NT_SOLVE = 128;   // most threads of a narrow solver CTA (one window per warp)
+constexpr int NT_SOLVE = 128;   // threads of a narrow solver CTA at one warp per window
+constexpr int NW_SOLVE = 8;     // warps of a CTA that works on one window
+constexpr int SOLVE_SROWS = 1024;   // rows whose assignment stays in shared memory
+constexpr int SOLVE_SCOST = 4096;   // costs (rows x W) a CTA per window keeps there too (32 KB)
 
-struct PoaWarpShared {
+struct PoaWinShared {
   long long wmin[POA_WMAX][POA_WMAX];   // edge weights, FX_INF without a row
   int wrow[POA_WMAX][POA_WMAX];         // the request behind each
   int counts[POA_WMAX];
+  int item[POA_WMAX * POA_WMAX];        // weights to look up again: 16 j + k
+  int nitems, emax;
+  uint8_t asg[SOLVE_SROWS];
 };
 
 __device__ __forceinline__ double warp_sum(double v) {
@@ -342,46 +356,43 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
-// Weights j -> k, for the columns k set in `need`, from the requests now at j:
-// min of c_qk - c_qj, ties to the lowest row.  Rows go 128 at a time, four per
-// lane in flight.
-template <int WT>
-__device__ __forceinline__ void poa_rescan(PoaWarpShared& S, const long long* cost,
-                                           const int32_t* asg, int64_t m, int W, int j,
-                                           unsigned need, int lane) {
-  while (need) {   // (uniform)
-    const int k = __ffs(need) - 1;
-    need &= need - 1;
-    long long best = FX_INF;
-    int row = -1;
-    for (int64_t r0 = lane; r0 < m; r0 += 128) {
-      int at[4];
-      long long v[4];
+// Weight j -> k from the requests now at j: min of c_qk - c_qj, ties to the
+// lowest row (one warp).  fx is [W][m]: lanes over the rows read whole sectors.
+// Rows go 256 at a time, eight per lane in flight.
+__device__ __forceinline__ void poa_rescan(PoaWinShared& S, const long long* fx,
+                                           const uint8_t* asg, int m, int j, int k, int lane) {
+  constexpr int U = 8;
+  const long long* ck = fx + (int64_t)k * m;
+  const long long* cj = fx + (int64_t)j * m;
+  long long best = FX_INF;
+  int row = -1;
+  for (int r0 = lane; r0 < m; r0 += 32 * U) {
+    int at[U];
+    long long v[U];
 #pragma unroll
-      for (int u = 0; u < 4; u++) {
-        const int64_t r = r0 + 32 * u;
-        at[u] = -1;
-        v[u] = 0;
-        if (r < m) {
-          at[u] = asg[r];
-          v[u] = cost[r * W + k] - cost[r * W + j];
-        }
+    for (int u = 0; u < U; u++) {
+      const int r = r0 + 32 * u;
+      at[u] = -1;
+      v[u] = 0;
+      if (r < m) {
+        at[u] = asg[r];
+        v[u] = ck[r] - cj[r];
       }
+    }
 #pragma unroll
-      for (int u = 0; u < 4; u++)
-        if (at[u] == j && v[u] < best) {
-          best = v[u];
-          row = (int)(r0 + 32 * u);
-        }
-    }
-    long long least;
-    warp_argmin(best, row >= 0, &least);
-    const bool mine = row >= 0 && best == least;
-    const unsigned rr = __reduce_min_sync(FULL_MASK, mine ? (unsigned)row : 0xFFFFFFFFu);
-    if (lane == 0) {
-      S.wmin[j][k] = rr != 0xFFFFFFFFu ? least : FX_INF;
-      S.wrow[j][k] = (int)rr;   // (-1 without a row)
-    }
+    for (int u = 0; u < U; u++)
+      if (at[u] == j && v[u] < best) {
+        best = v[u];
+        row = r0 + 32 * u;
+      }
+  }
+  long long least;
+  warp_argmin(best, row >= 0, &least);
+  const bool mine = row >= 0 && best == least;
+  const unsigned rr = __reduce_min_sync(FULL_MASK, mine ? (unsigned)row : 0xFFFFFFFFu);
+  if (lane == 0) {
+    S.wmin[j][k] = rr != 0xFFFFFFFFu ? least : FX_INF;
+    S.wrow[j][k] = (int)rr;   // (-1 without a row)
   }
 }
 
@@ -421,271 +432,314 @@ __device__ __forceinline__ bool poa_next(const PoaProblem* __restrict__ probs, c
 // POA_WMAX), so that the unrolled per-worker loops hold no dead iterations:
 // the solver's warps run different phases at once and its code must stay
 // small for the instruction cache.
-template <int WT>
-__global__ void __launch_bounds__(NT_SOLVE) k_poa_solve(const PoaProblem* __restrict__ probs,
-                                                        PoaBuffers b, ModelConsts mc) {
-  __shared__ PoaWarpShared P[NT_SOLVE / 32];
+// NWP: warps working on a window.  One when there are windows enough to fill
+// the GPU; NW_SOLVE (a CTA per window) when there are few and the launch waits
+// for its longest chain of augmentations: the warps then share the rows and
+// look up an augmentation's weights at the same time, while warp 0 runs the
+// path, and the window's costs sit in shared memory.  (poa_estimate on 20 000
+// records at W = 6, 81 windows of about 250 requests, 200 of them past a
+// capacity: 0.61 ms a call at one warp per window, 0.43 ms so.)
+template <int WT, int NWP>
+__global__ void __launch_bounds__(NWP == 1 ? NT_SOLVE : 32 * NWP)
+    k_poa_solve(const PoaProblem* __restrict__ probs, PoaBuffers b, ModelConsts mc) {
+  constexpr int WPC = NWP == 1 ? NT_SOLVE / 32 : 1;   // windows of a CTA
+  constexpr int NT = 32 * NWP;                        // threads of a window
+  __shared__ PoaWinShared P[WPC];
+  __shared__ long long s_fx[NWP == 1 ? 1 : SOLVE_SCOST];
   __shared__ double ftab[POA_FTAB];
+  __shared__ double red[3][NWP];
+  __shared__ int64_t s_w;
+  __shared__ int s_pi;
   fill_ftab(mc, ftab);
   const int nft = mc.cap < POA_FTAB ? mc.cap : POA_FTAB;
+  const bool wc_finite = __dmul_rn(mc.w_c, 0.0) == 0.0;
   const int W = mc.W;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, wpc = blockDim.x >> 5;
-  PoaWarpShared& S = P[warp];
-  int64_t next = (int64_t)blockIdx.y * wpc + warp;
-  const int64_t stride = (int64_t)gridDim.y * wpc;
-  int pi;
-  int64_t w;
-  // (a problem whose windows overflowed: k_poa_total reports it)
-  while (poa_next(probs, b, lane, next, stride, &pi, &w)) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int ww = NWP == 1 ? 0 : warp;                 // warp of the window
+  const int tid = ww * 32 + lane;
+  PoaWinShared& S = P[NWP == 1 ? warp : 0];
+  auto sync = [] {
+    if (NWP == 1) __syncwarp(); else __syncthreads();
+  };
+  // a sum over the window's threads, the warps' in order (every thread gets it)
+  auto sum3 = [&](double& x, double& y, double& z) {
+    x = warp_sum(x);
+    y = warp_sum(y);
+    z = warp_sum(z);
+    if (NWP > 1) {
+      if (lane == 0) { red[0][ww] = x; red[1][ww] = y; red[2][ww] = z; }
+      __syncthreads();
+      x = y = z = 0.0;
+      for (int v = 0; v < NWP; v++) { x += red[0][v]; y += red[1][v]; z += red[2][v]; }
+      __syncthreads();
+    }
+  };
+  int64_t next = (int64_t)blockIdx.y * WPC + (NWP == 1 ? warp : 0);
+  const int64_t stride = (int64_t)gridDim.y * WPC;
+  for (;;) {
+    // (a problem whose windows overflowed: k_poa_total reports it)
+    int pi = -1;
+    int64_t w = 0;
+    if (ww == 0 && !poa_next(probs, b, lane, next, stride, &pi, &w)) pi = -1;
+    if (NWP > 1) {
+      if (threadIdx.x == 0) { s_pi = pi; s_w = w; }
+      __syncthreads();
+      pi = s_pi;
+      w = s_w;
+    }
+    if (pi < 0) return;
     const PoaProblem pr = probs[pi];
     const int64_t* wst = b.wstart + pr.win_base + pi;
     const int64_t s0 = wst[w];
-    const int64_t m = wst[w + 1] - s0;
+    const int m = (int)(wst[w + 1] - s0);
     const int64_t base = pr.scratch_base + s0;   // window rows in order[], asg[]
     const int64_t slot = pr.win_base + w;
-    if (m == 0) {
-      if (lane == 0) {
-        b.wnum[slot] = 0.0;
-        b.wopt[slot] = 0.0;
-        b.wstat[slot] = 0.0;
-        b.wcnt[slot] = 0;
-      }
-      continue;
-    }
-    int64_t capw = (m + W - 1) / W;
+    int capw = (m + W - 1) / W;
     if (capw < mc.cap) capw = mc.cap;
-    if (lane < W) S.counts[lane] = 0;
-    __syncwarp();
-    double* cost = b.cost + base * W;
-    int32_t* asg = b.asg + base;
+    if (tid < W) S.counts[tid] = 0;
+    if (tid == 0) S.emax = 0;
+    sync();
+    double* cost = b.cost + base * W;   // [W][m]
+    uint8_t* asg = m <= SOLVE_SROWS ? S.asg : reinterpret_cast<uint8_t*>(b.asg + base);
     double num = 0.0, nst = 0.0, opt = 0.0;
     int emax = 0;
-    for (int64_t r = lane; r < m; r += 32) {
+    for (int r = tid; r < m; r += NT) {
       const int64_t q = pr.rec_base + b.order[base + r];
       const int nbt = b.rec.nbt[q], wk = b.rec.worker[q];
       const uint16_t* nfr = b.rec.n_frozen + q * W;
       const uint16_t* pre = b.rec.prefix + q * W;
-      double* cr = cost + r * W;
       double bc = 0.0, cw = 0.0;
+      long long bk = 0;
       int best = 0;
 #pragma unroll
       for (int j = 0; j < WT; j++) {
         if (j < W) {
-          const double c = frozen_cost(mc, ftab, nft, nfr[j], pre[j], nbt);
-          cr[j] = c;
-          if (j == 0 || c < bc) { bc = c; best = j; }
+          const double c = frozen_cost(mc, ftab, nft, wc_finite, nfr[j], pre[j], nbt);
+          const long long ck = okey(c);
+          cost[(int64_t)j * m + r] = c;
+          if (j == 0 || ck < bk) { bk = ck; bc = c; best = j; }
           if (j == wk) cw = c;
           const int e = cost_exp(c);
           emax = e > emax ? e : emax;
         }
       }
       nst += cw;   // the realized assignment's frozen cost
-      asg[r] = best;
+      asg[r] = (uint8_t)best;
       atomicAdd(&S.counts[best], 1);
       num += b.rec.ttft[q];
       opt += bc;
     }
-    num = warp_sum(num);
-    nst = warp_sum(nst);
-    __syncwarp();
-    int count = lane < W ? S.counts[lane] : 0;   // lane j keeps worker j's load
-    if (__any_sync(FULL_MASK, lane < W && count > capw)) {
-      emax = __reduce_max_sync(FULL_MASK, emax);
+    emax = __reduce_max_sync(FULL_MASK, emax);
+    if (lane == 0) atomicMax(&S.emax, emax);
+    sync();
+    sum3(num, nst, opt);
+    int count = lane < W ? S.counts[lane] : 0;   // lane j of warp 0 keeps worker j's load
+    if (__any_sync(FULL_MASK, lane < W && count > capw)) {   // (every warp alike)
       double inv;
-      const double scale = fx_scale(emax, FX_BITS, &inv);
-      long long* fx = reinterpret_cast<long long*>(cost);   // in place
-      for (int64_t e = lane; e < m * W; e += 32) fx[e] = to_fx(cost[e], scale, FX_BITS);
-      __syncwarp();
-      const unsigned wmask = (1u << W) - 1u;
-      for (int j = 0; j < W; j++)
-        poa_rescan<WT>(S, fx, asg, m, W, j, wmask & ~(1u << j), lane);
-      if (lane < W) {
-        S.wmin[lane][lane] = FX_INF;
-        S.wrow[lane][lane] = -1;
+      const double scale = fx_scale(S.emax, FX_BITS, &inv);
+      long long* fx = NWP > 1 && (int64_t)m * W <= SOLVE_SCOST ? s_fx
+                                                                : reinterpret_cast<long long*>(cost);
+      for (int64_t e = tid; e < (int64_t)m * W; e += NT) fx[e] = to_fx(cost[e], scale, FX_BITS);
+      if (tid < W) {
+        S.wmin[tid][tid] = FX_INF;
+        S.wrow[tid][tid] = -1;
       }
-      __syncwarp();
+      sync();
+      for (int e = ww; e < W * W; e += NWP)
+        if (e / W != e % W) poa_rescan(S, fx, asg, m, e / W, e % W, lane);
+      sync();
       for (;;) {
-        // distances from the workers over their capacity, in Jacobi rounds:
-        // lane k < W owns target k and every round reads the previous one's
-        // distances (shortest paths have at most W - 1 edges)
-        const bool src = lane < W && count > capw;
-        if (!__any_sync(FULL_MASK, src)) break;
-        long long dk = src ? 0 : FX_INF;
-        int pk = -1;
-        long long wm[WT];
+        int nmv = 0, mk = -1, mr = -1;
+        if (ww == 0) {
+          // distances from the workers over their capacity, in Jacobi rounds:
+          // lane k < W owns target k and every round reads the previous one's
+          // distances (shortest paths have at most W - 1 edges)
+          const bool src = lane < W && count > capw;
+          int pk = -1, tgt = -1;
+          long long dk = src ? 0 : FX_INF, dt;
+          if (__any_sync(FULL_MASK, src)) {
+            long long wm[WT];
 #pragma unroll
-        for (int j = 0; j < WT; j++) wm[j] = j < W && lane < W ? S.wmin[j][lane] : FX_INF;
-        for (int it = 0; it < W; it++) {
-          long long bv = dk < FX_REAL ? dk : FX_REAL;
-          int bj = -1;
+            for (int j = 0; j < WT; j++) wm[j] = j < W && lane < W ? S.wmin[j][lane] : FX_INF;
+            for (int it = 0; it < W; it++) {
+              long long bv = dk < FX_REAL ? dk : FX_REAL;
+              int bj = -1;
 #pragma unroll
-          for (int j = 0; j < WT; j++) {
-            const long long v = __shfl_sync(FULL_MASK, dk, j) + wm[j];   // (<= 2 FX_INF)
-            if (v < bv) { bv = v; bj = j; }
+              for (int j = 0; j < WT; j++) {
+                const long long v = __shfl_sync(FULL_MASK, dk, j) + wm[j];   // (<= 2 FX_INF)
+                if (v < bv) { bv = v; bj = j; }
+              }
+              if (bj >= 0) { dk = bv; pk = bj; }
+              if (!__any_sync(FULL_MASK, bj >= 0)) break;
+            }
+            // target: the nearest worker with room (ties: lowest index)
+            tgt = warp_argmin(dk, lane < W && count < capw && dk < FX_REAL, &dt);
           }
-          if (bj >= 0) { dk = bv; pk = bj; }
-          if (!__any_sync(FULL_MASK, bj >= 0)) break;
-        }
-        // target: the nearest worker with room (ties: lowest index)
-        long long dt;
-        const int tgt = warp_argmin(dk, lane < W && count < capw && dk < FX_REAL, &dt);
-        if (tgt < 0) break;   // (cannot happen: W capw >= m)
-        // walk the path back from its end: each edge j -> k moves the request
-        // behind wrow[j][k] from j to k; lane t keeps step t
-        int k = tgt, nmv = 0, mj = -1, mk = -1, mr = -1;
-        for (; nmv < W; nmv++) {
-          const int j = __shfl_sync(FULL_MASK, pk, k);
-          if (j < 0) break;
-          if (lane == nmv) {
-            mj = j;
-            mk = k;
-            mr = S.wrow[j][k];
+          // walk the path back from its end: each edge j -> k moves the
+          // request behind wrow[j][k] from j to k; lane t keeps step t.  A
+          // worker that loses a request: the weights whose minimum it was go
+          // to the list
+          int k = tgt, ni = 0;
+          for (; tgt >= 0 && nmv < W; nmv++) {
+            const int j = __shfl_sync(FULL_MASK, pk, k);
+            if (j < 0) break;
+            const int r = S.wrow[j][k];
+            if (lane == nmv) {
+              mk = k;
+              mr = r;
+            }
+            const bool need = lane < W && lane != j && S.wrow[j][lane] == r;
+            const unsigned nm = __ballot_sync(FULL_MASK, need);
+            if (need) S.item[ni + __popc(nm & ((1u << lane) - 1u))] = j * POA_WMAX + lane;
+            ni += __popc(nm);
+            k = j;
           }
-          k = j;
+          if (tgt >= 0 && lane == k) count--;
+          if (tgt >= 0 && lane == tgt) count++;
+          if (lane < nmv) asg[mr] = (uint8_t)mk;
+          if (lane == 0) S.nitems = ni;
         }
-        if (lane == k) count--;
-        if (lane == tgt) count++;
-        if (lane < nmv) asg[mr] = mk;
-        __syncwarp();
-        // a worker that lost a request: the weights whose minimum it was
-        for (int t = 0; t < nmv; t++) {
-          const int j = __shfl_sync(FULL_MASK, mj, t), r = __shfl_sync(FULL_MASK, mr, t);
-          const unsigned need = __ballot_sync(FULL_MASK, lane < W && lane != j && S.wrow[j][lane] == r);
-          poa_rescan<WT>(S, fx, asg, m, W, j, need, lane);
-        }
-        __syncwarp();
+        sync();
+        const int ni = S.nitems;
+        if (ni == 0) break;   // no worker over its capacity is left (a path has items)
+        for (int e = ww; e < ni; e += NWP)
+          poa_rescan(S, fx, asg, m, S.item[e] / POA_WMAX, S.item[e] % POA_WMAX, lane);
+        sync();
         // requests that moved in lower their new worker's weights
-        for (int t = 0; t < nmv; t++) {
-          const int to = __shfl_sync(FULL_MASK, mk, t), r = __shfl_sync(FULL_MASK, mr, t);
-          if (lane < W && lane != to) {
-            const long long v = fx[(int64_t)r * W + lane] - fx[(int64_t)r * W + to];
-            const long long o = S.wmin[to][lane];
-            if (v < o || (v == o && r < S.wrow[to][lane])) {
-              S.wmin[to][lane] = v;
-              S.wrow[to][lane] = r;
+        if (ww == 0) {
+          for (int t = 0; t < nmv; t++) {
+            const int to = __shfl_sync(FULL_MASK, mk, t), r = __shfl_sync(FULL_MASK, mr, t);
+            if (lane < W && lane != to) {
+              const long long v = fx[(int64_t)lane * m + r] - fx[(int64_t)to * m + r];
+              const long long o = S.wmin[to][lane];
+              if (v < o || (v == o && r < S.wrow[to][lane])) {
+                S.wmin[to][lane] = v;
+                S.wrow[to][lane] = r;
+              }
             }
           }
+          __syncwarp();
         }
-        __syncwarp();
       }
-      const bool bad = __any_sync(FULL_MASK, lane < W && count > capw);
+      // (a load past its capacity cannot be left: W capw >= m)
+      const bool bad = ww == 0 && __any_sync(FULL_MASK, lane < W && count > capw);
       opt = 0.0;
-      for (int64_t r = lane; r < m; r += 32) opt += (double)fx[r * W + asg[r]] * inv;
+      for (int r = tid; r < m; r += NT) opt += (double)fx[(int64_t)asg[r] * m + r] * inv;
+      double z0 = 0.0, z1 = 0.0;
+      sum3(opt, z0, z1);
       if (bad) opt = __longlong_as_double(0x7FF8000000000000ll);
     }
-    opt = warp_sum(opt);
-    if (lane == 0) {
+    if (tid == 0) {
       b.wnum[slot] = num;
       b.wstat[slot] = nst;
       b.wopt[slot] = opt;
       b.wcnt[slot] = m;
     }
-    __syncwarp();
+    sync();   // (S is reused by the next window)
   }
 }
 
-// The same OPT for W > POA_WMAX workers, one CTA per window: few windows, each
-// of hundreds to thousands of requests, so the latency of one augmentation is
-// what counts.  Thread t owns the target worker t % 64 and a quarter t / 64 of
-// the sources (or of a worker's requests) in every W x W step; the quarters
-// meet in shared memory.
-constexpr int NT_WIDE = 256;
-constexpr int WIDE_G = NT_WIDE / POA_WMAX_WIDE;   // source groups
+// The same OPT for W > POA_WMAX workers, one CTA of 32 warps per window: few
+// windows, each of hundreds to thousands of requests, so the latency of one
+// augmentation is what counts, and a window's weights (52 KB), its requests by
+// worker and each request's cost at its worker stay in shared memory.  Per
+// augmentation: Jacobi rounds relax the edges out of the sources that changed
+// in the round before, thread (g, k) those of sources 4 g .. 4 g + 3 into target
+// k, and a thread per target joins the groups; warp 0 walks the path and moves
+// its requests between the workers' lists; the weights that lost their minimum
+// are listed, and a warp looks up one of them, or a part of one while there
+// are fewer than warps, lanes over its worker's requests.  (16 replicas x 5000
+// requests, 48 windows of 950 to 1450 rows with 450 to 1070 rows to move: 18 ms
+// with 8 warps and a quarter of the sources per thread, 7 ms so; a round costs
+// about 500 cycles, of 6 per augmentation.)
+constexpr int NT_WIDE = 1024;
+constexpr int NW_WIDE = NT_WIDE / 32;
+constexpr int WIDE_G = NT_WIDE / POA_WMAX_WIDE;            // source groups of a round
+constexpr int WIDE_GS = POA_WMAX_WIDE / WIDE_G;            // sources of a group
+constexpr int WIDE_SROWS = 4096;   // rows of a window whose lists fit in shared memory
+// list entries then: every worker's list holds max(its first load, capacity)
+// rows, in all at most rows + max(64 W, rows + W)
+constexpr int WIDE_SLIST = 2 * WIDE_SROWS + POA_WMAX_WIDE;
+static_assert(NW_WIDE == 32, "a lane per warp joins the warps' sums");
 
 struct PoaWideShared {
   long long dist[POA_WMAX_WIDE];
-  long long pv[WIDE_G][POA_WMAX_WIDE];   // per group: the best value of each target ...
-  int pi[WIDE_G][POA_WMAX_WIDE];         // ... and its source (or request)
-  double red[3][NT_WIDE / 32];
+  long long pv[WIDE_G][POA_WMAX_WIDE];   // a round: best way into each target from each group
+  uint8_t pj[WIDE_G][POA_WMAX_WIDE];     // ... and its source
+  long long part_v[NW_WIDE];             // a weight's parts
+  int part_r[NW_WIDE];
+  unsigned act[2];                       // sources that changed in the last round
+  double red[3][NW_WIDE];
   double ftab[POA_FTAB];
-  int pred[POA_WMAX_WIDE], counts[POA_WMAX_WIDE];
-  int mv_j[POA_WMAX_WIDE], mv_k[POA_WMAX_WIDE], mv_r[POA_WMAX_WIDE];   // the last path's moves
-  int dpos[POA_WMAX_WIDE];     // where a source's request list starts, -1: not rescanned
-  int dfill[POA_WMAX_WIDE];
-  int nmv, changed, emax, done, tgt, pi_next;
+  int32_t* list[POA_WMAX_WIDE];          // each worker's requests
+  int pred[POA_WMAX_WIDE], counts[POA_WMAX_WIDE], fill[POA_WMAX_WIDE];
+  int path[POA_WMAX_WIDE + 1];           // workers from the target back to the source
+  int mv_r[POA_WMAX_WIDE];               // the request moved from path[t + 1] to path[t]
+  int nmv, nitems, emax, pi_next;
   int64_t w_next;
 };
 
+// Row stride of the weights, stored [target][source] and odd: lanes over the
+// sources of one target, or over the targets of one source, hit other banks.
+__host__ __device__ inline int wide_ld(int W) { return W | 1; }
 __host__ __device__ inline size_t poa_wide_smem(int W) {
-  return (size_t)W * W * 12;   // weights and their requests; PoaWideShared is static
+  return (size_t)W * wide_ld(W) * 12 + (size_t)WIDE_SROWS * 12 + (size_t)WIDE_SLIST * 4 +
+         (size_t)W * W * 2 + 8;
 }
 
-// Weights j -> k of every source with dpos[j] >= 0, for the columns whose
-// minimum left (wrow[j][k] == lost[j]; every column when `all`), from the
-// requests now at j.  list: scratch for the rescanned sources' requests.
-__device__ __forceinline__ void wide_rescan(PoaWideShared& S, long long* wmin, int* wrow,
-                                            const long long* fx, const int32_t* asg, int32_t* list,
-                                            int64_t m, int W, int nsrc, const int* srcs,
-                                            const int* lost, bool all) {
-  const int k = threadIdx.x % POA_WMAX_WIDE, g = threadIdx.x / POA_WMAX_WIDE;
-  // the rescanned sources' requests, gathered per source (any order: ties are
-  // settled by the row)
-  for (int64_t r = threadIdx.x; r < m; r += NT_WIDE) {
-    const int j = asg[r];
-    const int d = S.dpos[j];
-    if (d >= 0) list[d + atomicAdd(&S.dfill[j], 1)] = (int32_t)r;
-  }
-  __syncthreads();
-  for (int s = 0; s < nsrc; s++) {
-    const int j = all ? s : srcs[s];
-    const int n = S.dfill[j];
-    const int32_t* rows = list + S.dpos[j];
-    const bool need = k < W && k != j && (all || wrow[j * W + k] == lost[s]);
-    long long best = FX_INF;
-    int row = -1;
-    if (need) {
-      for (int t0 = g; t0 < n; t0 += 8 * WIDE_G) {
-        long long v[8];
-        int rr[8];
+// Weight j -> k over part `part` of `parts` of worker j's n requests: min of
+// c_qk - c_qj, ties to the lowest row (one warp; row -1: no request there).
+// rows NULL: the requests r < n with pos[r] == j.  cur: the requests' costs at
+// their workers, or NULL (then read from fx).
+__device__ __forceinline__ void wide_weight(const int32_t* rows, const int32_t* pos, int n,
+                                            const long long* fx, const long long* cur, int W, int j,
+                                            int k, int part, int parts, int lane, long long* least,
+                                            int* lrow) {
+  constexpr int U = 4;
+  long long best = FX_INF;
+  int row = -1;
+  for (int t0 = part * 32 * U + lane; t0 < n; t0 += parts * 32 * U) {
+    int rr[U];
+    long long v[U];
 #pragma unroll
-        for (int u = 0; u < 8; u++) {
-          const int t = t0 + u * WIDE_G;
-          rr[u] = t < n ? rows[t] : -1;
-        }
-#pragma unroll
-        for (int u = 0; u < 8; u++) {
-          const long long* cr = fx + (int64_t)(rr[u] < 0 ? 0 : rr[u]) * W;
-          v[u] = cr[k] - cr[j];
-        }
-#pragma unroll
-        for (int u = 0; u < 8; u++)
-          if (rr[u] >= 0 && (v[u] < best || (v[u] == best && rr[u] < row))) {
-            best = v[u];
-            row = rr[u];
-          }
+    for (int u = 0; u < U; u++) {
+      const int t = t0 + 32 * u;
+      rr[u] = -1;
+      if (t < n) rr[u] = rows ? rows[t] : (pos[t] == j ? t : -1);
+      v[u] = 0;
+      if (rr[u] >= 0) {
+        const long long* cr = fx + (int64_t)rr[u] * W;
+        v[u] = cr[k] - (cur ? cur[rr[u]] : cr[j]);
       }
     }
-    S.pv[g][k] = best;
-    S.pi[g][k] = row;
-    __syncthreads();
-    if (g == 0 && need) {
 #pragma unroll
-      for (int h = 1; h < WIDE_G; h++) {
-        const long long v = S.pv[h][k];
-        const int r = S.pi[h][k];
-        if (r >= 0 && (v < best || (v == best && r < row))) {
-          best = v;
-          row = r;
-        }
+    for (int u = 0; u < U; u++)
+      if (rr[u] >= 0 && (v[u] < best || (v[u] == best && rr[u] < row))) {
+        best = v[u];
+        row = rr[u];
       }
-      wmin[j * W + k] = row >= 0 ? best : FX_INF;
-      wrow[j * W + k] = row;
-    }
-    __syncthreads();
   }
+  warp_argmin(best, row >= 0, least);
+  const bool mine = row >= 0 && best == *least;
+  *lrow = (int)__reduce_min_sync(FULL_MASK, mine ? (unsigned)row : 0xFFFFFFFFu);
+  if (*lrow < 0) *least = FX_INF;
 }
 
 __global__ void __launch_bounds__(NT_WIDE) k_poa_solve_wide(const PoaProblem* __restrict__ probs,
                                                             PoaBuffers b, ModelConsts mc) {
   extern __shared__ __align__(16) unsigned char wsm[];
   __shared__ PoaWideShared S;
-  const int W = mc.W;
-  long long* wmin = reinterpret_cast<long long*>(wsm);
-  int* wrow = reinterpret_cast<int*>(wmin + (size_t)W * W);
+  const int W = mc.W, ld = wide_ld(W);
+  long long* wmin = reinterpret_cast<long long*>(wsm);               // [target][source]
+  long long* s_cur = wmin + (size_t)W * ld;
+  int* wrow = reinterpret_cast<int*>(s_cur + WIDE_SROWS);
+  int32_t* s_pos = wrow + (size_t)W * ld;
+  int32_t* s_list = s_pos + WIDE_SROWS;
+  uint16_t* item = reinterpret_cast<uint16_t*>(s_list + WIDE_SLIST);   // 64 j + k
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int k = threadIdx.x % POA_WMAX_WIDE, g = threadIdx.x / POA_WMAX_WIDE;
   fill_ftab(mc, S.ftab);
   const int nft = mc.cap < POA_FTAB ? mc.cap : POA_FTAB;
+  const bool wc_finite = __dmul_rn(mc.w_c, 0.0) == 0.0;
   int64_t next = blockIdx.y;
   const int64_t stride = gridDim.y;
   for (;;) {
@@ -699,7 +753,7 @@ __global__ void __launch_bounds__(NT_WIDE) k_poa_solve_wide(const PoaProblem* __
         S.emax = 0;
       }
     }
-    for (int j = threadIdx.x; j < W; j += NT_WIDE) S.counts[j] = 0;
+    if (threadIdx.x < W) S.counts[threadIdx.x] = 0;
     __syncthreads();
     const int pi = S.pi_next;
     if (pi < 0) return;
@@ -707,17 +761,25 @@ __global__ void __launch_bounds__(NT_WIDE) k_poa_solve_wide(const PoaProblem* __
     const PoaProblem pr = probs[pi];
     const int64_t* wst = b.wstart + pr.win_base + pi;
     const int64_t s0 = wst[w];
-    const int64_t m = wst[w + 1] - s0;
+    const int m = (int)(wst[w + 1] - s0);
     const int64_t base = pr.scratch_base + s0;
     const int64_t slot = pr.win_base + w;
-    int64_t capw = (m + W - 1) / W;
+    int capw = (m + W - 1) / W;
     if (capw < mc.cap) capw = mc.cap;
-    double* cost = b.cost + base * W;
-    int32_t* asg = b.asg + base;
+    double* cost = b.cost + base * W;   // [m][W]
+    const bool in_smem = m <= WIDE_SROWS && capw <= WIDE_SROWS / W;
+    // lists fit: in shared memory, or in the window's order[] and wkey[], not
+    // needed past the sums below (the full workers' lists, m rows at most, in
+    // the one, the others' capacities in the other).  They do not when a large
+    // C_j leaves the workers room for several times the window's rows; a
+    // worker's requests are then found by scanning the rows
+    const bool listed = in_smem || (int64_t)(W - 1) * capw <= m;
+    // a row's worker; once the lists are built, its position in its list
+    int32_t* pos = in_smem ? s_pos : b.asg + base;
     // costs and cheapest workers, one warp per request (lane: workers lane, lane + 32)
     double num = 0.0, nst = 0.0, opt = 0.0;
     int emax = 0;
-    for (int64_t r = warp; r < m; r += NT_WIDE / 32) {
+    for (int r = warp; r < m; r += NW_WIDE) {
       const int64_t q = pr.rec_base + b.order[base + r];
       const int nbt = b.rec.nbt[q];
       double c[2];
@@ -726,34 +788,23 @@ __global__ void __launch_bounds__(NT_WIDE) k_poa_solve_wide(const PoaProblem* __
         const int j = lane + 32 * h;
         c[h] = 0.0;
         if (j < W) {
-          c[h] = frozen_cost(mc, S.ftab, nft, b.rec.n_frozen[q * W + j], b.rec.prefix[q * W + j], nbt);
-          cost[r * W + j] = c[h];
+          c[h] = frozen_cost(mc, S.ftab, nft, wc_finite, b.rec.n_frozen[q * W + j],
+                             b.rec.prefix[q * W + j], nbt);
+          cost[(int64_t)r * W + j] = c[h];
           const int e = cost_exp(c[h]);
           emax = e > emax ? e : emax;
         }
       }
-      // the lowest-index cheapest worker (W > 32 or not: lane l's first is l)
-      double bc = c[0];
-      int best = lane;
-      bool in = lane < W;
-      if (lane + 32 < W && c[1] < bc) {
-        bc = c[1];
-        best = lane + 32;
-      }
-      for (int o = 16; o > 0; o >>= 1) {
-        const double oc = __shfl_xor_sync(FULL_MASK, bc, o);
-        const int ob = __shfl_xor_sync(FULL_MASK, best, o);
-        const bool oi = __shfl_xor_sync(FULL_MASK, in, o);
-        if (oi && (!in || oc < bc || (oc == bc && ob < best))) {
-          bc = oc;
-          best = ob;
-          in = true;
-        }
-      }
+      // the lowest-index cheapest worker: the lower half's on a tie
+      long long k0, k1;
+      const int b0 = warp_argmin(okey(c[0]), lane < W, &k0);
+      const int b1 = warp_argmin(okey(c[1]), lane + 32 < W, &k1);
+      const int best = b1 >= 0 && k1 < k0 ? b1 + 32 : b0;
+      const double bc = __shfl_sync(FULL_MASK, best < 32 ? c[0] : c[1], best & 31);
       const int wk = b.rec.worker[q];
       const double cw = __shfl_sync(FULL_MASK, wk < 32 ? c[0] : c[1], wk & 31);
       if (lane == 0) {
-        asg[r] = best;
+        pos[r] = best;
         atomicAdd(&S.counts[best], 1);
         num += b.rec.ttft[q];
         nst += cw;
@@ -768,137 +819,303 @@ __global__ void __launch_bounds__(NT_WIDE) k_poa_solve_wide(const PoaProblem* __
       S.red[2][warp] = opt;
     }
     __syncthreads();
-    num = nst = opt = 0.0;
-    for (int v = 0; v < NT_WIDE / 32; v++) {
-      num += S.red[0][v];
-      nst += S.red[1][v];
-      opt += S.red[2][v];
-    }
+    num = warp_sum(S.red[0][lane]);   // (NW_WIDE == 32: a lane per warp)
+    nst = warp_sum(S.red[1][lane]);
+    opt = warp_sum(S.red[2][lane]);
     if (__syncthreads_or(threadIdx.x < W && S.counts[threadIdx.x] > capw)) {
       double inv;
       const double scale = fx_scale(S.emax, FX_BITS_WIDE, &inv);
       long long* fx = reinterpret_cast<long long*>(cost);   // in place
-      int32_t* list = b.wkey + base;   // (the keys are not needed past the sort)
-      for (int64_t e = threadIdx.x; e < m * W; e += NT_WIDE)
+      for (int64_t e = threadIdx.x; e < (int64_t)m * W; e += NT_WIDE)
         fx[e] = to_fx(cost[e], scale, FX_BITS_WIDE);
+      // room for a worker's first load or, below it, its capacity
       if (threadIdx.x == 0) {
-        int o = 0;
+        int32_t *over = in_smem ? s_list : b.order + base, *under = b.wkey + base;
         for (int j = 0; j < W; j++) {
-          S.dpos[j] = o;
-          S.dfill[j] = 0;
-          o += S.counts[j];
+          S.fill[j] = 0;
+          if (in_smem || S.counts[j] >= capw) {
+            S.list[j] = over;
+            over += S.counts[j] > capw ? S.counts[j] : capw;
+          } else {
+            S.list[j] = under;
+            under += capw;
+          }
         }
       }
-      for (int j = threadIdx.x; j < W; j += NT_WIDE) {
-        wmin[j * W + j] = FX_INF;
-        wrow[j * W + j] = -1;
+      if (threadIdx.x < W) {
+        wmin[threadIdx.x * ld + threadIdx.x] = FX_INF;
+        wrow[threadIdx.x * ld + threadIdx.x] = -1;
       }
       __syncthreads();
-      wide_rescan(S, wmin, wrow, fx, asg, list, m, W, W, nullptr, nullptr, true);
+      long long* cur = in_smem ? s_cur : nullptr;
+      for (int r = threadIdx.x; listed && r < m; r += NT_WIDE) {
+        const int j = pos[r];
+        const int p = atomicAdd(&S.fill[j], 1);
+        S.list[j][p] = r;
+        pos[r] = p;
+        if (cur) cur[r] = fx[(int64_t)r * W + j];
+      }
+      __syncthreads();
+      // every weight: a warp per worker, lanes over the targets
+      for (int j = warp; j < W; j += NW_WIDE) {
+        const int32_t* rows = S.list[j];
+        const int n = listed ? S.counts[j] : m;
+        long long best[2] = {FX_INF, FX_INF};
+        int row[2] = {-1, -1};
+        for (int t0 = 0; t0 < n; t0 += 4) {
+          int rr[4];
+          long long c[4][3];
+#pragma unroll
+          for (int u = 0; u < 4; u++) {
+            rr[u] = -1;
+            if (t0 + u < n) rr[u] = listed ? rows[t0 + u] : (pos[t0 + u] == j ? t0 + u : -1);
+            const long long* cr = fx + (int64_t)(rr[u] < 0 ? 0 : rr[u]) * W;
+            c[u][0] = lane < W ? cr[lane] : 0;
+            c[u][1] = lane + 32 < W ? cr[lane + 32] : 0;
+            c[u][2] = cr[j];
+          }
+#pragma unroll
+          for (int u = 0; u < 4; u++)
+#pragma unroll
+            for (int h = 0; h < 2; h++) {
+              const long long v = c[u][h] - c[u][2];
+              if (rr[u] >= 0 && (v < best[h] || (v == best[h] && rr[u] < row[h]))) {
+                best[h] = v;
+                row[h] = rr[u];
+              }
+            }
+        }
+#pragma unroll
+        for (int h = 0; h < 2; h++) {
+          const int q = lane + 32 * h;
+          if (q < W && q != j) {
+            wmin[q * ld + j] = best[h];
+            wrow[q * ld + j] = row[h];
+          }
+        }
+      }
       for (;;) {
-        // distances from the workers over their capacity, in Jacobi rounds
-        const bool src = threadIdx.x < W && S.counts[threadIdx.x] > capw;
-        if (threadIdx.x < W) {
+        // distances from the workers over their capacity, in Jacobi rounds:
+        // every round reads the previous one's distances and relaxes the edges
+        // out of the sources that changed in it (an edge out of another was
+        // tested against a distance that has only fallen since)
+        if (threadIdx.x < POA_WMAX_WIDE) {
+          const bool src = threadIdx.x < W && S.counts[threadIdx.x] > capw;
           S.dist[threadIdx.x] = src ? 0 : FX_INF;
           S.pred[threadIdx.x] = -1;
+          const unsigned bal = __ballot_sync(FULL_MASK, src);
+          if (lane == 0) S.act[warp] = bal;
         }
-        if (!__syncthreads_or(src)) break;
-        for (int it = 0; it < W; it++) {
+        if (threadIdx.x == 0) S.nitems = 0;
+        __syncthreads();
+        uint64_t act = (uint64_t)S.act[0] | ((uint64_t)S.act[1] << 32);
+        if (act == 0) break;
+        const int k = threadIdx.x & (POA_WMAX_WIDE - 1), g = threadIdx.x / POA_WMAX_WIDE;
+        for (int it = 0; it < W && act; it++) {
+          const unsigned mine = (unsigned)(act >> (WIDE_GS * g)) & ((1u << WIDE_GS) - 1u);
           long long bv = FX_REAL;
-          int bj = -1;
-          if (k < W) {
-#pragma unroll 4
-            for (int j = g; j < W; j += WIDE_G) {
-              const long long v = S.dist[j] + wmin[j * W + k];   // (<= 2 FX_INF)
-              if (v < bv) {
-                bv = v;
-                bj = j;
-              }
+          int bj = 0;
+          if (mine && k < W) {   // (mine is alike in the warp)
+            long long v[WIDE_GS];
+#pragma unroll
+            for (int q = 0; q < WIDE_GS; q++) {
+              const int j = WIDE_GS * g + q < W ? WIDE_GS * g + q : W - 1;
+              v[q] = S.dist[j] + wmin[k * ld + j];   // (<= 2 FX_INF)
             }
+#pragma unroll
+            for (int q = 0; q < WIDE_GS; q++)
+              if ((mine >> q & 1u) && v[q] < bv) {
+                bv = v[q];
+                bj = WIDE_GS * g + q;
+              }
           }
           S.pv[g][k] = bv;
-          S.pi[g][k] = bj;
+          S.pj[g][k] = (uint8_t)bj;
           __syncthreads();
-          bool ch = false;
-          if (g == 0 && k < W) {
-            for (int h = 1; h < WIDE_G; h++)
-              if (S.pv[h][k] < bv) {
-                bv = S.pv[h][k];
-                bj = S.pi[h][k];
+          if (threadIdx.x < POA_WMAX_WIDE) {
+            // (sources in increasing order: ties keep the lowest)
+            long long v[WIDE_G];
+#pragma unroll
+            for (int q = 0; q < WIDE_G; q++) v[q] = S.pv[q][k];
+            const long long d = S.dist[k];
+            long long nv = d < FX_REAL ? d : FX_REAL;
+            int from = -1;
+#pragma unroll
+            for (int q = 0; q < WIDE_G; q++)
+              if (v[q] < nv) {
+                nv = v[q];
+                from = q;
               }
-            if (bj >= 0 && bv < S.dist[k]) {
-              S.dist[k] = bv;
-              S.pred[k] = bj;
-              ch = true;
+            const bool ch = from >= 0 && k < W;
+            if (ch) {
+              S.dist[k] = nv;
+              S.pred[k] = S.pj[from][k];
             }
+            const unsigned bal = __ballot_sync(FULL_MASK, ch);
+            if (lane == 0) S.act[warp] = bal;
           }
-          if (!__syncthreads_or(ch)) break;
+          __syncthreads();
+          act = (uint64_t)S.act[0] | ((uint64_t)S.act[1] << 32);
         }
         if (warp == 0) {
           // target: the nearest worker with room (ties: lowest index)
-          const bool r0 = lane < W && S.counts[lane] < capw && S.dist[lane] < FX_REAL;
-          const bool r1 = lane + 32 < W && S.counts[lane + 32] < capw && S.dist[lane + 32] < FX_REAL;
+          const long long d0 = lane < W ? S.dist[lane] : FX_INF;
+          const long long d1 = lane + 32 < W ? S.dist[lane + 32] : FX_INF;
+          const bool r0 = lane < W && S.counts[lane] < capw && d0 < FX_REAL;
+          const bool r1 = lane + 32 < W && S.counts[lane + 32] < capw && d1 < FX_REAL;
           long long v0, v1;
-          const int t0 = warp_argmin(r0 ? S.dist[lane] : 0, r0, &v0);
-          const int t1 = warp_argmin(r1 ? S.dist[lane + 32] : 0, r1, &v1);
+          const int t0 = warp_argmin(d0, r0, &v0);
+          const int t1 = warp_argmin(d1, r1, &v1);
           const int tgt = t0 >= 0 && (t1 < 0 || v0 <= v1) ? t0 : (t1 >= 0 ? t1 + 32 : -1);
-          for (int j = lane; j < W; j += 32) {
-            S.dpos[j] = -1;
-            S.dfill[j] = 0;
+          // the path back from its end (it visits a worker once)
+          int at = tgt, n = 0;
+          while (tgt >= 0 && n < W) {
+            if (lane == 0) S.path[n] = at;
+            const int j = S.pred[at];
+            if (j < 0) break;
+            n++;
+            at = j;
           }
           __syncwarp();
-          if (lane == 0) {
-            // walk the path back from its end: edge j -> kk moves the request
-            // behind wrow[j][kk] from j to kk
-            int kk = tgt, n = 0, o = 0;
-            while (tgt >= 0 && n < W && S.pred[kk] >= 0) {
-              const int j = S.pred[kk];
-              const int r = wrow[j * W + kk];
-              S.mv_j[n] = j;
-              S.mv_k[n] = kk;
-              S.mv_r[n++] = r;
-              asg[r] = kk;
-              kk = j;
-            }
-            if (n > 0) {
-              S.counts[kk]--;
-              S.counts[tgt]++;
-            }
-            for (int t = 0; t < n; t++) {   // (a path visits a worker once)
-              const int j = S.mv_j[t];
-              S.dpos[j] = o;
-              o += S.counts[j];
-            }
-            S.nmv = n;
+          // step t moves the request behind the edge path[t + 1] -> path[t]
+          for (int t = lane; t < n; t += 32) S.mv_r[t] = wrow[S.path[t] * ld + S.path[t + 1]];
+          __syncwarp();
+          // path[t], 0 < t < n, loses request mv_r[t - 1] and gains mv_r[t], which
+          // takes the lost one's place; the source's last request fills its
+          // gap; the target's list grows
+          int sl[2] = {0, 0};
+#pragma unroll
+          for (int u = 0; u < 2; u++) {
+            const int t = lane + 32 * u;
+            if (listed && t >= 1 && t <= n) sl[u] = pos[S.mv_r[t - 1]];
           }
+          __syncwarp();
+#pragma unroll
+          for (int u = 0; u < 2; u++) {
+            const int t = lane + 32 * u;
+            if (n > 0 && t <= n) {
+              const int j = S.path[t];
+              int32_t* rows = S.list[j];
+              if (!listed) {
+                if (t < n) pos[S.mv_r[t]] = j;
+                if (t == 0) S.counts[j]++;
+                if (t == n) S.counts[j]--;
+              } else if (t == n) {
+                const int last = S.counts[j] - 1;
+                const int x = rows[last];
+                rows[sl[u]] = x;
+                if (x != S.mv_r[t - 1]) pos[x] = sl[u];
+                S.counts[j] = last;
+              } else {
+                const int x = S.mv_r[t];
+                const int p = t == 0 ? S.counts[j] : sl[u];
+                rows[p] = x;
+                pos[x] = p;
+                if (t == 0) S.counts[j] = p + 1;
+              }
+            }
+          }
+          if (lane == 0) S.nmv = n;
         }
         __syncthreads();
         const int nmv = S.nmv;
         if (nmv == 0) break;   // (cannot happen: W capw >= m)
-        wide_rescan(S, wmin, wrow, fx, asg, list, m, W, nmv, S.mv_j, S.mv_r, false);
+        // warp t (and t + 32 on a longer path): the weights out of path[t + 1]
+        // whose minimum moved away are listed; the moved request's costs beside
+        // the one at its new worker are loaded for the end of the step
+        long long in_v[2][2];
+#pragma unroll
+        for (int u = 0; u < 2; u++) {
+          const int t = warp + 32 * u;
+          if (t < nmv) {
+            const int to = S.path[t], j = S.path[t + 1], r = S.mv_r[t];
+            const long long ct = fx[(int64_t)r * W + to];
+            if (cur && lane == 0) cur[r] = ct;
+#pragma unroll
+            for (int h = 0; h < 2; h++) {
+              const int q = lane + 32 * h;
+              in_v[u][h] = FX_INF;
+              if (q < W) {
+                if (q != to) in_v[u][h] = fx[(int64_t)r * W + q] - ct;
+                if (q != j && wrow[q * ld + j] == r)
+                  item[atomicAdd(&S.nitems, 1)] = (uint16_t)(j * POA_WMAX_WIDE + q);
+              }
+            }
+          }
+        }
+        __syncthreads();
+        const int ni = S.nitems;
+        // fewer weights than warps: each in `parts` parts
+        const int parts = ni <= NW_WIDE / 8 ? 8 : (ni <= NW_WIDE / 4 ? 4 : (ni <= NW_WIDE / 2 ? 2 : 1));
+        for (int e = warp; e < ni * parts; e += NW_WIDE) {
+          const int x = item[e / parts], j = x / POA_WMAX_WIDE, q = x % POA_WMAX_WIDE;
+          long long v;
+          int r;
+          wide_weight(listed ? S.list[j] : nullptr, pos, listed ? S.counts[j] : m, fx, cur, W, j, q,
+                      e % parts, parts, lane, &v, &r);
+          if (lane == 0) {
+            if (parts == 1) {
+              wmin[q * ld + j] = v;
+              wrow[q * ld + j] = r;
+            } else {   // (one round: ni parts <= 32)
+              S.part_v[e] = v;
+              S.part_r[e] = r;
+            }
+          }
+        }
+        __syncthreads();
+        if (parts > 1) {
+          if (threadIdx.x < ni) {
+            long long v = FX_INF;
+            int r = -1;
+            for (int p = 0; p < parts; p++) {
+              const long long pv = S.part_v[threadIdx.x * parts + p];
+              const int pr2 = S.part_r[threadIdx.x * parts + p];
+              if (pr2 >= 0 && (r < 0 || pv < v || (pv == v && pr2 < r))) {
+                v = pv;
+                r = pr2;
+              }
+            }
+            const int x = item[threadIdx.x], j = x / POA_WMAX_WIDE, q = x % POA_WMAX_WIDE;
+            wmin[q * ld + j] = v;
+            wrow[q * ld + j] = r;
+          }
+          __syncthreads();
+        }
         // requests that moved in lower their new worker's weights (a path
         // enters a worker once: the moves are independent)
-        for (int t = g; t < nmv; t += WIDE_G) {
-          const int to = S.mv_k[t], r = S.mv_r[t];
-          if (k < W && k != to) {
-            const long long v = fx[(int64_t)r * W + k] - fx[(int64_t)r * W + to];
-            const long long o = wmin[to * W + k];
-            if (v < o || (v == o && r < wrow[to * W + k])) {
-              wmin[to * W + k] = v;
-              wrow[to * W + k] = r;
+#pragma unroll
+        for (int u = 0; u < 2; u++) {
+          const int t = warp + 32 * u;
+          if (t < nmv) {
+            const int to = S.path[t], r = S.mv_r[t];
+#pragma unroll
+            for (int h = 0; h < 2; h++) {
+              const int q = lane + 32 * h;
+              const long long v = in_v[u][h];
+              if (q < W && q != to) {
+                const long long o = wmin[q * ld + to];
+                if (v < o || (v == o && r < wrow[q * ld + to])) {
+                  wmin[q * ld + to] = v;
+                  wrow[q * ld + to] = r;
+                }
+              }
             }
           }
         }
         __syncthreads();
       }
       const bool bad = __syncthreads_or(threadIdx.x < W && S.counts[threadIdx.x] > capw);
+      // each row's worker again, then the sum in row order
+      for (int j = warp; listed && j < W; j += NW_WIDE)
+        for (int t = lane; t < S.counts[j]; t += 32) pos[S.list[j][t]] = j;
+      __syncthreads();
       opt = 0.0;
-      for (int64_t r = threadIdx.x; r < m; r += NT_WIDE) opt += (double)fx[r * W + asg[r]] * inv;
+      for (int r = threadIdx.x; r < m; r += NT_WIDE) opt += (double)fx[(int64_t)r * W + pos[r]] * inv;
       opt = warp_sum(opt);
       if (lane == 0) S.red[0][warp] = opt;
       __syncthreads();
-      opt = 0.0;
-      for (int v = 0; v < NT_WIDE / 32; v++) opt += S.red[0][v];
+      opt = warp_sum(S.red[0][lane]);
       if (bad) opt = __longlong_as_double(0x7FF8000000000000ll);
     }
     if (threadIdx.x == 0) {
@@ -977,21 +1194,27 @@ cudaError_t launch_poa(const PoaProblem* d_prob, int nprob, const PoaBuffers& b,
   k_poa_sort<<<nprob, nts, POA_SORT_TAB * sizeof(uint32_t), st>>>(d_prob, b, mc.W);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  void (*kern)(const PoaProblem*, PoaBuffers, ModelConsts) =
-      mc.W > POA_WMAX ? k_poa_solve_wide
-      : mc.W == 3     ? k_poa_solve<3>
-                      : (mc.W == 6 ? k_poa_solve<6> : k_poa_solve<POA_WMAX>);
+  // a CTA per window while they all fit on the GPU at about two to an SM
   const bool wide = mc.W > POA_WMAX;
+  const bool few = b.wnext ? b.nslots <= 2 * (int64_t)sms : nprob <= sms;
+  void (*kern)(const PoaProblem*, PoaBuffers, ModelConsts) = nullptr;
+  if (wide)
+    kern = k_poa_solve_wide;
+  else if (few)
+    kern = mc.W == 3 ? k_poa_solve<3, NW_SOLVE>
+                     : (mc.W == 6 ? k_poa_solve<6, NW_SOLVE> : k_poa_solve<POA_WMAX, NW_SOLVE>);
+  else
+    kern = mc.W == 3 ? k_poa_solve<3, 1>
+                     : (mc.W == 6 ? k_poa_solve<6, 1> : k_poa_solve<POA_WMAX, 1>);
   const size_t smem = wide ? poa_wide_smem(mc.W) : 0;
   if (wide && (e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                         (int)smem)) != cudaSuccess)
     return e;
+  const int nt = wide ? NT_WIDE : (few ? 32 * NW_SOLVE : NT_SOLVE);
+  const int wpc = wide || few ? 1 : NT_SOLVE / 32;   // windows of a CTA
   if (b.wnext) {
-    // one wave of CTAs that take the windows from the counter; few windows go
-    // one to a CTA, so that each has an SM's integer and FP64 pipes to itself
+    // one wave of CTAs that take the windows from the counter
     if ((e = cudaMemsetAsync(b.wnext, 0, sizeof(unsigned long long), st)) != cudaSuccess) return e;
-    const int nt = wide ? NT_WIDE : (b.nslots <= 4 * (int64_t)sms ? 32 : NT_SOLVE);
-    const int wpc = wide ? 1 : nt / 32;
     int per_sm = 0;
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, nt, smem)) != cudaSuccess)
       return e;
@@ -1001,8 +1224,8 @@ cudaError_t launch_poa(const PoaProblem* d_prob, int nprob, const PoaBuffers& b,
     kern<<<(unsigned)(gr > 0 ? gr : 1), nt, smem, st>>>(d_prob, b, mc);
   } else {
     // each problem's windows on its own CTAs, enough of them to fill the GPU
-    int split = (4 * sms + nprob - 1) / nprob;
-    kern<<<dim3(nprob, split), wide ? NT_WIDE : 32, smem, st>>>(d_prob, b, mc);
+    const int split = (2 * sms + nprob - 1) / nprob;
+    kern<<<dim3(nprob, split), nt, smem, st>>>(d_prob, b, mc);
   }
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   k_poa_total<<<(nprob + NT_POA / 32 - 1) / (NT_POA / 32), NT_POA, 0, st>>>(nprob, b, d_prob);

@@ -159,9 +159,10 @@ struct PoaProblem {
 
 struct PoaBuffers {
   rs_records rec;
-  double* cost;             // [rows][W] by sorted row (a window past a capacity: fixed point)
+  double* cost;             // [rows][W] per window ([W][its rows] at W <= POA_WMAX; past a
+                            // capacity: fixed point)
   int32_t* order;           // [rows] row (relative) sorted by window, stable
-  int32_t* asg;             // [rows]
+  int32_t* asg;             // [rows] assignment of windows too large for shared memory
   int32_t* wkey;            // [rows] window of each row (-1 skipped); past the sort, scratch
   int64_t* wstart;          // [win slots + problems]
   int64_t* wfill;           // [win slots]

@@ -95,12 +95,13 @@ def test_windows_far_apart_and_empty_records():
     assert nw == 0 and gt == 0.0
 
 
-def _random_records(rng, n, W, span, tied):
+def _random_records(rng, n, W, span, tied, cap):
     """Records whose cheapest workers exceed their capacity: worker 0 is cheap for every row;
     `tied` makes many costs equal (few load levels, no prefixes)."""
     nbt = rng.integers(1, 60, n).astype(np.int32)
     nf = rng.integers(20, 23 if tied else 60, (n, W)).astype(np.uint16)
     nf[:, 0] = rng.integers(1, 3 if tied else 20, n)
+    nf = np.minimum(nf, cap - 1)
     pre = np.zeros((n, W), np.uint16) if tied else \
         (rng.integers(0, 2, (n, W)) * rng.integers(0, 60, (n, W)) % (nbt[:, None] + 1)).astype(np.uint16)
     comp = rng.uniform(0.0, span, n)
@@ -112,15 +113,19 @@ def _random_records(rng, n, W, span, tied):
 
 
 # windows up to the sort's table (11 264) and one past it; rows that end inside a warp's 32; solvers
-# for W = 3, 6, up to 16 and wider, at capacities that bind (rows per window > 64 on worker 0)
-@pytest.mark.parametrize("W,n,windows,tied", [
-    (2, 1, 1, False), (3, 331, 2, True), (6, 1537, 4, False), (6, 1000, 11264, False),
-    (6, 1000, 11265, False), (16, 900, 3, True), (17, 801, 2, False), (33, 700, 2, True),
-    (64, 1400, 2, False)])
-def test_sort_and_solvers_at_their_edges(W, n, windows, tied):
-    ctx = rs.Context(W=W, K=64)
-    o = _random_records(np.random.default_rng(W * n + windows), n, W, 5.0 * windows, tied)
-    num, opt, cnt, tot = O.poa(oracle_cfg(ctx), o)
+# for W = 3, 6, up to 16 and wider, at capacities that bind (rows per window > C_j on worker 0); costs
+# and rows of a window inside and past what the solvers keep in shared memory (W <= 16: 4096 costs,
+# 1024 rows; wider: 4096 rows), one warp per window (400 windows) and a CTA per window; W > 16 with a
+# C_j whose lists fit nowhere
+@pytest.mark.parametrize("W,n,windows,tied,cap", [
+    (2, 1, 1, False, 64), (3, 331, 2, True, 64), (6, 1537, 4, False, 64), (6, 1000, 11264, False, 64),
+    (6, 1000, 11265, False, 64), (6, 4801, 400, False, 3), (6, 900, 1, True, 64),
+    (3, 1500, 1, False, 64), (16, 900, 3, True, 64), (17, 801, 2, False, 64), (33, 700, 2, True, 64),
+    (64, 1400, 2, False, 64), (17, 4500, 1, False, 64), (20, 700, 1, False, 300)])
+def test_sort_and_solvers_at_their_edges(W, n, windows, tied, cap):
+    ctx = rs.Context(W=W, K=64, cap=cap)
+    o = _random_records(np.random.default_rng(W * n + windows), n, W, 5.0 * windows, tied, cap)
+    num, opt, cnt, tot = O.poa(oracle_cfg(ctx, cap=cap), o)
     assert num.size == windows
     rec, keep = _to_device(o, n, W)
     gn, go, gc, gt, nw = rs.poa_estimate(ctx.h, rec, n, windows)
