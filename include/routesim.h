@@ -315,7 +315,10 @@ typedef struct {
   double* kv_cost;        /* [rows] Eq. kv-cost of the request on its worker (tiered; optional) */
 } rs_records;
 
-enum { RS_SIM_NO_POA = 1 };   /* flags of simulate_replicas */
+/* Flags of simulate_replicas.  RS_SIM_TABLES: the workers' caches as hash
+ * tables even where block ids apply (same results; the form that a call whose
+ * ids would take more memory than the tables uses). */
+enum { RS_SIM_NO_POA = 1, RS_SIM_TABLES = 2 };
 
 /* Runs n_replicas independent replicas (one per CTA) and, unless
  * RS_SIM_NO_POA, the Eq. (12) estimate per replica.  traces: host array of

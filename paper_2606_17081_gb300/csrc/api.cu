@@ -27,7 +27,7 @@ struct DevBuf {
 struct rs_ctx {
   rs_config cfg;
   cudaStream_t st = nullptr;
-  int device = 0;
+  int device = 0, sms = 0;
   std::string err;
   TableGeom g;    // the live routers' caches (cache_blocks)
   TableGeom gs;   // the simulated workers' caches (all tiers)
@@ -38,6 +38,9 @@ struct rs_ctx {
   // simulation scratch (grow-only)
   DevBuf keys, stamp, log, tmp, pend, meta_out, res, desc, hashes, stats, hjobs, dstat, wco, slots;
   DevBuf fexp, tmpe;   // frequency eviction state and its rebuild scratch
+  // simulation on block ids: the sets of the numbering step, then ids, requests'
+  // last block seen before, counts, the replicas' stamps and update scratch
+  DevBuf i_jobs, i_keys, i_first, i_num, i_ids, i_nz, i_count, i_stamps, i_scratch;
   DevBuf dupf;         // per request: a chained hash repeats within the prompt
   DevBuf djobs;        // every trace in use, for the block-count and flag kernels
   DevBuf h_hashes;     // staged block hashes of host traces given by their hashes
@@ -51,6 +54,16 @@ struct rs_ctx {
   size_t pinned_n = 0;
   // last simulate_replicas call
   int32_t last_nsim = 0;
+  // where its caches are, per replica, when it ran on block ids (else empty)
+  struct IdCache {
+    const uint64_t* hashes;   // of its trace
+    const uint32_t* ids;
+    int64_t blocks;           // positions of the trace
+    const uint32_t* stamps;   // [W][nre]
+    int64_t nre;
+  };
+  std::vector<IdCache> last_ids;
+  uint32_t last_ids_rmask = 0;
   cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};
   rs_timing timing;
 };
@@ -255,6 +268,7 @@ rs_status route_init(rs_ctx** out, const rs_config* cfg, int32_t n_instances, vo
   ctx->g = table_geom(cfg->cache_blocks);
   ctx->gs = cfg->tiered ? table_geom(cfg->cache_blocks + cfg->tier_k2 + cfg->tier_k3) : ctx->g;
   ctx->mc = make_consts(*cfg);
+  cudaDeviceGetAttribute(&ctx->sms, cudaDevAttrMultiProcessorCount, ctx->device);
   memset(&ctx->timing, 0, sizeof ctx->timing);
   for (auto& ev : ctx->ev) {
     e = cudaEventCreate(&ev);
@@ -311,7 +325,9 @@ void route_destroy(rs_ctx* ctx) {
                    &ctx->h_tokens, &ctx->h_offsets,
                    &ctx->h_release, &ctx->h_outlen, &ctx->k_rows, &ctx->k_load, &ctx->k_sweep,
                    &ctx->k_stat, &ctx->k_d1, &ctx->k_d2, &ctx->k_kload, &ctx->k_kidx,
-                   &ctx->fexp, &ctx->tmpe, &ctx->djobs, &ctx->h_hashes};
+                   &ctx->fexp, &ctx->tmpe, &ctx->djobs, &ctx->h_hashes, &ctx->i_jobs, &ctx->i_keys,
+                   &ctx->i_first, &ctx->i_num, &ctx->i_ids, &ctx->i_nz, &ctx->i_count,
+                   &ctx->i_stamps, &ctx->i_scratch};
   for (DevBuf* b : all) release(*b);
   if (ctx->pinned) cudaFreeHost(ctx->pinned);
   for (auto& ev : ctx->ev)
@@ -562,6 +578,13 @@ static rs_status records_effective(rs_ctx* ctx, const rs_records* user, int64_t 
 // Eq. (12) for every problem in probs (rec_base, n, scratch_base set; the
 // window slots are sized here): the last window of each problem is found on
 // the device first, so that every window its records span gets a slot.
+// Block ids of one trace of a call.
+struct TraceIds {
+  const uint32_t* ids = nullptr;
+  const int32_t* nz = nullptr;
+  int64_t nre = 8;   // numbered blocks, rounded up to whole sectors
+};
+
 static rs_status run_poa(rs_ctx* ctx, const rs_records& rec, std::vector<PoaProblem>& probs,
                          int64_t rows, rs_replica_result* res_dev) {
   const int W = ctx->cfg.W;
@@ -631,6 +654,96 @@ static rs_status run_poa(rs_ctx* ctx, const rs_records& rec, std::vector<PoaProb
   b.wnext = P<unsigned long long>(ctx->p_wnext);
   b.nslots = win_slots;
   CK(launch_poa(P<PoaProblem>(ctx->p_prob), np, b, ctx->mc, ctx->st), "poa launch");
+  return RS_OK;
+}
+
+// Block ids of every trace in use (jobs `all`, request bases rbase): tids[t]
+// and the words of all replicas' stamps.  Reads the counts (synchronises).
+static rs_status trace_ids(rs_ctx* ctx, const rs_trace* traces, const std::vector<char>& used,
+                           const std::vector<int64_t>& tot, const std::vector<HashJob>& all,
+                           int64_t req_total, const rs_replica_params* params, int32_t n_replicas,
+                           std::vector<TraceIds>& tids, size_t* stamp_words, int64_t* launches) {
+  rs_status r;
+  std::vector<int> tr;   // trace of each job
+  for (size_t t = 0; t < used.size(); t++)
+    if (used[t] && traces[t].n_req > 0) tr.push_back((int)t);
+  const size_t nj = tr.size();
+  size_t pos = 0;
+  std::vector<IdJob> jobs(nj);
+  for (size_t k = 0; k < nj; k++) {
+    const int64_t blocks = tot[tr[k]] / 16 + 1;
+    uint64_t cap = 32;
+    while (cap < 2 * (uint64_t)blocks) cap <<= 1;
+    jobs[k].hashes = all[k].out;
+    jobs[k].offsets = all[k].offsets;
+    jobs[k].n_req = all[k].n_req;
+    jobs[k].tmask = (uint32_t)(cap - 1);
+    pos += (size_t)blocks;
+  }
+  // launches: up to IDS_MAX_JOBS traces whose sets take at most 8 GB together
+  std::vector<size_t> start{0};
+  size_t slots = 0, most = 0;
+  for (size_t k = 0; k < nj; k++) {
+    const size_t cap = (size_t)jobs[k].tmask + 1;
+    if (k > start.back() && (k - start.back() == IDS_MAX_JOBS || (slots + cap) * 16 > (size_t)8 << 30)) {
+      start.push_back(k);
+      slots = 0;
+    }
+    slots += cap;
+    most = std::max(most, slots);
+  }
+  start.push_back(nj);
+  if ((r = ensure(ctx, ctx->i_jobs, sizeof(IdJob) * std::max<size_t>(nj, 1), "id jobs")) ||
+      (r = ensure(ctx, ctx->i_keys, most * 8, "block sets")) ||
+      (r = ensure(ctx, ctx->i_first, most * 4, "block sets")) ||
+      (r = ensure(ctx, ctx->i_num, most * 4, "block sets")) ||
+      (r = ensure(ctx, ctx->i_ids, pos * 4, "block ids")) ||
+      (r = ensure(ctx, ctx->i_nz, (size_t)req_total * 4, "block ids")) ||
+      (r = ensure(ctx, ctx->i_count, nj * 4, "block counts")) || (r = ensure_pinned(ctx, nj + 1)))
+    return r;
+  pos = 0;
+  for (size_t g = 0; g + 1 < start.size(); g++) {
+    slots = 0;
+    for (size_t k = start[g]; k < start[g + 1]; k++) {
+      IdJob& J = jobs[k];
+      J.req_base = all[k].req_base - all[start[g]].req_base;
+      J.keys = P<unsigned long long>(ctx->i_keys) + slots;
+      J.first = P<uint32_t>(ctx->i_first) + slots;
+      J.num = P<uint32_t>(ctx->i_num) + slots;
+      J.ids = P<uint32_t>(ctx->i_ids) + pos;
+      J.nz = P<int32_t>(ctx->i_nz) + all[k].req_base;
+      J.count = P<uint32_t>(ctx->i_count) + k;
+      tids[tr[k]].ids = J.ids;
+      tids[tr[k]].nz = J.nz;
+      slots += (size_t)J.tmask + 1;
+      pos += (size_t)(tot[tr[k]] / 16 + 1);
+    }
+  }
+  if (nj > 0) {
+    CK(cudaMemcpyAsync(ctx->i_jobs.p, jobs.data(), sizeof(IdJob) * nj, cudaMemcpyHostToDevice, ctx->st),
+       "copy id jobs");
+    CK(cudaMemsetAsync(ctx->i_count.p, 0, nj * 4, ctx->st), "memset");
+    CK(cudaMemsetAsync(ctx->i_ids.p, 0, pos * 4, ctx->st), "memset");   // (places between prompts)
+  }
+  for (size_t g = 0; g + 1 < start.size(); g++) {
+    const size_t a = start[g], b = start[g + 1];
+    if (a == b) continue;
+    slots = 0;
+    for (size_t k = a; k < b; k++) slots += (size_t)jobs[k].tmask + 1;
+    CK(cudaMemsetAsync(ctx->i_keys.p, 0, slots * 8, ctx->st), "memset");
+    CK(cudaMemsetAsync(ctx->i_first.p, 0xFF, slots * 4, ctx->st), "memset");
+    const int64_t total = jobs[b - 1].req_base + jobs[b - 1].n_req;
+    CK(launch_block_ids(P<IdJob>(ctx->i_jobs) + a, (int)(b - a), total, ctx->st), "block id launch");
+    *launches += 4;
+  }
+  uint32_t* cnt = reinterpret_cast<uint32_t*>(ctx->pinned);
+  if (nj > 0)
+    CK(cudaMemcpyAsync(cnt, ctx->i_count.p, nj * 4, cudaMemcpyDeviceToHost, ctx->st), "read counts");
+  CK(cudaStreamSynchronize(ctx->st), "sync");
+  for (size_t k = 0; k < nj; k++) tids[tr[k]].nre = ((int64_t)cnt[k] + 8) & ~(int64_t)7;
+  *stamp_words = 0;
+  for (int32_t k = 0; k < n_replicas; k++)
+    *stamp_words += (size_t)ctx->cfg.W * (size_t)tids[params[k].trace].nre;
   return RS_OK;
 }
 
@@ -757,72 +870,33 @@ rs_status simulate_replicas(rs_ctx* ctx, const rs_trace* traces, int32_t n_trace
       no += n;
     }
   } else {
-    if ((r = ensure_pinned(ctx, (size_t)n_traces + 1)) != RS_OK) return r;
     for (int t = 0; t < n_traces; t++) {
       dtok[t] = traces[t].tokens;
       dhash[t] = prehashed(t) ? traces[t].hashes : nullptr;
       doff[t] = traces[t].offsets;
       drel[t] = traces[t].release;
       dol[t] = traces[t].out_len;
-      if (used[t] && traces[t].n_req > 0)
-        CK(cudaMemcpyAsync(ctx->pinned + t, traces[t].offsets + traces[t].n_req, 8,
-                           cudaMemcpyDeviceToHost, ctx->st), "read offsets");
     }
-    CK(cudaStreamSynchronize(ctx->st), "sync");
-    for (int t = 0; t < n_traces; t++)
-      if (used[t] && traces[t].n_req > 0) tot[t] = ctx->pinned[t];
   }
-  size_t hash_total = 0;
-  for (int t = 0; t < n_traces; t++) {
-    if (tot[t] < 0) return fail(ctx, RS_ERR_INVALID, "trace %d: offsets[n_req] < 0", t);
-    hoff[t] = (int64_t)hash_total;
-    if (used[t] && !dhash[t]) hash_total += (size_t)(tot[t] / 16 + 1);
-  }
-  if ((r = ensure(ctx, ctx->hashes, hash_total * 8, "block hashes")) ||
-      (r = ensure(ctx, ctx->stats, (size_t)n_traces * 8, "trace stats")) ||
-      (r = ensure_pinned(ctx, (size_t)n_traces + 1)))
-    return r;
-  // ---- K1: block hashes of every trace in use that comes as tokens.  The
-  // hash jobs number their requests among themselves; the per-request flags
-  // number the requests of every trace in use (rbase).
+  // the longest prompt's full blocks over every trace in use, and (device
+  // traces) the traces' lengths
   int64_t launches = 0, hashed_tokens = 0;
   std::vector<HashJob> jobs, all;
   int64_t req_total = 0, hreq = 0;
   for (int t = 0; t < n_traces; t++) {
     if (!used[t] || traces[t].n_req == 0) continue;
     rbase[t] = req_total;
-    uint64_t* hp = dhash[t] ? const_cast<uint64_t*>(dhash[t]) : P<uint64_t>(ctx->hashes) + hoff[t];
-    all.push_back(HashJob{dtok[t], doff[t], hp, traces[t].n_req, req_total});
-    if (!dhash[t]) {
-      jobs.push_back(HashJob{dtok[t], doff[t], hp, traces[t].n_req, hreq});
-      hreq += traces[t].n_req;
-      hashed_tokens += tot[t];
-    }
+    all.push_back(HashJob{dtok[t], doff[t], nullptr, traces[t].n_req, req_total});
     req_total += traces[t].n_req;
   }
-  if ((r = ensure(ctx, ctx->hjobs, sizeof(HashJob) * std::max<size_t>(jobs.size(), 1), "hash jobs")) ||
-      (r = ensure(ctx, ctx->djobs, sizeof(HashJob) * std::max<size_t>(all.size(), 1), "trace jobs")))
+  if ((r = ensure(ctx, ctx->djobs, sizeof(HashJob) * std::max<size_t>(all.size(), 1), "trace jobs")) ||
+      (r = ensure(ctx, ctx->stats, (size_t)n_traces * 8, "trace stats")) ||
+      (r = ensure_pinned(ctx, (size_t)n_traces + 1)))
     return r;
-  std::vector<HashJob> hj = group_jobs(jobs);
-  if (!jobs.empty())
-    CK(cudaMemcpyAsync(ctx->hjobs.p, hj.data(), sizeof(HashJob) * hj.size(), cudaMemcpyHostToDevice,
-                       ctx->st), "copy hash jobs");
   std::vector<HashJob> aj = group_jobs(all);
   CK(cudaMemcpyAsync(ctx->djobs.p, aj.data(), sizeof(HashJob) * aj.size(), cudaMemcpyHostToDevice,
                      ctx->st), "copy trace jobs");
   CK(cudaMemsetAsync(ctx->stats.p, 0, (size_t)n_traces * 8, ctx->st), "memset");
-  // the events time the hash launches alone
-  CK(cudaEventRecord(ctx->ev[0], ctx->st), "event");
-  for (size_t g0 = 0; g0 < jobs.size(); g0 += HASH_MAX_JOBS) {
-    const size_t g1 = std::min(jobs.size(), g0 + HASH_MAX_JOBS);
-    const int64_t total = jobs[g1 - 1].req_base + jobs[g1 - 1].n_req - jobs[g0].req_base;
-    CK(launch_block_hash(P<HashJob>(ctx->hjobs) + g0, (int)(g1 - g0), total, ctx->cfg.hash_seed,
-                         nullptr, ctx->st),
-       "block hash launch");
-    launches++;
-  }
-  CK(cudaEventRecord(ctx->ev[1], ctx->st), "event");
-  // the longest prompt's full blocks, over every trace in use
   for (size_t g0 = 0; g0 < all.size(); g0 += HASH_MAX_JOBS) {
     const size_t g1 = std::min(all.size(), g0 + HASH_MAX_JOBS);
     const int64_t total = all[g1 - 1].req_base + all[g1 - 1].n_req - all[g0].req_base;
@@ -831,9 +905,20 @@ rs_status simulate_replicas(rs_ctx* ctx, const rs_trace* traces, int32_t n_trace
        "block count launch");
     launches++;
   }
-  CK(cudaMemcpyAsync(ctx->pinned, ctx->stats.p, 8, cudaMemcpyDeviceToHost, ctx->st), "read stats");
+  if (!host)
+    for (int t = 0; t < n_traces; t++)
+      if (used[t] && traces[t].n_req > 0)
+        CK(cudaMemcpyAsync(ctx->pinned + t, traces[t].offsets + traces[t].n_req, 8,
+                           cudaMemcpyDeviceToHost, ctx->st), "read offsets");
+  CK(cudaMemcpyAsync(ctx->pinned + n_traces, ctx->stats.p, 8, cudaMemcpyDeviceToHost, ctx->st),
+     "read stats");
   CK(cudaStreamSynchronize(ctx->st), "sync");
-  int64_t nbmax = std::max<int64_t>(1, ctx->pinned[0]);
+  if (!host)
+    for (int t = 0; t < n_traces; t++)
+      if (used[t] && traces[t].n_req > 0) tot[t] = ctx->pinned[t];
+  for (int t = 0; t < n_traces; t++)
+    if (tot[t] < 0) return fail(ctx, RS_ERR_INVALID, "trace %d: offsets[n_req] < 0", t);
+  int64_t nbmax = std::max<int64_t>(1, ctx->pinned[n_traces]);
   if (nbmax > (int64_t)g.K) nbmax = g.K;   // longer prompts stop their replica with RS_ERR_CAPACITY
   int maxsmem = 0;
   cudaDeviceGetAttribute(&maxsmem, cudaDevAttrMaxSharedMemoryPerBlockOptin, ctx->device);
@@ -854,13 +939,95 @@ rs_status simulate_replicas(rs_ctx* ctx, const rs_trace* traces, int32_t n_trace
     return fail(ctx, RS_ERR_CAPACITY,
                 "prompt of %lld blocks needs %zu bytes of shared memory per replica",
                 (long long)nbmax, smem);
-  // ---- scratch
+  // block ids instead of hash tables: exact LRU replicas on traces whose
+  // positions fit 31 bits (run_ids falls back to the tables when the ids'
+  // memory would exceed the tables')
   const size_t nsim = n_replicas;
+  bool use_ids = !tiered && !any_freq && !(flags & RS_SIM_TABLES);
+  for (int t = 0; t < n_traces; t++)
+    if (used[t] && tot[t] / 16 + 1 > (int64_t)1 << 30) use_ids = false;
+  // the kernel on block ids: its own arrays (smaller except for the window of
+  // the log that it keeps per worker)
+  bool ids_slots_global = false;
+  {
+    const int ntu = 32 * sim_ids_update_warps(n_replicas, ctx->sms);
+    if (sim_ids_smem_bytes(W, (int)nbmax, cmax, ctx->cfg.cap, ntu, false) > smem_room) {
+      ids_slots_global = true;
+      if (sim_ids_smem_bytes(W, (int)nbmax, cmax, ctx->cfg.cap, ntu, true) > smem_room) use_ids = false;
+    }
+  }
+  size_t hash_total = 0;
+  for (int t = 0; t < n_traces; t++) {
+    hoff[t] = (int64_t)hash_total;
+    // (a device trace's own hashes are copied when the caches will refer to them)
+    if (used[t] && (!dhash[t] || (use_ids && !host))) hash_total += (size_t)(tot[t] / 16 + 1);
+  }
+  if ((r = ensure(ctx, ctx->hashes, hash_total * 8, "block hashes")) != RS_OK) return r;
+  ctx->last_nsim = 0;   // the last call's caches are overwritten from here on
+  ctx->last_ids.clear();
+  // ---- K1: block hashes of every trace in use that comes as tokens.  The
+  // hash jobs number their requests among themselves; the per-request flags
+  // number the requests of every trace in use (rbase).
+  all.clear();
+  for (int t = 0; t < n_traces; t++) {
+    if (!used[t] || traces[t].n_req == 0) continue;
+    uint64_t* hp = P<uint64_t>(ctx->hashes) + hoff[t];
+    if (!dhash[t]) {
+      jobs.push_back(HashJob{dtok[t], doff[t], hp, traces[t].n_req, hreq});
+      hreq += traces[t].n_req;
+      hashed_tokens += tot[t];
+    } else if (use_ids && !host) {
+      CK(cudaMemcpyAsync(hp, dhash[t], (size_t)(tot[t] / 16) * 8, cudaMemcpyDeviceToDevice, ctx->st),
+         "copy hashes");
+      dhash[t] = hp;
+    } else {
+      hp = const_cast<uint64_t*>(dhash[t]);
+    }
+    all.push_back(HashJob{dtok[t], doff[t], hp, traces[t].n_req, rbase[t]});
+  }
+  if ((r = ensure(ctx, ctx->hjobs, sizeof(HashJob) * std::max<size_t>(jobs.size(), 1), "hash jobs")) != RS_OK)
+    return r;
+  std::vector<HashJob> hj = group_jobs(jobs);
+  if (!jobs.empty())
+    CK(cudaMemcpyAsync(ctx->hjobs.p, hj.data(), sizeof(HashJob) * hj.size(), cudaMemcpyHostToDevice,
+                       ctx->st), "copy hash jobs");
+  aj = group_jobs(all);
+  CK(cudaMemcpyAsync(ctx->djobs.p, aj.data(), sizeof(HashJob) * aj.size(), cudaMemcpyHostToDevice,
+                     ctx->st), "copy trace jobs");
+  // the events time the hash launches alone
+  CK(cudaEventRecord(ctx->ev[0], ctx->st), "event");
+  for (size_t g0 = 0; g0 < jobs.size(); g0 += HASH_MAX_JOBS) {
+    const size_t g1 = std::min(jobs.size(), g0 + HASH_MAX_JOBS);
+    const int64_t total = jobs[g1 - 1].req_base + jobs[g1 - 1].n_req - jobs[g0].req_base;
+    CK(launch_block_hash(P<HashJob>(ctx->hjobs) + g0, (int)(g1 - g0), total, ctx->cfg.hash_seed,
+                         nullptr, ctx->st),
+       "block hash launch");
+    launches++;
+  }
+  CK(cudaEventRecord(ctx->ev[1], ctx->st), "event");
+  std::vector<TraceIds> tids(n_traces);
+  if (use_ids) {
+    size_t stamp_words = 0;
+    r = trace_ids(ctx, traces, used, tot, all, req_total, params, n_replicas, tids, &stamp_words,
+                  &launches);
+    if (r == RS_OK && stamp_words * 4 > std::max<size_t>(nsim * W * g.slots * 12, (size_t)4 << 30))
+      r = RS_ERR_OOM;
+    if (r == RS_OK) r = ensure(ctx, ctx->i_stamps, stamp_words * 4, "block stamps");
+    if (r == RS_OK)
+      r = ensure(ctx, ctx->i_scratch, nsim * sim_ids_scratch_bytes((int)nbmax), "update scratch");
+    if (r == RS_ERR_OOM) {   // no room for the ids: the tables
+      use_ids = false;
+      ctx->err.clear();
+    } else if (r != RS_OK) {
+      return r;
+    }
+  }
+  // ---- scratch
   const size_t nsl = nsim * W * g.slots;
-  if ((r = ensure(ctx, ctx->keys, nsl * 8, "cache keys")) ||
-      (r = ensure(ctx, ctx->stamp, nsl * 4, "cache stamps")) ||
+  if ((!use_ids && ((r = ensure(ctx, ctx->keys, nsl * 8, "cache keys")) ||
+                    (r = ensure(ctx, ctx->stamp, nsl * 4, "cache stamps")) ||
+                    (r = ensure(ctx, ctx->tmp, nsim * g.K * 8, "rebuild scratch")))) ||
       (r = ensure(ctx, ctx->log, nsim * W * g.R * 4, "cache logs")) ||
-      (r = ensure(ctx, ctx->tmp, nsim * g.K * 8, "rebuild scratch")) ||
       (r = ensure(ctx, ctx->pend, nsim * 5 * (size_t)std::max<int64_t>(pend_cap, 1) * 8, "controller windows")) ||
       (r = ensure(ctx, ctx->meta_out, nsim * W * sizeof(CacheMeta), "cache meta")) ||
       (r = ensure(ctx, ctx->res, nsim * sizeof(rs_replica_result), "results")) ||
@@ -869,14 +1036,16 @@ rs_status simulate_replicas(rs_ctx* ctx, const rs_trace* traces, int32_t n_trace
       (r = ensure(ctx, ctx->dstat, (size_t)std::max<int64_t>(rows, 1) * 6 * sizeof(float),
                   "decision statistics")))
     return r;
+  if (use_ids) slots_global = ids_slots_global;
   if (slots_global &&
-      (r = ensure(ctx, ctx->slots, nsim * sim_slot_bytes(cmax), "request slots")) != RS_OK)
+      (r = ensure(ctx, ctx->slots, nsim * (use_ids ? sim_ids_slot_bytes(cmax) : sim_slot_bytes(cmax)),
+                  "request slots")) != RS_OK)
     return r;
   if (any_freq && ((r = ensure(ctx, ctx->fexp, nsl * 4, "frequency state")) ||
                    (r = ensure(ctx, ctx->tmpe, nsim * g.K * 4, "frequency rebuild scratch"))))
     return r;
   // w_c * (m / nbt) table for prompts up to nbmax blocks (none beyond 2048)
-  const bool use_tab = nbmax <= 2048;
+  const bool use_tab = nbmax <= 2048 && !use_ids;
   if (use_tab &&
       (r = ensure(ctx, ctx->wco, (size_t)(nbmax + 1) * (nbmax + 2) * sizeof(double), "w_c o table")))
     return r;
@@ -886,13 +1055,23 @@ rs_status simulate_replicas(rs_ctx* ctx, const rs_trace* traces, int32_t n_trace
   std::vector<SimDesc> desc(nsim);
   std::vector<PoaProblem> probs(nsim);
   int64_t rb = 0;
+  size_t sw = 0;
+  if (use_ids) ctx->last_ids.resize(nsim);
   for (size_t k = 0; k < nsim; k++) {
     const rs_replica_params& p = params[k];
     SimDesc& d = desc[k];
+    const TraceIds& ti = tids[p.trace];
+    d.ids = ti.ids;
+    d.nz = ti.nz;
+    d.nre = ti.nre;
+    d.stamps = use_ids ? P<uint32_t>(ctx->i_stamps) + sw : nullptr;
+    sw += (size_t)W * ti.nre;
     d.offsets = doff[p.trace];
     d.release = drel[p.trace];
     d.out_len = dol[p.trace];
     d.hashes = dhash[p.trace] ? dhash[p.trace] : P<uint64_t>(ctx->hashes) + hoff[p.trace];
+    if (use_ids)
+      ctx->last_ids[k] = rs_ctx::IdCache{d.hashes, ti.ids, tot[p.trace] / 16 + 1, d.stamps, ti.nre};
     d.dupflag = P<uint8_t>(ctx->dupf) + rbase[p.trace];
     d.n_req = p.n_req;
     d.rec_base = rb;
@@ -932,6 +1111,7 @@ rs_status simulate_replicas(rs_ctx* ctx, const rs_trace* traces, int32_t n_trace
   sb.dstat = P<float>(ctx->dstat);
   sb.wco_tab = use_tab ? P<double>(ctx->wco) : nullptr;
   sb.wco_dim = (int)nbmax + 2;
+  sb.scratch = use_ids ? P<unsigned char>(ctx->i_scratch) : nullptr;
   sb.slotmem = slots_global ? P<unsigned char>(ctx->slots) : nullptr;
   SimLaunch L;
   L.nsim = (int)nsim;
@@ -942,6 +1122,16 @@ rs_status simulate_replicas(rs_ctx* ctx, const rs_trace* traces, int32_t n_trace
   L.cmax = cmax;
   L.slots_global = slots_global ? 1 : 0;
   L.g = g;
+  // The log ring of the simulation on block ids: 4 K entries as the tables',
+  // but 2 K for a small cache, where a compaction in place is one pass of a
+  // few log entries per thread and the shorter ring stays in L1.
+  {
+    uint64_t R = g.R;
+    if (g.K < 512)
+      for (R = 1; R < 2 * (uint64_t)g.K; R <<= 1) {}
+    L.ids_rmask = (uint32_t)(R - 1);
+    ctx->last_ids_rmask = L.ids_rmask;
+  }
   L.mc = ctx->mc;
   L.mc.write_cost = want_cost ? 1 : 0;
   if (use_tab) {
@@ -958,7 +1148,8 @@ rs_status simulate_replicas(rs_ctx* ctx, const rs_trace* traces, int32_t n_trace
        "duplicate flags launch");
     launches++;
   }
-  CK(launch_sim(P<SimDesc>(ctx->desc), sb, L, ctx->st), "simulation launch");
+  CK((use_ids ? launch_sim_ids : launch_sim)(P<SimDesc>(ctx->desc), sb, L, ctx->st),
+     "simulation launch");
   CK(launch_decision_stats(P<SimDesc>(ctx->desc), sb, L, ctx->st), "statistics launch");
   launches += 2;
   CK(cudaEventRecord(ctx->ev[2], ctx->st), "event");
@@ -1085,6 +1276,51 @@ rs_status sweep_knee(rs_ctx* ctx, const rs_records* records, const int64_t* row_
   return RS_OK;
 }
 
+// The cache of a replica that ran on block ids: its live log entries' hashes.
+static rs_status dump_ids(rs_ctx* ctx, int32_t index, int32_t worker, uint64_t* keys_host,
+                          int64_t capacity, int64_t* size) {
+  const rs_ctx::IdCache& ic = ctx->last_ids[index];
+  const size_t wi = (size_t)index * ctx->cfg.W + worker;
+  std::vector<uint32_t> stamps(ic.nre), log((size_t)ctx->last_ids_rmask + 1);
+  std::vector<uint32_t> ids(ic.blocks);
+  std::vector<uint64_t> hashes(ic.blocks);
+  CacheMeta m;
+  CK(cudaMemcpyAsync(stamps.data(), ic.stamps + (size_t)worker * ic.nre, (size_t)ic.nre * 4,
+                     cudaMemcpyDeviceToHost, ctx->st), "read");
+  CK(cudaMemcpyAsync(log.data(), P<uint32_t>(ctx->log) + wi * ctx->gs.R, log.size() * 4,
+                     cudaMemcpyDeviceToHost, ctx->st), "read");
+  CK(cudaMemcpyAsync(&m, P<CacheMeta>(ctx->meta_out) + wi, sizeof m, cudaMemcpyDeviceToHost, ctx->st),
+     "read");
+  if (ic.blocks > 1) {   // (the last position is never a full block's)
+    CK(cudaMemcpyAsync(ids.data(), ic.ids, (size_t)(ic.blocks - 1) * 4, cudaMemcpyDeviceToHost, ctx->st),
+       "read");
+    CK(cudaMemcpyAsync(hashes.data(), ic.hashes, (size_t)(ic.blocks - 1) * 8, cudaMemcpyDeviceToHost,
+                       ctx->st), "read");
+  }
+  CK(cudaStreamSynchronize(ctx->st), "sync");
+  std::vector<uint64_t> of(ic.nre, 0);   // a numbered block's hash: that of its first occurrence
+  for (size_t q = 0; q < ids.size(); q++)
+    if ((ids[q] >> 31) && (ids[q] & 0x7FFFFFFFu) < (uint32_t)ic.nre) of[ids[q] & 0x7FFFFFFFu] = hashes[q];
+  int64_t k = 0;
+  for (uint32_t t = m.head; t < m.T; t++) {
+    const uint32_t x = log[t & ctx->last_ids_rmask];
+    uint64_t h;
+    if (x >> 31)
+      h = hashes[x & 0x7FFFFFFFu];
+    else if (stamps[x] == t)
+      h = of[x];
+    else
+      continue;
+    if (k < capacity) keys_host[k] = h;
+    k++;
+  }
+  *size = k;
+  if (k != (int64_t)m.size)
+    return fail(ctx, RS_ERR_STATE, "cache of worker %d holds %lld live entries, size says %u", worker,
+                (long long)k, m.size);
+  return RS_OK;
+}
+
 rs_status route_cache_dump(rs_ctx* ctx, int32_t source, int32_t index, int32_t worker,
                            uint64_t* keys_host, int64_t capacity, int64_t* size) {
   if (!ctx) return fail(nullptr, RS_ERR_INVALID, "ctx is NULL");
@@ -1115,6 +1351,8 @@ rs_status route_cache_dump(rs_ctx* ctx, int32_t source, int32_t index, int32_t w
   } else {
     return fail(ctx, RS_ERR_INVALID, "source must be 0 or 1");
   }
+  if (source == 1 && !ctx->last_ids.empty())
+    return dump_ids(ctx, index, worker, keys_host, capacity, size);
   std::vector<uint64_t> keys(g.slots);
   std::vector<uint32_t> stamps(g.slots), log(g.R);
   CacheMeta m;

@@ -67,6 +67,12 @@ struct SimDesc {
   const int32_t* out_len;
   const uint64_t* hashes;   // block hashes of the replica's trace
   const uint8_t* dupflag;   // per request: 1 when two blocks share a chained hash
+  // the simulation on block ids (else NULL): the trace's ids and blocks up to
+  // the last not fresh one per request, the replica's stamps [W][nre]
+  const uint32_t* ids;
+  const int32_t* nz;
+  uint32_t* stamps;
+  int64_t nre;
   int64_t n_req;
   int64_t rec_base;         // first record row
   int32_t C, policy, controller, eviction;   // eviction: RS_EVICT_*
@@ -102,6 +108,7 @@ struct SimBuffers {
   const double* wco_tab;    // [(nbmax+1)(nbmax+2)] w_c * (m / nbt), or NULL
   int wco_dim;              // nbmax + 2 (row length of wco_tab)
   unsigned char* slotmem;   // [nsim][sim_slot_bytes(cmax)] when SimLaunch::slots_global
+  unsigned char* scratch;   // [nsim][sim_ids_scratch_bytes(nbmax)] (simulation on block ids)
 };
 
 struct SimLaunch {
@@ -111,6 +118,7 @@ struct SimLaunch {
   int slots_global;         // 1: per-request slot arrays in SimBuffers::slotmem
   int tiered;               // 1: Game 2 tiers (g.K = all tiers of a worker)
   int64_t k1, k12;          // G1 capacity, G1 + G2 capacity (k1 = g.K without tiers)
+  uint32_t ids_rmask;       // log ring of the simulation on block ids, less 1 (within g.R)
   TableGeom g;
   ModelConsts mc;
 };
@@ -144,6 +152,29 @@ cudaError_t launch_dup_flags(const HashJob* jobs_dev, int njobs, int64_t total_r
                              uint8_t* flags, cudaStream_t st);
 cudaError_t launch_sim(const SimDesc* d_desc, const SimBuffers& b, const SimLaunch& L,
                        cudaStream_t st);
+// One trace for the block-id kernels (requests numbered as in HashJob).
+struct IdJob {
+  const uint64_t* hashes;
+  const int64_t* offsets;
+  int64_t n_req;
+  int64_t req_base;
+  unsigned long long* keys;   // [tmask + 1] set of the trace's hashes, cleared to 0
+  uint32_t* first;            // [tmask + 1] least position (bit 31: occurs again), cleared to ~0
+  uint32_t* num;              // [tmask + 1] numbers of the hashes that occur again
+  uint32_t tmask;
+  uint32_t* ids;              // out, in the layout of hashes
+  int32_t* nz;                // out, [n_req]
+  uint32_t* count;            // hashes that occur again, cleared to 0
+};
+constexpr int IDS_MAX_JOBS = 64;
+cudaError_t launch_block_ids(const IdJob* jobs_dev, int njobs, int64_t total_req, cudaStream_t st);
+// The simulation on block ids (exact LRU replicas).
+cudaError_t launch_sim_ids(const SimDesc* d_desc, const SimBuffers& b, const SimLaunch& L,
+                           cudaStream_t st);
+size_t sim_ids_smem_bytes(int W, int nbmax, int cmax, int cap, int ntu, bool slots_global);
+size_t sim_ids_slot_bytes(int cmax);
+size_t sim_ids_scratch_bytes(int nbmax);
+int sim_ids_update_warps(int nsim, int sms);
 cudaError_t launch_wco_table(double* tab, int nbmax, double w_c, cudaStream_t st);
 cudaError_t launch_decision_stats(const SimDesc* d_desc, const SimBuffers& b, const SimLaunch& L,
                                   cudaStream_t st);

@@ -24,6 +24,7 @@ RS_POLICY_ROUNDROBIN, RS_POLICY_RANDOM, RS_POLICY_P2C = 2, 3, 4
 RS_MEM_DEVICE, RS_MEM_HOST = 0, 1
 RS_EVICT_LRU, RS_EVICT_FREQ = 0, 1
 RS_SIM_NO_POA = 1
+RS_SIM_TABLES = 2
 
 
 class rs_config(C.Structure):

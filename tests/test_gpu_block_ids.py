@@ -1,0 +1,119 @@
+"""The simulation on block ids against the simulation on hash tables
+(RS_SIM_TABLES): the same records, results and final caches, bit for bit, over
+the shapes at which the kernel on block ids changes its course: one worker, a
+worker per update warp, more workers than update warps, the most workers;
+enough replicas for the launch with two update warps; prompts with more
+victims than the window of the log holds; caches with exact-sequence updates
+and compactions of both ring sizes; slot arrays in global memory; block hashes
+given by the caller; a prompt that repeats a block; a prompt longer than the
+cache."""
+import numpy as np
+import pytest
+
+from paper_2606_17081_gb300 import routesim as rs
+from paper_2606_17081_gb300 import workloads as wk
+
+from gpu_helpers import gpu_run
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("needs a CUDA device", allow_module_level=True)
+
+OWN_COUNTS = ("probes", "slow_path", "rebuilds", "reserved0")   # of each form's own operations
+
+
+def _trace(n, seed, groups=12, lo=0, hi=3000, pre=(64, 1500), rate=None):
+    return wk.make_trace(wk.TraceSpec(n_req=n, len_kind="uniform", len_min=lo, len_max=hi, n_groups=groups,
+                                      prefix_min=pre[0], prefix_max=pre[1], zipf_s=0.8, out_kind="uniform",
+                                      out_min=0, out_max=400, rate=rate), seed)
+
+
+def _both(ctx, traces, reps, caches=()):
+    out = []
+    for flags in (0, rs.RS_SIM_TABLES):
+        st, g = gpu_run(ctx, traces, reps, flags=flags)
+        out.append((st, g, [rs.route_cache_dump(ctx.h, 1, r, j, ctx.K) for r, j in caches]))
+    (sa, a, ca), (sb, b, cb) = out
+    assert sa == sb
+    for x, y in zip(a, b):
+        if x["result"]["status"] == 0:
+            for f in x:
+                if f != "result":
+                    assert np.array_equal(x[f], y[f]), f
+        for f, v in x["result"].items():
+            if f not in OWN_COUNTS and (x["result"]["status"] == 0 or f == "status"):
+                w = y["result"][f]
+                if f in ("sum_ttft", "sum_e2e"):   # n summands, taken by 128 threads or 256
+                    assert abs(v - w) <= x["result"]["n_routed"] * 2.0 ** -53 * abs(w), (f, v, w)
+                    continue
+                assert (list(v) == list(w)) if hasattr(v, "__len__") else v == w, (f, v, w)
+    for x, y in zip(ca, cb):
+        assert x.size and np.array_equal(x, y)
+    return sa, a
+
+
+@pytest.mark.parametrize("W,K,C,tau,policy,hi", [
+    (1, 700, 9, 0.0, wk.POLICY_DYNAMO, 3000),
+    (3, 190, 40, 0.7, wk.POLICY_DYNAMO, 3000),       # ring of 2 K: every update evicts
+    (6, 511, 33, 0.0, wk.POLICY_LOADBAL, 7000),      # more victims than the window
+    (6, 512, 33, 0.0, wk.POLICY_DYNAMO, 7000),       # ring of 4 K
+    (7, 900, 64, 0.5, wk.POLICY_DYNAMO, 1040),      # past one worker per warp
+    (24, 300, 200, 0.0, wk.POLICY_DYNAMO, 3000),
+    (25, 300, 200, 1.0, wk.POLICY_P2C, 3000),
+    (64, 400, 500, 0.3, wk.POLICY_DYNAMO, 3000),
+    (33, 100, 5000, 0.0, wk.POLICY_RANDOM, 500),    # slot arrays in global memory
+])
+def test_ids_equal_tables(W, K, C, tau, policy, hi):
+    tr = _trace(900, W + K, hi=hi)
+    rep = wk.Replica(0, C, policy, int(tau > 0), 1.0, tau, 5, tr.n_req)
+    st, g = _both(rs.Context(W=W, K=K), [tr], [rep], [(0, j) for j in range(0, W, 5)])
+    assert st == rs.RS_OK and g[0]["result"]["evicted_blocks"] > 0
+
+
+def test_ids_equal_tables_many_replicas():
+    # two update warps per replica, traces of unequal length, truncated replicas, an idle one
+    trs = [_trace(150, 1), _trace(90, 2, groups=3, hi=900), _trace(40, 3, lo=0, hi=40)]
+    reps = [wk.Replica(r % 3, 1 + r % 50, wk.POLICY_DYNAMO if r % 4 else wk.POLICY_LOADBAL, r % 2, 1.0,
+                       0.25 * (r % 3), r, (trs[r % 3].n_req, 0, 30)[0 if r % 7 else r % 3]) for r in range(330)]
+    st, _ = _both(rs.Context(W=5, K=600), trs, reps, [(1, 0), (329, 4)])
+    assert st == rs.RS_OK
+
+
+def test_ids_from_given_hashes_repeated_block_and_long_prompt():
+    tr = _trace(300, 9, hi=900)
+    ctx = rs.Context(W=3, K=200)
+    d = rs.device_trace(tr)
+    h = torch.zeros(int(tr.offsets[-1]) // 16 + 1, dtype=torch.int64, device="cuda")
+    rs.route_hash_blocks(ctx.h, d.tokens, d.offsets, tr.n_req, h)
+
+    def run(hashes, n, flags):
+        t = d.desc()
+        t.tokens, t.hashes = None, hashes.data_ptr()
+        p = [rs.replica_params(wk.Replica(0, 8, wk.POLICY_DYNAMO, 0, 1.0, 0.0, 0, n))]
+        try:
+            return rs.simulate_replicas(ctx.h, [t], rs.RS_MEM_DEVICE, p, None, flags)[0].as_dict()
+        except rs.RoutesimError as e:
+            return e.results[0].as_dict()
+
+    mine = h.clone()
+    a = run(mine, tr.n_req, 0)
+    mine.zero_()   # the caches that the call left do not refer to the caller's array
+    torch.cuda.synchronize()
+    got = [rs.route_cache_dump(ctx.h, 1, 0, j, 200) for j in range(3)]
+    b = run(h, tr.n_req, rs.RS_SIM_TABLES)
+    assert a["status"] == b["status"] == 0 and a["hit_blocks"] == b["hit_blocks"] and a["sum_ttft"] == b["sum_ttft"]
+    for j in range(3):
+        assert np.array_equal(got[j], rs.route_cache_dump(ctx.h, 1, 0, j, 200))
+    nb = np.diff(tr.offsets) // 16
+    i = int(np.nonzero(nb >= 4)[0][40])
+    base = int(tr.offsets[i]) // 16
+    h[base + 3] = h[base + 1]
+    for f in (0, rs.RS_SIM_TABLES):
+        r = run(h, tr.n_req, f)
+        assert r["status"] == rs.RS_ERR_COLLISION and r["n_routed"] == i + 1, f
+    small = rs.Context(W=2, K=int(nb.max()) - 1)
+    tr2 = wk.Replica(0, 8, wk.POLICY_DYNAMO, 0, 1.0, 0.0, 0, tr.n_req)
+    st, _ = _both(small, [tr], [tr2])
+    assert st == rs.RS_ERR_CAPACITY
