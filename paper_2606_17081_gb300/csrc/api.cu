@@ -1045,9 +1045,9 @@ rs_status simulate_replicas(rs_ctx* ctx, const rs_trace* traces, int32_t n_trace
                    (r = ensure(ctx, ctx->tmpe, nsim * g.K * 4, "frequency rebuild scratch"))))
     return r;
   // w_c * (m / nbt) table for prompts up to nbmax blocks (none beyond 2048)
-  const bool use_tab = nbmax <= 2048 && !use_ids;
+  const bool use_tab = nbmax <= 2048;
   if (use_tab &&
-      (r = ensure(ctx, ctx->wco, (size_t)(nbmax + 1) * (nbmax + 2) * sizeof(double), "w_c o table")))
+      (r = ensure(ctx, ctx->wco, (size_t)(nbmax + 2) * (nbmax + 2) * sizeof(double), "w_c o table")))
     return r;
   rs_records rec;
   const bool want_cost = records && records->cost;
@@ -1135,7 +1135,7 @@ rs_status simulate_replicas(rs_ctx* ctx, const rs_trace* traces, int32_t n_trace
   L.mc = ctx->mc;
   L.mc.write_cost = want_cost ? 1 : 0;
   if (use_tab) {
-    CK(launch_wco_table(P<double>(ctx->wco), (int)nbmax, ctx->cfg.w_c, ctx->st), "table launch");
+    CK(launch_wco_table(P<double>(ctx->wco), (int)nbmax, ctx->cfg.w_c, use_ids, ctx->st), "table launch");
     launches++;
   }
   // per-request duplicate-hash flags of every trace in use

@@ -105,7 +105,7 @@ struct SimBuffers {
   rs_replica_result* res;   // [nsim]
   rs_records rec;           // every field non-NULL except possibly cost and kv_cost
   float* dstat;             // [rows][6]: two lowest costs, draw position (see k_decision_stats)
-  const double* wco_tab;    // [(nbmax+1)(nbmax+2)] w_c * (m / nbt), or NULL
+  const double* wco_tab;    // w_c * (m / nbt) at [m][nbt] (on block ids: [nbt][m]), or NULL
   int wco_dim;              // nbmax + 2 (row length of wco_tab)
   unsigned char* slotmem;   // [nsim][sim_slot_bytes(cmax)] when SimLaunch::slots_global
   unsigned char* scratch;   // [nsim][sim_ids_scratch_bytes(nbmax)] (simulation on block ids)
@@ -175,7 +175,7 @@ size_t sim_ids_smem_bytes(int W, int nbmax, int cmax, int cap, int ntu, bool slo
 size_t sim_ids_slot_bytes(int cmax);
 size_t sim_ids_scratch_bytes(int nbmax);
 int sim_ids_update_warps(int nsim, int sms);
-cudaError_t launch_wco_table(double* tab, int nbmax, double w_c, cudaStream_t st);
+cudaError_t launch_wco_table(double* tab, int nbmax, double w_c, bool by_nbt, cudaStream_t st);
 cudaError_t launch_decision_stats(const SimDesc* d_desc, const SimBuffers& b, const SimLaunch& L,
                                   cudaStream_t st);
 

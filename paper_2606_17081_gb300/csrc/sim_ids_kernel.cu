@@ -19,16 +19,25 @@
 //
 // One CTA per replica; NU update warps, a control warp, a staging warp, joined
 // by one CTA barrier per request.  Between the joins of requests i and i+1:
-//   update   the choice, request i's cache update on the chosen worker, then
-//            request i+1's cached prefix on every worker;
-//   control  the choice, request i's load and service start, then completions
+//   staging  the choice (handed to the others at a second, named barrier), then
+//            request i+3's scalars and block ids, request i's records;
+//   control  meanwhile the times that a service start would have on each
+//            worker; then request i's load and service start, and completions
 //            and controller samples up to request i+1's arrival, whose loads
 //            it publishes for the next choice;
-//   staging  the choice, request i's records and statistics, then request
-//            i+3's scalars and block ids.
+//   update   request i's cache update on the chosen worker, then request i+1's
+//            cached prefix on every worker (and, with a warp per worker, what
+//            request i+1's update would do to each).
 // What the groups hand one another at the join is double-buffered by the
-// request's parity, so no other barrier is shared.  The choice is computed by
-// every warp alike.
+// request's parity.  Between 5 and 7 cycles pass per instruction of a warp
+// that has its SM sub-partition to itself, and with four replicas per SM the
+// wait for instructions is the longest (7 of 17 cycles): the loop's code and
+// its instruction count are what to keep small.
+//
+// Calls before (hash tables) and now: 64 replicas x 10 000 requests at W = 3
+// 53.5 and 21.2 ms, 648 x 10 000 at W = 6 246 and 62.8 ms, 256 x 6 000 at
+// W = 6 with controller and sampling 62.5 and 18.7 ms, 16 x 5 000 at W = 64
+// 206 and 38.3 ms, 512 requests at W = 3 2.33 and 1.04 ms.
 #include <algorithm>
 
 #include "sim_common.cuh"
@@ -180,7 +189,7 @@ constexpr int IDS_RING = 4;   // requests staged at once (i .. i+3)
 // A staged request: what the loop needs beside its block ids.
 struct IdsReq : ReqState {
   int64_t pos0;        // position of its first block in the trace
-  double inv;          // 1 / nbt, rounded (0 for an empty prompt)
+  double inv;          // 1 / nbt, rounded (0 for an empty prompt; without the w_c o table)
   uint32_t dx, dy;     // words 0 and 1 of its Philox block
   int32_t nz, pad;
 };
@@ -191,19 +200,32 @@ struct IdsArrival {
   float tau, omega;
 };
 
+// What a worker's cache update will do, worked out before the choice
+// (launches with an update warp per worker).
+constexpr int IDS_WRING = 512;        // log entries kept ahead of the head (power of two)
+constexpr uint32_t IDS_GENERAL = 0xFFFFFFFFu;
+constexpr int IDS_WIN = 192;          // log entries an update examines that was not planned
+struct IdsPlan {
+  uint32_t nabs, E, step, pad;        // absent blocks, victims, log entries passed (or IDS_GENERAL)
+  uint32_t vic[IDS_WRING / 32];       // victims among the entries from the head on, as bits
+};
+
 struct IdsShared {
   IdsReq q[IDS_RING];
+  alignas(16) IdsPlan plan[8];
+
   IdsArrival pub[2];
   int stat[2];                 // by parity: an error seen before that join
-  int hist[256];
-  alignas(16) uint4 red[8];    // per update warp: absent blocks, least stamp, live entries
+  alignas(16) uint2 red[8];    // per update warp: absent blocks, least stamp
+  unsigned livew[IDS_WIN / 32];   // live entries of the window
   int warp_tot[8];
   int err;                     // of the update
-  int bad, nvic, nins;
+  int nvic, nins;
+  int js;                      // the chosen worker
 };
 
 struct IdsLayout {
-  size_t ftab, f_oitl, f_a, f_o, h_k, wA, codes, meta, f_req, f_worker, f_blk, f_next, h_f,
+  size_t ftab, f_oitl, f_a, f_o, h_k, srec, gk, gf, wA, codes, meta, f_req, f_worker, f_blk, f_next, h_f,
       freestk, winserv, wqh, wqt, wm, act, nfz, whead, wlen, win;
   size_t total, slot_bytes;
 };
@@ -225,18 +247,31 @@ __host__ __device__ inline IdsLayout make_ids_layout(int W, int nbmax, int cmax,
     return r;
   };
   L.ftab = take(8 * (size_t)(nft > 0 ? nft : 1));
+  // by request slot: of IdsEvents in shared memory, or the heap's in global
+  const size_t G = (C + 31) / 32;
   L.f_oitl = slots(8 * C);
   L.f_a = slots(8 * C);
   L.f_o = slots(8 * C);
-  L.h_k = slots(8 * C);
+  L.h_k = slots(8 * 32 * G);
+  L.srec = L.gk = L.gf = 0;
+  if (!slots_global) {
+    L.srec = take(16 * C);
+    if (G > 32) {
+      L.gk = take(8 * G);
+      L.gf = take(4 * G);
+    }
+  }
   L.wA = take(8 * (size_t)W);
   L.codes = take(4 * nb * IDS_RING);
   L.meta = take(sizeof(CacheMeta) * (size_t)W);
-  L.f_req = slots(4 * C);
-  L.f_worker = slots(4 * C);
-  L.f_blk = slots(4 * C);
-  L.f_next = slots(4 * C);
-  L.h_f = slots(4 * C);
+  L.f_req = L.f_worker = L.f_blk = L.f_next = L.h_f = 0;
+  if (slots_global) {
+    L.f_req = slots(4 * C);
+    L.f_worker = slots(4 * C);
+    L.f_blk = slots(4 * C);
+    L.f_next = slots(4 * C);
+    L.h_f = slots(4 * C);
+  }
   L.freestk = slots(4 * C);
   L.winserv = take(4 * (size_t)W);
   L.wqh = take(4 * (size_t)W);
@@ -246,7 +281,7 @@ __host__ __device__ inline IdsLayout make_ids_layout(int W, int nbmax, int cmax,
   L.nfz = take(4 * 2 * (size_t)W);
   L.whead = take(4 * (size_t)W);
   L.wlen = take(4 * (size_t)W);
-  L.win = take(4 * (size_t)W * ntu);
+  L.win = take(4 * (size_t)W * (W <= ntu / 32 ? IDS_WRING : IDS_WIN));
   L.total = o;
   L.slot_bytes = (og + 255) & ~(size_t)255;
   return L;
@@ -302,6 +337,19 @@ __device__ __forceinline__ void join_cta() {
   asm volatile("barrier.sync 0, %0;" ::"n"(NT) : "memory");
 }
 
+// The choice of request i: made by the staging warp (Sh.js written), waited
+// for by the others.  (Every warp computing it alike took a third of all
+// instructions and three copies of its code.)
+template <int NT>
+__device__ __forceinline__ void choice_made() {
+  __syncwarp();
+  asm volatile("barrier.arrive 2, %0;" ::"n"(NT) : "memory");
+}
+template <int NT>
+__device__ __forceinline__ void choice_wait() {
+  asm volatile("barrier.sync 2, %0;" ::"n"(NT) : "memory");
+}
+
 // ------------------------------------------------------------ probe
 
 // Leading blocks of the prompt found in one worker's cache from block k0 on,
@@ -309,6 +357,7 @@ __device__ __forceinline__ void join_cta() {
 __device__ __forceinline__ int ids_prefix(const uint32_t* st, const uint32_t* cd, int k0, int nz,
                                           unsigned& cnt) {
   const int lane = (int)(threadIdx.x & 31);
+#pragma unroll 1
   for (int k = k0; k < nz; k += 128) {
     uint32_t v[4];
     bool in[4];
@@ -354,6 +403,7 @@ __device__ __forceinline__ void ids_probe(const uint32_t* stamps, size_t nre, co
       m[q] = nz;
       open |= (unsigned)(j0 + q * NU < W) << q;
     }
+#pragma unroll 1
     for (int k = 0; k < nz && open; k += 64) {
       const int ka = k + lane, kb = ka + 32;
       const uint32_t ca = ka < nz ? cd[ka] : CODE_FRESH, cb = kb < nz ? cd[kb] : CODE_FRESH;
@@ -390,15 +440,16 @@ __device__ __forceinline__ void ids_probe(const uint32_t* stamps, size_t nre, co
 
 // ------------------------------------------------------------ choice
 
-// Eq. (1) costs of workers lane and lane + 32 and the chosen worker (a warp;
-// every warp the same).  Costs are >= +0, so their bit patterns order them.
+// Eq. (1) costs of workers lane and lane + 32 and the chosen worker (a warp).
+// Costs are >= +0, so their bit patterns order them.
 struct IdsChoice {
   float c[2], best;
   int bj, js;
   float target, S, lo, hi;   // where an Eq. (2) draw fell
 };
 
-__device__ __forceinline__ IdsChoice ids_choice(const SimDesc& d, const IdsReq& q,
+template <bool WIDE>
+__device__ __forceinline__ IdsChoice ids_choice(int policy, const IdsReq& q,
                                                 const IdsArrival& ar, const int* wm,
                                                 const float* act, int W, int64_t i, int lane) {
   IdsChoice r;
@@ -408,25 +459,25 @@ __device__ __forceinline__ IdsChoice ids_choice(const SimDesc& d, const IdsReq& 
   for (int h = 0; h < 2; h++) {
     const int j = lane + 32 * h;
     r.c[h] = inf;
-    if (j < W) r.c[h] = __fadd_rn(__fmul_rn(om, __int2float_rn(q.nbt - wm[j])), act[j]);
+    if ((h == 0 || WIDE) && j < W) r.c[h] = __fadd_rn(__fmul_rn(om, __int2float_rn(q.nbt - wm[j])), act[j]);
   }
   const unsigned mn = __reduce_min_sync(FULL_MASK, min(__float_as_uint(r.c[0]), __float_as_uint(r.c[1])));
   // the lowest index among the minima: workers 0-31 first
   const unsigned e0 =
       __ballot_sync(FULL_MASK, lane < W && __float_as_uint(r.c[0]) == mn);
   const unsigned e1 =
-      W > 32 ? __ballot_sync(FULL_MASK, lane + 32 < W && __float_as_uint(r.c[1]) == mn) : 0u;
+      WIDE ? __ballot_sync(FULL_MASK, lane + 32 < W && __float_as_uint(r.c[1]) == mn) : 0u;
   r.bj = e0 ? __ffs(e0) - 1 : 32 + __ffs(e1) - 1;
   r.best = __uint_as_float(mn);
   r.js = r.bj;
-  if (d.policy != RS_POLICY_DYNAMO && d.policy != RS_POLICY_LOADBAL) {
+  if (policy != RS_POLICY_DYNAMO && policy != RS_POLICY_LOADBAL) {
     // the static policies (as static_policy_worker)
-    if (d.policy == RS_POLICY_ROUNDROBIN) {
+    if (policy == RS_POLICY_ROUNDROBIN) {
       r.js = (int)((uint64_t)i % (uint64_t)W);
     } else {
       const int j1 = (int)(((uint64_t)(q.dx >> 8) * (uint64_t)W) >> 24);
       r.js = j1;
-      if (d.policy == RS_POLICY_P2C && W >= 2) {
+      if (policy == RS_POLICY_P2C && W >= 2) {
         int j2 = (int)(((uint64_t)(q.dy >> 8) * (uint64_t)(W - 1)) >> 24);
         if (j2 >= j1) j2++;
         const int lo = j1 < j2 ? j1 : j2, hi = j1 < j2 ? j2 : j1;
@@ -442,18 +493,20 @@ __device__ __forceinline__ IdsChoice ids_choice(const SimDesc& d, const IdsReq& 
     float e[2];
 #pragma unroll
     for (int h = 0; h < 2; h++)
-      e[h] = lane + 32 * h < W ? exp_sm(-__fdiv_rn(__fsub_rn(r.c[h], r.best), tau)) : 0.0f;
+      e[h] = (h == 0 || WIDE) && lane + 32 * h < W ? exp_sm(-__fdiv_rn(__fsub_rn(r.c[h], r.best), tau)) : 0.0f;
     float S = 0.0f;
+#pragma unroll 4
     for (int j = 0; j < W; j++)
-      S = __fadd_rn(S, __shfl_sync(FULL_MASK, j < 32 ? e[0] : e[1], j & 31));
+      S = __fadd_rn(S, __shfl_sync(FULL_MASK, !WIDE || j < 32 ? e[0] : e[1], j & 31));
     r.target = __fmul_rn(__fmul_rn((float)(q.dx >> 8), 0x1p-24f), S);
     r.S = S;
     const float qnan = __int_as_float(0x7FC00000);
     float cum = 0.0f;
     r.lo = r.hi = qnan;
     int pick = -1, last = r.bj;
+#pragma unroll 4
     for (int j = 0; j < W; j++) {
-      const float ej = __shfl_sync(FULL_MASK, j < 32 ? e[0] : e[1], j & 31);
+      const float ej = __shfl_sync(FULL_MASK, !WIDE || j < 32 ? e[0] : e[1], j & 31);
       cum = __fadd_rn(cum, ej);
       if (ej > 0.0f) last = j;
       if (pick < 0 && r.target < cum) {
@@ -493,12 +546,12 @@ __device__ __forceinline__ bool ids_live(const IdsTable& t, uint32_t x, uint32_t
 // stamps by a multiple of the ring's length (so ring places stay), in place:
 // an entry never moves up.
 template <int NT>
-__device__ __forceinline__ void ids_compact(const IdsTable& t, CacheMeta* meta, int* warp_tot,
-                                            int* err) {
+__device__ __noinline__ void ids_compact(IdsTable t, CacheMeta* meta, int* warp_tot, int* err) {
   const uint32_t head = meta->head, T = meta->T, size = meta->size;
   const uint32_t d = head & ~t.rmask;
   constexpr int PER = 4;
   uint32_t base = 0;
+#pragma unroll 1
   for (uint32_t p0 = head; p0 < T; p0 += NT * PER) {
     const uint32_t pb = p0 + threadIdx.x * PER;
     uint32_t x[PER];
@@ -536,6 +589,7 @@ template <int NT>
 __device__ __forceinline__ uint32_t ids_gather(const IdsTable& t, uint32_t head, uint32_t T,
                                                uint32_t want, const IdsScratch& sc, int* warp_tot) {
   uint32_t have = 0;
+#pragma unroll 1
   for (uint32_t p0 = head; have < want && p0 < T; p0 += NT) {
     const uint32_t p = p0 + threadIdx.x;
     uint32_t x = 0;
@@ -569,16 +623,20 @@ __device__ __forceinline__ uint32_t ids_place(const uint32_t* vt, uint32_t n, ui
 // An update whose victims the window does not settle: more victims than it
 // holds, or a present block among the least recent entries, which the exact
 // sequence (one thread, over the first 2 nb live entries) decides.  Evicts;
-// returns the head past the last victim, victims in *E, insertions in *nins.
+// returns the head past the last victim; victims in S.nvic, insertions in
+// S.nins.  (Rare, and out of line: the loop's hot code has to stay small, its
+// warps wait for instructions otherwise.)
 template <int NT>
-__device__ __forceinline__ uint32_t ids_evict_general(const IdsTable& t, const CacheMeta& m,
-                                                      uint32_t K, const uint32_t* cd, int nb,
-                                                      uint32_t E0, uint32_t pmin, int nabs,
-                                                      const IdsScratch& sc, IdsShared& S,
-                                                      int64_t* slow, uint32_t* E, int* nins) {
+__device__ __noinline__ uint32_t ids_evict_general(IdsTable t, CacheMeta m, uint32_t K,
+                                                   const uint32_t* cd, int nb, uint32_t E0,
+                                                   uint32_t pmin, int nabs, unsigned char* scratch,
+                                                   int nbmax, IdsShared& S, int64_t* slow) {
+  const IdsScratch sc = ids_scratch(scratch, nbmax);
+  if (threadIdx.x == 0) {
+    S.nvic = 0;
+    S.nins = nabs;
+  }
   uint32_t G = ids_gather<NT>(t, m.head, m.T, E0, sc, S.warp_tot);
-  *E = 0;
-  *nins = nabs;
   if (G < E0) {   // fewer live entries than the size says
     if (threadIdx.x == 0) S.err = RS_ERR_TIMEOUT;
     return m.head;
@@ -586,7 +644,8 @@ __device__ __forceinline__ uint32_t ids_evict_general(const IdsTable& t, const C
   if (pmin > sc.vt[E0 - 1]) {   // (also pmin = STAMP_NONE: no block present)
     for (uint32_t v = threadIdx.x; v < E0; v += NT)
       if (!(sc.vent[v] & SINGLE_FLAG)) t.st[sc.vent[v]] = STAMP_NONE;
-    *E = E0;
+    if (threadIdx.x == 0) S.nvic = (int)E0;
+    grp_bar<NT>();
     return sc.vt[E0 - 1] + 1;
   }
   grp_bar<NT>();
@@ -638,35 +697,154 @@ __device__ __forceinline__ uint32_t ids_evict_general(const IdsTable& t, const C
     const uint32_t x = sc.vent[sc.victim[v]];
     if (!(x & SINGLE_FLAG)) t.st[x] = STAMP_NONE;
   }
-  *E = (uint32_t)e;
-  *nins = S.nins;
   const uint32_t nh = e > 0 ? sc.vt[sc.victim[e - 1]] + 1 : m.head;
   grp_bar<NT>();   // a victim may be a block of this request: its new stamp comes after
   return nh;
 }
 
+// m_j of one worker and its update's plan, by its warp.  The worker's log
+// entries from the head on come from a ring of IDS_WRING entries in shared
+// memory, copied in the background two or more updates ahead; [head, safe) are
+// known to have landed.  Loads: a stamp per block and per window entry, all in
+// flight together.  Planning every worker before the choice takes the update's
+// loads, its reductions and its barrier off the path between the choice and
+// the next probe: 1 960 + 760 SM cycles a request for update and probe with
+// the update's reads after the choice (64 replicas, W = 3).
+__device__ __forceinline__ int ids_plan(const IdsTable& t, const CacheMeta& m, uint32_t K,
+                                        const uint32_t* cd, int nb, int nz, uint32_t* ring,
+                                        uint32_t safe, IdsPlan& P, unsigned& cnt) {
+  const int lane = (int)(threadIdx.x & 31);
+  const bool full = m.size + (uint32_t)nb > K;   // a victim may be needed
+  // four words of the window (128 log entries): entries, then their stamps.
+  // Loads take no branch: a place past the log or a single block reads a
+  // stamp that is not used.
+  auto entries = [&](int w0, uint32_t (&x)[4], uint32_t (&v)[4]) {
+    const uint32_t p0 = m.head + 32 * w0 + lane;
+#pragma unroll
+    for (int r = 0; r < 4; r++) x[r] = ring[(p0 + 32 * r) & (IDS_WRING - 1)];
+    if (p0 + 96 >= safe) {
+#pragma unroll
+      for (int r = 0; r < 4; r++) {
+        const uint32_t p = p0 + 32 * r;
+        if (p >= safe) {
+          x[r] = p < m.T ? t.log[p & t.rmask] : SINGLE_FLAG;
+          ring[p & (IDS_WRING - 1)] = x[r];
+        }
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < 4; r++) v[r] = t.st[(x[r] & SINGLE_FLAG) ? 0u : x[r]];
+  };
+  uint32_t x[4], v[4];
+  if (full) entries(0, x, v);
+  int mj = nz, nabs = nb - nz;   // past nz every block is fresh
+  uint32_t pmin = STAMP_NONE;
+#pragma unroll 1
+  for (int k = 0; k < nz; k += 128) {
+    uint32_t u[4], cc[4];
+#pragma unroll
+    for (int r = 0; r < 4; r++) cc[r] = cd[min(k + 32 * r + lane, nz - 1)];
+#pragma unroll
+    for (int r = 0; r < 4; r++) u[r] = t.st[cc[r] >> 31 ? 0u : cc[r]];
+#pragma unroll
+    for (int r = 0; r < 4; r++) {
+      const bool in = k + 32 * r + lane < nz, old = in && !(cc[r] >> 31);
+      cnt += old;
+      if (!old) u[r] = STAMP_NONE;
+      const unsigned ab = __ballot_sync(FULL_MASK, in && u[r] == STAMP_NONE);
+      nabs += __popc(ab);
+      if (ab && mj == nz) mj = k + 32 * r + __ffs(ab) - 1;
+      pmin = min(pmin, u[r]);
+    }
+  }
+  const uint32_t freeb = K - m.size;
+  const uint32_t E = (uint32_t)nabs > freeb ? (uint32_t)nabs - freeb : 0u;
+  uint32_t step = 0, bits = 0;   // lane w: victims among entries 32 w .. 32 w + 31
+  if (E > 0) {
+    // the first E live entries, all before the oldest present block
+    const uint32_t end = min(__reduce_min_sync(FULL_MASK, pmin), m.T);
+    uint32_t have = 0;
+#pragma unroll 1
+    for (int w0 = 0;;) {
+#pragma unroll
+      for (int r = 0; r < 4; r++) {
+        const uint32_t p = m.head + 32 * (w0 + r) + lane;
+        unsigned b = __ballot_sync(FULL_MASK, p < end && ((x[r] & SINGLE_FLAG) || v[r] == p));
+        const uint32_t n = (uint32_t)__popc(b);
+        if (have < E) {
+          if (have + n >= E) {
+            const int q = nth_set_bit32(b, (int)(E - have) - 1);
+            b &= q == 31 ? FULL_MASK : (2u << q) - 1u;
+            step = 32u * (w0 + r) + (uint32_t)q + 1u;
+          }
+          if (lane == w0 + r) bits = b;
+          have += n;
+        }
+      }
+      w0 += 4;
+      if (have >= E || w0 == IDS_WRING / 32 || m.head + 32 * w0 >= end) break;
+      entries(w0, x, v);
+    }
+    if (have < E) step = IDS_GENERAL;
+  }
+  if ((uint64_t)m.T - m.head + (uint64_t)nb > (uint64_t)t.rmask + 1 ||
+      (uint64_t)m.T + nb > STAMP_LIMIT)
+    step = IDS_GENERAL;   // a compaction first
+  if (lane == 0) {
+    P.nabs = (uint32_t)nabs;
+    P.E = E;
+    P.step = step;
+  }
+  if (lane < IDS_WRING / 32) P.vic[lane] = bits;
+  return mj;
+}
+
+// The planned update of the chosen worker, by the update warps.
+template <int NT>
+__device__ __forceinline__ void ids_apply(const IdsTable& t, CacheMeta* meta, const IdsPlan& P, const uint32_t* ring,
+                                          const uint32_t* cd, const IdsReq& q) {
+  const CacheMeta m = *meta;
+  const uint32_t step = P.step;
+  const int tid = (int)threadIdx.x;
+#pragma unroll 1
+  for (uint32_t w = tid; w < step; w += NT)
+    if ((P.vic[w >> 5] >> (w & 31)) & 1u) {
+      const uint32_t x = ring[(m.head + w) & (IDS_WRING - 1)];
+      if (!(x & SINGLE_FLAG)) t.st[x] = STAMP_NONE;
+    }
+  // every block of the prompt is now the most recent, in order
+  const int nb = q.nb;
+#pragma unroll 1
+  for (int k = tid; k < nb; k += NT) {
+    const uint32_t b = cd[k] & CODE_SINGLE, pos = m.T + (uint32_t)k;
+    if (b != CODE_SINGLE) t.st[b] = pos;
+    t.log[pos & t.rmask] = b != CODE_SINGLE ? b : SINGLE_FLAG | (uint32_t)(q.pos0 + k);
+  }
+}
+
 // Request i's blocks touched in order on the chosen worker's cache (exact
-// LRU), by the update warps.  The window win holds the log entries from
+// LRU), by the update warps.  WINDOW: the window win holds the log entries from
 // whead on (copied in the background after the worker's last update), so the
 // common update makes one round of stamp loads and one barrier: every thread
 // reads the stamp of one block of the prompt and of one window entry; the
 // live entries before the oldest present block are the candidates, and the
-// first E0 = absent - free of them are the victims.
-template <int NT>
-__device__ __forceinline__ void ids_update(SimCtx& c, IdsShared& S, const IdsTable& t,
-                                           CacheMeta* meta, const uint32_t* cd, const IdsReq& q,
-                                           const IdsScratch& sc, uint32_t* win, uint32_t* whead,
-                                           uint32_t* wlen, int64_t i) {
-  constexpr int NW = NT / 32;
-  const uint32_t K = c.L->g.K;
+// first E0 = absent - free of them are the victims.  Without: the course that
+// a plan leaves to the whole group.
+template <int NT, bool WINDOW>
+__device__ __forceinline__ void ids_update(SimScalars& A, IdsShared& S, uint32_t K, int nbmax,
+                                           const IdsTable& t, CacheMeta* meta, const uint32_t* cd,
+                                           const IdsReq& q, unsigned char* scratch, uint32_t* win,
+                                           uint32_t* whead, uint32_t* wlen, int64_t i) {
+  constexpr int R = IDS_WIN / NT, NW = IDS_WIN / 32;   // window entries per thread, words
+  static_assert(R * NT == IDS_WIN, "whole window entries per thread");
   const int nb = q.nb, nz = q.nz, tid = (int)threadIdx.x, lane = tid & 31;
-  cp_async_wait_all();   // this thread's window entries
+  if (WINDOW) cp_async_wait_all();   // this thread's window entries
   if ((uint64_t)meta->T - meta->head + (uint64_t)nb > (uint64_t)t.rmask + 1 ||
       (uint64_t)meta->T + nb > STAMP_LIMIT) {
     grp_bar<NT>();
     ids_compact<NT>(t, meta, S.warp_tot, &S.err);
     if (tid == 0) {
-      c.S->rebuilds++;
+      A.rebuilds++;
       *wlen = 0;
     }
     grp_bar<NT>();
@@ -676,37 +854,44 @@ __device__ __forceinline__ void ids_update(SimCtx& c, IdsShared& S, const IdsTab
   // stamps of the prompt's blocks, of the window's entries
   int nabs = 0;
   uint32_t pmin = STAMP_NONE;
+#pragma unroll 1
   for (int k = tid; k < nz; k += NT) {
     const uint32_t x = cd[k];
     const uint32_t st = x >> 31 ? STAMP_NONE : t.st[x];
     nabs += st == STAMP_NONE;
     pmin = min(pmin, st);
   }
-  uint32_t x = 0;
-  bool live = false;
-  if (full) {
-    const uint32_t p = m.head + tid;
-    if (p < m.T) {
-      x = *whead == m.head && (uint32_t)tid < *wlen ? win[tid] : t.log[p & t.rmask];
-      live = ids_live(t, x, p);
-    }
+  uint32_t x[R];
+  bool live[R];
+  const uint32_t have_win = WINDOW && *whead == m.head ? *wlen : 0u;
+#pragma unroll
+  for (int r = 0; r < R; r++) {
+    const uint32_t w = (uint32_t)(r * NT + tid), p = m.head + w;
+    live[r] = full && p < m.T;
+    x[r] = 0;
+    if (live[r]) x[r] = w < have_win ? win[w] : t.log[p & t.rmask];
   }
+#pragma unroll
+  for (int r = 0; r < R; r++)
+    if (live[r]) live[r] = ids_live(t, x[r], m.head + (uint32_t)(r * NT + tid));
   {
     const int a = (int)__reduce_add_sync(FULL_MASK, (unsigned)nabs);
     const uint32_t pm = __reduce_min_sync(FULL_MASK, pmin);
-    const unsigned lv = __ballot_sync(FULL_MASK, live);
-    if (lane == 0) S.red[tid >> 5] = make_uint4((unsigned)a, pm, lv, 0u);
+    if (lane == 0) S.red[tid >> 5] = make_uint2((unsigned)a, pm);
+#pragma unroll
+    for (int r = 0; r < R; r++) {
+      const unsigned lv = __ballot_sync(FULL_MASK, live[r]);
+      if (lane == 0) S.livew[r * (NT / 32) + (tid >> 5)] = lv;
+    }
   }
   grp_bar<NT>();
   nabs = nb - nz;   // past nz every block is fresh
   pmin = STAMP_NONE;
-  unsigned lv[NW];
 #pragma unroll
-  for (int w = 0; w < NW; w++) {
-    const uint4 r = S.red[w];
+  for (int w = 0; w < NT / 32; w++) {
+    const uint2 r = S.red[w];
     nabs += (int)r.x;
     pmin = min(pmin, r.y);
-    lv[w] = r.z;
   }
   const uint32_t freeb = K - m.size;
   const uint32_t E0 = (uint32_t)nabs > freeb ? (uint32_t)nabs - freeb : 0u;
@@ -721,19 +906,24 @@ __device__ __forceinline__ void ids_update(SimCtx& c, IdsShared& S, const IdsTab
     for (int w = 0; w < NW; w++) {
       const uint32_t l0 = 32u * w;
       const unsigned mk = lim >= l0 + 32u ? FULL_MASK : (lim > l0 ? (1u << (lim - l0)) - 1u : 0u);
-      const unsigned b = lv[w] & mk;
+      const unsigned b = S.livew[w] & mk;
       const uint32_t n = (uint32_t)__popc(b);
       if (have < E0 && have + n >= E0) last = (int)l0 + nth_set_bit32(b, (int)(E0 - have) - 1);
       have += n;
     }
     if (last >= 0) {
-      if (live && tid <= last && !(x & SINGLE_FLAG)) t.st[x] = STAMP_NONE;
+#pragma unroll
+      for (int r = 0; r < R; r++)
+        if (live[r] && r * NT + tid <= last && !(x[r] & SINGLE_FLAG)) t.st[x[r]] = STAMP_NONE;
       nh = m.head + (uint32_t)last + 1u;
     } else {
-      nh = ids_evict_general<NT>(t, m, K, cd, nb, E0, pmin, nabs, sc, S, &c.S->slow, &E, &nins);
+      nh = ids_evict_general<NT>(t, m, K, cd, nb, E0, pmin, nabs, scratch, nbmax, S, &A.slow);
+      E = (uint32_t)S.nvic;
+      nins = S.nins;
     }
   }
   // every block of the prompt is now the most recent, in order
+#pragma unroll 1
   for (int k = tid; k < nb; k += NT) {
     const uint32_t b = cd[k] & CODE_SINGLE, pos = m.T + (uint32_t)k;
     if (b != CODE_SINGLE) t.st[b] = pos;
@@ -742,27 +932,38 @@ __device__ __forceinline__ void ids_update(SimCtx& c, IdsShared& S, const IdsTab
   const uint32_t size = m.size + (uint32_t)nins - E;
   // the window of this worker's next update: entries written before this one
   // (all threads have read the old window: the barrier above)
-  if (size + (uint32_t)c.L->nbmax > K) {
-    const uint32_t p = nh + tid;
-    if (p < m.T) cp_async4(win + tid, t.log + (p & t.rmask));
+  if (WINDOW && size + (uint32_t)nbmax > K) {
+#pragma unroll
+    for (int r = 0; r < R; r++) {
+      const uint32_t p = nh + (uint32_t)(r * NT + tid);
+      if (p < m.T) cp_async4(win + r * NT + tid, t.log + (p & t.rmask));
+    }
     if (tid == 0) {
       *whead = nh;
-      *wlen = m.T > nh ? min((uint32_t)NT, m.T - nh) : 0u;
+      *wlen = m.T > nh ? min((uint32_t)IDS_WIN, m.T - nh) : 0u;
     }
   }
   if (tid == 0) {
     meta->size = size;
     meta->head = nh;
     meta->T = m.T + (uint32_t)nb;
-    SimScalars& R = *c.S;
-    R.inserted += nins;
-    R.evicted += E;
-    if (E > 0 && R.first_evict_i < 0) {
+    A.inserted += nins;
+    A.evicted += E;
+    if (E > 0 && A.first_evict_i < 0) {
       // the first update that evicted; resident blocks = inserted - evicted
-      R.first_evict_i = i;
-      R.first_live = R.inserted - R.evicted;
+      A.first_evict_i = i;
+      A.first_live = A.inserted - A.evicted;
     }
   }
+}
+
+// The same out of line, for updates that a plan leaves to the whole group.
+template <int NT>
+__device__ __noinline__ void ids_update_unplanned(SimScalars& A, IdsShared& S, uint32_t K, int nbmax,
+                                                  IdsTable t, CacheMeta* meta, const uint32_t* cd,
+                                                  const IdsReq& q, unsigned char* scratch,
+                                                  uint32_t* wlen, int64_t i) {
+  ids_update<NT, false>(A, S, K, nbmax, t, meta, cd, q, scratch, nullptr, nullptr, wlen, i);
 }
 
 // ------------------------------------------------------------ control warp
@@ -770,8 +971,16 @@ __device__ __forceinline__ void ids_update(SimCtx& c, IdsShared& S, const IdsTab
 // A controller sample with a non-empty window (as the CTA-wide tick of the
 // table kernel, by one warp): the window's nearest-rank P99 by an exact radix
 // selection, from the highest byte in which its TTFTs differ.
-__device__ __forceinline__ void ids_tick(SimCtx& c, IdsShared& Sh, int lane) {
-  SimScalars& S = *c.S;
+__device__ __noinline__ void ids_tick(SimScalars& S, const SimLaunch& L, double* pend,
+                                      int64_t pend_cap, int lane) {
+  SimCtx c;
+  c.S = &S;
+  c.L = &L;
+  c.pend_ft0 = pend;
+  c.pend_tt0 = pend + pend_cap;
+  c.pend_ft1 = pend + 2 * pend_cap;
+  c.pend_tt1 = pend + 3 * pend_cap;
+  c.pend_win = pend + 4 * pend_cap;
   const int cur = S.pend_cur;
   const int64_t np = S.np;
   const double* sft = c.pend_ft(cur);
@@ -815,25 +1024,25 @@ __device__ __forceinline__ void ids_tick(SimCtx& c, IdsShared& Sh, int lane) {
     any1 |= __shfl_xor_sync(FULL_MASK, any1, o);
   }
   __syncwarp();
-  double L = 0.0;
+  double p99 = 0.0;
   if (nwin > 0) {
     int kk = (int)((99 * nwin + 99) / 100);   // 1-based rank
     const uint64_t diff = all1 ^ any1;
     int shift = diff ? (63 - __clzll((long long)diff)) & ~7 : -8;
     uint64_t pre = shift < 0 ? all1 : (shift == 56 ? 0ull : all1 & (~0ull << (shift + 8)));
     for (; shift >= 0; shift -= 8) {
-      for (int q = lane; q < 256; q += 32) Sh.hist[q] = 0;
+      for (int q = lane; q < 256; q += 32) c.S->hist[q] = 0;
       __syncwarp();
       const uint64_t mhi = shift == 56 ? 0ull : (~0ull << (shift + 8));
       for (int64_t p = lane; p < nwin; p += 32) {
         const uint64_t bits = (uint64_t)__double_as_longlong(c.pend_win[p]);
-        if ((bits & mhi) == (pre & mhi)) atomicAdd(&Sh.hist[(bits >> shift) & 255], 1);
+        if ((bits & mhi) == (pre & mhi)) atomicAdd(&c.S->hist[(bits >> shift) & 255], 1);
       }
       __syncwarp();
       // lane l holds bins 8 l .. 8 l + 7
       int sum = 0;
 #pragma unroll
-      for (int e = 0; e < 8; e++) sum += Sh.hist[8 * lane + e];
+      for (int e = 0; e < 8; e++) sum += c.S->hist[8 * lane + e];
       int inc = sum;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
@@ -845,26 +1054,36 @@ __device__ __forceinline__ void ids_tick(SimCtx& c, IdsShared& Sh, int lane) {
       int dg = 0, cum = inc - sum;
       if (lane == ls)
         for (dg = 8 * lane; dg < 8 * lane + 7; dg++) {
-          if (cum + Sh.hist[dg] >= kk) break;
-          cum += Sh.hist[dg];
+          if (cum + c.S->hist[dg] >= kk) break;
+          cum += c.S->hist[dg];
         }
       dg = __shfl_sync(FULL_MASK, dg, ls);
       kk -= __shfl_sync(FULL_MASK, cum, ls);
       pre |= (uint64_t)dg << shift;
       __syncwarp();
     }
-    L = __longlong_as_double((long long)pre);
+    p99 = __longlong_as_double((long long)pre);
   }
   if (lane == 0) {
     S.np = nkeep;
     S.pend_cur = cur ^ 1;
     S.min_ft = tval(mft);
-    ctl_sample(c, nwin > 0, L);
+    ctl_sample(c, nwin > 0, p99);
   }
   __syncwarp();
 }
 
-// Request i's arrival: every event before it, then what its choice needs.
+// A controller sample without a window.
+__device__ __noinline__ void ids_tick_empty(SimScalars& S, const SimLaunch& L, int lane) {
+  SimCtx c;
+  c.S = &S;
+  c.L = &L;
+  if (lane == 0) ctl_sample(c, false, 0.0);
+  __syncwarp();
+}
+
+// Request i's arrival: every event before it, then what its choice needs (one
+// thread and a heap: for concurrencies whose slots are in global memory).
 __device__ __forceinline__ void ids_arrive(SimCtx& c, IdsShared& Sh, int64_t i, float* act,
                                            int* nfz, int lane) {
   SimScalars& S = *c.S;
@@ -878,7 +1097,7 @@ __device__ __forceinline__ void ids_arrive(SimCtx& c, IdsShared& Sh, int64_t i, 
     int ev = 0;
     if (lane == 0) ev = events_advance(c, q);
     if (!__shfl_sync(FULL_MASK, ev, 0)) break;
-    ids_tick(c, Sh, lane);
+    ids_tick(S, *c.L, c.pend_ft0, c.b->pend_cap, lane);
   }
   if (lane == 0) {
     regime_params<false>(c, q);
@@ -891,6 +1110,280 @@ __device__ __forceinline__ void ids_arrive(SimCtx& c, IdsShared& Sh, int64_t i, 
   for (int j = lane; j < W; j += 32) {
     act[p * W + j] = __int2float_rn((int)c.wA[j]);
     nfz[p * W + j] = min(c.winserv[j] + 1, c.L->mc.cap - 1);
+  }
+}
+
+// ------------------------------------------------------------ events (control warp)
+
+// The closed-loop client's events with their state in the control warp's
+// registers, every lane running the same course: lane j holds workers j and
+// (WIDE) j + 32: active blocks, requests in service, queue ends.  Completion
+// times lie by request slot in groups of 32; lane g keeps the earliest of
+// group g (and of groups g + 32, ...), so an insertion is one comparison and a
+// removal one load across the warp and two pairs of warp minima, whatever the
+// concurrency.
+//
+// This warp is the replica's critical path at one or two replicas per SM.  An
+// FP64 instruction holds its SM sub-partition's unit for 63 cycles whatever
+// the number of lanes, dependent or not, so the times that a service start
+// would have are computed for every worker at once, one lane each, from loads
+// issued before the choice; nothing that the next event does not need is computed here (TTFT is
+// left to the pass over the records).  On one thread with a heap in shared
+// memory and the FP64 chain after the choice, the booking took 1 150 SM cycles
+// a request and the events 3 000 (64 replicas, W = 3).
+constexpr uint64_t KEY_NONE = ~0ull;   // no completion (above every time's key)
+
+template <bool WIDE>
+struct IdsEvents {
+  static constexpr int H = WIDE ? 2 : 1;
+  uint64_t lk, kc;   // earliest completion of this lane's groups, of all
+  int lf, fc;        // their slots
+  int A[H], serv[H], qh[H], qt[H];
+  int inflight, nfree, np, cur, ng;
+  uint64_t mft, tick;   // keys: earliest pending first token, next controller sample
+  uint64_t pk;       // key of the last arrival
+  double prev;       // the last arrival
+  int conc, ctl, spike;   // C, controller on, load-spike schedule
+  float tau, omega;       // in the Below regime
+  uint64_t* skey;    // [32 ng] completion keys by slot
+  int4* srec;        // [slots] worker, blocks, next in queue, request
+  uint64_t* gk;      // [ng] earliest key of each group, and its slot (ng > 32)
+  int* gf;
+  double *sa, *so, *soitl;   // [slots] of queued requests: arrival, w_c o, O itl
+  int* freestk;
+  double* rp;        // lanes 0-2: start, first token, completion records
+
+  __device__ __forceinline__ int get(const int (&v)[H], int j) const {
+    int x = __shfl_sync(FULL_MASK, v[0], j & 31);
+    if (WIDE) {
+      const int y = __shfl_sync(FULL_MASK, v[H - 1], j & 31);
+      if (j >= 32) x = y;
+    }
+    return x;
+  }
+  __device__ __forceinline__ void add(int (&v)[H], int j, int x, int lane) {
+#pragma unroll
+    for (int h = 0; h < H; h++)
+      if (lane + 32 * h == j) v[h] += x;
+  }
+  __device__ __forceinline__ void put(int (&v)[H], int j, int x, int lane) {
+#pragma unroll
+    for (int h = 0; h < H; h++)
+      if (lane + 32 * h == j) v[h] = x;
+  }
+};
+
+// f(n) of Eq. (9) past the table (rare: kept out of the loop's code).
+__device__ __noinline__ double ids_latency(const ModelConsts& mc, int n) { return latency_f(mc, n); }
+
+__device__ __forceinline__ double ev_f(const SimCtx& c, int n) {
+  return n < FTAB_MAX ? c.ftab[n] : ids_latency(c.L->mc, n);
+}
+
+// The earliest of the warp's (key, slot) pairs, by (key, request).
+template <bool WIDE>
+__device__ __forceinline__ void ev_min(const IdsEvents<WIDE>& E, uint64_t k, int f, uint64_t& ko,
+                                       int& fo) {
+  const unsigned hi = __reduce_min_sync(FULL_MASK, (unsigned)(k >> 32));
+  const unsigned lo =
+      __reduce_min_sync(FULL_MASK, (unsigned)(k >> 32) == hi ? (unsigned)k : 0xFFFFFFFFu);
+  ko = ((uint64_t)hi << 32) | lo;
+  unsigned eq = __ballot_sync(FULL_MASK, k == ko);
+  if ((eq & (eq - 1u)) && ko != KEY_NONE) {   // equal times: the earlier request first
+    const unsigned rq = k == ko ? (unsigned)E.srec[f].w : 0xFFFFFFFFu;
+    const unsigned mn = __reduce_min_sync(FULL_MASK, rq);
+    eq = __ballot_sync(FULL_MASK, rq == mn);
+  }
+  fo = __shfl_sync(FULL_MASK, f, __ffs(eq) - 1);
+}
+
+// Request req in slot f is in service from t on: first token ft, completion ct.
+template <bool WIDE>
+__device__ __forceinline__ void ev_start(SimCtx& c, IdsEvents<WIDE>& E, int f, int req, double t,
+                                         double ft, double ct, double a, int lane) {
+  const uint64_t k = tkey(ct);
+  const int g = f >> 5;
+  if (lane == (g & 31)) {
+    E.skey[f] = k;
+    if (E.ng > 32 && (k < E.gk[g] || (k == E.gk[g] && req < E.srec[E.gf[g]].w))) {
+      E.gk[g] = k;
+      E.gf[g] = f;
+    }
+    if (k < E.lk || (k == E.lk && req < E.srec[E.lf].w)) {
+      E.lk = k;
+      E.lf = f;
+    }
+  }
+  if (k < E.kc || (k == E.kc && req < E.srec[E.fc].w)) {
+    E.kc = k;
+    E.fc = f;
+  }
+  if (lane < 3) E.rp[req] = lane == 0 ? t : (lane == 1 ? ft : ct);
+  if (E.ctl) {
+    if (lane == 0) {
+      c.pend_ft(E.cur)[E.np] = ft;
+      c.pend_tt(E.cur)[E.np] = __dsub_rn(ft, a);
+    }
+    E.np++;
+    const uint64_t kf = tkey(ft);
+    if (kf < E.mft) E.mft = kf;
+  }
+  __syncwarp();
+}
+
+// Takes the earliest completion out and completes it: the slot is free, the
+// worker's next queued request starts.
+template <bool WIDE>
+__device__ __forceinline__ void ev_complete(SimCtx& c, IdsEvents<WIDE>& E, int lane) {
+  const int f = E.fc, g = f >> 5;
+  const double t = tval(E.kc);
+  const int4 r = E.srec[f];
+  const int j = r.x;
+  // the group without f, then the earliest of all groups
+  const int s = 32 * g + lane;
+  uint64_t k = E.skey[s];
+  if (s == f) {
+    k = KEY_NONE;
+    E.skey[s] = KEY_NONE;
+  }
+  ev_min(E, k, s, E.kc, E.fc);
+  if (E.ng > 1) {
+    if (lane == (g & 31)) {
+      E.lk = E.kc;
+      E.lf = E.fc;
+      if (E.ng > 32) {
+        E.gk[g] = E.kc;
+        E.gf[g] = E.fc;
+        for (int q = lane; q < E.ng; q += 32) {
+          const uint64_t kq = E.gk[q];
+          if (kq < E.lk || (kq == E.lk && kq != KEY_NONE && E.srec[E.gf[q]].w < E.srec[E.lf].w)) {
+            E.lk = kq;
+            E.lf = E.gf[q];
+          }
+        }
+      }
+    }
+    ev_min(E, E.lk, E.lf, E.kc, E.fc);
+  } else if (lane == 0) {
+    E.lk = E.kc;
+    E.lf = E.fc;
+  }
+  if (lane == 0) E.freestk[E.nfree] = f;
+  E.nfree++;
+  E.inflight--;
+  E.add(E.A, j, -r.y, lane);
+  const int f2 = E.get(E.qh, j);
+  if (f2 < 0) {
+    E.add(E.serv, j, -1, lane);
+    __syncwarp();
+  } else {   // (as many in service as before)
+    const int4 r2 = E.srec[f2];
+    E.put(E.qh, j, r2.z, lane);
+    if (r2.z < 0) E.put(E.qt, j, -1, lane);
+    const double ft = __dadd_rn(t, __dsub_rn(ev_f(c, E.get(E.serv, j)), E.so[f2]));
+    ev_start(c, E, f2, r2.w, t, ft, __dadd_rn(ft, E.soitl[f2]), E.sa[f2], lane);
+  }
+}
+
+// A controller sample is due (at E.tick): with first tokens before it the
+// window's P99, else none.
+template <bool WIDE>
+__device__ __forceinline__ void ev_sample(SimCtx& c, IdsEvents<WIDE>& E, int lane) {
+  SimScalars& S = *c.S;
+  if (E.mft >= E.tick) {
+    ids_tick_empty(S, *c.L, lane);
+  } else {
+    if (lane == 0) {
+      S.np = E.np;
+      S.pend_cur = E.cur;
+    }
+    __syncwarp();
+    ids_tick(S, *c.L, c.pend_ft0, c.b->pend_cap, lane);
+    E.np = (int)S.np;
+    E.cur = S.pend_cur;
+    E.mft = tkey(S.min_ft);
+  }
+  E.tick = tkey(S.tick_t);
+}
+
+// Request i's arrival: every event before it in time order (completions,
+// controller samples, steps of the load-spike schedule; ties in that order),
+// then what its choice needs.  drain: past the last request, the completions
+// that remain (they start the queued requests).
+template <bool WIDE>
+__device__ __forceinline__ void ev_arrive(SimCtx& c, IdsShared& Sh, IdsEvents<WIDE>& E, int64_t i,
+                                          bool drain, float* act, int* nfz, int lane) {
+  SimScalars& S = *c.S;
+  const IdsReq& q = Sh.q[i & (IDS_RING - 1)];
+  const int p = (int)(i & 1), W = c.L->mc.W;
+  if (!drain && q.nb > (int)c.L->g.K) {
+    if (lane == 0) Sh.stat[p] = S.status = RS_ERR_CAPACITY;
+    return;
+  }
+  const uint64_t krel = tkey(q.rel);
+  uint64_t ka = E.pk;              // while waiting: the time reached
+  uint64_t lim = drain ? KEY_NONE - 1 : KEY_INF - 1;   // events up to here are due
+  if (drain) E.tick = KEY_NONE;
+  int conc = E.conc;
+  bool wait = !drain, mid = false, step = false, ok = true;
+  for (;;) {
+    if (wait) {
+      // closed-loop client (§7.4): until fewer than C(t) requests are in flight
+      if (E.spike) {
+        const SimDesc& d = *c.d;
+        mid = ka >= tkey(d.c_t1);
+        const bool end = ka >= tkey(d.c_t2);
+        step = !end;
+        conc = end ? d.c_end : (mid ? d.c_mid : d.C);
+        lim = end ? KEY_INF - 1 : tkey(mid ? d.c_t2 : d.c_t1);
+      }
+      if (E.inflight < conc) {
+        wait = false;
+        if (krel > ka) ka = krel;
+        lim = ka < KEY_INF ? ka : KEY_INF - 1;
+      }
+    }
+    if (E.kc <= lim && E.kc <= E.tick) {
+      if (wait && E.kc > ka) ka = E.kc;
+      ev_complete(c, E, lane);
+    } else if (E.tick <= lim) {
+      ev_sample(c, E, lane);
+      if (S.status != RS_OK) {
+        ok = false;
+        break;
+      }
+    } else if (!wait) {
+      break;
+    } else if (step) {
+      ka = tkey(mid ? c.d->c_t2 : c.d->c_t1);   // the schedule steps
+    } else {   // cannot happen: a request in flight is in service
+      if (lane == 0) S.status = RS_ERR_TIMEOUT;
+      ok = false;
+      break;
+    }
+  }
+  if (drain) return;
+  E.pk = ka;
+  E.prev = tval(ka);
+#pragma unroll
+  for (int h = 0; h < IdsEvents<WIDE>::H; h++) {
+    const int j = lane + 32 * h;
+    if (j < W) {
+      act[p * W + j] = __int2float_rn(E.A[h]);
+      nfz[p * W + j] = min(E.serv[h] + 1, c.L->mc.cap - 1);
+    }
+  }
+  if (lane == 0) {
+    IdsArrival ar;
+    ar.a = E.prev;
+    ar.tau = E.tau;
+    ar.omega = E.omega;
+    if (E.ctl && c.d->policy != RS_POLICY_LOADBAL && S.regime > 0) {
+      ar.tau = c.L->mc.regime_tau[S.regime];
+      ar.omega = c.L->mc.regime_omega[S.regime];
+    }
+    Sh.pub[p] = ar;
+    if (!ok) Sh.stat[p] = S.status;
   }
 }
 
@@ -938,7 +1431,7 @@ __device__ __forceinline__ void ids_stage(const SimCtx& c, IdsShared& Sh, const 
     q.nbt = (int)((L + 15) >> 4);
     q.blk = (L + r.O + 15) >> 4;
     q.phase = 0;
-    q.inv = q.nbt > 0 ? __ddiv_rn(1.0, (double)q.nbt) : 0.0;
+    if (!c.b->wco_tab) q.inv = q.nbt > 0 ? __ddiv_rn(1.0, (double)q.nbt) : 0.0;
     const uint4 x = philox4x32_10(make_uint4((uint32_t)i, (uint32_t)((uint64_t)i >> 32), 0u, TAG_SIM),
                                   make_uint2((uint32_t)c.d->seed, (uint32_t)(c.d->seed >> 32)));
     q.dx = x.x;
@@ -948,11 +1441,13 @@ __device__ __forceinline__ void ids_stage(const SimCtx& c, IdsShared& Sh, const 
 
 // ------------------------------------------------------------ the kernel
 
-template <int NU, int MINB, bool SG>
+// VAR 0: an update warp per worker (planned updates); 1: up to 32 workers; 2: up to 64.
+template <int NU, int MINB, bool SG, int VAR>
 __global__ void __launch_bounds__((NU + 2) * 32, MINB)
     k_sim_ids(const SimDesc* __restrict__ descs, const __grid_constant__ SimBuffers b,
               const __grid_constant__ SimLaunch L) {
   constexpr int NT = (NU + 2) * 32, NTU = NU * 32;
+  constexpr bool WIDE = VAR == 2, PLAN = VAR == 0;
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ SimScalars S;
   __shared__ IdsShared Sh;
@@ -1008,6 +1503,9 @@ __global__ void __launch_bounds__((NU + 2) * 32, MINB)
   const size_t nre = d.nre;
   const int64_t n = d.n_req;
 
+  int policy = d.policy;
+  asm volatile("" : "+r"(policy));   // (held in a register)
+
   // ---- initial state: empty caches, idle workers
   {
     const size_t nst = (size_t)W * nre;   // (nre: a multiple of 4)
@@ -1037,109 +1535,269 @@ __global__ void __launch_bounds__((NU + 2) * 32, MINB)
       Sh.err = 0;
     }
   }
-  // ---- prologue: the first requests staged
-  IdsRaw raw;   // (staging warp) the request after the last one staged
-  if (warp == NU + 1) {
-    for (int64_t i = 0; i < 3 && i < n; i++) {
-      raw = ids_read(d, i);
-      ids_stage(c, Sh, raw, i, codes, nbcap, lane);
-    }
-    if (n > 3) raw = ids_read(d, 3);
-    cp_async_wait_all();
-  }
   __syncthreads();
 
   if (warp < NU) {
     // ================ update warps
-    const IdsScratch sc = ids_scratch(b.scratch + (size_t)sid * ids_scratch_bytes(L.nbmax), L.nbmax);
+    unsigned char* scratch = b.scratch + (size_t)sid * ids_scratch_bytes(L.nbmax);
     unsigned cnt = 0;
-    if (n > 0 && Sh.q[0].nb <= (int)L.g.K)
-      ids_probe<NU>(stamps, nre, codes, Sh.q[0].nz, W, wm, cnt);
-    for (int64_t i = 0; i < n; i++) {
-      const int p = (int)(i & 1), e = (int)(i & (IDS_RING - 1));
-      join_cta<NT>();
-      if (Sh.stat[p] != RS_OK) break;
-      const IdsReq& q = Sh.q[e];
-      const int js = ids_choice(d, q, Sh.pub[p], wm + p * W, act + p * W, W, i, lane).js;
-      if (q.dup) {
-        // two blocks of the prompt with one chained hash (a 64-bit collision)
-        if (threadIdx.x == 0) Sh.stat[p ^ 1] = RS_ERR_COLLISION;
+    auto table = [&](int j) {
+      IdsTable t;
+      t.st = stamps + j * nre;
+      t.log = b.log + ((size_t)sid * W + j) * L.g.R;
+      t.rmask = L.ids_rmask;
+      return t;
+    };
+    // request k's cached prefix on every worker (parity pk), and the plans
+    auto probe = [&](int64_t k, int pk) {
+      const int ek = (int)(k & (IDS_RING - 1));
+      const IdsReq& qk = Sh.q[ek];
+      if (qk.nb > (int)L.g.K) return;
+      const uint32_t* cd = codes + (size_t)ek * nbcap;
+      if constexpr (PLAN) {
+        if (warp >= W) return;
+        const IdsTable t = table(warp);
+        const CacheMeta m = c.wmeta[warp];
+        uint32_t* ring = win + warp * IDS_WRING;
+        uint32_t wend = max(wlen[warp], m.head);   // (a compaction sets it to 0)
+        // the ring's next entries, once a victim may be needed soon; those
+        // copied before the last time have landed
+        const uint32_t safe = wend;
+        const uint32_t to = min(m.T, m.head + IDS_WRING);
+        if (m.size + 2 * (uint32_t)L.nbmax > L.g.K && wend < to) {
+          for (uint32_t p = wend + lane; p < to; p += 32)
+            cp_async4(ring + (p & (IDS_WRING - 1)), t.log + (p & t.rmask));
+          wend = to;
+        }
+        if (lane == 0) wlen[warp] = wend;
+        asm volatile("cp.async.commit_group;\ncp.async.wait_group 1;" ::: "memory");
+        __syncwarp();
+        const int mj = ids_plan(t, m, L.g.K, cd, qk.nb, qk.nz, ring, safe, Sh.plan[warp], cnt);
+        if (lane == 0) wm[pk * W + warp] = mj;
       } else {
-        IdsTable t;
-        t.st = stamps + js * nre;
-        t.log = b.log + ((size_t)sid * W + js) * L.g.R;
-        t.rmask = L.ids_rmask;
-        ids_update<NTU>(c, Sh, t, c.wmeta + js, codes + (size_t)e * nbcap, q, sc,
-                        win + (size_t)js * NTU, whead + js, wlen + js, i);
-        if (threadIdx.x == 0 && Sh.err) Sh.stat[p ^ 1] = Sh.err;
+        ids_probe<NU>(stamps, nre, cd, qk.nz, W, wm + pk * W, cnt);
       }
-      grp_bar<NTU>();   // the update's stamps, before the next probe
-      if (i + 1 < n) {
-        const int e1 = (int)((i + 1) & (IDS_RING - 1));
-        const IdsReq& q1 = Sh.q[e1];
-        if (q1.nb <= (int)L.g.K)
-          ids_probe<NU>(stamps, nre, codes + (size_t)e1 * nbcap, q1.nz, W, wm + (p ^ 1) * W, cnt);
+    };
+    join_cta<NT>();   // the first requests are staged
+#pragma unroll 1
+    for (int64_t i = -1; i < n; i++) {
+      const int p = (int)(i & 1), e = (int)(i & (IDS_RING - 1));
+      if (i >= 0) {
+        join_cta<NT>();
+        if (Sh.stat[p] != RS_OK) break;
+        const IdsReq& q = Sh.q[e];
+        choice_wait<NT>();
+        const int js = Sh.js;
+        if (q.dup) {
+          // two blocks of the prompt with one chained hash (a 64-bit collision)
+          if (threadIdx.x == 0) Sh.stat[p ^ 1] = RS_ERR_COLLISION;
+        } else {
+          const IdsTable t = table(js);
+          const uint32_t* cd = codes + (size_t)e * nbcap;
+          if (PLAN && Sh.plan[js].step != IDS_GENERAL) {
+            ids_apply<NTU>(t, c.wmeta + js, Sh.plan[js], win + js * IDS_WRING, cd, q);
+          } else {
+            if constexpr (PLAN)
+              ids_update_unplanned<NTU>(S, Sh, L.g.K, L.nbmax, t, c.wmeta + js, cd, q, scratch, wlen + js, i);
+            else
+              ids_update<NTU, true>(S, Sh, L.g.K, L.nbmax, t, c.wmeta + js, cd, q, scratch,
+                                    win + (size_t)js * IDS_WIN, whead + js, wlen + js, i);
+            if (threadIdx.x == 0 && Sh.err) Sh.stat[p ^ 1] = Sh.err;
+          }
+        }
+        grp_bar<NTU>();   // the update's stamps, before the next probe
+        if (PLAN && warp == js && Sh.plan[js].step != IDS_GENERAL && !q.dup) {
+          // (every update warp has read the old state)
+          if (lane == 0) {
+            CacheMeta m = c.wmeta[js];
+            const IdsPlan& P = Sh.plan[js];
+            m.size += P.nabs - P.E;
+            m.head += P.step;
+            m.T += (uint32_t)q.nb;
+            c.wmeta[js] = m;
+            S.inserted += P.nabs;
+            if (P.E > 0) {
+              S.evicted += P.E;
+              if (S.first_evict_i < 0) {
+                // the first update that evicted; resident blocks = inserted - evicted
+                S.first_evict_i = i;
+                S.first_live = S.inserted - S.evicted;
+              }
+            }
+          }
+          __syncwarp();
+        }
       }
+      if (i + 1 < n) probe(i + 1, p ^ 1);
     }
     cp_async_wait_all();
     cnt = __reduce_add_sync(FULL_MASK, cnt);
     if (lane == 0) atomicAdd(&S.probes, (unsigned long long)cnt);
   } else if (warp == NU) {
     // ================ control warp
-    if (n > 0) ids_arrive(c, Sh, 0, act, nfz, lane);
-    for (int64_t i = 0; i < n; i++) {
-      const int p = (int)(i & 1), e = (int)(i & (IDS_RING - 1));
-      join_cta<NT>();
-      if (Sh.stat[p] != RS_OK) break;
-      const IdsReq& q = Sh.q[e];
-      // w_c o_ij of every worker: m / nbt correctly rounded from the rounded
-      // reciprocal (one exact remainder and one correction: Markstein 1990)
-      double wco[2];
+    IdsEvents<WIDE> E;
+    if constexpr (!SG) {
+      E.lk = E.kc = KEY_NONE;
+      E.lf = E.fc = 0;
 #pragma unroll
-      for (int h = 0; h < 2; h++) {
-        const int j = lane + 32 * h;
-        wco[h] = 0.0;
-        if (j < W) {
-          const double m = (double)wm[p * W + j], nd = (double)q.nbt;
-          const double q0 = __dmul_rn(m, q.inv);
-          const double r = __fma_rn(-q0, nd, m);
-          wco[h] = __dmul_rn(mc.w_c, __fma_rn(r, q.inv, q0));
+      for (int h = 0; h < E.H; h++) {
+        E.A[h] = E.serv[h] = 0;
+        E.qh[h] = E.qt[h] = -1;
+      }
+      E.inflight = E.np = E.cur = 0;
+      E.nfree = max(d.C, max(d.c_mid, d.c_end));
+      E.ng = (E.nfree + 31) >> 5;
+      E.mft = KEY_INF;
+      E.tick = d.controller ? tkey(mc.dt) : KEY_INF;
+      E.prev = 0.0;
+      E.pk = tkey(0.0);
+      // held in registers: a later load of the descriptor would be on the path
+      E.conc = d.C;
+      E.ctl = d.controller;
+      E.spike = d.c_mid > 0;
+      E.tau = d.policy == RS_POLICY_LOADBAL ? 0.0f : d.tau;
+      E.omega = d.policy == RS_POLICY_LOADBAL ? 0.0f : d.omega;
+      asm volatile("" : "+r"(E.conc), "+r"(E.ctl), "+r"(E.spike), "+f"(E.tau), "+f"(E.omega));
+      E.skey = c.h_k;
+      E.srec = reinterpret_cast<int4*>(smem + lay.srec);
+      E.gk = reinterpret_cast<uint64_t*>(smem + lay.gk);
+      E.gf = reinterpret_cast<int*>(smem + lay.gf);
+      E.sa = c.f_a;
+      E.so = c.f_o;
+      E.soitl = c.f_oitl;
+      E.freestk = c.freestk;
+      E.rp = (lane == 0 ? b.rec.start : (lane == 1 ? b.rec.first_token : b.rec.completion)) + d.rec_base;
+      for (int f = lane; f < 32 * E.ng; f += 32) E.skey[f] = KEY_NONE;
+      if (E.ng > 32)
+        for (int g = lane; g < E.ng; g += 32) {
+          E.gk[g] = KEY_NONE;
+          E.gf[g] = 0;
+        }
+      __syncwarp();
+    }
+    join_cta<NT>();   // the first requests are staged
+#pragma unroll 1
+    for (int64_t i = -1; i < n; i++) {
+      const int p = (int)(i & 1), e = (int)(i & (IDS_RING - 1));
+      if (i >= 0) {
+        join_cta<NT>();
+        if (Sh.stat[p] != RS_OK) break;
+        const IdsReq& q = Sh.q[e];
+        // w_c o_ij of workers lane, lane + 32: from the table of every (nbt, m),
+        // or m / nbt correctly rounded from the rounded reciprocal (one exact
+        // remainder and one correction: Markstein 1990)
+        constexpr int H = IdsEvents<WIDE>::H;
+        double wco[H];
+#pragma unroll
+        for (int h = 0; h < H; h++) {
+          const int j = lane + 32 * h;
+          const int m = j < W ? wm[p * W + j] : 0;
+          if (b.wco_tab) {
+            wco[h] = __ldg(b.wco_tab + (size_t)q.nbt * b.wco_dim + m);
+          } else {
+            const double md = (double)m, nd = (double)q.nbt;
+            const double q0 = __dmul_rn(md, q.inv);
+            wco[h] = __dmul_rn(mc.w_c, __fma_rn(__fma_rn(-q0, nd, md), q.inv, q0));
+          }
+        }
+        double ft[H], ct[H];
+        if constexpr (!SG) {
+          // first token and completion of a service that starts on each worker now
+#pragma unroll
+          for (int h = 0; h < H; h++) {
+            const int ns = min(E.serv[h] + 1, mc.cap - 1);
+            ft[h] = __dadd_rn(E.prev, __dsub_rn(ev_f(c, ns), wco[h]));
+            ct[h] = __dadd_rn(ft[h], q.oitl);
+          }
+        }
+        choice_wait<NT>();
+        const int js = Sh.js;
+        auto of = [&](const double (&v)[H]) {
+          double x = __shfl_sync(FULL_MASK, v[0], js & 31);
+          if (WIDE) {
+            const double y = __shfl_sync(FULL_MASK, v[H - 1], js & 31);
+            if (js >= 32) x = y;
+          }
+          return x;
+        };
+        if constexpr (!SG) {
+          // request i's load and service start on worker js
+          const int f = E.freestk[--E.nfree];
+          E.inflight++;
+          E.add(E.A, js, (int)q.blk, lane);
+          if (lane == 0) E.srec[f] = make_int4(js, (int)q.blk, -1, (int)i);
+          if (E.get(E.serv, js) < mc.cap - 1) {
+            E.add(E.serv, js, 1, lane);
+            ev_start(c, E, f, (int)i, E.prev, of(ft), of(ct), E.prev, lane);
+          } else {
+            const int qt = E.get(E.qt, js);
+            const double w = of(wco);
+            if (lane == 0) {
+              E.sa[f] = E.prev;
+              E.so[f] = w;
+              E.soitl[f] = q.oitl;
+              if (qt >= 0) E.srec[qt].z = f;
+            }
+            if (qt < 0) E.put(E.qh, js, f, lane);
+            E.put(E.qt, js, f, lane);
+            __syncwarp();
+          }
+          if (lane == 0) S.n_routed = i + 1;
+        } else {
+          const double w = of(wco);
+          if (lane == 0) {
+            S.jstar = js;
+            book_request<false>(c, q, i, w);
+          }
+          __syncwarp();
         }
       }
-      const int js = ids_choice(d, q, Sh.pub[p], wm + p * W, act + p * W, W, i, lane).js;
-      const double w0 = __shfl_sync(FULL_MASK, wco[0], js & 31);
-      const double w1 = __shfl_sync(FULL_MASK, wco[1], js & 31);
-      if (lane == 0) {
-        S.jstar = js;
-        book_request<false>(c, q, i, js < 32 ? w0 : w1);
-      }
-      __syncwarp();
-      if (i + 1 < n) ids_arrive(c, Sh, i + 1, act, nfz, lane);
+      if constexpr (!SG)
+        ev_arrive(c, Sh, E, i + 1, i + 1 == n, act, nfz, lane);
+      else if (i + 1 < n)
+        ids_arrive(c, Sh, i + 1, act, nfz, lane);
     }
-    // drain: remaining completions start the queued requests
-    if (lane == 0 && S.status == RS_OK && Sh.stat[0] == RS_OK && Sh.stat[1] == RS_OK)
-      while (S.nheap > 0) {
-        uint64_t k;
-        int f;
-        heap_pop(c, &k, &f);
-        complete(c, f, tval(k));
-      }
+    if constexpr (SG) {
+      // drain: remaining completions start the queued requests
+      if (lane == 0 && S.status == RS_OK && Sh.stat[0] == RS_OK && Sh.stat[1] == RS_OK)
+        while (S.nheap > 0) {
+          uint64_t k;
+          int f;
+          heap_pop(c, &k, &f);
+          complete(c, f, tval(k));
+        }
+    }
   } else {
     // ================ staging warp
     int64_t hit = 0, pbl = 0, hashed = 0, sampled = 0;
     const bool eq2 = d.policy == RS_POLICY_DYNAMO || d.policy == RS_POLICY_LOADBAL;
-    for (int64_t i = 0; i < n; i++) {
+    IdsRaw raw;   // the request after the last one staged
+    if (n > 0) raw = ids_read(d, 0);
+    // (from request 0 - 3: each turn stages three requests ahead)
+#pragma unroll 1
+    for (int64_t i = -3; i < n; i++) {
       const int p = (int)(i & 1), e = (int)(i & (IDS_RING - 1));
-      join_cta<NT>();
-      if (Sh.stat[p] != RS_OK) break;
-      // request i+3 first: its copies run beside the records
+      const IdsReq& q = Sh.q[e];
+      IdsChoice ch;
+      if (i >= 0) {
+        join_cta<NT>();
+        if (Sh.stat[p] != RS_OK) break;
+        ch = ids_choice<WIDE>(policy, q, Sh.pub[p], wm + p * W, act + p * W, W, i, lane);
+        if (lane == 0) Sh.js = ch.js;
+        choice_made<NT>();
+      }
       if (i + 3 < n) {
         ids_stage(c, Sh, raw, i + 3, codes, nbcap, lane);
         if (i + 4 < n) raw = ids_read(d, i + 4);
       }
       asm volatile("cp.async.commit_group;" ::: "memory");
-      const IdsReq& q = Sh.q[e];
-      const IdsChoice ch = ids_choice(d, q, Sh.pub[p], wm + p * W, act + p * W, W, i, lane);
+      if (i < 0) {
+        if (i == -1) {
+          cp_async_wait_all();
+          join_cta<NT>();
+        }
+        continue;
+      }
       const int64_t row = d.rec_base + i;
       int pb = 0;
       float c2 = __int_as_float(0x7F800000);
@@ -1196,9 +1854,11 @@ __global__ void __launch_bounds__((NU + 2) * 32, MINB)
     if (S.status == RS_OK)
       for (int64_t q = threadIdx.x; q < S.n_routed; q += NT) {
         const int64_t row = d.rec_base + q;
-        const double ct = b.rec.completion[row];
-        st = __dadd_rn(st, b.rec.ttft[row]);
-        se = __dadd_rn(se, __dsub_rn(ct, b.rec.arrival[row]));
+        const double ct = b.rec.completion[row], a = b.rec.arrival[row];
+        const double tt = __dsub_rn(b.rec.first_token[row], a);
+        b.rec.ttft[row] = tt;
+        st = __dadd_rn(st, tt);
+        se = __dadd_rn(se, __dsub_rn(ct, a));
         mk = fmax(mk, ct);
       }
     for (int o = 16; o > 0; o >>= 1) {
@@ -1246,10 +1906,15 @@ cudaError_t launch_sim_ids(const SimDesc* d_desc, const SimBuffers& b, const Sim
   const bool sg = L.slots_global != 0;
   const size_t smem = sim_ids_smem_bytes(L.mc.W, L.nbmax, L.cmax, L.mc.cap, 32 * nu, sg);
   void (*kern)(const SimDesc*, const SimBuffers, const SimLaunch);
+  const int var = L.mc.W <= nu ? 0 : (L.mc.W <= 32 ? 1 : 2);
   if (nu == 6)
-    kern = sg ? k_sim_ids<6, 2, true> : k_sim_ids<6, 2, false>;
+    kern = var == 0 ? (sg ? k_sim_ids<6, 2, true, 0> : k_sim_ids<6, 2, false, 0>)
+                    : (sg ? k_sim_ids<6, 2, true, 2>
+                          : (var == 1 ? k_sim_ids<6, 2, false, 1> : k_sim_ids<6, 2, false, 2>));
   else
-    kern = sg ? k_sim_ids<2, 5, true> : k_sim_ids<2, 5, false>;
+    kern = var == 0 ? (sg ? k_sim_ids<2, 5, true, 0> : k_sim_ids<2, 5, false, 0>)
+                    : (sg ? k_sim_ids<2, 5, true, 2>
+                          : (var == 1 ? k_sim_ids<2, 5, false, 1> : k_sim_ids<2, 5, false, 2>));
   e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   kern<<<L.nsim, (nu + 2) * 32, smem, st>>>(d_desc, b, L);

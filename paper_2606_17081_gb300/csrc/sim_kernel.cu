@@ -1066,20 +1066,22 @@ __global__ void __launch_bounds__(NT_SIM, MINB) k_sim(const SimDesc* __restrict_
 }
 
 // w_c * (m / nbt) for every cached-prefix length m <= nbmax and prompt
-// length nbt <= nbmax + 1 blocks, rounded as the latency of Eq. (9) uses it.
-__global__ void k_wco_table(double* tab, int nbmax, double w_c) {
+// length nbt <= nbmax + 1 blocks, rounded as the latency of Eq. (9) uses it:
+// rows of one m, or (by_nbt) rows of one nbt, of nbmax + 2 entries.
+__global__ void k_wco_table(double* tab, int nbmax, double w_c, bool by_nbt) {
   const int dim = nbmax + 2;
-  const int64_t total = (int64_t)(nbmax + 1) * dim;
+  const int64_t total = (int64_t)(by_nbt ? dim : nbmax + 1) * dim;
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
        e += (int64_t)gridDim.x * blockDim.x) {
-    const int m = (int)(e / dim), nbt = (int)(e % dim);
+    const int row = (int)(e / dim), col = (int)(e % dim);
+    const int m = by_nbt ? col : row, nbt = by_nbt ? row : col;
     const double o = nbt > 0 ? __ddiv_rn((double)m, (double)nbt) : 0.0;
     tab[e] = __dmul_rn(w_c, o);
   }
 }
 
-cudaError_t launch_wco_table(double* tab, int nbmax, double w_c, cudaStream_t st) {
-  k_wco_table<<<152 * 4, 256, 0, st>>>(tab, nbmax, w_c);
+cudaError_t launch_wco_table(double* tab, int nbmax, double w_c, bool by_nbt, cudaStream_t st) {
+  k_wco_table<<<152 * 4, 256, 0, st>>>(tab, nbmax, w_c, by_nbt);
   return cudaGetLastError();
 }
 
