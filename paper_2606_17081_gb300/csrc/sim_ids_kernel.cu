@@ -224,6 +224,9 @@ struct IdsShared {
   int js;                      // the chosen worker
 };
 
+// Workers per update warp up to which updates are planned before the choice.
+__host__ __device__ constexpr int ids_plan_workers(int) { return 1; }
+
 struct IdsLayout {
   size_t ftab, f_oitl, f_a, f_o, h_k, srec, gk, gf, wA, codes, meta, f_req, f_worker, f_blk, f_next, h_f,
       freestk, winserv, wqh, wqt, wm, act, nfz, whead, wlen, win;
@@ -281,7 +284,8 @@ __host__ __device__ inline IdsLayout make_ids_layout(int W, int nbmax, int cmax,
   L.nfz = take(4 * 2 * (size_t)W);
   L.whead = take(4 * (size_t)W);
   L.wlen = take(4 * (size_t)W);
-  L.win = take(4 * (size_t)W * (W <= ntu / 32 ? IDS_WRING : IDS_WIN));
+  const int nu = ntu / 32;
+  L.win = take(4 * (size_t)W * (W <= nu * ids_plan_workers(nu) ? IDS_WRING : IDS_WIN));
   L.total = o;
   L.slot_bytes = (og + 255) & ~(size_t)255;
   return L;
@@ -381,12 +385,57 @@ __device__ __forceinline__ int ids_prefix(const uint32_t* st, const uint32_t* cd
   return nz;
 }
 
-// m_j of every worker (the NU update warps); wm[j] = m_j.  Up to NU workers:
-// a warp each.  More: a warp walks four workers at a time, two chunks of 32
+// The same for the workers j[q] of the set bits of `open`, four at a time, 64
 // blocks of each in flight, until each has its first miss.
+__device__ __forceinline__ void ids_prefix4(const uint32_t* stamps, size_t nre, const int (&j)[4],
+                                            unsigned open, const uint32_t* cd, int k0, int nz,
+                                            int (&m)[4], unsigned& cnt) {
+  const int lane = (int)(threadIdx.x & 31);
+#pragma unroll
+  for (int q = 0; q < 4; q++) m[q] = nz;
+#pragma unroll 1
+  for (int k = k0; k < nz && open; k += 64) {
+    const int ka = k + lane, kb = ka + 32;
+    const uint32_t ca = ka < nz ? cd[ka] : CODE_FRESH, cb = kb < nz ? cd[kb] : CODE_FRESH;
+    uint32_t va[4], vb[4];
+#pragma unroll
+    for (int q = 0; q < 4; q++) {
+      const uint32_t* st = stamps + (size_t)j[q] * nre;
+      va[q] = vb[q] = STAMP_NONE;
+      if ((open >> q) & 1u) {
+        if (!(ca >> 31)) {
+          va[q] = st[ca];
+          cnt++;
+        }
+        if (!(cb >> 31)) {
+          vb[q] = st[cb];
+          cnt++;
+        }
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < 4; q++) {
+      const unsigned ma = __ballot_sync(FULL_MASK, ka < nz && va[q] == STAMP_NONE);
+      const unsigned mb = __ballot_sync(FULL_MASK, kb < nz && vb[q] == STAMP_NONE);
+      if (((open >> q) & 1u) && (ma | mb)) {
+        m[q] = ma ? k + __ffs(ma) - 1 : k + 32 + __ffs(mb) - 1;
+        open &= ~(1u << q);
+      }
+    }
+  }
+}
+
+// m_j of every worker (the NU update warps); wm[j] = m_j.  Up to NU workers: a
+// warp each.  Up to 4 NU: a warp walks its workers together.  More: a warp
+// looks up the first 32 blocks of B workers at once (most workers miss among
+// them: one round of loads for all), then walks those where all are present,
+// four together.  At W = 64 walks from block 0 on take 7 300 SM cycles a
+// request; at W = 6 and NU = 2 the round of first blocks takes 5 200 against
+// 3 200 for the walk.
 template <int NU>
 __device__ __forceinline__ void ids_probe(const uint32_t* stamps, size_t nre, const uint32_t* cd,
                                           int nz, int W, int* wm, unsigned& cnt) {
+  constexpr int B = NU >= 6 ? 11 : 8;
   const int warp = (int)(threadIdx.x >> 5), lane = (int)(threadIdx.x & 31);
   if (W <= NU) {
     if (warp < W) {
@@ -395,46 +444,55 @@ __device__ __forceinline__ void ids_probe(const uint32_t* stamps, size_t nre, co
     }
     return;
   }
-  for (int j0 = warp; j0 < W; j0 += 4 * NU) {
-    unsigned open = 0;   // (uniform) bit q: worker j0 + q NU still all present
-    int m[4];
+  int j[4], m[4];
+  if (W <= 4 * NU) {
+    unsigned open = 0;
 #pragma unroll
     for (int q = 0; q < 4; q++) {
-      m[q] = nz;
-      open |= (unsigned)(j0 + q * NU < W) << q;
+      j[q] = warp + q * NU;
+      open |= (unsigned)(j[q] < W) << q;
     }
+    ids_prefix4(stamps, nre, j, open, cd, 0, nz, m, cnt);
+    if (lane < 4 && warp + lane * NU < W)
+      wm[warp + lane * NU] = lane == 0 ? m[0] : (lane == 1 ? m[1] : (lane == 2 ? m[2] : m[3]));
+    return;
+  }
+  const uint32_t c = lane < nz ? cd[lane] : CODE_FRESH;
+  const bool old = !(c >> 31);
+  const uint32_t x = old ? c : 0u;
 #pragma unroll 1
-    for (int k = 0; k < nz && open; k += 64) {
-      const int ka = k + lane, kb = ka + 32;
-      const uint32_t ca = ka < nz ? cd[ka] : CODE_FRESH, cb = kb < nz ? cd[kb] : CODE_FRESH;
-      uint32_t va[4], vb[4];
+  for (int j0 = warp; j0 < W; j0 += B * NU) {
+    uint32_t v[B];
 #pragma unroll
-      for (int q = 0; q < 4; q++) {
-        const uint32_t* st = stamps + (size_t)(j0 + q * NU) * nre;
-        va[q] = vb[q] = STAMP_NONE;
-        if ((open >> q) & 1u) {
-          if (!(ca >> 31)) {
-            va[q] = st[ca];
-            cnt++;
-          }
-          if (!(cb >> 31)) {
-            vb[q] = st[cb];
-            cnt++;
-          }
-        }
-      }
+    for (int q = 0; q < B; q++)
+      v[q] = j0 + q * NU < W ? stamps[(size_t)(j0 + q * NU) * nre + x] : STAMP_NONE;
+    int mine = nz;       // lane q: m of worker j0 + q NU
+    unsigned open = 0;   // (uniform) bit q: its first 32 blocks are all present
 #pragma unroll
-      for (int q = 0; q < 4; q++) {
-        const unsigned ma = __ballot_sync(FULL_MASK, ka < nz && va[q] == STAMP_NONE);
-        const unsigned mb = __ballot_sync(FULL_MASK, kb < nz && vb[q] == STAMP_NONE);
-        if (((open >> q) & 1u) && (ma | mb)) {
-          m[q] = ma ? k + __ffs(ma) - 1 : k + 32 + __ffs(mb) - 1;
-          open &= ~(1u << q);
-        }
-      }
+    for (int q = 0; q < B; q++) {
+      const unsigned ms = __ballot_sync(FULL_MASK, lane < nz && (!old || v[q] == STAMP_NONE));
+      if (lane == q && ms) mine = __ffs(ms) - 1;
+      if (!ms && j0 + q * NU < W) open |= 1u << q;
     }
-    if (lane < 4 && j0 + lane * NU < W)
-      wm[j0 + lane * NU] = lane == 0 ? m[0] : (lane == 1 ? m[1] : (lane == 2 ? m[2] : m[3]));
+    if (old) cnt += (unsigned)min(B, (W - j0 + NU - 1) / NU);
+    if (nz <= 32) open = 0;
+#pragma unroll 1
+    while (open) {
+      int w[4];
+      unsigned some = 0;
+#pragma unroll
+      for (int q = 0; q < 4; q++) {
+        w[q] = open ? __ffs(open) - 1 : 0;
+        some |= (unsigned)(open != 0) << q;
+        open &= open - 1u;
+        j[q] = j0 + w[q] * NU;
+      }
+      ids_prefix4(stamps, nre, j, some, cd, 32, nz, m, cnt);
+#pragma unroll
+      for (int q = 0; q < 4; q++)
+        if (((some >> q) & 1u) && lane == w[q]) mine = m[q];
+    }
+    if (lane < B && j0 + lane * NU < W) wm[j0 + lane * NU] = mine;
   }
 }
 
@@ -489,32 +547,43 @@ __device__ __forceinline__ IdsChoice ids_choice(int policy, const IdsReq& q,
       }
     }
   } else if (tau > 0.0f) {
-    // Eq. (2), as select_worker_warp: one weight per lane, sums in worker order
-    float e[2];
+    // Eq. (2), as select_worker_warp: one weight per lane, summed in worker
+    // order; each lane keeps the sum at its worker, so one pass gives S, the
+    // worker where the draw falls and the sums around it
+    float e[2], at[2] = {0.0f, 0.0f};
 #pragma unroll
     for (int h = 0; h < 2; h++)
       e[h] = (h == 0 || WIDE) && lane + 32 * h < W ? exp_sm(-__fdiv_rn(__fsub_rn(r.c[h], r.best), tau)) : 0.0f;
-    float S = 0.0f;
-#pragma unroll 4
-    for (int j = 0; j < W; j++)
-      S = __fadd_rn(S, __shfl_sync(FULL_MASK, !WIDE || j < 32 ? e[0] : e[1], j & 31));
-    r.target = __fmul_rn(__fmul_rn((float)(q.dx >> 8), 0x1p-24f), S);
-    r.S = S;
-    const float qnan = __int_as_float(0x7FC00000);
     float cum = 0.0f;
-    r.lo = r.hi = qnan;
-    int pick = -1, last = r.bj;
 #pragma unroll 4
     for (int j = 0; j < W; j++) {
-      const float ej = __shfl_sync(FULL_MASK, !WIDE || j < 32 ? e[0] : e[1], j & 31);
-      cum = __fadd_rn(cum, ej);
-      if (ej > 0.0f) last = j;
-      if (pick < 0 && r.target < cum) {
-        pick = j;
-        r.hi = cum;
-      }
-      if (!(r.target < cum)) r.lo = cum;
+      cum = __fadd_rn(cum, __shfl_sync(FULL_MASK, !WIDE || j < 32 ? e[0] : e[1], j & 31));
+      if (lane == (j & 31)) at[!WIDE || j < 32 ? 0 : 1] = cum;
     }
+    r.S = cum;
+    r.target = __fmul_rn(__fmul_rn((float)(q.dx >> 8), 0x1p-24f), cum);
+    unsigned long long past = __ballot_sync(FULL_MASK, lane < W && r.target < at[0]);
+    unsigned long long some = __ballot_sync(FULL_MASK, e[0] > 0.0f);
+    if (WIDE) {
+      past |= (unsigned long long)__ballot_sync(FULL_MASK, lane + 32 < W && r.target < at[1]) << 32;
+      some |= (unsigned long long)__ballot_sync(FULL_MASK, e[1] > 0.0f) << 32;
+    }
+    const int pick = past ? __ffsll((long long)past) - 1 : -1;
+    const int last = some ? 63 - __clzll((long long)some) : r.bj;
+    // the sums do not decrease: those at or below the target come before pick
+    auto sum_at = [&](int j) {
+      float x = __shfl_sync(FULL_MASK, at[0], j & 31);
+      if (WIDE) {
+        const float y = __shfl_sync(FULL_MASK, at[1], j & 31);
+        if (j >= 32) x = y;
+      }
+      return x;
+    };
+    const float qnan = __int_as_float(0x7FC00000);
+    const int below = (pick >= 0 ? pick : W) - 1;
+    const float lo = sum_at(below >= 0 ? below : 0), hi = sum_at(pick >= 0 ? pick : 0);
+    r.lo = below >= 0 ? lo : qnan;
+    r.hi = pick >= 0 ? hi : qnan;
     r.js = pick >= 0 ? pick : last;
   }
   return r;
@@ -1441,13 +1510,14 @@ __device__ __forceinline__ void ids_stage(const SimCtx& c, IdsShared& Sh, const 
 
 // ------------------------------------------------------------ the kernel
 
-// VAR 0: an update warp per worker (planned updates); 1: up to 32 workers; 2: up to 64.
+// VAR 0: planned updates (few workers per update warp); 1: up to 32 workers; 2: up to 64.
 template <int NU, int MINB, bool SG, int VAR>
 __global__ void __launch_bounds__((NU + 2) * 32, MINB)
     k_sim_ids(const SimDesc* __restrict__ descs, const __grid_constant__ SimBuffers b,
               const __grid_constant__ SimLaunch L) {
   constexpr int NT = (NU + 2) * 32, NTU = NU * 32;
   constexpr bool WIDE = VAR == 2, PLAN = VAR == 0;
+  constexpr int PW = ids_plan_workers(NU);   // workers per update warp with planned updates
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ SimScalars S;
   __shared__ IdsShared Sh;
@@ -1555,25 +1625,40 @@ __global__ void __launch_bounds__((NU + 2) * 32, MINB)
       if (qk.nb > (int)L.g.K) return;
       const uint32_t* cd = codes + (size_t)ek * nbcap;
       if constexpr (PLAN) {
-        if (warp >= W) return;
-        const IdsTable t = table(warp);
-        const CacheMeta m = c.wmeta[warp];
-        uint32_t* ring = win + warp * IDS_WRING;
-        uint32_t wend = max(wlen[warp], m.head);   // (a compaction sets it to 0)
-        // the ring's next entries, once a victim may be needed soon; those
+        // the rings' next entries, once a victim may be needed soon; those
         // copied before the last time have landed
-        const uint32_t safe = wend;
-        const uint32_t to = min(m.T, m.head + IDS_WRING);
-        if (m.size + 2 * (uint32_t)L.nbmax > L.g.K && wend < to) {
-          for (uint32_t p = wend + lane; p < to; p += 32)
-            cp_async4(ring + (p & (IDS_WRING - 1)), t.log + (p & t.rmask));
-          wend = to;
+        uint32_t safe[PW];
+#pragma unroll
+        for (int w = 0; w < PW; w++) {
+          const int j = warp + w * NU;
+          if (j >= W) break;
+          const CacheMeta m = c.wmeta[j];
+          uint32_t wend = max(wlen[j], m.head);   // (a compaction sets it to 0)
+          safe[w] = wend;
+          const uint32_t to = min(m.T, m.head + IDS_WRING);
+          if (m.size + 2 * (uint32_t)L.nbmax > L.g.K && wend < to) {
+            const uint32_t* lg = table(j).log;
+#pragma unroll 1
+            for (uint32_t p = wend + lane; p < to; p += 32)
+              cp_async4(win + j * IDS_WRING + (p & (IDS_WRING - 1)), lg + (p & L.ids_rmask));
+            wend = to;
+          }
+          if (lane == 0) wlen[j] = wend;
         }
-        if (lane == 0) wlen[warp] = wend;
         asm volatile("cp.async.commit_group;\ncp.async.wait_group 1;" ::: "memory");
         __syncwarp();
-        const int mj = ids_plan(t, m, L.g.K, cd, qk.nb, qk.nz, ring, safe, Sh.plan[warp], cnt);
-        if (lane == 0) wm[pk * W + warp] = mj;
+#pragma unroll 1
+        for (int w = 0; w < PW; w++) {
+          const int j = warp + w * NU;
+          if (j >= W) break;
+          uint32_t sf = safe[0];
+#pragma unroll
+          for (int v = 1; v < PW; v++)
+            if (w == v) sf = safe[v];
+          const int mj = ids_plan(table(j), c.wmeta[j], L.g.K, cd, qk.nb, qk.nz, win + j * IDS_WRING, sf,
+                                  Sh.plan[j], cnt);
+          if (lane == 0) wm[pk * W + j] = mj;
+        }
       } else {
         ids_probe<NU>(stamps, nre, cd, qk.nz, W, wm + pk * W, cnt);
       }
@@ -1606,7 +1691,7 @@ __global__ void __launch_bounds__((NU + 2) * 32, MINB)
           }
         }
         grp_bar<NTU>();   // the update's stamps, before the next probe
-        if (PLAN && warp == js && Sh.plan[js].step != IDS_GENERAL && !q.dup) {
+        if (PLAN && warp == js % NU && Sh.plan[js].step != IDS_GENERAL && !q.dup) {
           // (every update warp has read the old state)
           if (lane == 0) {
             CacheMeta m = c.wmeta[js];
@@ -1906,7 +1991,7 @@ cudaError_t launch_sim_ids(const SimDesc* d_desc, const SimBuffers& b, const Sim
   const bool sg = L.slots_global != 0;
   const size_t smem = sim_ids_smem_bytes(L.mc.W, L.nbmax, L.cmax, L.mc.cap, 32 * nu, sg);
   void (*kern)(const SimDesc*, const SimBuffers, const SimLaunch);
-  const int var = L.mc.W <= nu ? 0 : (L.mc.W <= 32 ? 1 : 2);
+  const int var = L.mc.W <= nu * ids_plan_workers(nu) ? 0 : (L.mc.W <= 32 ? 1 : 2);
   if (nu == 6)
     kern = var == 0 ? (sg ? k_sim_ids<6, 2, true, 0> : k_sim_ids<6, 2, false, 0>)
                     : (sg ? k_sim_ids<6, 2, true, 2>
