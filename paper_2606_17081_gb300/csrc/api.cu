@@ -1245,6 +1245,8 @@ rs_status sweep_knee(rs_ctx* ctx, const rs_records* records, const int64_t* row_
       return fail(ctx, RS_ERR_INVALID, "sweep_start decreases at sweep %d", s);
   if (sweep_start[n_sweeps] > n_replicas)
     return fail(ctx, RS_ERR_INVALID, "sweeps reach past the replicas");
+  int64_t max_rows = 0;   // of a replica
+  for (int32_t r = 0; r < n_replicas; r++) max_rows = std::max(max_rows, row_start[r + 1] - row_start[r]);
   const size_t nr = (size_t)n_replicas, ns = (size_t)n_sweeps;
   rs_status r;
   if ((r = ensure(ctx, ctx->k_rows, (nr + 1) * 8, "knee rows")) != RS_OK) return r;
@@ -1258,7 +1260,7 @@ rs_status sweep_knee(rs_ctx* ctx, const rs_records* records, const int64_t* row_
   CK(cudaMemcpyAsync(ctx->k_rows.p, row_start, (nr + 1) * 8, cudaMemcpyHostToDevice, ctx->st), "copy");
   if (nr) CK(cudaMemcpyAsync(ctx->k_load.p, load, nr * 8, cudaMemcpyHostToDevice, ctx->st), "copy");
   CK(cudaMemcpyAsync(ctx->k_sweep.p, sweep_start, (ns + 1) * 4, cudaMemcpyHostToDevice, ctx->st), "copy");
-  CK(launch_sweep_knee(records->worker, records->ttft, P<int64_t>(ctx->k_rows), n_replicas,
+  CK(launch_sweep_knee(records->worker, records->ttft, P<int64_t>(ctx->k_rows), n_replicas, max_rows,
                        P<double>(ctx->k_load), P<int32_t>(ctx->k_sweep), n_sweeps, pct, theta,
                        P<double>(ctx->k_stat), P<double>(ctx->k_d1), P<double>(ctx->k_d2),
                        P<double>(ctx->k_kload), P<int32_t>(ctx->k_kidx), ctx->st),

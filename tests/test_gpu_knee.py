@@ -107,3 +107,23 @@ def test_knee_of_a_simulated_concurrency_sweep():
     assert np.array_equal(g["knee_index"], o["knee_index"])
     # the P99 grows with the concurrency level on the static sweep
     assert o["stat"][8] > o["stat"][0]
+
+
+@pytest.mark.parametrize("rows", [1, 255, 256, 257, 1023, 1025, 24576, 24577, 60000])
+def test_percentile_selection_edges(rows):
+    # around the direct ranking, one pass of the threads, the rows held on chip; values that
+    # agree in all but their lowest bits, on few distinct values, over every binade, infinities
+    rng = np.random.default_rng(rows)
+    sets = [1.0 + rng.integers(0, 1 << 12, rows) * 2.0 ** -52, rng.choice([0.25, 0.5, np.inf], rows),
+            np.full(rows, 3.5), rng.normal(0, 1, rows) * 2.0 ** rng.integers(-1000, 1000, rows),
+            np.where(rng.random(rows) < 0.5, -0.0, 0.0), rng.lognormal(-2.0, 1.0, rows)]
+    ttft = np.concatenate(sets)
+    worker = np.where(rng.random(ttft.size) < 0.1, -1, 0).astype(np.int32)
+    worker[::rows] = 0
+    start = np.arange(len(sets) + 1, dtype=np.int64) * rows
+    ctx = rs.Context(W=1, K=16)
+    rec, _ = _device_records(worker, ttft)
+    for pct in (1, 37, 99, 100):
+        g = rs.sweep_knee(ctx.h, rec, start, np.arange(6.0), [0, 6], pct=pct)
+        o = O.sweep_knee(worker, ttft, start, np.arange(6.0), [0, 6], pct=pct)
+        assert _same(g["stat"], o["stat"]) and _same(g["d1"], o["d1"]), pct
