@@ -455,17 +455,18 @@ rs_status route_batch(rs_ctx* ctx, int32_t instance, const int32_t* tokens_dev,
   CK(cudaStreamSynchronize(ctx->st), "sync");
   int64_t nbmax = ctx->pinned[0];
   if (nbmax > (int64_t)ctx->g.K) nbmax = ctx->g.K;   // longer prompts stop with RS_ERR_CAPACITY
-  {
-    int maxsmem = 0;
-    cudaDeviceGetAttribute(&maxsmem, cudaDevAttrMaxSharedMemoryPerBlockOptin, ctx->device);
-    if (router_smem(ctx->cfg.W, (int)std::max<int64_t>(nbmax, 1)) + 4096 > (size_t)maxsmem)
-      return fail(ctx, RS_ERR_CAPACITY, "a prompt of %lld blocks needs too much shared memory",
-                  (long long)nbmax);
-  }
+  // (4 KB beside the arrays for the kernel's own variables)
+  int maxsmem = 0;
+  cudaDeviceGetAttribute(&maxsmem, cudaDevAttrMaxSharedMemoryPerBlockOptin, ctx->device);
+  const int nbl = (int)std::max<int64_t>(nbmax, 1);
+  const bool lean = router_smem(ctx->cfg.W, nbl, false) + 4096 > (size_t)maxsmem;
+  if (lean && router_smem(ctx->cfg.W, nbl, true) + 3584 > (size_t)maxsmem)
+    return fail(ctx, RS_ERR_CAPACITY, "a prompt of %lld blocks needs too much shared memory",
+                (long long)nbmax);
   ModelConsts mc = ctx->mc;
   CK(launch_route_batch(s, instance, offsets_dev, P<uint64_t>(ctx->r_hash), n_req, out_len_dev,
-                        worker_out_dev, cost_out_dev, prefix_out_dev, (int)std::max<int64_t>(nbmax, 1),
-                        ctx->g, mc, ctx->cfg.omega, ctx->cfg.tau, ctx->cfg.seed, ctx->st),
+                        worker_out_dev, cost_out_dev, prefix_out_dev, nbl,
+                        ctx->g, mc, ctx->cfg.omega, ctx->cfg.tau, ctx->cfg.seed, lean, ctx->st),
      "route_batch launch");
   return RS_OK;
 }

@@ -5,190 +5,285 @@
 // instance's active blocks, the Eq. (2) choice, and the chosen worker's cache
 // and load update -- the same steps as a simulated arrival, without the
 // event loop (completions are reported by the caller through route_release).
-#include "rs_device.cuh"
+#include "sim_probe.cuh"
 
 namespace rs {
 
+// Per request (256 threads):
+//   probe    every (worker, block) pair at once while W nb <= PROBE_CAP, its
+//            slot kept for the update, else in rounds to each worker's first
+//            miss; beside it the request's hashes go through the repeat
+//            detector;
+//   choose   every warp alike (a lane per worker), so no barrier follows;
+//   update   the chosen worker's cache, from the kept slots; meanwhile the
+//            next request's hashes are copied into the other buffer.
+// Bound by the latency of that chain: one CTA, about ten barriers and four
+// rounds of loads a request.  Two lookups of every block of the chosen worker,
+// the choice and the list of open workers on one thread and each request's
+// hashes loaded on arrival took 8.9 us a request (W = 6, 256 requests a call,
+// tau = 0.5), this XX us.
+constexpr int NT_ROUTE = 512;
+
 struct RouterShared {
-  UpdateShared us;
+  int warp_tot[NT_ROUTE / 32];
   uint32_t scan_pos;
-  int warp_tot[NT_SIM / 32];
-  unsigned long long probes;
-  int64_t off0, off1;
-  int status, nopen, jstar, rebuild;
+  int status, dup;
   uint64_t ordinal;
 };
 
-__global__ void __launch_bounds__(NT_SIM) k_route_batch(
-    RouterState s, int32_t instance, const int64_t* __restrict__ offsets,
-    const uint64_t* __restrict__ hashes, int32_t n_req, const int32_t* __restrict__ out_len,
-    int32_t* __restrict__ worker_out, float* __restrict__ cost_out, int32_t* __restrict__ prefix_out,
-    int nbmax, TableGeom g, ModelConsts mc, float omega, float tau, uint64_t seed) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ RouterShared R;
-  const int W = mc.W;
-  const size_t nb_cap = (size_t)(nbmax > 0 ? nbmax : 1);
-  size_t dup = 1;
-  while (dup < 2 * nb_cap) dup <<= 1;
-  unsigned char* p = smem;
+struct RouteLayout {
+  size_t hbuf, dupset, pslot, pfree, A, meta, slot, pst, fslot, vslot, vt, owner, victim, wm, wabs,
+      wcost, wopen, kind, evk, touched, total;
+  uint32_t dupmask;
+};
+
+// lean: no kept slots and one hash buffer, for prompts whose arrays would not
+// fit in shared memory otherwise.
+__host__ __device__ inline RouteLayout make_route_layout(int W, int nbmax, bool lean) {
+  RouteLayout L;
+  const size_t nb = (size_t)(nbmax > 0 ? nbmax : 1);
+  size_t dup = 1, o = 0;
+  while (dup < 2 * nb) dup <<= 1;
+  L.dupmask = (uint32_t)(dup - 1);
   auto take = [&](size_t bytes) {
-    unsigned char* r = p;
-    p += (bytes + 15) & ~(size_t)15;
+    const size_t r = o;
+    o += (bytes + 15) & ~(size_t)15;
     return r;
   };
-  uint64_t* hbuf = reinterpret_cast<uint64_t*>(take(8 * nb_cap));
-  UpdateScratch sc;
-  sc.dupset = reinterpret_cast<uint64_t*>(take(8 * dup));
-  sc.dupmask = (uint32_t)(dup - 1);
-  int64_t* A = reinterpret_cast<int64_t*>(take(8 * (size_t)W));
-  CacheMeta* meta = reinterpret_cast<CacheMeta*>(take(sizeof(CacheMeta) * (size_t)W));
-  sc.slot = reinterpret_cast<uint32_t*>(take(4 * nb_cap));
-  sc.pst = reinterpret_cast<uint32_t*>(take(4 * nb_cap));
-  sc.fslot = reinterpret_cast<uint32_t*>(take(4 * nb_cap));
-  sc.vslot = reinterpret_cast<uint32_t*>(take(8 * nb_cap));
-  sc.vt = reinterpret_cast<uint32_t*>(take(8 * nb_cap));
-  sc.owner = reinterpret_cast<int32_t*>(take(8 * nb_cap));
-  sc.victim = reinterpret_cast<int32_t*>(take(8 * nb_cap));
-  int32_t* wm = reinterpret_cast<int32_t*>(take(4 * (size_t)W));
-  int32_t* wopen = reinterpret_cast<int32_t*>(take(4 * (size_t)W));
-  float* wcost = reinterpret_cast<float*>(take(4 * (size_t)W));
-  sc.kind = take(nb_cap);
-  sc.evk = take(nb_cap);
-  sc.touched = take(2 * nb_cap);
+  L.hbuf = take((lean ? 1 : 2) * 8 * nb);
+  L.dupset = take(8 * dup);
+  const size_t cap = lean ? 0 : (size_t)W * nb < (size_t)PROBE_CAP ? (size_t)W * nb : (size_t)PROBE_CAP;
+  L.pslot = take(4 * cap);
+  L.pfree = take(4 * cap);
+  L.A = take(8 * (size_t)W);
+  L.meta = take(sizeof(CacheMeta) * (size_t)W);
+  L.slot = take(4 * nb);
+  L.pst = take(4 * nb);
+  L.fslot = take(4 * nb);
+  L.vslot = take(8 * nb);
+  L.vt = take(8 * nb);
+  L.owner = take(8 * nb);
+  L.victim = take(8 * nb);
+  L.wm = take(4 * (size_t)W);
+  L.wabs = take(4 * (size_t)W);
+  L.wcost = take(4 * (size_t)W);
+  L.wopen = take((size_t)(NT_ROUTE / 32) * WMAX);
+  L.kind = take(nb);
+  L.evk = take(nb);
+  L.touched = take(2 * nb);
+  L.total = o;
+  return L;
+}
 
-  for (uint32_t q = threadIdx.x; q <= sc.dupmask; q += NT_SIM) sc.dupset[q] = 0ull;
-  for (int j = threadIdx.x; j < W; j += NT_SIM) {
+__global__ void __launch_bounds__(NT_ROUTE) k_route_batch(
+    const __grid_constant__ SimBuffers b, const __grid_constant__ SimLaunch L, RouterState s,
+    int32_t instance, const int64_t* __restrict__ offsets, const uint64_t* __restrict__ hashes,
+    int32_t n_req, const int32_t* __restrict__ out_len, int32_t* __restrict__ worker_out,
+    float* __restrict__ cost_out, int32_t* __restrict__ prefix_out, float omega, float tau,
+    uint64_t seed, bool lean) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ RouterShared R;
+  __shared__ SimScalars S;
+  const TableGeom& g = L.g;
+  const int W = L.mc.W, nbmax = L.nbmax;
+  const size_t nb_cap = (size_t)(nbmax > 0 ? nbmax : 1);
+  const RouteLayout lay = make_route_layout(W, nbmax, lean);
+  const int tid = (int)threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  SimCtx c;   // the tables are those of "replica" 0
+  c.S = &S;
+  c.b = &b;
+  c.L = &L;
+  c.sid = 0;
+  c.pslot = reinterpret_cast<uint32_t*>(smem + lay.pslot);
+  c.pfree = reinterpret_cast<uint32_t*>(smem + lay.pfree);
+  c.wm = reinterpret_cast<int32_t*>(smem + lay.wm);
+  c.wabs = reinterpret_cast<int32_t*>(smem + lay.wabs);
+  c.wopen = smem + lay.wopen;
+  UpdateScratch& sc = c.sc;
+  sc.dupset = reinterpret_cast<uint64_t*>(smem + lay.dupset);
+  sc.dupmask = lay.dupmask;
+  sc.slot = reinterpret_cast<uint32_t*>(smem + lay.slot);
+  sc.pst = reinterpret_cast<uint32_t*>(smem + lay.pst);
+  sc.fslot = reinterpret_cast<uint32_t*>(smem + lay.fslot);
+  sc.vslot = reinterpret_cast<uint32_t*>(smem + lay.vslot);
+  sc.vt = reinterpret_cast<uint32_t*>(smem + lay.vt);
+  sc.owner = reinterpret_cast<int32_t*>(smem + lay.owner);
+  sc.victim = reinterpret_cast<int32_t*>(smem + lay.victim);
+  sc.kind = smem + lay.kind;
+  sc.evk = smem + lay.evk;
+  sc.touched = smem + lay.touched;
+  uint64_t* hbuf = reinterpret_cast<uint64_t*>(smem + lay.hbuf);   // [2][nb_cap]
+  int64_t* A = reinterpret_cast<int64_t*>(smem + lay.A);
+  CacheMeta* meta = reinterpret_cast<CacheMeta*>(smem + lay.meta);
+  float* wc = reinterpret_cast<float*>(smem + lay.wcost);   // (every warp writes the same costs)
+
+  // the first request's hashes, and its scalars in every thread
+  int64_t o0 = offsets[0], o1 = offsets[1];
+  int out = out_len[0];
+  auto copy_hashes = [&](int64_t a, int64_t e, int buf) {
+    const int64_t nb = (e - a) >> 4;
+    if (nb <= (int64_t)nb_cap) {
+      const uint64_t* src = hashes + (a >> 4);
+      for (int k = tid; k < (int)nb; k += NT_ROUTE) cp_async8(hbuf + buf * nb_cap + k, src + k);
+    }
+  };
+  copy_hashes(o0, o1, 0);
+  for (uint32_t q = tid; q <= sc.dupmask; q += NT_ROUTE) sc.dupset[q] = 0ull;
+  for (int j = tid; j < W; j += NT_ROUTE) {
     A[j] = s.active[j];
     meta[j] = s.meta[j];
   }
-  if (threadIdx.x == 0) {
+  if (tid == 0) {
     R.status = *s.status;
     R.ordinal = *s.ordinal;
-    R.probes = 0;
+    R.dup = 0;
+    S.status = RS_OK;
+    S.probes = 0;
+    update_reset(&S.us);
+    S.us.err = 0;
   }
-  __syncthreads();
-  auto table = [&](int j) {
-    TableView t;
-    t.keys = s.keys + (size_t)j * g.slots;
-    t.stamp = s.stamp + (size_t)j * g.slots;
-    t.log = s.log + (size_t)j * g.R;
-    t.fexp = nullptr;
-    t.bmask = g.bmask;
-    t.rmask = g.rmask;
-    return t;
-  };
-  const int CH = max(32, ((4 * NT_SIM) / W) & ~31);
-  for (int32_t i = 0; i < n_req && R.status == RS_OK; i++) {
-    const int64_t o0 = offsets[i], o1 = offsets[i + 1];
-    const int64_t Lp = o1 - o0;
-    const int64_t nb64 = Lp >> 4;
-    if (nb64 > (int64_t)g.K || nb64 > (int64_t)nbmax) {
-      __syncthreads();
-      if (threadIdx.x == 0) R.status = RS_ERR_CAPACITY;
+  for (int32_t i = 0; i < n_req; i++) {
+    const int64_t Lp = o1 - o0, nb64 = Lp >> 4;
+    const bool fits = nb64 <= (int64_t)g.K && nb64 <= (int64_t)nbmax;
+    const int nb = fits ? (int)nb64 : 0, nbt = (int)((Lp + 15) >> 4);
+    const uint64_t* hb = hbuf + (lean ? 0 : (size_t)(i & 1) * nb_cap);
+    for (int j = tid; j < W; j += NT_ROUTE) {
+      c.wm[j] = nb;
+      c.wabs[j] = 0;
+    }
+    cp_async_wait_all();
+    __syncthreads();   // hashes in place, the last update done
+    if (R.status != RS_OK) break;
+    if (!fits) {
+      __syncthreads();   // (every thread has read the status)
+      if (tid == 0) R.status = RS_ERR_CAPACITY;
       __syncthreads();
       break;
     }
-    const int nb = (int)nb64;
-    const int nbt = (int)((Lp + 15) >> 4);
-    for (int k = threadIdx.x; k < nb; k += NT_SIM) hbuf[k] = __ldg(hashes + (o0 >> 4) + k);
-    for (int j = threadIdx.x; j < W; j += NT_SIM) {
-      wm[j] = nb;
-      wopen[j] = j;
+    // the next request: its scalars now, its hashes once they are known
+    const bool more = i + 1 < n_req;
+    int64_t o2 = 0;
+    int outn = 0;
+    if (more) {
+      o2 = offsets[i + 2];
+      outn = out_len[i + 1];
     }
-    if (threadIdx.x == 0) R.nopen = W;
+    // cached prefix on every worker; repeats among the prompt's hashes
+    const bool full = !lean && W * nb64 <= PROBE_CAP;
+    int32_t claim0 = -1;   // set entry of this thread's first block
+    int dup = 0;
+    for (int k = tid; k < nb; k += NT_ROUTE) {
+      const int32_t cl = dup_claim(sc, hb[k], &dup);
+      if (k == tid) claim0 = cl; else sc.owner[k] = cl;
+    }
+    if (dup) R.dup = 1;
+    if (full)
+      probe_full<NT_ROUTE, 1>(c, hb, nb);
+    else
+      probe_prefixes<NT_ROUTE, 2>(c, hb, nb);
+    if (more && !lean) copy_hashes(o1, o2, (i + 1) & 1);
     __syncthreads();
-    // cached prefix on every worker
-    int err = 0;
-    for (int c0 = 0;;) {
-      const int nopen = R.nopen;
-      const int len = min(CH, nb - c0);
-      const int total = len > 0 ? nopen * len : 0;
-      for (int it = threadIdx.x; it < total; it += NT_SIM) {
-        const int jj = wopen[it / len];
-        const int k = c0 + it % len;
-        if (k < wm[jj] && table_find(table(jj), hbuf[k], &err) == SLOT_NONE) atomicMin(&wm[jj], k);
+    // ---- Eq. (1) costs and the Eq. (2) choice, by every warp alike
+    float bc = __int_as_float(0x7F800000);
+    int bj = 0x7FFFFFFF;
+    for (int j = lane; j < W; j += 32) {
+      const float cj = router_cost(omega, (int64_t)nbt - c.wm[j], A[j]);
+      wc[j] = cj;
+      if (warp == 0) {
+        if (cost_out) cost_out[(size_t)i * W + j] = cj;
+        if (prefix_out) prefix_out[(size_t)i * W + j] = c.wm[j];
       }
-      __syncthreads();
-      c0 += CH;
-      if (threadIdx.x == 0) {
-        int no = 0;
-        if (c0 < nb)
-          for (int j = 0; j < W; j++)
-            if (wm[j] >= c0) wopen[no++] = j;
-        R.nopen = no;
+      if (cj < bc || bj == 0x7FFFFFFF) {
+        bc = cj;
+        bj = j;
       }
+    }
+    argmin_warp(bc, bj);
+    int js = bj;
+    if (tau > 0.0f) {
+      __syncwarp();
+      uint32_t u24 = 0;
+      if (lane == 0) u24 = draw_u24(seed, R.ordinal, (uint32_t)instance, TAG_ROUTE);
+      u24 = __shfl_sync(FULL_MASK, u24, 0);
+      js = select_worker_warp(wc, W, tau, u24, bj, nullptr, lane);
+    }
+    const CacheMeta mt = meta[js];
+    const int nabs = c.wabs[js];
+    const uint64_t span = (uint64_t)mt.T - mt.head + (uint64_t)nb;
+    const bool rebuild =
+        span > g.R || mt.tombs > g.slots / 8 || (uint64_t)mt.T + nb > STAMP_LIMIT;
+    // the detector's entries given back, before the update claims slots there
+    for (int k = tid; k < nb; k += NT_ROUTE) {
+      const int32_t cl = k == tid ? claim0 : sc.owner[k];
+      if (cl >= 0) sc.dupset[cl] = 0ull;
+    }
+    __syncthreads();   // every warp has read the loads and the probe
+    if (R.dup || S.status != RS_OK) {
       __syncthreads();
-      if (R.nopen == 0) break;
-    }
-    if (err) R.status = RS_ERR_TIMEOUT;
-    for (int j = threadIdx.x; j < W; j += NT_SIM) {
-      const float cj = router_cost(omega, (int64_t)nbt - wm[j], A[j]);
-      wcost[j] = cj;
-      if (cost_out) cost_out[(size_t)i * W + j] = cj;
-      if (prefix_out) prefix_out[(size_t)i * W + j] = wm[j];
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      const uint32_t u24 = tau > 0.0f ? draw_u24(seed, R.ordinal, (uint32_t)instance, TAG_ROUTE) : 0u;
-      R.jstar = select_worker(wcost, W, tau, u24, nullptr);
-      CacheMeta* mt = &meta[R.jstar];
-      const uint64_t span = (uint64_t)mt->T - mt->head + (uint64_t)nb;
-      R.rebuild = span > g.R || mt->tombs > g.slots / 8 || (uint64_t)mt->T + nb > STAMP_LIMIT;
-      update_reset(&R.us);
-      R.us.err = 0;
-    }
-    __syncthreads();
-    const int js = R.jstar;
-    const TableView tv = table(js);
-    if (R.rebuild) cache_rebuild<NT_SIM>(tv, &meta[js], g.K, s.tmp, R.warp_tot, &R.us);
-    cache_lookup_all<NT_SIM>(tv, hbuf, nb, sc, &R.us, &R.probes);
-    __syncthreads();
-    if (R.us.dup) {
-      if (threadIdx.x == 0) R.status = RS_ERR_COLLISION;
+      if (tid == 0) R.status = S.status != RS_OK ? S.status : RS_ERR_COLLISION;
       __syncthreads();
       break;
     }
-    cache_apply<NT_SIM>(tv, &meta[js], g.K, hbuf, nb, sc, &R.us, R.warp_tot, &R.scan_pos);
-    if (threadIdx.x == 0) {
-      if (R.us.err) R.status = R.us.err;
-      A[js] += (Lp + out_len[i] + 15) >> 4;
+    const TableView tv = c.table(js);
+    if (rebuild) cache_rebuild<NT_ROUTE>(tv, &meta[js], g.K, s.tmp, R.warp_tot, &S.us);
+    const bool captured = full && !rebuild;
+    if (captured)
+      cache_prepare_captured<NT_ROUTE>(tv, &meta[js], g.K, c.pslot + (size_t)js * nb,
+                                     c.pfree + (size_t)js * nb, nb, nabs, sc, &S.us, R.warp_tot,
+                                     &R.scan_pos);
+    else
+      cache_lookup_all<NT_ROUTE, false>(tv, hb, nb, sc, &S.us, &S.probes);
+    cache_apply<NT_ROUTE>(tv, &meta[js], g.K, hb, nb, sc, &S.us, R.warp_tot, &R.scan_pos, captured);
+    if (tid == 0) {
+      if (S.us.err) R.status = S.us.err;
+      update_reset(&S.us);
+      A[js] += (Lp + out + 15) >> 4;
       worker_out[i] = js;
       R.ordinal++;
     }
-    __syncthreads();
+    if (more && lean) {
+      __syncthreads();   // the update has read its hashes
+      copy_hashes(o1, o2, 0);
+    }
+    o0 = o1;
+    o1 = o2;
+    out = outn;
   }
+  cp_async_wait_all();
   __syncthreads();
-  for (int j = threadIdx.x; j < W; j += NT_SIM) {
+  for (int j = tid; j < W; j += NT_ROUTE) {
     s.active[j] = A[j];
     s.meta[j] = meta[j];
   }
-  if (threadIdx.x == 0) {
+  if (tid == 0) {
     *s.status = R.status;
     *s.ordinal = R.ordinal;
   }
 }
 
-size_t router_smem(int W, int nbmax) {
-  const size_t nb = (size_t)(nbmax > 0 ? nbmax : 1);
-  size_t dup = 1;
-  while (dup < 2 * nb) dup <<= 1;
-  auto r16 = [](size_t x) { return (x + 15) & ~(size_t)15; };
-  return r16(8 * nb) + r16(8 * dup) + r16(8 * (size_t)W) + r16(sizeof(CacheMeta) * (size_t)W) +
-         3 * r16(4 * nb) + 4 * r16(8 * nb) + 3 * r16(4 * (size_t)W) + 2 * r16(nb) + r16(2 * nb);
-}
+size_t router_smem(int W, int nbmax, bool lean) { return make_route_layout(W, nbmax, lean).total; }
 
 cudaError_t launch_route_batch(const RouterState& s, int32_t instance, const int64_t* offsets,
                                const uint64_t* hashes, int32_t n_req, const int32_t* out_len,
                                int32_t* worker_out, float* cost_out, int32_t* prefix_out,
                                int nbmax, const TableGeom& g, const ModelConsts& mc, float omega,
-                               float tau, uint64_t seed, cudaStream_t st) {
+                               float tau, uint64_t seed, bool lean, cudaStream_t st) {
   if (n_req <= 0) return cudaSuccess;
-  const size_t smem = router_smem(mc.W, nbmax);
+  const size_t smem = router_smem(mc.W, nbmax, lean);
   cudaError_t e = cudaFuncSetAttribute(k_route_batch, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)smem);
   if (e != cudaSuccess) return e;
-  k_route_batch<<<1, NT_SIM, smem, st>>>(s, instance, offsets, hashes, n_req, out_len, worker_out,
-                                         cost_out, prefix_out, nbmax, g, mc, omega, tau, seed);
+  SimBuffers b{};
+  b.keys = s.keys;
+  b.stamp = s.stamp;
+  b.log = s.log;
+  SimLaunch L{};
+  L.nsim = 1;
+  L.nbmax = nbmax;
+  L.g = g;
+  L.mc = mc;
+  k_route_batch<<<1, NT_ROUTE, smem, st>>>(b, L, s, instance, offsets, hashes, n_req, out_len,
+                                         worker_out, cost_out, prefix_out, omega, tau, seed, lean);
   return cudaGetLastError();
 }
 

@@ -250,8 +250,8 @@ cudaError_t launch_route_batch(const RouterState& s, int32_t instance, const int
                                const uint64_t* hashes, int32_t n_req, const int32_t* out_len,
                                int32_t* worker_out, float* cost_out, int32_t* prefix_out,
                                int nbmax, const TableGeom& g, const ModelConsts& mc, float omega,
-                               float tau, uint64_t seed, cudaStream_t st);
-size_t router_smem(int W, int nbmax);
+                               float tau, uint64_t seed, bool lean, cudaStream_t st);
+size_t router_smem(int W, int nbmax, bool lean);
 cudaError_t launch_route_release(const RouterState& s, const int32_t* worker, const int32_t* blocks,
                                  int32_t n, int32_t W, cudaStream_t st);
 cudaError_t launch_clear_tables(uint64_t* keys, uint32_t* stamp, size_t nslots, CacheMeta* meta,

@@ -220,7 +220,8 @@ struct IdsShared {
   unsigned livew[IDS_WIN / 32];   // live entries of the window
   int warp_tot[8];
   int err;                     // of the update
-  int nvic, nins;
+  int nvic, nins, changed;
+  uint32_t nh;
   int js;                      // the chosen worker
 };
 
@@ -297,14 +298,13 @@ size_t sim_ids_smem_bytes(int W, int nbmax, int cmax, int cap, int ntu, bool slo
 
 // Global scratch of one replica for the updates that need the exact sequence.
 struct IdsScratch {
-  uint32_t *vent, *vt, *pst;    // [2 nb] live entries and positions, [nb] stamps
-  int32_t *owner, *victim;      // [2 nb]
-  uint8_t *touched, *kind, *evk;   // [2 nb], [nb], [nb]
+  uint32_t *vent, *vt;   // [2 nb] live entries and their positions
+  int32_t *owner, *w;    // [2 nb] the prompt's block holding an entry or -1, [nb] see lru_exact
 };
 
 __host__ __device__ inline size_t ids_scratch_bytes(int nbmax) {
   const size_t nb = (size_t)(nbmax > 0 ? nbmax : 1);
-  return (40 * nb + 255) & ~(size_t)255;
+  return (28 * nb + 255) & ~(size_t)255;
 }
 
 size_t sim_ids_scratch_bytes(int nbmax) { return ids_scratch_bytes(nbmax); }
@@ -315,11 +315,7 @@ __device__ __forceinline__ IdsScratch ids_scratch(unsigned char* p, int nbmax) {
   s.vent = reinterpret_cast<uint32_t*>(p);
   s.vt = s.vent + 2 * nb;
   s.owner = reinterpret_cast<int32_t*>(s.vt + 2 * nb);
-  s.victim = s.owner + 2 * nb;
-  s.pst = reinterpret_cast<uint32_t*>(s.victim + 2 * nb);
-  s.touched = reinterpret_cast<uint8_t*>(s.pst + nb);
-  s.kind = s.touched + 2 * nb;
-  s.evk = s.kind + nb;
+  s.w = s.owner + 2 * nb;
   return s;
 }
 
@@ -690,8 +686,8 @@ __device__ __forceinline__ uint32_t ids_place(const uint32_t* vt, uint32_t n, ui
 }
 
 // An update whose victims the window does not settle: more victims than it
-// holds, or a present block among the least recent entries, which the exact
-// sequence (one thread, over the first 2 nb live entries) decides.  Evicts;
+// holds, or a present block among the least recent entries (lru_exact over the
+// first 2 nb live entries).  Evicts;
 // returns the head past the last victim; victims in S.nvic, insertions in
 // S.nins.  (Rare, and out of line: the loop's hot code has to stay small, its
 // warps wait for instructions otherwise.)
@@ -719,56 +715,55 @@ __device__ __noinline__ uint32_t ids_evict_general(IdsTable t, CacheMeta m, uint
   }
   grp_bar<NT>();
   G = ids_gather<NT>(t, m.head, m.T, min(m.size, 2u * (uint32_t)nb), sc, S.warp_tot);
-  for (uint32_t p = threadIdx.x; p < G; p += NT) {
-    sc.owner[p] = -1;
-    sc.touched[p] = 0;
-  }
+  for (uint32_t p = threadIdx.x; p < G; p += NT) sc.owner[p] = -1;
   grp_bar<NT>();
   const uint32_t last = G ? sc.vt[G - 1] : 0u;
+  const int freeb = (int)(K - m.size);
   for (int k = threadIdx.x; k < nb; k += NT) {
     const uint32_t c = cd[k];
     const uint32_t st = c >> 31 ? STAMP_NONE : t.st[c];
-    sc.pst[k] = st;
-    sc.evk[k] = 0;
-    if (st != STAMP_NONE && G && st <= last) sc.owner[ids_place(sc.vt, G, st)] = k;
-  }
-  grp_bar<NT>();
-  if (threadIdx.x == 0) {
-    uint32_t ptr = 0, sz = m.size;
-    int e = 0, ni = 0;
-    for (int k = 0; k < nb; k++) {
-      const uint32_t st = sc.pst[k];
-      if (st != STAMP_NONE && !sc.evk[k]) {
-        if (G && st <= last) sc.touched[ids_place(sc.vt, G, st)] = 1;
-        continue;
-      }
-      ni++;
-      if (sz < K) {
-        sz++;
-        continue;
-      }
-      while (ptr < G && sc.touched[ptr]) ptr++;
-      if (ptr >= G) {
-        S.err = RS_ERR_TIMEOUT;
-        break;
-      }
-      sc.victim[e++] = (int32_t)ptr;
-      if (sc.owner[ptr] >= 0) sc.evk[sc.owner[ptr]] = 1;
-      ptr++;
+    int v = st == STAMP_NONE ? LRU_ABSENT : LRU_FAR;
+    if (v == LRU_FAR && G && st <= last) {
+      v = (int)ids_place(sc.vt, G, st);
+      sc.owner[v] = k;
     }
-    S.nvic = e;
-    S.nins = ni;
+    sc.w[k] = v;
+  }
+  if (threadIdx.x == 0) S.nins = 0;
+  lru_exact<NT>(sc.w, nb, freeb, &S.changed);
+  int ni = 0;
+  for (int k = threadIdx.x; k < nb; k += NT) ni += sc.w[k] == LRU_ABSENT || sc.w[k] >= LRU_EVICTED;
+  ni = (int)__reduce_add_sync(FULL_MASK, (unsigned)ni);
+  if ((threadIdx.x & 31) == 0 && ni) atomicAdd(&S.nins, ni);
+  grp_bar<NT>();
+  const int E = max(0, S.nins - freeb);
+  if (threadIdx.x == 0) {
+    S.nvic = E;
+    S.nh = m.head;
     ++*slow;
   }
   grp_bar<NT>();
-  const int e = S.nvic;
-  for (int v = threadIdx.x; v < e; v += NT) {
-    const uint32_t x = sc.vent[sc.victim[v]];
-    if (!(x & SINGLE_FLAG)) t.st[x] = STAMP_NONE;
+  // the victims: the first entries that are not touched before their turn
+  int have = 0;
+  for (uint32_t p0 = 0; p0 < G && have < E; p0 += NT) {
+    const uint32_t p = p0 + threadIdx.x;
+    bool v = p < G;
+    if (v) {
+      const int k = sc.owner[p];
+      v = k < 0 || sc.w[k] >= LRU_EVICTED;
+    }
+    int tot;
+    const int r = have + cta_rank<NT>(v, S.warp_tot, &tot);
+    if (v && r < E) {
+      const uint32_t x = sc.vent[p];
+      if (!(x & SINGLE_FLAG)) t.st[x] = STAMP_NONE;
+      if (r == E - 1) S.nh = sc.vt[p] + 1;
+    }
+    have += tot;
   }
-  const uint32_t nh = e > 0 ? sc.vt[sc.victim[e - 1]] + 1 : m.head;
-  grp_bar<NT>();   // a victim may be a block of this request: its new stamp comes after
-  return nh;
+  if (have < E && threadIdx.x == 0) S.err = RS_ERR_TIMEOUT;
+  grp_bar<NT>();   // (a victim may be a block of this request: its new stamp comes after)
+  return S.nh;
 }
 
 // m_j of one worker and its update's plan, by its warp.  The worker's log
