@@ -14,20 +14,22 @@ namespace rs {
 //            slot kept for the update, else in rounds to each worker's first
 //            miss; beside it the request's hashes go through the repeat
 //            detector;
-//   choose   every warp alike (a lane per worker), so no barrier follows;
+//   choose   the first warp, a lane per worker;
 //   update   the chosen worker's cache, from the kept slots; meanwhile the
 //            next request's hashes are copied into the other buffer.
-// Bound by the latency of that chain: one CTA, about ten barriers and four
-// rounds of loads a request.  Two lookups of every block of the chosen worker,
-// the choice and the list of open workers on one thread and each request's
-// hashes loaded on arrival took 8.9 us a request (W = 6, 256 requests a call,
-// tau = 0.5), this XX us.
+// Bound by the latency of that chain on one SM: of 14 300 cycles a request
+// (W = 6, tau = 0.5) the probe takes 4 600, the choice 3 000, the update's reads
+// 2 600 and its writes 3 700.  With two lookups of every block of the chosen
+// worker, the choice on one thread and each request's hashes loaded on arrival
+// a call of 256 requests took 2.39 ms, now 1.76; 256 threads with two lookups
+// each in flight take the same.
 constexpr int NT_ROUTE = 512;
 
 struct RouterShared {
   int warp_tot[NT_ROUTE / 32];
   uint32_t scan_pos;
-  int status, dup;
+  int status, dup, js, rebuild;
+  uint32_t u24;   // the request's draw
   uint64_t ordinal;
 };
 
@@ -181,43 +183,41 @@ __global__ void __launch_bounds__(NT_ROUTE) k_route_batch(
       probe_full<NT_ROUTE, 1>(c, hb, nb);
     else
       probe_prefixes<NT_ROUTE, 2>(c, hb, nb);
+    if (tau > 0.0f && tid == NT_ROUTE - 1) R.u24 = draw_u24(seed, R.ordinal, (uint32_t)instance, TAG_ROUTE);
     if (more && !lean) copy_hashes(o1, o2, (i + 1) & 1);
     __syncthreads();
-    // ---- Eq. (1) costs and the Eq. (2) choice, by every warp alike
-    float bc = __int_as_float(0x7F800000);
-    int bj = 0x7FFFFFFF;
-    for (int j = lane; j < W; j += 32) {
-      const float cj = router_cost(omega, (int64_t)nbt - c.wm[j], A[j]);
-      wc[j] = cj;
-      if (warp == 0) {
+    // ---- Eq. (1) costs and the Eq. (2) choice, by the first warp
+    if (warp == 0) {
+      float bc = __int_as_float(0x7F800000);
+      int bj = 0x7FFFFFFF;
+      for (int j = lane; j < W; j += 32) {
+        const float cj = router_cost(omega, (int64_t)nbt - c.wm[j], A[j]);
+        wc[j] = cj;
         if (cost_out) cost_out[(size_t)i * W + j] = cj;
         if (prefix_out) prefix_out[(size_t)i * W + j] = c.wm[j];
+        if (cj < bc || bj == 0x7FFFFFFF) {
+          bc = cj;
+          bj = j;
+        }
       }
-      if (cj < bc || bj == 0x7FFFFFFF) {
-        bc = cj;
-        bj = j;
-      }
-    }
-    argmin_warp(bc, bj);
-    int js = bj;
-    if (tau > 0.0f) {
+      argmin_warp(bc, bj);
       __syncwarp();
-      uint32_t u24 = 0;
-      if (lane == 0) u24 = draw_u24(seed, R.ordinal, (uint32_t)instance, TAG_ROUTE);
-      u24 = __shfl_sync(FULL_MASK, u24, 0);
-      js = select_worker_warp(wc, W, tau, u24, bj, nullptr, lane);
+      const int j = select_worker_warp(wc, W, tau, R.u24, bj, nullptr, lane);
+      if (lane == 0) {
+        const CacheMeta mt = meta[j];
+        const uint64_t span = (uint64_t)mt.T - mt.head + (uint64_t)nb;
+        R.js = j;
+        R.rebuild = span > g.R || mt.tombs > g.slots / 8 || (uint64_t)mt.T + nb > STAMP_LIMIT;
+      }
     }
-    const CacheMeta mt = meta[js];
-    const int nabs = c.wabs[js];
-    const uint64_t span = (uint64_t)mt.T - mt.head + (uint64_t)nb;
-    const bool rebuild =
-        span > g.R || mt.tombs > g.slots / 8 || (uint64_t)mt.T + nb > STAMP_LIMIT;
     // the detector's entries given back, before the update claims slots there
     for (int k = tid; k < nb; k += NT_ROUTE) {
       const int32_t cl = k == tid ? claim0 : sc.owner[k];
       if (cl >= 0) sc.dupset[cl] = 0ull;
     }
-    __syncthreads();   // every warp has read the loads and the probe
+    __syncthreads();
+    const int js = R.js, nabs = c.wabs[js];
+    const bool rebuild = R.rebuild;
     if (R.dup || S.status != RS_OK) {
       __syncthreads();
       if (tid == 0) R.status = S.status != RS_OK ? S.status : RS_ERR_COLLISION;

@@ -192,41 +192,45 @@ __device__ __forceinline__ int select_worker(const float* c, int W, float tau, u
 
 // select_worker computed by a whole warp (W <= 64; every lane returns the
 // same worker): lane l computes the weights of workers l and l + 32, each
-// once, and every lane then accumulates them in worker order from shuffles,
-// so the sums, the draw and the statistics are those of select_worker bit
-// for bit.  b: the lowest-index argmin of c.  ds (nullable) is written by
-// lane 0.
+// once; every lane then sums them in worker order from shuffles and keeps the
+// sum at its own workers, so one pass gives S, the worker where the draw falls
+// and the sums around it, those of select_worker bit for bit.  b: the
+// lowest-index argmin of c.  ds (nullable) is written by lane 0.
 __device__ __forceinline__ int select_worker_warp(const float* c, int W, float tau, uint32_t u24,
                                                   int b, float* ds, int lane) {
   if (tau == 0.0f) return b;
   const float cmin = c[b];
-  float e[2];
+  float e[2], at[2] = {0.0f, 0.0f};
 #pragma unroll
   for (int h = 0; h < 2; h++) {
     const int j = lane + 32 * h;
     e[h] = j < W ? exp_sm(-__fdiv_rn(__fsub_rn(c[j], cmin), tau)) : 0.0f;
   }
   float S = 0.0f;
-  for (int j = 0; j < W; j++) S = __fadd_rn(S, __shfl_sync(FULL_MASK, e[j >> 5], j & 31));
-  const float target = __fmul_rn(__fmul_rn((float)u24, 0x1p-24f), S);
-  const float qnan = __int_as_float(0x7FC00000);
-  float cum = 0.0f, lo = qnan, hi = qnan;
-  int pick = -1, last = b;
+#pragma unroll 4
   for (int j = 0; j < W; j++) {
-    const float ej = __shfl_sync(FULL_MASK, e[j >> 5], j & 31);
-    cum = __fadd_rn(cum, ej);
-    if (ej > 0.0f) last = j;
-    if (pick < 0 && target < cum) {
-      pick = j;
-      hi = cum;
-    }
-    if (!(target < cum)) lo = cum;
+    S = __fadd_rn(S, __shfl_sync(FULL_MASK, j < 32 ? e[0] : e[1], j & 31));
+    if (lane == (j & 31)) at[j >> 5] = S;
   }
-  if (ds && lane == 0) {
-    ds[0] = target;
-    ds[1] = S;
-    ds[2] = lo;
-    ds[3] = hi;
+  const float target = __fmul_rn(__fmul_rn((float)u24, 0x1p-24f), S);
+  const unsigned long long past =
+      __ballot_sync(FULL_MASK, lane < W && target < at[0]) |
+      (unsigned long long)__ballot_sync(FULL_MASK, lane + 32 < W && target < at[1]) << 32;
+  const unsigned long long some = __ballot_sync(FULL_MASK, e[0] > 0.0f) |
+                                  (unsigned long long)__ballot_sync(FULL_MASK, e[1] > 0.0f) << 32;
+  const int pick = past ? __ffsll((long long)past) - 1 : -1;
+  const int last = some ? 63 - __clzll((long long)some) : b;
+  if (ds) {   // (uniform) the sums do not decrease: those at or below the target come before pick
+    const float qnan = __int_as_float(0x7FC00000);
+    const int below = (pick >= 0 ? pick : W) - 1, lo_j = below >= 0 ? below : 0, hi_j = pick >= 0 ? pick : 0;
+    const float l0 = __shfl_sync(FULL_MASK, at[0], lo_j & 31), l1 = __shfl_sync(FULL_MASK, at[1], lo_j & 31);
+    const float h0 = __shfl_sync(FULL_MASK, at[0], hi_j & 31), h1 = __shfl_sync(FULL_MASK, at[1], hi_j & 31);
+    if (lane == 0) {
+      ds[0] = target;
+      ds[1] = S;
+      ds[2] = below >= 0 ? (lo_j < 32 ? l0 : l1) : qnan;
+      ds[3] = pick >= 0 ? (hi_j < 32 ? h0 : h1) : qnan;
+    }
   }
   return pick >= 0 ? pick : last;
 }
@@ -784,9 +788,7 @@ __device__ __forceinline__ void cache_prepare_captured(const TableView& t, const
 // E > o - T.  Every block depends on earlier ones only: the blocks are evaluated
 // together until none changes (at least one more is final after each turn, in
 // practice all after two to four).  One thread replaying the sequence took
-// most of a request's time where prompts recur after about a cache's worth of
-// others: live router, 256 requests a call at W = 6, K = 8192, 1.98 ms a call
-// against X.XX ms.
+// about 300 cycles a block.
 constexpr int LRU_ABSENT = -1, LRU_FAR = -2, LRU_EVICTED = 0x40000000;
 
 template <int NT>
