@@ -48,7 +48,7 @@ struct rs_ctx {
       rec_prefix;
   DevBuf p_cost, p_order, p_asg, p_wkey, p_wstart, p_wfill, p_wnum, p_wopt, p_wcnt, p_total,
       p_nwin, p_prob, p_wstat, p_tstat, p_wprob, p_wnext;
-  DevBuf k_rows, k_load, k_sweep, k_stat, k_d1, k_d2, k_kload, k_kidx;
+  DevBuf k_in, k_out;
   DevBuf h_tokens, h_offsets, h_release, h_outlen;
   int64_t* pinned = nullptr;   // small host staging for device -> host reads
   size_t pinned_n = 0;
@@ -323,8 +323,7 @@ void route_destroy(rs_ctx* ctx) {
                    &ctx->p_wnum, &ctx->p_wopt, &ctx->p_wcnt, &ctx->p_total, &ctx->p_nwin,
                    &ctx->p_prob, &ctx->p_wstat, &ctx->p_tstat, &ctx->p_wprob, &ctx->p_wnext,
                    &ctx->h_tokens, &ctx->h_offsets,
-                   &ctx->h_release, &ctx->h_outlen, &ctx->k_rows, &ctx->k_load, &ctx->k_sweep,
-                   &ctx->k_stat, &ctx->k_d1, &ctx->k_d2, &ctx->k_kload, &ctx->k_kidx,
+                   &ctx->h_release, &ctx->h_outlen, &ctx->k_in, &ctx->k_out,
                    &ctx->fexp, &ctx->tmpe, &ctx->djobs, &ctx->h_hashes, &ctx->i_jobs, &ctx->i_keys,
                    &ctx->i_first, &ctx->i_num, &ctx->i_ids, &ctx->i_nz, &ctx->i_count,
                    &ctx->i_stamps, &ctx->i_scratch};
@@ -335,8 +334,6 @@ void route_destroy(rs_ctx* ctx) {
   delete ctx;
 }
 
-static rs_status hash_jobs(rs_ctx* ctx, std::vector<HashJob>& jobs, int64_t* nbmax_dev);
-
 rs_status route_hash_blocks(rs_ctx* ctx, const int32_t* tokens_dev, const int64_t* offsets_dev,
                             int64_t n_req, uint64_t* hashes_dev) {
   if (!ctx) return fail(nullptr, RS_ERR_INVALID, "ctx is NULL");
@@ -345,9 +342,10 @@ rs_status route_hash_blocks(rs_ctx* ctx, const int32_t* tokens_dev, const int64_
   if (n_req == 0) return RS_OK;
   if (!tokens_dev || !offsets_dev || !hashes_dev) return fail(ctx, RS_ERR_INVALID, "NULL pointer");
   if (!aligned16(tokens_dev)) return fail(ctx, RS_ERR_INVALID, "tokens must be 16-byte aligned");
-  std::vector<HashJob> jobs(1);
-  jobs[0] = HashJob{tokens_dev, offsets_dev, hashes_dev, n_req, 0};
-  return hash_jobs(ctx, jobs, nullptr);
+  CK(launch_block_hash_one(HashJob{tokens_dev, offsets_dev, hashes_dev, n_req, 0},
+                           ctx->cfg.hash_seed, ctx->st),
+     "block hash launch");
+  return RS_OK;
 }
 
 rs_status route_dup_flags(rs_ctx* ctx, const uint64_t* hashes_dev, const int64_t* offsets_dev,
@@ -382,41 +380,40 @@ static std::vector<HashJob> group_jobs(const std::vector<HashJob>& jobs) {
   return out;
 }
 
-// Hashes every job (trace) in launches of up to HASH_MAX_JOBS traces.
-static rs_status hash_jobs(rs_ctx* ctx, std::vector<HashJob>& jobs, int64_t* nbmax_dev) {
-  if (jobs.empty()) return RS_OK;
-  rs_status r = ensure(ctx, ctx->hjobs, sizeof(HashJob) * jobs.size(), "hash jobs");
-  if (r != RS_OK) return r;
-  const std::vector<HashJob> grp = group_jobs(jobs);
-  CK(cudaMemcpyAsync(ctx->hjobs.p, grp.data(), sizeof(HashJob) * grp.size(),
-                     cudaMemcpyHostToDevice, ctx->st),
-     "copy hash jobs");
-  for (size_t g0 = 0; g0 < jobs.size(); g0 += HASH_MAX_JOBS) {
-    const size_t g1 = std::min(jobs.size(), g0 + HASH_MAX_JOBS);
-    const int64_t total = jobs[g1 - 1].req_base + jobs[g1 - 1].n_req - jobs[g0].req_base;
-    CK(launch_block_hash(P<HashJob>(ctx->hjobs) + g0, (int)(g1 - g0), total, ctx->cfg.hash_seed,
-                         nbmax_dev, ctx->st),
-       "block hash launch");
-  }
-  return RS_OK;
-}
+// Block hashes of one batch of a router instance into ctx->r_hash, sized from
+// the end of its last prompt, which is read first (synchronises), with the
+// longest prompt's full blocks into *nbmax (nullable).
+constexpr int64_t SMALL_BATCH = 4096;   // requests up to which one CTA reads the sizes
 
-// Block hashes of one batch of a router instance into ctx->r_hash (sized from
-// offsets_dev[n_req], read with a synchronising copy); nbmax_dev (nullable)
-// receives the longest prompt's full blocks.
 static rs_status hash_batch(rs_ctx* ctx, const int32_t* tokens_dev, const int64_t* offsets_dev,
-                            int64_t n_req, int64_t* nbmax_dev) {
+                            int64_t n_req, int64_t* nbmax) {
   rs_status r = ensure_pinned(ctx, 4);
   if (r != RS_OK) return r;
-  CK(cudaMemcpyAsync(ctx->pinned, offsets_dev + n_req, 8, cudaMemcpyDeviceToHost, ctx->st),
-     "read offsets");
+  const HashJob job{tokens_dev, offsets_dev, nullptr, n_req, 0};
+  if (n_req <= SMALL_BATCH) {   // straight into pinned memory
+    CK(launch_batch_sizes(offsets_dev, (int)n_req, ctx->pinned, ctx->st), "batch sizes launch");
+  } else {
+    if (nbmax) {
+      if ((r = ensure(ctx, ctx->hjobs, sizeof(HashJob), "hash jobs")) != RS_OK) return r;
+      CK(cudaMemcpyAsync(ctx->hjobs.p, &job, sizeof(HashJob), cudaMemcpyHostToDevice, ctx->st),
+         "copy hash job");
+      CK(cudaMemsetAsync(ctx->r_stats.p, 0, 8, ctx->st), "memset");
+      CK(launch_nbmax(P<HashJob>(ctx->hjobs), 1, n_req, P<int64_t>(ctx->r_stats), ctx->st),
+         "block count launch");
+      CK(cudaMemcpyAsync(ctx->pinned, ctx->r_stats.p, 8, cudaMemcpyDeviceToHost, ctx->st), "read stats");
+    }
+    CK(cudaMemcpyAsync(ctx->pinned + 1, offsets_dev + n_req, 8, cudaMemcpyDeviceToHost, ctx->st),
+       "read offsets");
+  }
   CK(cudaStreamSynchronize(ctx->st), "sync");
-  const int64_t total = ctx->pinned[0];
+  if (nbmax) *nbmax = ctx->pinned[0];
+  const int64_t total = ctx->pinned[1];
   if (total < 0) return fail(ctx, RS_ERR_INVALID, "offsets[n_req] < 0");
   if ((r = ensure(ctx, ctx->r_hash, (size_t)(total / 16 + 1) * 8, "batch hashes")) != RS_OK) return r;
-  std::vector<HashJob> jobs(1);
-  jobs[0] = HashJob{tokens_dev, offsets_dev, P<uint64_t>(ctx->r_hash), n_req, 0};
-  return hash_jobs(ctx, jobs, nbmax_dev);
+  CK(launch_block_hash_one(HashJob{tokens_dev, offsets_dev, P<uint64_t>(ctx->r_hash), n_req, 0},
+                           ctx->cfg.hash_seed, ctx->st),
+     "block hash launch");
+  return RS_OK;
 }
 
 // ---------------------------------------------------------------- live router
@@ -448,12 +445,8 @@ rs_status route_batch(rs_ctx* ctx, int32_t instance, const int32_t* tokens_dev,
   if (!tokens_dev || !offsets_dev || !out_len_dev || !worker_out_dev)
     return fail(ctx, RS_ERR_INVALID, "NULL pointer");
   if (!aligned16(tokens_dev)) return fail(ctx, RS_ERR_INVALID, "tokens must be 16-byte aligned");
-  CK(cudaMemsetAsync(ctx->r_stats.p, 0, 8, ctx->st), "memset");
-  if ((r = hash_batch(ctx, tokens_dev, offsets_dev, n_req, P<int64_t>(ctx->r_stats))) != RS_OK)
-    return r;
-  CK(cudaMemcpyAsync(ctx->pinned, ctx->r_stats.p, 8, cudaMemcpyDeviceToHost, ctx->st), "read stats");
-  CK(cudaStreamSynchronize(ctx->st), "sync");
-  int64_t nbmax = ctx->pinned[0];
+  int64_t nbmax = 0;
+  if ((r = hash_batch(ctx, tokens_dev, offsets_dev, n_req, &nbmax)) != RS_OK) return r;
   if (nbmax > (int64_t)ctx->g.K) nbmax = ctx->g.K;   // longer prompts stop with RS_ERR_CAPACITY
   // (4 KB beside the arrays for the kernel's own variables)
   int maxsmem = 0;
@@ -489,6 +482,12 @@ rs_status route_probe(rs_ctx* ctx, int32_t instance, const int32_t* tokens_dev,
   return RS_OK;
 }
 
+static rs_status router_status(rs_ctx* ctx, int32_t instance, int32_t st) {
+  if (st != RS_OK)
+    return fail(ctx, (rs_status)st, "router instance %d stopped on a device error (%d)", instance, st);
+  return RS_OK;
+}
+
 static rs_status router_sync_status(rs_ctx* ctx, int32_t instance, int* bad) {
   rs_status r = ensure_pinned(ctx, 4);
   if (r != RS_OK) return r;
@@ -498,10 +497,7 @@ static rs_status router_sync_status(rs_ctx* ctx, int32_t instance, int* bad) {
   CK(cudaStreamSynchronize(ctx->st), "sync");
   const int32_t* st = reinterpret_cast<const int32_t*>(ctx->pinned);
   if (bad) *bad = st[1];
-  if (st[0] != RS_OK)
-    return fail(ctx, (rs_status)st[0], "router instance %d stopped on a device error (%d)", instance,
-                st[0]);
-  return RS_OK;
+  return router_status(ctx, instance, st[0]);
 }
 
 rs_status route_release(rs_ctx* ctx, int32_t instance, const int32_t* worker_dev,
@@ -513,10 +509,17 @@ rs_status route_release(rs_ctx* ctx, int32_t instance, const int32_t* worker_dev
   if (r != RS_OK) return r;
   if (n < 0) return fail(ctx, RS_ERR_INVALID, "n < 0");
   if (n > 0 && (!worker_dev || !blocks_dev)) return fail(ctx, RS_ERR_INVALID, "NULL pointer");
-  CK(launch_route_release(s, worker_dev, blocks_dev, n, ctx->cfg.W, ctx->st), "release launch");
   int bad = 0;
-  r = router_sync_status(ctx, instance, &bad);
-  if (r != RS_OK) return r;
+  if (n == 0) {
+    if ((r = router_sync_status(ctx, instance, &bad)) != RS_OK) return r;
+  } else {
+    if ((r = ensure_pinned(ctx, 4)) != RS_OK) return r;
+    int32_t* host = reinterpret_cast<int32_t*>(ctx->pinned);
+    CK(launch_route_release(s, worker_dev, blocks_dev, n, ctx->cfg.W, host, ctx->st), "release launch");
+    CK(cudaStreamSynchronize(ctx->st), "sync");
+    bad = host[1];
+    if ((r = router_status(ctx, instance, host[0])) != RS_OK) return r;
+  }
   if (bad) {
     CK(cudaMemsetAsync(s.status + 1, 0, 4, ctx->st), "memset");
     CK(cudaStreamSynchronize(ctx->st), "sync");
@@ -1199,24 +1202,32 @@ rs_status poa_estimate(rs_ctx* ctx, const rs_records* records, int64_t n, double
   probs[0].scratch_base = 0;
   rs_status r = run_poa(ctx, u, probs, std::max<int64_t>(n, 1), nullptr);
   if (r != RS_OK) return r;
+  // the windows are known (run_poa has read the last one): every output in one
+  // set of copies through pinned memory
   const int64_t cap = *n_windows_inout;
-  if ((r = ensure_pinned(ctx, 2)) != RS_OK) return r;
-  CK(cudaMemcpyAsync(ctx->pinned, ctx->p_nwin.p, 8, cudaMemcpyDeviceToHost, ctx->st), "read");
-  CK(cudaMemcpyAsync(ctx->pinned + 1, ctx->p_total.p, 8, cudaMemcpyDeviceToHost, ctx->st), "read");
+  const int64_t k = std::max<int64_t>(0, std::min(cap, probs[0].win_cap - 1));
+  if ((r = ensure_pinned(ctx, 2 + 3 * (size_t)k)) != RS_OK) return r;
+  int64_t* p = ctx->pinned;
+  CK(cudaMemcpyAsync(p, ctx->p_nwin.p, 8, cudaMemcpyDeviceToHost, ctx->st), "read");
+  CK(cudaMemcpyAsync(p + 1, ctx->p_total.p, 8, cudaMemcpyDeviceToHost, ctx->st), "read");
+  if (k > 0) {
+    if (numer_host) CK(cudaMemcpyAsync(p + 2, ctx->p_wnum.p, k * 8, cudaMemcpyDeviceToHost, ctx->st), "read");
+    if (opt_host) CK(cudaMemcpyAsync(p + 2 + k, ctx->p_wopt.p, k * 8, cudaMemcpyDeviceToHost, ctx->st), "read");
+    if (count_host) CK(cudaMemcpyAsync(p + 2 + 2 * k, ctx->p_wcnt.p, k * 8, cudaMemcpyDeviceToHost, ctx->st), "read");
+  }
   CK(cudaStreamSynchronize(ctx->st), "sync");
-  const int64_t nw = ctx->pinned[0];
+  const int64_t nw = p[0];
   double tot;
-  memcpy(&tot, ctx->pinned + 1, 8);
+  memcpy(&tot, p + 1, 8);
   if (nw < 0)
     return fail(ctx, RS_ERR_INVALID, "a routed row has a negative or non-finite completion time");
   *n_windows_inout = nw;
   *poa_total_host = tot;
-  const int64_t k = std::min(cap, nw);
-  if (k > 0) {
-    if (numer_host) CK(cudaMemcpyAsync(numer_host, ctx->p_wnum.p, k * 8, cudaMemcpyDeviceToHost, ctx->st), "read");
-    if (opt_host) CK(cudaMemcpyAsync(opt_host, ctx->p_wopt.p, k * 8, cudaMemcpyDeviceToHost, ctx->st), "read");
-    if (count_host) CK(cudaMemcpyAsync(count_host, ctx->p_wcnt.p, k * 8, cudaMemcpyDeviceToHost, ctx->st), "read");
-    CK(cudaStreamSynchronize(ctx->st), "sync");
+  const int64_t got = std::min(k, nw);
+  if (got > 0) {
+    if (numer_host) memcpy(numer_host, p + 2, got * 8);
+    if (opt_host) memcpy(opt_host, p + 2 + k, got * 8);
+    if (count_host) memcpy(count_host, p + 2 + 2 * k, got * 8);
   }
   return RS_OK;
 }
@@ -1250,32 +1261,35 @@ rs_status sweep_knee(rs_ctx* ctx, const rs_records* records, const int64_t* row_
   for (int32_t r = 0; r < n_replicas; r++) max_rows = std::max(max_rows, row_start[r + 1] - row_start[r]);
   const size_t nr = (size_t)n_replicas, ns = (size_t)n_sweeps;
   rs_status r;
-  if ((r = ensure(ctx, ctx->k_rows, (nr + 1) * 8, "knee rows")) != RS_OK) return r;
-  if ((r = ensure(ctx, ctx->k_load, nr * 8, "knee load")) != RS_OK) return r;
-  if ((r = ensure(ctx, ctx->k_sweep, (ns + 1) * 4, "knee sweeps")) != RS_OK) return r;
-  if ((r = ensure(ctx, ctx->k_stat, nr * 8, "knee stat")) != RS_OK) return r;
-  if ((r = ensure(ctx, ctx->k_d1, nr * 8, "knee d1")) != RS_OK) return r;
-  if ((r = ensure(ctx, ctx->k_d2, nr * 8, "knee d2")) != RS_OK) return r;
-  if ((r = ensure(ctx, ctx->k_kload, ns * 8, "knee load out")) != RS_OK) return r;
-  if ((r = ensure(ctx, ctx->k_kidx, ns * 4, "knee index out")) != RS_OK) return r;
-  CK(cudaMemcpyAsync(ctx->k_rows.p, row_start, (nr + 1) * 8, cudaMemcpyHostToDevice, ctx->st), "copy");
-  if (nr) CK(cudaMemcpyAsync(ctx->k_load.p, load, nr * 8, cudaMemcpyHostToDevice, ctx->st), "copy");
-  CK(cudaMemcpyAsync(ctx->k_sweep.p, sweep_start, (ns + 1) * 4, cudaMemcpyHostToDevice, ctx->st), "copy");
-  CK(launch_sweep_knee(records->worker, records->ttft, P<int64_t>(ctx->k_rows), n_replicas, max_rows,
-                       P<double>(ctx->k_load), P<int32_t>(ctx->k_sweep), n_sweeps, pct, theta,
-                       P<double>(ctx->k_stat), P<double>(ctx->k_d1), P<double>(ctx->k_d2),
-                       P<double>(ctx->k_kload), P<int32_t>(ctx->k_kidx), ctx->st),
+  // inputs and outputs each in one block, one copy in and one out through
+  // pinned memory: row starts, loads, sweep starts | percentiles, quotients,
+  // second differences, knee loads, knee indexes
+  const size_t in_n = (nr + 1) + nr + (ns + 2) / 2, out_n = 3 * nr + ns + (ns + 1) / 2;
+  if ((r = ensure(ctx, ctx->k_in, in_n * 8, "knee inputs")) ||
+      (r = ensure(ctx, ctx->k_out, out_n * 8, "knee outputs")) ||
+      (r = ensure_pinned(ctx, in_n + out_n)))
+    return r;
+  int64_t *hin = ctx->pinned, *hout = ctx->pinned + in_n;
+  memcpy(hin, row_start, (nr + 1) * 8);
+  if (nr) memcpy(hin + nr + 1, load, nr * 8);
+  memcpy(hin + 2 * nr + 1, sweep_start, (ns + 1) * 4);
+  CK(cudaMemcpyAsync(ctx->k_in.p, hin, in_n * 8, cudaMemcpyHostToDevice, ctx->st), "copy");
+  int64_t* din = P<int64_t>(ctx->k_in);
+  double* dout = P<double>(ctx->k_out);
+  CK(launch_sweep_knee(records->worker, records->ttft, din, n_replicas, max_rows,
+                       reinterpret_cast<double*>(din + nr + 1),
+                       reinterpret_cast<int32_t*>(din + 2 * nr + 1), n_sweeps, pct, theta, dout,
+                       dout + nr, dout + 2 * nr, dout + 3 * nr,
+                       reinterpret_cast<int32_t*>(dout + 3 * nr + ns), ctx->st),
      "knee launch");
-  if (nr) {
-    if (stat_host) CK(cudaMemcpyAsync(stat_host, ctx->k_stat.p, nr * 8, cudaMemcpyDeviceToHost, ctx->st), "read");
-    if (d1_host) CK(cudaMemcpyAsync(d1_host, ctx->k_d1.p, nr * 8, cudaMemcpyDeviceToHost, ctx->st), "read");
-    if (d2_host) CK(cudaMemcpyAsync(d2_host, ctx->k_d2.p, nr * 8, cudaMemcpyDeviceToHost, ctx->st), "read");
-  }
-  if (ns) {
-    if (knee_load_host) CK(cudaMemcpyAsync(knee_load_host, ctx->k_kload.p, ns * 8, cudaMemcpyDeviceToHost, ctx->st), "read");
-    if (knee_index_host) CK(cudaMemcpyAsync(knee_index_host, ctx->k_kidx.p, ns * 4, cudaMemcpyDeviceToHost, ctx->st), "read");
-  }
+  if (out_n)
+    CK(cudaMemcpyAsync(hout, dout, out_n * 8, cudaMemcpyDeviceToHost, ctx->st), "read");
   CK(cudaStreamSynchronize(ctx->st), "sync");
+  if (stat_host) memcpy(stat_host, hout, nr * 8);
+  if (d1_host) memcpy(d1_host, hout + nr, nr * 8);
+  if (d2_host) memcpy(d2_host, hout + 2 * nr, nr * 8);
+  if (knee_load_host) memcpy(knee_load_host, hout + 3 * nr, ns * 8);
+  if (knee_index_host) memcpy(knee_index_host, hout + 3 * nr + ns, ns * 4);
   return RS_OK;
 }
 

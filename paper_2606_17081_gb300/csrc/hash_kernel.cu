@@ -70,13 +70,19 @@ __host__ __device__ constexpr uint64_t p_pow2(int s) {
   return x;
 }
 
+// jobs: device array of njobs traces, or NULL: the one trace `one`.
 __global__ void __launch_bounds__(HASH_NT) k_block_hash(const HashJob* __restrict__ jobs,
-                                                        int njobs, int64_t total_req,
+                                                        const HashJob one, int njobs,
+                                                        int64_t total_req,
                                                         uint64_t seed,
                                                         int64_t* __restrict__ nbmax) {
   __shared__ HashJob s_jobs[HASH_MAX_JOBS];
   __shared__ int64_t s_max[HASH_NT / 32];
-  for (int j = threadIdx.x; j < njobs; j += HASH_NT) s_jobs[j] = jobs[j];
+  if (jobs) {
+    for (int j = threadIdx.x; j < njobs; j += HASH_NT) s_jobs[j] = jobs[j];
+  } else if (threadIdx.x == 0) {
+    s_jobs[0] = one;
+  }
   __syncthreads();
   const int lane = threadIdx.x & 31;
   // P^(lane + 1): the factor of the carry H_{k0-1} at this lane's block
@@ -130,8 +136,9 @@ __global__ void __launch_bounds__(HASH_NT) k_block_hash(const HashJob* __restric
   }
 }
 
-cudaError_t launch_block_hash(const HashJob* jobs_dev, int njobs, int64_t total_req, uint64_t seed,
-                              int64_t* nbmax_out, cudaStream_t st) {
+static cudaError_t hash_launch(const HashJob* jobs_dev, const HashJob& one, int njobs,
+                               int64_t total_req, uint64_t seed, int64_t* nbmax_out,
+                               cudaStream_t st) {
   if (total_req <= 0) return cudaSuccess;
   if (njobs < 1 || njobs > HASH_MAX_JOBS) return cudaErrorInvalidValue;
   int dev = 0, sms = 0;
@@ -143,7 +150,45 @@ cudaError_t launch_block_hash(const HashJob* jobs_dev, int njobs, int64_t total_
   // tail than long ones (the cap was chosen by measurement)
   int64_t nblk = (total_req + HASH_NT / 32 - 1) / (HASH_NT / 32);
   if (nblk > (int64_t)sms * 64) nblk = (int64_t)sms * 64;
-  k_block_hash<<<(unsigned)nblk, HASH_NT, 0, st>>>(jobs_dev, njobs, total_req, seed, nbmax_out);
+  k_block_hash<<<(unsigned)nblk, HASH_NT, 0, st>>>(jobs_dev, one, njobs, total_req, seed, nbmax_out);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_block_hash(const HashJob* jobs_dev, int njobs, int64_t total_req, uint64_t seed,
+                              int64_t* nbmax_out, cudaStream_t st) {
+  return hash_launch(jobs_dev, HashJob{}, njobs, total_req, seed, nbmax_out, st);
+}
+
+cudaError_t launch_block_hash_one(const HashJob& job, uint64_t seed, cudaStream_t st) {
+  return hash_launch(nullptr, job, 1, job.n_req, seed, nullptr, st);
+}
+
+// A small batch's sizes, written to (pinned host) out: the longest prompt's
+// full blocks and the end of the last prompt.  One CTA.
+__global__ void __launch_bounds__(1024) k_batch_sizes(const int64_t* __restrict__ offsets, int n,
+                                                      int64_t* out) {
+  __shared__ long long s_max[32];
+  long long m = 0;
+  for (int i = threadIdx.x; i < n; i += blockDim.x) {
+    const long long nb = (offsets[i + 1] - offsets[i]) >> 4;
+    m = nb > m ? nb : m;
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const long long v = __shfl_xor_sync(FULL_MASK, m, o);
+    m = v > m ? v : m;
+  }
+  if ((threadIdx.x & 31) == 0) s_max[threadIdx.x >> 5] = m;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 0; w < (int)(blockDim.x >> 5); w++) m = s_max[w] > m ? s_max[w] : m;
+    out[0] = m;
+    out[1] = offsets[n];
+  }
+}
+
+cudaError_t launch_batch_sizes(const int64_t* offsets, int n, int64_t* out, cudaStream_t st) {
+  k_batch_sizes<<<1, n < 1024 ? (n + 31) / 32 * 32 : 1024, 0, st>>>(offsets, n, out);
   return cudaGetLastError();
 }
 

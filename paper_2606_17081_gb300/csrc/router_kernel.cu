@@ -292,7 +292,8 @@ cudaError_t launch_route_batch(const RouterState& s, int32_t instance, const int
 // and flagged in *bad.
 __global__ void k_route_release(int64_t* active, const int32_t* __restrict__ worker,
                                 const int32_t* __restrict__ blocks, int32_t n, int32_t W,
-                                int32_t* bad) {
+                                int32_t* status, int32_t* host) {
+  int32_t* bad = status + 1;
   for (int32_t i = threadIdx.x; i < n; i += blockDim.x) {
     const int w = worker[i];
     if (w < 0 || w >= W) {
@@ -305,12 +306,15 @@ __global__ void k_route_release(int64_t* active, const int32_t* __restrict__ wor
   __syncthreads();
   for (int j = threadIdx.x; j < W; j += blockDim.x)
     if (active[j] < 0) active[j] = 0;
+  if (threadIdx.x == 0) {
+    host[0] = status[0];
+    host[1] = __ldcg(bad);   // (set by any thread of this CTA, through L2)
+  }
 }
 
 cudaError_t launch_route_release(const RouterState& s, const int32_t* worker, const int32_t* blocks,
-                                 int32_t n, int32_t W, cudaStream_t st) {
-  if (n <= 0) return cudaSuccess;
-  k_route_release<<<1, 256, 0, st>>>(s.active, worker, blocks, n, W, s.status + 1);
+                                 int32_t n, int32_t W, int32_t* host, cudaStream_t st) {
+  k_route_release<<<1, 256, 0, st>>>(s.active, worker, blocks, n, W, s.status, host);
   return cudaGetLastError();
 }
 

@@ -141,6 +141,10 @@ struct HashJob {
 constexpr int HASH_MAX_JOBS = 64;
 cudaError_t launch_block_hash(const HashJob* jobs_dev, int njobs, int64_t total_req, uint64_t seed,
                               int64_t* nbmax_out, cudaStream_t st);
+cudaError_t launch_block_hash_one(const HashJob& job, uint64_t seed, cudaStream_t st);
+// out[0] = the longest prompt's full blocks, out[1] = offsets[n] (out: device
+// memory or pinned host memory; small n).
+cudaError_t launch_batch_sizes(const int64_t* offsets, int n, int64_t* out, cudaStream_t st);
 // *nbmax = max(*nbmax, the largest floor(L/16) over the jobs' requests).
 cudaError_t launch_nbmax(const HashJob* jobs_dev, int njobs, int64_t total_req, int64_t* nbmax,
                          cudaStream_t st);
@@ -252,8 +256,10 @@ cudaError_t launch_route_batch(const RouterState& s, int32_t instance, const int
                                int nbmax, const TableGeom& g, const ModelConsts& mc, float omega,
                                float tau, uint64_t seed, bool lean, cudaStream_t st);
 size_t router_smem(int W, int nbmax, bool lean);
+// host: pinned, receives the instance's sticky status and whether entries were
+// skipped (then the flag stays set on the device).
 cudaError_t launch_route_release(const RouterState& s, const int32_t* worker, const int32_t* blocks,
-                                 int32_t n, int32_t W, cudaStream_t st);
+                                 int32_t n, int32_t W, int32_t* host, cudaStream_t st);
 cudaError_t launch_clear_tables(uint64_t* keys, uint32_t* stamp, size_t nslots, CacheMeta* meta,
                                 size_t nmeta, cudaStream_t st);
 
