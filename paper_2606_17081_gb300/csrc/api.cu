@@ -943,11 +943,11 @@ rs_status simulate_replicas(rs_ctx* ctx, const rs_trace* traces, int32_t n_trace
     return fail(ctx, RS_ERR_CAPACITY,
                 "prompt of %lld blocks needs %zu bytes of shared memory per replica",
                 (long long)nbmax, smem);
-  // block ids instead of hash tables: exact LRU replicas on traces whose
-  // positions fit 31 bits (run_ids falls back to the tables when the ids'
-  // memory would exceed the tables')
+  // block ids instead of hash tables: without tiers, on traces whose positions
+  // fit 31 bits (and the tables after all when the ids' memory would exceed
+  // theirs)
   const size_t nsim = n_replicas;
-  bool use_ids = !tiered && !any_freq && !(flags & RS_SIM_TABLES);
+  bool use_ids = !tiered && !(flags & RS_SIM_TABLES);
   for (int t = 0; t < n_traces; t++)
     if (used[t] && tot[t] / 16 + 1 > (int64_t)1 << 30) use_ids = false;
   // the kernel on block ids: its own arrays (smaller except for the window of
@@ -955,9 +955,9 @@ rs_status simulate_replicas(rs_ctx* ctx, const rs_trace* traces, int32_t n_trace
   bool ids_slots_global = false;
   {
     const int ntu = 32 * sim_ids_update_warps(n_replicas, ctx->sms);
-    if (sim_ids_smem_bytes(W, (int)nbmax, cmax, ctx->cfg.cap, ntu, false) > smem_room) {
+    if (sim_ids_smem_bytes(W, (int)nbmax, cmax, ctx->cfg.cap, ntu, false, any_freq) > smem_room) {
       ids_slots_global = true;
-      if (sim_ids_smem_bytes(W, (int)nbmax, cmax, ctx->cfg.cap, ntu, true) > smem_room) use_ids = false;
+      if (any_freq || sim_ids_smem_bytes(W, (int)nbmax, cmax, ctx->cfg.cap, ntu, true) > smem_room) use_ids = false;
     }
   }
   size_t hash_total = 0;
@@ -1010,13 +1010,13 @@ rs_status simulate_replicas(rs_ctx* ctx, const rs_trace* traces, int32_t n_trace
   }
   CK(cudaEventRecord(ctx->ev[1], ctx->st), "event");
   std::vector<TraceIds> tids(n_traces);
+  size_t stamp_words = 0;
   if (use_ids) {
-    size_t stamp_words = 0;
     r = trace_ids(ctx, traces, used, tot, all, req_total, params, n_replicas, tids, &stamp_words,
                   &launches);
-    if (r == RS_OK && stamp_words * 4 > std::max<size_t>(nsim * W * g.slots * 12, (size_t)4 << 30))
+    if (r == RS_OK && stamp_words * 4 * (any_freq ? 2 : 1) > std::max<size_t>(nsim * W * g.slots * 12, (size_t)4 << 30))
       r = RS_ERR_OOM;
-    if (r == RS_OK) r = ensure(ctx, ctx->i_stamps, stamp_words * 4, "block stamps");
+    if (r == RS_OK) r = ensure(ctx, ctx->i_stamps, stamp_words * 4 * (any_freq ? 2 : 1), "block stamps");
     if (r == RS_OK)
       r = ensure(ctx, ctx->i_scratch, nsim * sim_ids_scratch_bytes((int)nbmax), "update scratch");
     if (r == RS_ERR_OOM) {   // no room for the ids: the tables
@@ -1045,7 +1045,7 @@ rs_status simulate_replicas(rs_ctx* ctx, const rs_trace* traces, int32_t n_trace
       (r = ensure(ctx, ctx->slots, nsim * (use_ids ? sim_ids_slot_bytes(cmax) : sim_slot_bytes(cmax)),
                   "request slots")) != RS_OK)
     return r;
-  if (any_freq && ((r = ensure(ctx, ctx->fexp, nsl * 4, "frequency state")) ||
+  if (any_freq && !use_ids && ((r = ensure(ctx, ctx->fexp, nsl * 4, "frequency state")) ||
                    (r = ensure(ctx, ctx->tmpe, nsim * g.K * 4, "frequency rebuild scratch"))))
     return r;
   // w_c * (m / nbt) table for prompts up to nbmax blocks (none beyond 2048)
@@ -1069,6 +1069,7 @@ rs_status simulate_replicas(rs_ctx* ctx, const rs_trace* traces, int32_t n_trace
     d.nz = ti.nz;
     d.nre = ti.nre;
     d.stamps = use_ids ? P<uint32_t>(ctx->i_stamps) + sw : nullptr;
+    d.fexp = use_ids && any_freq ? P<uint32_t>(ctx->i_stamps) + stamp_words + sw : nullptr;
     sw += (size_t)W * ti.nre;
     d.offsets = doff[p.trace];
     d.release = drel[p.trace];
@@ -1105,7 +1106,7 @@ rs_status simulate_replicas(rs_ctx* ctx, const rs_trace* traces, int32_t n_trace
   sb.stamp = P<uint32_t>(ctx->stamp);
   sb.log = P<uint32_t>(ctx->log);
   sb.tmp = P<uint64_t>(ctx->tmp);
-  sb.fexp = any_freq ? P<uint32_t>(ctx->fexp) : nullptr;
+  sb.fexp = any_freq ? P<uint32_t>(use_ids ? ctx->i_stamps : ctx->fexp) : nullptr;
   sb.tmpe = any_freq ? P<uint32_t>(ctx->tmpe) : nullptr;
   sb.pend = P<double>(ctx->pend);
   sb.pend_cap = std::max<int64_t>(pend_cap, 1);
@@ -1324,7 +1325,7 @@ static rs_status dump_ids(rs_ctx* ctx, int32_t index, int32_t worker, uint64_t* 
     uint64_t h;
     if (x >> 31)
       h = hashes[x & 0x7FFFFFFFu];
-    else if (stamps[x] == t)
+    else if ((int64_t)x < ic.nre && stamps[x] == t)   // (else dead)
       h = of[x];
     else
       continue;

@@ -72,6 +72,7 @@ struct SimDesc {
   const uint32_t* ids;
   const int32_t* nz;
   uint32_t* stamps;
+  uint32_t* fexp;           // [W][nre] frequency eviction state, or NULL
   int64_t nre;
   int64_t n_req;
   int64_t rec_base;         // first record row
@@ -172,10 +173,12 @@ struct IdJob {
 };
 constexpr int IDS_MAX_JOBS = 64;
 cudaError_t launch_block_ids(const IdJob* jobs_dev, int njobs, int64_t total_req, cudaStream_t st);
-// The simulation on block ids (exact LRU replicas).
+// The simulation on block ids (exact LRU; frequency eviction when b.fexp is set,
+// then with the request slots in shared memory only).
 cudaError_t launch_sim_ids(const SimDesc* d_desc, const SimBuffers& b, const SimLaunch& L,
                            cudaStream_t st);
-size_t sim_ids_smem_bytes(int W, int nbmax, int cmax, int cap, int ntu, bool slots_global);
+size_t sim_ids_smem_bytes(int W, int nbmax, int cmax, int cap, int ntu, bool slots_global,
+                          bool freq = false);
 size_t sim_ids_slot_bytes(int cmax);
 size_t sim_ids_scratch_bytes(int nbmax);
 int sim_ids_update_warps(int nsim, int sms);

@@ -47,6 +47,7 @@ namespace rs {
 constexpr uint32_t CODE_FRESH = 0x80000000u;    // first occurrence in the trace
 constexpr uint32_t CODE_SINGLE = 0x7FFFFFFFu;   // (low bits) occurs once
 constexpr uint32_t SINGLE_FLAG = 0x80000000u;   // log entry: a single block's position
+constexpr uint32_t LOG_DEAD = 0x7FFFFFFFu;      // log entry: evicted before the head passed it
 
 // ------------------------------------------------------------ block ids
 
@@ -198,6 +199,7 @@ struct IdsReq : ReqState {
 struct IdsArrival {
   double a;
   float tau, omega;
+  uint32_t D;          // decay step (frequency eviction)
 };
 
 // What a worker's cache update will do, worked out before the choice
@@ -217,7 +219,10 @@ struct IdsShared {
   IdsArrival pub[2];
   int stat[2];                 // by parity: an error seen before that join
   alignas(16) uint2 red[8];    // per update warp: absent blocks, least stamp
-  unsigned livew[IDS_WIN / 32];   // live entries of the window
+  unsigned livew[IDS_WIN / 32];   // live entries of the window (frequency eviction: cold ones)
+  uint2 hot[8];                // per update warp: least e and position of the hot entries passed
+  FreqShared fs;
+  FreqMeta fnew;
   int warp_tot[8];
   int err;                     // of the update
   int nvic, nins, changed;
@@ -230,12 +235,12 @@ __host__ __device__ constexpr int ids_plan_workers(int) { return 1; }
 
 struct IdsLayout {
   size_t ftab, f_oitl, f_a, f_o, h_k, srec, gk, gf, wA, codes, meta, f_req, f_worker, f_blk, f_next, h_f,
-      freestk, winserv, wqh, wqt, wm, act, nfz, whead, wlen, win;
+      freestk, winserv, wqh, wqt, wm, act, nfz, whead, wlen, win, wfreq;
   size_t total, slot_bytes;
 };
 
 __host__ __device__ inline IdsLayout make_ids_layout(int W, int nbmax, int cmax, int nft, int ntu,
-                                                     bool slots_global) {
+                                                     bool slots_global, bool freq = false) {
   IdsLayout L;
   size_t o = 0, og = 0;
   const size_t nb = (size_t)(nbmax > 0 ? nbmax : 1), C = (size_t)(cmax > 0 ? cmax : 1);
@@ -286,25 +291,32 @@ __host__ __device__ inline IdsLayout make_ids_layout(int W, int nbmax, int cmax,
   L.whead = take(4 * (size_t)W);
   L.wlen = take(4 * (size_t)W);
   const int nu = ntu / 32;
-  L.win = take(4 * (size_t)W * (W <= nu * ids_plan_workers(nu) ? IDS_WRING : IDS_WIN));
+  L.win = take(4 * (size_t)W * (!freq && W <= nu * ids_plan_workers(nu) ? IDS_WRING : IDS_WIN));
+  L.wfreq = take(freq ? sizeof(FreqMeta) * (size_t)W : 0);
   L.total = o;
   L.slot_bytes = (og + 255) & ~(size_t)255;
   return L;
 }
 
-size_t sim_ids_smem_bytes(int W, int nbmax, int cmax, int cap, int ntu, bool slots_global) {
-  return make_ids_layout(W, nbmax, cmax, ftab_size(cap), ntu, slots_global).total;
+size_t sim_ids_smem_bytes(int W, int nbmax, int cmax, int cap, int ntu, bool slots_global, bool freq) {
+  return make_ids_layout(W, nbmax, cmax, ftab_size(cap), ntu, slots_global, freq).total;
 }
 
 // Global scratch of one replica for the updates that need the exact sequence.
 struct IdsScratch {
   uint32_t *vent, *vt;   // [2 nb] live entries and their positions
   int32_t *owner, *w;    // [2 nb] the prompt's block holding an entry or -1, [nb] see lru_exact
+  // frequency eviction: [2 nb] hot entries (position << 32 | id), [2 nb] victims,
+  // [nb] stamps and e, [2 nb] touched entries, [nb] kinds, [nb] evicted early
+  uint64_t* hot;
+  int32_t* victim;
+  uint32_t *pst, *e;
+  uint8_t *touched, *kind, *evk;
 };
 
 __host__ __device__ inline size_t ids_scratch_bytes(int nbmax) {
   const size_t nb = (size_t)(nbmax > 0 ? nbmax : 1);
-  return (28 * nb + 255) & ~(size_t)255;
+  return (64 * nb + 255) & ~(size_t)255;
 }
 
 size_t sim_ids_scratch_bytes(int nbmax) { return ids_scratch_bytes(nbmax); }
@@ -312,16 +324,24 @@ size_t sim_ids_scratch_bytes(int nbmax) { return ids_scratch_bytes(nbmax); }
 __device__ __forceinline__ IdsScratch ids_scratch(unsigned char* p, int nbmax) {
   const size_t nb = (size_t)(nbmax > 0 ? nbmax : 1);
   IdsScratch s;
-  s.vent = reinterpret_cast<uint32_t*>(p);
+  s.hot = reinterpret_cast<uint64_t*>(p);
+  s.vent = reinterpret_cast<uint32_t*>(s.hot + 2 * nb);
   s.vt = s.vent + 2 * nb;
   s.owner = reinterpret_cast<int32_t*>(s.vt + 2 * nb);
   s.w = s.owner + 2 * nb;
+  s.victim = s.w + nb;
+  s.pst = reinterpret_cast<uint32_t*>(s.victim + 2 * nb);
+  s.e = s.pst + nb;
+  s.touched = reinterpret_cast<uint8_t*>(s.e + nb);
+  s.kind = s.touched + 2 * nb;
+  s.evk = s.kind + nb;
   return s;
 }
 
 // One worker's cache.
 struct IdsTable {
   uint32_t* st;    // [nre] stamps
+  uint32_t* fe;    // [nre] frequency eviction: e, the decay step from which a block is cold
   uint32_t* log;   // [rmask + 1]
   uint32_t rmask;
 };
@@ -604,7 +624,7 @@ __device__ __forceinline__ int nth_set_bit32(unsigned x, int n) {
 
 // Whether log entry x at position p is live.
 __device__ __forceinline__ bool ids_live(const IdsTable& t, uint32_t x, uint32_t p) {
-  return (x & SINGLE_FLAG) || t.st[x] == p;
+  return (x & SINGLE_FLAG) || (x != LOG_DEAD && t.st[x] == p);
 }
 
 // Moves the live entries of the log down to the head, in order, and renumbers
@@ -1030,6 +1050,401 @@ __device__ __noinline__ void ids_update_unplanned(SimScalars& A, IdsShared& S, u
   ids_update<NT, false>(A, S, K, nbmax, t, meta, cd, q, scratch, nullptr, nullptr, wlen, i);
 }
 
+// ------------------------------------------------------------ frequency eviction
+//
+// The KV Block Manager's rule as in rs_device.cuh (a block is cold iff e <= D;
+// e = D on insertion, raised on a hit).  A single block is never hit, so it is
+// cold for good.  Victims beyond hot entries leave the head where it is: a
+// single one's log entry becomes LOG_DEAD.
+
+// The first `want` live cold entries from `start` on into vent / vt (hot ones
+// passed lower S.fs); returns how many.
+template <int NT>
+__device__ __forceinline__ uint32_t ids_gather_cold(const IdsTable& t, uint32_t start, uint32_t T,
+                                                    uint32_t want, uint32_t D, const IdsScratch& sc,
+                                                    IdsShared& S) {
+  uint32_t have = 0, he = 0xFFFFFFFFu, hp = 0xFFFFFFFFu;
+#pragma unroll 1
+  for (uint32_t p0 = start; have < want && p0 < T; p0 += NT) {
+    const uint32_t p = p0 + threadIdx.x;
+    uint32_t x = 0;
+    bool cold = false;
+    if (p < T) {
+      x = t.log[p & t.rmask];
+      cold = ids_live(t, x, p);
+      if (cold && !(x & SINGLE_FLAG)) {
+        const uint32_t e = t.fe[x];
+        if (e > D) {
+          cold = false;
+          he = min(he, e);
+          hp = min(hp, p);
+        }
+      }
+    }
+    int tot;
+    const int r = cta_rank<NT>(cold, S.warp_tot, &tot);
+    if (cold && have + r < want) {
+      sc.vent[have + r] = x;
+      sc.vt[have + r] = p;
+    }
+    have = min(want, have + (uint32_t)tot);
+  }
+  he = __reduce_min_sync(FULL_MASK, he);
+  hp = __reduce_min_sync(FULL_MASK, hp);
+  if ((threadIdx.x & 31) == 0) {
+    if (he != 0xFFFFFFFFu) atomicMin(&S.fs.femin, he);
+    if (hp != 0xFFFFFFFFu) atomicMin(&S.fs.fhot, hp);
+  }
+  grp_bar<NT>();
+  return have;
+}
+
+// An update that the window does not settle.  With enough cold entries before
+// the oldest present cold block, those are the victims; else one thread replays
+// the sequence over the first 2 nb cold entries, the first 2 nb hot ones (only
+// when the cold ones run out) and the prompt's own blocks.  Evicts; kinds in
+// sc.kind (0 touched, 1 inserted, 2 / 3 inserted / touched and evicted again),
+// victims in S.nvic, insertions in S.nins, S.changed = 1 when replayed, S.nh =
+// one past the last victim otherwise.
+template <int NT>
+__device__ __noinline__ void ids_freq_general(IdsTable t, CacheMeta m, uint32_t start, uint32_t K,
+                                              const uint32_t* cd, int nb, uint32_t E0, uint32_t pmin,
+                                              int nabs, uint32_t D, uint32_t fmax,
+                                              unsigned char* scratch, int nbmax, IdsShared& S,
+                                              int64_t* slow) {
+  const IdsScratch sc = ids_scratch(scratch, nbmax);
+  if (threadIdx.x == 0) {
+    S.fs.femin = S.fs.fhot = 0xFFFFFFFFu;
+    S.changed = 0;
+  }
+  grp_bar<NT>();
+  uint32_t G = ids_gather_cold<NT>(t, start, m.T, E0, D, sc, S);
+  for (int k = threadIdx.x; k < nb; k += NT) {
+    const uint32_t c = cd[k];
+    const uint32_t st = c >> 31 ? STAMP_NONE : t.st[c];
+    sc.pst[k] = st;
+    sc.e[k] = st == STAMP_NONE ? 0u : t.fe[c];
+    sc.evk[k] = 0;
+    sc.kind[k] = st == STAMP_NONE;
+  }
+  grp_bar<NT>();
+  if (G >= E0 && pmin > sc.vt[E0 - 1]) {
+    for (uint32_t v = threadIdx.x; v < E0; v += NT) {
+      const uint32_t x = sc.vent[v];
+      if (x & SINGLE_FLAG) t.log[sc.vt[v] & t.rmask] = LOG_DEAD; else t.st[x] = STAMP_NONE;
+    }
+    if (threadIdx.x == 0) {
+      S.nvic = (int)E0;
+      S.nins = nabs;
+      S.nh = sc.vt[E0 - 1] + 1;
+    }
+    grp_bar<NT>();
+    return;
+  }
+  grp_bar<NT>();
+  const uint32_t want = min(m.size, 2u * (uint32_t)nb);
+  G = ids_gather_cold<NT>(t, start, m.T, want, D, sc, S);
+  // hot entries, when the cold ones run out
+  uint32_t GB = 0;
+  if (G < want) {
+#pragma unroll 1
+    for (uint32_t p0 = m.head; GB < want && p0 < m.T; p0 += NT) {
+      const uint32_t p = p0 + threadIdx.x;
+      uint32_t x = 0;
+      bool hot = false;
+      if (p < m.T) {
+        x = t.log[p & t.rmask];
+        hot = !(x & SINGLE_FLAG) && ids_live(t, x, p) && t.fe[x] > D;
+      }
+      int tot;
+      const int r = cta_rank<NT>(hot, S.warp_tot, &tot);
+      if (hot && GB + r < want) sc.hot[GB + r] = ((uint64_t)p << 32) | x;
+      GB = min(want, GB + (uint32_t)tot);
+    }
+  }
+  for (uint32_t q = threadIdx.x; q < G; q += NT) {
+    sc.owner[q] = -1;
+    sc.touched[q] = 0;
+  }
+  grp_bar<NT>();
+  const uint32_t last = G ? sc.vt[G - 1] : 0u;
+  for (int k = threadIdx.x; k < nb; k += NT) {
+    const uint32_t st = sc.pst[k];
+    if (st != STAMP_NONE && G && st <= last && sc.e[k] <= D) {
+      const uint32_t lo = ids_place(sc.vt, G, st);
+      if (lo < G && sc.vt[lo] == st) sc.owner[lo] = k;
+    }
+  }
+  grp_bar<NT>();
+  if (threadIdx.x == 0) {
+    const bool hits_cold = fmax < 2u;   // a hit at cap 1 leaves the block cold
+    uint32_t pa = 0, pb = 0, sz = m.size;
+    int qc = 0, qh = 0, E = 0, ni = 0;
+    for (int k = 0; k < nb; k++) {
+      if (sc.pst[k] != STAMP_NONE && !sc.evk[k]) {
+        sc.kind[k] = 0;
+        const uint32_t st = sc.pst[k];
+        if (sc.e[k] <= D) {   // a cold entry: in the list if old enough
+          if (G && st <= last) {
+            const uint32_t lo = ids_place(sc.vt, G, st);
+            if (lo < G && sc.vt[lo] == st) sc.touched[lo] = 1;
+          }
+        } else if (GB) {      // a hot entry: in the hot list if old enough
+          uint32_t lo = 0, hi = GB;
+          while (lo < hi) {
+            const uint32_t mid = (lo + hi) >> 1;
+            if ((uint32_t)(sc.hot[mid] >> 32) < st) lo = mid + 1; else hi = mid;
+          }
+          if (lo < GB && (uint32_t)(sc.hot[lo] >> 32) == st) sc.hot[lo] |= 0x80000000ull;   // touched
+        }
+        continue;
+      }
+      sc.kind[k] = 1;
+      ni++;
+      if (sz < K) {
+        sz++;
+        continue;
+      }
+      // the victim: old cold, own cold, old hot, own hot -- each oldest first
+      while (pa < G && sc.touched[pa]) pa++;
+      if (pa < G) {
+        sc.victim[E++] = (int32_t)pa;
+        if (sc.owner[pa] >= 0) sc.evk[sc.owner[pa]] = 1;   // evicted before its turn
+        pa++;
+        continue;
+      }
+      while (qc < k && !(sc.kind[qc] == 1 || (hits_cold && sc.kind[qc] == 0))) qc++;
+      if (qc < k) {
+        if (sc.kind[qc] == 1) {
+          sc.kind[qc] = 2;
+          sc.victim[E++] = VICTIM_OWN_INSERT;
+        } else {
+          sc.kind[qc] = 3;
+          sc.victim[E++] = -(int32_t)(cd[qc] & CODE_SINGLE) - 2;
+        }
+        qc++;
+        continue;
+      }
+      while (pb < GB && (sc.hot[pb] & 0x80000000ull)) pb++;
+      if (pb < GB) {
+        const uint32_t x = (uint32_t)sc.hot[pb];
+        sc.victim[E++] = -(int32_t)x - 2;
+        for (int k2 = k + 1; k2 < nb; k2++)   // a present hot block evicted before its turn
+          if (cd[k2] == x && !sc.evk[k2]) sc.evk[k2] = 1;
+        pb++;
+        continue;
+      }
+      while (qh < k && sc.kind[qh] != 0) qh++;
+      if (qh < k) {
+        sc.kind[qh] = 3;
+        sc.victim[E++] = -(int32_t)(cd[qh] & CODE_SINGLE) - 2;
+        qh++;
+        continue;
+      }
+      S.err = RS_ERR_TIMEOUT;   // nothing to evict: inconsistent state
+      break;
+    }
+    S.nvic = E;
+    S.nins = ni;
+    S.changed = 1;
+    ++*slow;
+  }
+  grp_bar<NT>();
+  const int E = S.nvic;
+  for (int v = threadIdx.x; v < E; v += NT) {
+    const int32_t iv = sc.victim[v];
+    if (iv == VICTIM_OWN_INSERT) continue;
+    if (iv >= 0) {
+      const uint32_t x = sc.vent[iv];
+      if (x & SINGLE_FLAG) t.log[sc.vt[iv] & t.rmask] = LOG_DEAD; else t.st[x] = STAMP_NONE;
+    } else {
+      t.st[(uint32_t)(-(iv + 2))] = STAMP_NONE;
+    }
+  }
+  grp_bar<NT>();   // (a victim may be a block of this request: its new stamp comes after)
+}
+
+// As ids_update under the frequency rule at decay step D (known with the
+// arrival, so nothing is planned before the choice).  The window starts where
+// the last search ended while the hot entries passed there are still hot.
+template <int NT>
+__device__ __forceinline__ void ids_update_freq(SimScalars& A, IdsShared& S, uint32_t K, int nbmax,
+                                                const IdsTable& t, CacheMeta* meta, FreqMeta* fm,
+                                                const uint32_t* cd, const IdsReq& q, uint32_t D,
+                                                uint32_t fmax, unsigned char* scratch, uint32_t* win,
+                                                uint32_t* whead, uint32_t* wlen, int64_t i) {
+  constexpr int R = IDS_WIN / NT, NW = IDS_WIN / 32;
+  const int nb = q.nb, nz = q.nz, tid = (int)threadIdx.x, lane = tid & 31;
+  cp_async_wait_all();
+  if ((uint64_t)meta->T - meta->head + (uint64_t)nb > (uint64_t)t.rmask + 1 ||
+      (uint64_t)meta->T + nb > STAMP_LIMIT) {
+    grp_bar<NT>();
+    ids_compact<NT>(t, meta, S.warp_tot, &S.err);
+    if (tid == 0) {
+      A.rebuilds++;
+      *wlen = 0;
+      *fm = FreqMeta{0u, 0u};
+    }
+    grp_bar<NT>();
+  }
+  const CacheMeta m = *meta;
+  const FreqMeta f = *fm;
+  const uint32_t start = D < f.fmin ? f.fscan : m.head;
+  const bool full = m.size + (uint32_t)nb > K;
+  int nabs = 0;
+  uint32_t pmin = STAMP_NONE;   // least stamp of a present cold block
+#pragma unroll 1
+  for (int k = tid; k < nz; k += NT) {
+    const uint32_t x = cd[k];
+    const uint32_t st = x >> 31 ? STAMP_NONE : t.st[x];
+    nabs += st == STAMP_NONE;
+    if (st != STAMP_NONE && t.fe[x] <= D) pmin = min(pmin, st);
+  }
+  uint32_t x[R], he = 0xFFFFFFFFu, hp = 0xFFFFFFFFu;
+  bool cold[R];
+  const uint32_t have_win = *whead == start ? *wlen : 0u;
+#pragma unroll
+  for (int r = 0; r < R; r++) {
+    const uint32_t w = (uint32_t)(r * NT + tid), p = start + w;
+    x[r] = LOG_DEAD;
+    if (full && p < m.T) x[r] = w < have_win ? win[w] : t.log[p & t.rmask];
+  }
+#pragma unroll
+  for (int r = 0; r < R; r++) {
+    const uint32_t p = start + (uint32_t)(r * NT + tid);
+    cold[r] = ids_live(t, x[r], p);
+    if (cold[r] && !(x[r] & SINGLE_FLAG)) {
+      const uint32_t e = t.fe[x[r]];
+      if (e > D) {
+        cold[r] = false;
+        he = min(he, e);
+        hp = min(hp, p);
+      }
+    }
+  }
+  {
+    const int a = (int)__reduce_add_sync(FULL_MASK, (unsigned)nabs);
+    const uint32_t pm = __reduce_min_sync(FULL_MASK, pmin);
+    he = __reduce_min_sync(FULL_MASK, he);
+    hp = __reduce_min_sync(FULL_MASK, hp);
+    if (lane == 0) {
+      S.red[tid >> 5] = make_uint2((unsigned)a, pm);
+      S.hot[tid >> 5] = make_uint2(he, hp);
+    }
+#pragma unroll
+    for (int r = 0; r < R; r++) {
+      const unsigned cv = __ballot_sync(FULL_MASK, cold[r]);
+      if (lane == 0) S.livew[r * (NT / 32) + (tid >> 5)] = cv;
+    }
+  }
+  grp_bar<NT>();
+  nabs = nb - nz;   // past nz every block is fresh
+  pmin = he = hp = 0xFFFFFFFFu;
+#pragma unroll
+  for (int w = 0; w < NT / 32; w++) {
+    nabs += (int)S.red[w].x;
+    pmin = min(pmin, S.red[w].y);
+    he = min(he, S.hot[w].x);
+    hp = min(hp, S.hot[w].y);
+  }
+  const uint32_t freeb = K - m.size;
+  const uint32_t E0 = (uint32_t)nabs > freeb ? (uint32_t)nabs - freeb : 0u;
+  uint32_t E = E0, next = start;
+  int nins = nabs;
+  bool general = false, replayed = false;
+  if (E0 > 0) {
+    // the first E0 cold entries, all before the oldest present cold block
+    const uint32_t lim = pmin > start ? pmin - start : 0u;
+    uint32_t have = 0;
+    int last = -1;
+#pragma unroll
+    for (int w = 0; w < NW; w++) {
+      const uint32_t l0 = 32u * w;
+      const unsigned mk = lim >= l0 + 32u ? FULL_MASK : (lim > l0 ? (1u << (lim - l0)) - 1u : 0u);
+      const unsigned b = S.livew[w] & mk;
+      const uint32_t n = (uint32_t)__popc(b);
+      if (have < E0 && have + n >= E0) last = (int)l0 + nth_set_bit32(b, (int)(E0 - have) - 1);
+      have += n;
+    }
+    if (last >= 0) {
+#pragma unroll
+      for (int r = 0; r < R; r++)
+        if (cold[r] && r * NT + tid <= last) {
+          if (x[r] & SINGLE_FLAG)
+            t.log[(start + (uint32_t)(r * NT + tid)) & t.rmask] = LOG_DEAD;
+          else
+            t.st[x[r]] = STAMP_NONE;
+        }
+      next = start + (uint32_t)last + 1u;
+    } else {
+      ids_freq_general<NT>(t, m, start, K, cd, nb, E0, pmin, nabs, D, fmax, scratch, nbmax, S, &A.slow);
+      general = true;
+      replayed = S.changed != 0;
+      E = (uint32_t)S.nvic;
+      nins = S.nins;
+      next = S.nh;
+      he = S.fs.femin;
+      hp = S.fs.fhot;
+    }
+  }
+  const IdsScratch sc = ids_scratch(scratch, nbmax);
+#pragma unroll 1
+  for (int k = tid; k < nb; k += NT) {
+    const uint32_t b = cd[k] & CODE_SINGLE, pos = m.T + (uint32_t)k;
+    const int kind = general ? sc.kind[k] : -1;
+    if (kind >= 2) {   // evicted within this request
+      t.log[pos & t.rmask] = LOG_DEAD;
+      continue;
+    }
+    if (b != CODE_SINGLE) {
+      const bool ins = kind >= 0 ? kind == 1 : (cd[k] >> 31) != 0u || t.st[b] == STAMP_NONE;
+      t.fe[b] = ins ? D : freq_hit(t.fe[b], D, fmax);
+      t.st[b] = pos;
+    }
+    t.log[pos & t.rmask] = b != CODE_SINGLE ? b : SINGLE_FLAG | (uint32_t)(q.pos0 + k);
+  }
+  const uint32_t size = m.size + (uint32_t)nins - E;
+  FreqMeta fn = f;
+  uint32_t nh = m.head;
+  if (replayed) {
+    fn = FreqMeta{m.head, 0u};   // the next search starts at the head
+  } else if (E > 0) {
+    if (start == m.head) {
+      nh = min(hp, next);
+      fn.fmin = he;
+    } else {
+      fn.fmin = min(f.fmin, he);
+    }
+    fn.fscan = next;
+  }
+  // the window of this worker's next update, from where its search will start
+  const uint32_t ws = fn.fmin > D ? fn.fscan : nh;
+  const bool refresh = size + (uint32_t)nbmax > K && !replayed;
+  if (refresh) {
+#pragma unroll
+    for (int r = 0; r < R; r++) {
+      const uint32_t p = ws + (uint32_t)(r * NT + tid);
+      if (p < m.T) cp_async4(win + r * NT + tid, t.log + (p & t.rmask));
+    }
+  }
+  grp_bar<NT>();   // (every thread has read the old state)
+  if (tid == 0) {
+    // (a window that starts before this update's victims would miss their marks)
+    *whead = ws;
+    *wlen = refresh && ws >= next && m.T > ws ? min((uint32_t)IDS_WIN, m.T - ws) : 0u;
+    *fm = fn;
+    meta->size = size;
+    meta->head = nh;
+    meta->T = m.T + (uint32_t)nb;
+    A.inserted += nins;
+    A.evicted += E;
+    if (E > 0 && A.first_evict_i < 0) {
+      A.first_evict_i = i;
+      A.first_live = A.inserted - A.evicted;
+    }
+  }
+}
+
 // ------------------------------------------------------------ control warp
 
 // A controller sample with a non-empty window (as the CTA-wide tick of the
@@ -1208,6 +1623,8 @@ struct IdsEvents {
   uint64_t pk;       // key of the last arrival
   double prev;       // the last arrival
   int conc, ctl, spike;   // C, controller on, load-spike schedule
+  uint64_t dhi;           // (frequency eviction) key up to which the decay step is surely D
+  uint32_t D;
   float tau, omega;       // in the Below regime
   uint64_t* skey;    // [32 ng] completion keys by slot
   int4* srec;        // [slots] worker, blocks, next in queue, request
@@ -1374,7 +1791,7 @@ __device__ __forceinline__ void ev_sample(SimCtx& c, IdsEvents<WIDE>& E, int lan
 // controller samples, steps of the load-spike schedule; ties in that order),
 // then what its choice needs.  drain: past the last request, the completions
 // that remain (they start the queued requests).
-template <bool WIDE>
+template <bool WIDE, bool FREQ>
 __device__ __forceinline__ void ev_arrive(SimCtx& c, IdsShared& Sh, IdsEvents<WIDE>& E, int64_t i,
                                           bool drain, float* act, int* nfz, int lane) {
   SimScalars& S = *c.S;
@@ -1429,6 +1846,13 @@ __device__ __forceinline__ void ev_arrive(SimCtx& c, IdsShared& Sh, IdsEvents<WI
   if (drain) return;
   E.pk = ka;
   E.prev = tval(ka);
+  if (FREQ && ka >= E.dhi) {
+    // decay step of the arrival, floor(a / decay_s); the division (650 cycles)
+    // only where a has come near the next step (arrivals do not decrease)
+    const double s = c.d->decay_s, fl = floor(__ddiv_rn(E.prev, s));
+    E.D = fl < 2147483648.0 ? (uint32_t)fl : 2147483648u;
+    E.dhi = fl < 2147483648.0 ? tkey(__dmul_rn(__dmul_rn(fl + 1.0, s), 1.0 - 0x1p-40)) : KEY_NONE;
+  }
 #pragma unroll
   for (int h = 0; h < IdsEvents<WIDE>::H; h++) {
     const int j = lane + 32 * h;
@@ -1442,6 +1866,7 @@ __device__ __forceinline__ void ev_arrive(SimCtx& c, IdsShared& Sh, IdsEvents<WI
     ar.a = E.prev;
     ar.tau = E.tau;
     ar.omega = E.omega;
+    ar.D = FREQ ? E.D : 0u;
     if (E.ctl && c.d->policy != RS_POLICY_LOADBAL && S.regime > 0) {
       ar.tau = c.L->mc.regime_tau[S.regime];
       ar.omega = c.L->mc.regime_omega[S.regime];
@@ -1505,8 +1930,9 @@ __device__ __forceinline__ void ids_stage(const SimCtx& c, IdsShared& Sh, const 
 
 // ------------------------------------------------------------ the kernel
 
-// VAR 0: planned updates (few workers per update warp); 1: up to 32 workers; 2: up to 64.
-template <int NU, int MINB, bool SG, int VAR>
+// VAR 0: planned updates (a worker per update warp); 1: up to 32 workers; 2: up to 64.
+// FREQ: launches that hold replicas which evict by frequency (not SG, not VAR 0).
+template <int NU, int MINB, bool SG, int VAR, bool FREQ = false>
 __global__ void __launch_bounds__((NU + 2) * 32, MINB)
     k_sim_ids(const SimDesc* __restrict__ descs, const __grid_constant__ SimBuffers b,
               const __grid_constant__ SimLaunch L) {
@@ -1522,7 +1948,7 @@ __global__ void __launch_bounds__((NU + 2) * 32, MINB)
   const int W = mc.W;
   const int nft = ftab_size(mc.cap);
   const int nbcap = L.nbmax > 0 ? L.nbmax : 1;
-  const IdsLayout lay = make_ids_layout(W, L.nbmax, L.cmax, nft, NTU, SG);
+  const IdsLayout lay = make_ids_layout(W, L.nbmax, L.cmax, nft, NTU, SG, FREQ);
   unsigned char* slotbase;
   if constexpr (SG)
     slotbase = b.slotmem + (size_t)sid * lay.slot_bytes;
@@ -1563,7 +1989,8 @@ __global__ void __launch_bounds__((NU + 2) * 32, MINB)
   int* nfz = reinterpret_cast<int*>(smem + lay.nfz);                 // [2][W]
   uint32_t* whead = reinterpret_cast<uint32_t*>(smem + lay.whead);
   uint32_t* wlen = reinterpret_cast<uint32_t*>(smem + lay.wlen);
-  uint32_t* win = reinterpret_cast<uint32_t*>(smem + lay.win);       // [W][NTU]
+  uint32_t* win = reinterpret_cast<uint32_t*>(smem + lay.win);       // [W][IDS_WIN or IDS_WRING]
+  FreqMeta* wfreq = reinterpret_cast<FreqMeta*>(smem + lay.wfreq);
   uint32_t* stamps = d.stamps;
   const size_t nre = d.nre;
   const int64_t n = d.n_req;
@@ -1587,6 +2014,7 @@ __global__ void __launch_bounds__((NU + 2) * 32, MINB)
       c.wqt[j] = -1;
       whead[j] = 0;
       wlen[j] = 0;
+      if (FREQ) wfreq[j] = FreqMeta{0u, 0u};
     }
     if (threadIdx.x == 0) {
       memset(&S, 0, sizeof(SimScalars));
@@ -1609,6 +2037,7 @@ __global__ void __launch_bounds__((NU + 2) * 32, MINB)
     auto table = [&](int j) {
       IdsTable t;
       t.st = stamps + j * nre;
+      t.fe = FREQ ? d.fexp + j * nre : nullptr;
       t.log = b.log + ((size_t)sid * W + j) * L.g.R;
       t.rmask = L.ids_rmask;
       return t;
@@ -1677,7 +2106,11 @@ __global__ void __launch_bounds__((NU + 2) * 32, MINB)
           if (PLAN && Sh.plan[js].step != IDS_GENERAL) {
             ids_apply<NTU>(t, c.wmeta + js, Sh.plan[js], win + js * IDS_WRING, cd, q);
           } else {
-            if constexpr (PLAN)
+            if (FREQ && d.eviction == RS_EVICT_FREQ)
+              ids_update_freq<NTU>(S, Sh, L.g.K, L.nbmax, t, c.wmeta + js, wfreq + js, cd, q, Sh.pub[p].D,
+                                   (uint32_t)d.freq_max, scratch, win + (size_t)js * IDS_WIN, whead + js,
+                                   wlen + js, i);
+            else if constexpr (PLAN)
               ids_update_unplanned<NTU>(S, Sh, L.g.K, L.nbmax, t, c.wmeta + js, cd, q, scratch, wlen + js, i);
             else
               ids_update<NTU, true>(S, Sh, L.g.K, L.nbmax, t, c.wmeta + js, cd, q, scratch,
@@ -1731,6 +2164,8 @@ __global__ void __launch_bounds__((NU + 2) * 32, MINB)
       E.tick = d.controller ? tkey(mc.dt) : KEY_INF;
       E.prev = 0.0;
       E.pk = tkey(0.0);
+      E.D = 0u;
+      E.dhi = 0ull;
       // held in registers: a later load of the descriptor would be on the path
       E.conc = d.C;
       E.ctl = d.controller;
@@ -1833,7 +2268,7 @@ __global__ void __launch_bounds__((NU + 2) * 32, MINB)
         }
       }
       if constexpr (!SG)
-        ev_arrive(c, Sh, E, i + 1, i + 1 == n, act, nfz, lane);
+        ev_arrive<WIDE, FREQ>(c, Sh, E, i + 1, i + 1 == n, act, nfz, lane);
       else if (i + 1 < n)
         ids_arrive(c, Sh, i + 1, act, nfz, lane);
     }
@@ -1984,10 +2419,15 @@ cudaError_t launch_sim_ids(const SimDesc* d_desc, const SimBuffers& b, const Sim
   if (e != cudaSuccess) return e;
   const int nu = sim_ids_update_warps(L.nsim, sms);
   const bool sg = L.slots_global != 0;
-  const size_t smem = sim_ids_smem_bytes(L.mc.W, L.nbmax, L.cmax, L.mc.cap, 32 * nu, sg);
+  const bool freq = b.fexp != nullptr;
+  if (freq && sg) return cudaErrorInvalidValue;   // (such launches use the tables)
+  const size_t smem = sim_ids_smem_bytes(L.mc.W, L.nbmax, L.cmax, L.mc.cap, 32 * nu, sg, freq);
   void (*kern)(const SimDesc*, const SimBuffers, const SimLaunch);
   const int var = L.mc.W <= nu * ids_plan_workers(nu) ? 0 : (L.mc.W <= 32 ? 1 : 2);
-  if (nu == 6)
+  if (freq)
+    kern = nu == 6 ? (var == 2 ? k_sim_ids<6, 2, false, 2, true> : k_sim_ids<6, 2, false, 1, true>)
+                   : (var == 2 ? k_sim_ids<2, 5, false, 2, true> : k_sim_ids<2, 5, false, 1, true>);
+  else if (nu == 6)
     kern = var == 0 ? (sg ? k_sim_ids<6, 2, true, 0> : k_sim_ids<6, 2, false, 0>)
                     : (sg ? k_sim_ids<6, 2, true, 2>
                           : (var == 1 ? k_sim_ids<6, 2, false, 1> : k_sim_ids<6, 2, false, 2>));

@@ -117,3 +117,23 @@ def test_ids_from_given_hashes_repeated_block_and_long_prompt():
     tr2 = wk.Replica(0, 8, wk.POLICY_DYNAMO, 0, 1.0, 0.0, 0, tr.n_req)
     st, _ = _both(small, [tr], [tr2])
     assert st == rs.RS_ERR_CAPACITY
+
+
+@pytest.mark.parametrize("W,K,nrep,hi,decay,fmax", [
+    (3, 190, 4, 3000, 0.5, 64),       # ring of 2 K, frequencies that decay between requests
+    (6, 900, 5, 7000, 50.0, 1 << 20),  # mostly hot: the sequence is replayed, hot victims
+    (2, 120, 3, 1900, 5.0, 2),         # a request evicts its own blocks
+    (33, 300, 2, 3000, 1.0, 8),
+    (4, 400, 310, 1500, 2.0, 16),      # two update warps
+])
+def test_frequency_eviction_ids_equal_tables(W, K, nrep, hi, decay, fmax):
+    tr = _trace(600 if nrep < 300 else 150, W + K, groups=6 if fmax > 64 else 12, hi=hi)
+    reps = []
+    for r in range(nrep):
+        rep = wk.Replica(0, 40 + 9 * (r % 7), wk.POLICY_DYNAMO if r % 3 else wk.POLICY_LOADBAL, r % 2, 1.0, 0.3 * (r % 2),
+                         r, tr.n_req)
+        if r % 4 != 3:   # exact LRU replicas in the same launch
+            rep.eviction, rep.freq_max, rep.decay_s = rs.RS_EVICT_FREQ, fmax, decay * (1 + r % 2)
+        reps.append(rep)
+    st, g = _both(rs.Context(W=W, K=K), [tr], reps, [(r, j) for r in (0, nrep - 1) for j in (0, W - 1)])
+    assert st == rs.RS_OK and min(x["result"]["evicted_blocks"] for x in g) > 0
