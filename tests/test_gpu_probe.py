@@ -110,3 +110,29 @@ def test_probe_arguments():
         with pytest.raises(rs.RoutesimError) as e:
             rs.route_probe(ctx.h, inst, d.tokens, d.offsets, n, out)
         assert e.value.status == rs.RS_ERR_INVALID
+
+
+@pytest.mark.parametrize("W", [1, 2, 31, 32, 33, 63, 64])
+def test_probe_walk_edges(W):
+    # walks that end at, before and after a chunk of 32 blocks and at the prompt's end, on every
+    # count of workers around a warp: routed prompts (spread by tau) probed again, cut and extended
+    rng = np.random.default_rng(W)
+    base = rng.integers(0, 32000, 16 * 140).astype(np.int32)
+    blocks = [0, 1, 2, 31, 32, 33, 34, 64, 65, 66, 97, 128, 129]
+
+    def trace(parts):
+        off = np.concatenate([[0], np.cumsum([p.size for p in parts])]).astype(np.int64)
+        tok = np.concatenate(parts).astype(np.int32)
+        tok = np.concatenate([tok, np.zeros(-tok.size % 4 + 4, np.int32)])
+        n = len(parts)
+        return wk.Trace(tok, off, np.zeros(n), np.ones(n, np.int32), np.zeros(n, np.int32))
+
+    routed = trace([base[:16 * b + int(rng.integers(0, 16))] for b in blocks for _ in range(4)])
+    ctx = rs.Context(W=W, K=200, n_instances=1, tau=200.0, omega=1.0, seed=3)
+    ref = O.Router(O.OracleConfig(W=W, K=200), 1.0, 200.0, 3)
+    _route(ctx, ref, 0, routed, W)
+    other = rng.integers(0, 32000, 16 * 140).astype(np.int32)
+    probed = trace([np.concatenate([base[:16 * b + int(rng.integers(0, 16))], other[:16 * e]]) for b in blocks for e in (0, 1, 33)])
+    got = _probe(ctx, 0, probed, W)
+    st, want = ref.probe(0, probed.tokens, probed.offsets)
+    assert st == 0 and np.array_equal(got, want) and got.max() >= 128
