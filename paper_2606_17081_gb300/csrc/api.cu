@@ -1004,7 +1004,7 @@ rs_status simulate_replicas(rs_ctx* ctx, const rs_trace* traces, int32_t n_trace
     const size_t g1 = std::min(jobs.size(), g0 + HASH_MAX_JOBS);
     const int64_t total = jobs[g1 - 1].req_base + jobs[g1 - 1].n_req - jobs[g0].req_base;
     CK(launch_block_hash(P<HashJob>(ctx->hjobs) + g0, (int)(g1 - g0), total, ctx->cfg.hash_seed,
-                         nullptr, ctx->st),
+                         ctx->st),
        "block hash launch");
     launches++;
   }

@@ -141,7 +141,7 @@ struct HashJob {
 };
 constexpr int HASH_MAX_JOBS = 64;
 cudaError_t launch_block_hash(const HashJob* jobs_dev, int njobs, int64_t total_req, uint64_t seed,
-                              int64_t* nbmax_out, cudaStream_t st);
+                              cudaStream_t st);
 cudaError_t launch_block_hash_one(const HashJob& job, uint64_t seed, cudaStream_t st);
 // out[0] = the longest prompt's full blocks, out[1] = offsets[n] (out: device
 // memory or pinned host memory; small n).
