@@ -264,7 +264,7 @@ __host__ __device__ inline IdsLayout make_ids_layout(int W, int nbmax, int cmax,
   L.h_k = slots(8 * 32 * G);
   L.srec = L.gk = L.gf = 0;
   if (!slots_global) {
-    L.srec = take(16 * C);
+    L.srec = take(16 * 32 * G);   // (whole groups: read past the slots for no completion)
     if (G > 32) {
       L.gk = take(8 * G);
       L.gf = take(4 * G);
@@ -1617,12 +1617,15 @@ struct IdsEvents {
   static constexpr int H = WIDE ? 2 : 1;
   uint64_t lk, kc;   // earliest completion of this lane's groups, of all
   int lf, fc;        // their slots
+  int4 cr;           // srec[fc]
+  int fnext;         // the free slot taken next
   int A[H], serv[H], qh[H], qt[H];
   int inflight, nfree, np, cur, ng;
   uint64_t mft, tick;   // keys: earliest pending first token, next controller sample
   uint64_t pk;       // key of the last arrival
   double prev;       // the last arrival
-  int conc, ctl, spike;   // C, controller on, load-spike schedule
+  int conc, ctl, spike, regimes;   // C, controller on, load-spike schedule, the policy takes regimes
+  int64_t row0;           // first record row
   uint64_t dhi;           // (frequency eviction) key up to which the decay step is surely D
   uint32_t D;
   float tau, omega;       // in the Below regime
@@ -1632,7 +1635,6 @@ struct IdsEvents {
   int* gf;
   double *sa, *so, *soitl;   // [slots] of queued requests: arrival, w_c o, O itl
   int* freestk;
-  double* rp;        // lanes 0-2: start, first token, completion records
 
   __device__ __forceinline__ int get(const int (&v)[H], int j) const {
     int x = __shfl_sync(FULL_MASK, v[0], j & 31);
@@ -1678,38 +1680,41 @@ __device__ __forceinline__ void ev_min(const IdsEvents<WIDE>& E, uint64_t k, int
   fo = __shfl_sync(FULL_MASK, f, __ffs(eq) - 1);
 }
 
-// Request req in slot f is in service from t on: first token ft, completion ct.
+// The request of record r, in slot f, completes at the time of key k.
 template <bool WIDE>
-__device__ __forceinline__ void ev_start(SimCtx& c, IdsEvents<WIDE>& E, int f, int req, double t,
-                                         double ft, double ct, double a, int lane) {
-  const uint64_t k = tkey(ct);
+__device__ __forceinline__ void ev_push(IdsEvents<WIDE>& E, int f, uint64_t k, const int4& r,
+                                        int lane) {
   const int g = f >> 5;
   if (lane == (g & 31)) {
     E.skey[f] = k;
-    if (E.ng > 32 && (k < E.gk[g] || (k == E.gk[g] && req < E.srec[E.gf[g]].w))) {
+    if (E.ng > 32 && (k < E.gk[g] || (k == E.gk[g] && r.w < E.srec[E.gf[g]].w))) {
       E.gk[g] = k;
       E.gf[g] = f;
     }
-    if (k < E.lk || (k == E.lk && req < E.srec[E.lf].w)) {
+    if (k < E.lk || (k == E.lk && r.w < E.srec[E.lf].w)) {
       E.lk = k;
       E.lf = f;
     }
   }
-  if (k < E.kc || (k == E.kc && req < E.srec[E.fc].w)) {
+  if (k < E.kc || (k == E.kc && r.w < E.cr.w)) {
     E.kc = k;
     E.fc = f;
+    E.cr = r;
   }
-  if (lane < 3) E.rp[req] = lane == 0 ? t : (lane == 1 ? ft : ct);
+}
+
+// A service's records, and its place in the controller's window (one lane).
+template <bool WIDE>
+__device__ __forceinline__ void ev_records(const SimCtx& c, const IdsEvents<WIDE>& E, int req,
+                                           double t, double ft, double ct, double a) {
+  const int64_t row = E.row0 + req;
+  c.b->rec.start[row] = t;
+  c.b->rec.first_token[row] = ft;
+  c.b->rec.completion[row] = ct;
   if (E.ctl) {
-    if (lane == 0) {
-      c.pend_ft(E.cur)[E.np] = ft;
-      c.pend_tt(E.cur)[E.np] = __dsub_rn(ft, a);
-    }
-    E.np++;
-    const uint64_t kf = tkey(ft);
-    if (kf < E.mft) E.mft = kf;
+    c.pend_ft(E.cur)[E.np] = ft;
+    c.pend_tt(E.cur)[E.np] = __dsub_rn(ft, a);
   }
-  __syncwarp();
 }
 
 // Takes the earliest completion out and completes it: the slot is free, the
@@ -1718,7 +1723,7 @@ template <bool WIDE>
 __device__ __forceinline__ void ev_complete(SimCtx& c, IdsEvents<WIDE>& E, int lane) {
   const int f = E.fc, g = f >> 5;
   const double t = tval(E.kc);
-  const int4 r = E.srec[f];
+  const int4 r = E.cr;
   const int j = r.x;
   // the group without f, then the earliest of all groups
   const int s = 32 * g + lane;
@@ -1749,8 +1754,10 @@ __device__ __forceinline__ void ev_complete(SimCtx& c, IdsEvents<WIDE>& E, int l
     E.lk = E.kc;
     E.lf = E.fc;
   }
+  E.cr = E.srec[E.fc];
   if (lane == 0) E.freestk[E.nfree] = f;
   E.nfree++;
+  E.fnext = f;
   E.inflight--;
   E.add(E.A, j, -r.y, lane);
   const int f2 = E.get(E.qh, j);
@@ -1762,7 +1769,14 @@ __device__ __forceinline__ void ev_complete(SimCtx& c, IdsEvents<WIDE>& E, int l
     E.put(E.qh, j, r2.z, lane);
     if (r2.z < 0) E.put(E.qt, j, -1, lane);
     const double ft = __dadd_rn(t, __dsub_rn(ev_f(c, E.get(E.serv, j)), E.so[f2]));
-    ev_start(c, E, f2, r2.w, t, ft, __dadd_rn(ft, E.soitl[f2]), E.sa[f2], lane);
+    const double ct = __dadd_rn(ft, E.soitl[f2]);
+    ev_push(E, f2, tkey(ct), r2, lane);
+    if (lane == 0) ev_records(c, E, r2.w, t, ft, ct, E.sa[f2]);
+    if (E.ctl) {
+      E.np++;
+      E.mft = min(E.mft, tkey(ft));
+    }
+    __syncwarp();
   }
 }
 
@@ -1803,11 +1817,26 @@ __device__ __forceinline__ void ev_arrive(SimCtx& c, IdsShared& Sh, IdsEvents<WI
   }
   const uint64_t krel = tkey(q.rel);
   uint64_t ka = E.pk;              // while waiting: the time reached
-  uint64_t lim = drain ? KEY_NONE - 1 : KEY_INF - 1;   // events up to here are due
-  if (drain) E.tick = KEY_NONE;
+  uint64_t lim = KEY_INF - 1;      // events up to here are due
   int conc = E.conc;
-  bool wait = !drain, mid = false, step = false, ok = true;
-  for (;;) {
+  bool wait = true, mid = false, step = false, ok = true;
+  if (drain || !(E.ctl | E.spike)) {
+    // no samples, one concurrency (or the end): completions alone, in a loop of
+    // few branches (1 430 cycles a request at W = 3; 1 560 with the samples' test in it,
+    // 1 730 in the loop below)
+    if (drain) ka = KEY_NONE - 1;
+    for (;;) {
+      const bool w = !drain && E.inflight >= conc;
+      if (!w && !drain && krel > ka) ka = krel;   // (a free place, once there, stays)
+      if (E.kc > (w ? KEY_INF - 1 : ka)) {
+        if (w && lane == 0) S.status = RS_ERR_TIMEOUT;   // cannot happen, as below
+        ok = !w;
+        break;
+      }
+      if (w && E.kc > ka) ka = E.kc;
+      ev_complete(c, E, lane);
+    }
+  } else for (;;) {
     if (wait) {
       // closed-loop client (§7.4): until fewer than C(t) requests are in flight
       if (E.spike) {
@@ -1862,16 +1891,14 @@ __device__ __forceinline__ void ev_arrive(SimCtx& c, IdsShared& Sh, IdsEvents<WI
     }
   }
   if (lane == 0) {
-    IdsArrival ar;
+    IdsArrival& ar = Sh.pub[p];
     ar.a = E.prev;
-    ar.tau = E.tau;
-    ar.omega = E.omega;
-    ar.D = FREQ ? E.D : 0u;
-    if (E.ctl && c.d->policy != RS_POLICY_LOADBAL && S.regime > 0) {
-      ar.tau = c.L->mc.regime_tau[S.regime];
-      ar.omega = c.L->mc.regime_omega[S.regime];
+    if (FREQ) ar.D = E.D;
+    if (E.ctl) {   // (else written once)
+      const bool shift = E.regimes && S.regime > 0;
+      ar.tau = shift ? c.L->mc.regime_tau[S.regime] : E.tau;
+      ar.omega = shift ? c.L->mc.regime_omega[S.regime] : E.omega;
     }
-    Sh.pub[p] = ar;
     if (!ok) Sh.stat[p] = S.status;
   }
 }
@@ -1991,12 +2018,12 @@ __global__ void __launch_bounds__((NU + 2) * 32, MINB)
   uint32_t* wlen = reinterpret_cast<uint32_t*>(smem + lay.wlen);
   uint32_t* win = reinterpret_cast<uint32_t*>(smem + lay.win);       // [W][IDS_WIN or IDS_WRING]
   FreqMeta* wfreq = reinterpret_cast<FreqMeta*>(smem + lay.wfreq);
+  // held in registers: the compiler would load them again from the descriptor
+  // where they are used, on the path between two joins
   uint32_t* stamps = d.stamps;
-  const size_t nre = d.nre;
-  const int64_t n = d.n_req;
-
+  int64_t nre = d.nre, n = d.n_req;
   int policy = d.policy;
-  asm volatile("" : "+r"(policy));   // (held in a register)
+  asm volatile("" : "+r"(policy), "+l"(stamps), "+l"(nre), "+l"(n));
 
   // ---- initial state: empty caches, idle workers
   {
@@ -2170,9 +2197,11 @@ __global__ void __launch_bounds__((NU + 2) * 32, MINB)
       E.conc = d.C;
       E.ctl = d.controller;
       E.spike = d.c_mid > 0;
+      E.regimes = d.policy != RS_POLICY_LOADBAL;
       E.tau = d.policy == RS_POLICY_LOADBAL ? 0.0f : d.tau;
       E.omega = d.policy == RS_POLICY_LOADBAL ? 0.0f : d.omega;
-      asm volatile("" : "+r"(E.conc), "+r"(E.ctl), "+r"(E.spike), "+f"(E.tau), "+f"(E.omega));
+      E.row0 = d.rec_base;
+      asm volatile("" : "+r"(E.conc), "+r"(E.ctl), "+r"(E.spike), "+r"(E.regimes), "+f"(E.tau), "+f"(E.omega), "+l"(E.row0));
       E.skey = c.h_k;
       E.srec = reinterpret_cast<int4*>(smem + lay.srec);
       E.gk = reinterpret_cast<uint64_t*>(smem + lay.gk);
@@ -2181,7 +2210,13 @@ __global__ void __launch_bounds__((NU + 2) * 32, MINB)
       E.so = c.f_o;
       E.soitl = c.f_oitl;
       E.freestk = c.freestk;
-      E.rp = (lane == 0 ? b.rec.start : (lane == 1 ? b.rec.first_token : b.rec.completion)) + d.rec_base;
+      E.cr = make_int4(0, 0, -1, 0);
+      E.fnext = 0;   // (freestk[cslots - 1])
+      if (lane < 2) {
+        Sh.pub[lane].tau = E.tau;
+        Sh.pub[lane].omega = E.omega;
+        Sh.pub[lane].D = 0u;
+      }
       for (int f = lane; f < 32 * E.ng; f += 32) E.skey[f] = KEY_NONE;
       if (E.ng > 32)
         for (int g = lane; g < E.ng; g += 32) {
@@ -2216,6 +2251,8 @@ __global__ void __launch_bounds__((NU + 2) * 32, MINB)
           }
         }
         double ft[H], ct[H];
+        uint64_t kt[H];
+        unsigned can[H];   // workers below the service limit
         if constexpr (!SG) {
           // first token and completion of a service that starts on each worker now
 #pragma unroll
@@ -2223,8 +2260,11 @@ __global__ void __launch_bounds__((NU + 2) * 32, MINB)
             const int ns = min(E.serv[h] + 1, mc.cap - 1);
             ft[h] = __dadd_rn(E.prev, __dsub_rn(ev_f(c, ns), wco[h]));
             ct[h] = __dadd_rn(ft[h], q.oitl);
+            kt[h] = tkey(ct[h]);
+            can[h] = __ballot_sync(FULL_MASK, E.serv[h] < mc.cap - 1);
           }
         }
+        const int blk = (int)q.blk;
         choice_wait<NT>();
         const int js = Sh.js;
         auto of = [&](const double (&v)[H]) {
@@ -2237,14 +2277,31 @@ __global__ void __launch_bounds__((NU + 2) * 32, MINB)
         };
         if constexpr (!SG) {
           // request i's load and service start on worker js
-          const int f = E.freestk[--E.nfree];
+          const int f = E.fnext;
           E.inflight++;
-          E.add(E.A, js, (int)q.blk, lane);
-          if (lane == 0) E.srec[f] = make_int4(js, (int)q.blk, -1, (int)i);
-          if (E.get(E.serv, js) < mc.cap - 1) {
-            E.add(E.serv, js, 1, lane);
-            ev_start(c, E, f, (int)i, E.prev, of(ft), of(ct), E.prev, lane);
+          if (--E.nfree > 0) E.fnext = E.freestk[E.nfree - 1];
+          const int4 r = make_int4(js, blk, -1, (int)i);
+          if (lane == 0) E.srec[f] = r;
+          const int hj = WIDE ? js >> 5 : 0;
+          const bool mine = lane == (js & 31);
+          if ((((WIDE && hj) ? can[H - 1] : can[0]) >> (js & 31)) & 1u) {
+            const uint64_t kj = (WIDE && hj) ? kt[H - 1] : kt[0];
+            const unsigned hi = __shfl_sync(FULL_MASK, (unsigned)(kj >> 32), js & 31);
+            const unsigned lo = __shfl_sync(FULL_MASK, (unsigned)kj, js & 31);
+            ev_push(E, f, ((uint64_t)hi << 32) | lo, r, lane);
+#pragma unroll
+            for (int h = 0; h < H; h++)
+              if (mine && h == hj) {
+                E.A[h] += blk;
+                E.serv[h]++;
+                ev_records(c, E, (int)i, E.prev, ft[h], ct[h], E.prev);
+              }
+            if (E.ctl) {
+              E.np++;
+              E.mft = min(E.mft, tkey(of(ft)));
+            }
           } else {
+            E.add(E.A, js, blk, lane);
             const int qt = E.get(E.qt, js);
             const double w = of(wco);
             if (lane == 0) {
@@ -2255,8 +2312,8 @@ __global__ void __launch_bounds__((NU + 2) * 32, MINB)
             }
             if (qt < 0) E.put(E.qh, js, f, lane);
             E.put(E.qt, js, f, lane);
-            __syncwarp();
           }
+          __syncwarp();
           if (lane == 0) S.n_routed = i + 1;
         } else {
           const double w = of(wco);
