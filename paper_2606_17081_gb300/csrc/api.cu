@@ -674,13 +674,16 @@ static rs_status trace_ids(rs_ctx* ctx, const rs_trace* traces, const std::vecto
   const size_t nj = tr.size();
   size_t pos = 0;
   std::vector<IdJob> jobs(nj);
+  std::vector<int64_t> routed(used.size(), 0);   // requests of a trace that some replica routes
+  for (int32_t k = 0; k < n_replicas; k++)
+    routed[params[k].trace] = std::max(routed[params[k].trace], params[k].n_req);
   for (size_t k = 0; k < nj; k++) {
     const int64_t blocks = tot[tr[k]] / 16 + 1;
     uint64_t cap = 32;
     while (cap < 2 * (uint64_t)blocks) cap <<= 1;
     jobs[k].hashes = all[k].out;
     jobs[k].offsets = all[k].offsets;
-    jobs[k].n_req = all[k].n_req;
+    jobs[k].n_req = routed[tr[k]];
     jobs[k].tmask = (uint32_t)(cap - 1);
     pos += (size_t)blocks;
   }
@@ -708,9 +711,11 @@ static rs_status trace_ids(rs_ctx* ctx, const rs_trace* traces, const std::vecto
   pos = 0;
   for (size_t g = 0; g + 1 < start.size(); g++) {
     slots = 0;
+    int64_t base = 0;
     for (size_t k = start[g]; k < start[g + 1]; k++) {
       IdJob& J = jobs[k];
-      J.req_base = all[k].req_base - all[start[g]].req_base;
+      J.req_base = base;
+      base += J.n_req;
       J.keys = P<unsigned long long>(ctx->i_keys) + slots;
       J.first = P<uint32_t>(ctx->i_first) + slots;
       J.num = P<uint32_t>(ctx->i_num) + slots;
@@ -822,6 +827,8 @@ rs_status simulate_replicas(rs_ctx* ctx, const rs_trace* traces, int32_t n_trace
   auto prehashed = [&](int t) { return traces[t].tokens == nullptr; };
   std::vector<const uint64_t*> dhash(n_traces, nullptr);
   if (host) {
+    ctx->last_nsim = 0;   // the last call's caches may refer to its staged hashes
+    ctx->last_ids.clear();
     size_t tb = 0, ob = 0, nb = 0, hb = 0;
     for (int t = 0; t < n_traces; t++) {
       if (!used[t] || traces[t].n_req == 0) continue;
