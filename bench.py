@@ -174,9 +174,18 @@ class ClockSampler:
                 "samples": len(rows)}
 
 
+def _log_bytes(K: int) -> int:
+    """Device bytes of one simulated worker's log (>= 4K entries); its stamps,
+    one per block that recurs in the trace, are a few percent of that."""
+    ring = 1
+    while ring < 4 * K:
+        ring <<= 1
+    return ring * 4
+
+
 def _table_bytes(K: int) -> int:
-    """Device bytes of one worker's cache: keys + stamps (>= 4K slots in
-    buckets of 8) and the stamp log (>= 4K entries)."""
+    """Device bytes of one live-router worker's cache: keys + stamps (>= 4K
+    slots in buckets of 8) and the stamp log (>= 4K entries)."""
     slots = 8
     while slots < 4 * K:
         slots <<= 1
@@ -186,27 +195,24 @@ def _table_bytes(K: int) -> int:
     return slots * 12 + ring * 4
 
 
-# DRAM bytes (read + write) of one full-size k_sim launch of the headline
+# DRAM bytes (read + write) of one full-size k_sim_ids launch of the headline
 # workload (dram__bytes_read.sum + dram__bytes_write.sum), with the SHA-256 of
-# the simulation kernel's sources it was taken with; None until such a
-# capture exists for these sources.  The full grid holds about 103 GB of
-# cache tables, so the capture ran on 304 of its 8192 simulations (one
-# resident wave, two per SM, 10 000 requests each: 234.69 GB) and is scaled by
-# 8192 / 304; every simulation's tables and requests are of the same kind.
-SIM_TRAFFIC = {"bytes": 234692720384 * 8192 / 304,
-               "sources_sha256": "188fdf42bea8a811467ab449087524e9d353034642b819cda337c020b3f84b3f",
-               "summary": "profiles/k_sim_grid.md",
-               "scaled_from": "304 simulations x 10 000 requests, times 8192 / 304"}
+# the simulation kernel's sources it was taken with.  The capture ran on 760 of
+# its 8192 simulations (one resident wave, five per SM) and is scaled.
+SIM_TRAFFIC = {"bytes": (3742924544 + 4207784448) * 8192 / 760,
+               "sources_sha256": "2277c66bc86672f04db7f8c64cb98e8dff21747e4cbdfb214705b18b3621d74d",
+               "summary": "profiles/k_sim_ids.md",
+               "scaled_from": "760 simulations x 10 000 requests, times 8192 / 760"}
 
 
 def _sim_traffic(full_size: bool):
-    """The captured DRAM traffic per k_sim launch, or None when the kernel
+    """The captured DRAM traffic per k_sim_ids launch, or None when the kernel
     changed since the capture (or the workload is not the full-size one)."""
     import hashlib
     if SIM_TRAFFIC["bytes"] is None:
         return None
     h = hashlib.sha256()
-    for f in ("sim_kernel.cu", "rs_device.cuh", "rs_internal.h"):
+    for f in ("sim_ids_kernel.cu", "sim_common.cuh", "rs_device.cuh", "rs_internal.h"):
         with open(os.path.join(ROOT, "paper_2606_17081_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     if not full_size or h.hexdigest() != SIM_TRAFFIC["sources_sha256"]:
@@ -215,22 +221,21 @@ def _sim_traffic(full_size: bool):
 
 
 def _alg_bytes(results, W: int) -> float:
-    """Algorithmic bytes of the simulation kernel for one launch (per-unit
-    figures: 32 B per first-miss probe of a bucketed table, 8 B per block hash
-    read, 32 B key sector + 16 B LRU stamp/log per inserted block, 64 B per
-    eviction, 16 B per touched block, per-request record bytes)."""
+    """Algorithmic bytes of the simulation on block ids for one launch (per-unit
+    figures: 4 B stamp per first-miss probe, 4 B block id read, 4 B log entry
+    and 4 B stamp written per block of a routed prompt, 4 B log entry and 4 B
+    stamp per eviction, per-request record bytes)."""
     b = 0.0
     for r in results:
-        touched = r.hashed_blocks - r.inserted_blocks
-        b += (32.0 * r.probe_blocks + 8.0 * r.hashed_blocks + 48.0 * r.inserted_blocks +
-              64.0 * r.evicted_blocks + 16.0 * touched + (48.0 + 4.0 * W) * r.n_routed)
+        b += (4.0 * r.probe_blocks + 12.0 * r.hashed_blocks + 8.0 * r.evicted_blocks +
+              (48.0 + 4.0 * W) * r.n_routed)
     return b
 
 
 def _roofline(results, W, sim_ms, peak, peak_kind):
     alg = _alg_bytes(results, W)
     ach = alg / (sim_ms / 1e3) / 1e9
-    return {"kernel": "k_sim (replica simulation, one CTA per replica)", "bound": "hbm",
+    return {"kernel": "k_sim_ids (replica simulation, one CTA per replica)", "bound": "hbm",
             "achieved": ach, "peak": peak, "unit": "GB/s", "frac": ach / peak,
             "peak_kind": peak_kind, "alg_bytes_per_launch": alg}
 
@@ -545,7 +550,7 @@ def run_gpu(args):
     roof["traffic_source"] = SIM_TRAFFIC["summary"]
     roof["traffic_scaled_from"] = SIM_TRAFFIC["scaled_from"]
     roof["note"] = (f"latency-bound event loop: {len(params)} simulations, "
-                    f"{'two' if len(params) > 152 else 'one'} resident per SM")
+                    f"{'five' if len(params) > 304 else 'two' if len(params) > 152 else 'one'} resident per SM")
     hash_avg = statistics.mean(hash_ms)
     nblocks = sum(int(np.sum(np.diff(t.offsets) // 16)) for t in traces)
     hash_bytes = 4.0 * hashed_tokens + 8.0 * nblocks
@@ -566,9 +571,9 @@ def run_gpu(args):
                    "cache_blocks": p.K,
                    "parallelism": f"replicas of one plan partitioned over {ws} GPU(s)",
                    "l2": "inputs larger than L2 every step (%.0f MB of tokens read, %.0f MB of "
-                         "cache tables cleared and rebuilt per step; L2 129 MB)" % (
+                         "cache logs per step; L2 129 MB)" % (
                              sum(t.tokens.nbytes for t in traces) / 1e6,
-                             _table_bytes(p.K) * p.W * len(params) / 1e6)},
+                             _log_bytes(p.K) * p.W * len(params) / 1e6)},
         "replicas_per_s": total_replicas / per_step_s,
         "requests_per_s": total_decisions / p.W / per_step_s,
         "kernels_ms_per_step": {"block_hash": hash_avg, "simulate": sim_avg,

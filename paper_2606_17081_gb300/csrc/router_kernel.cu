@@ -232,7 +232,7 @@ __global__ void __launch_bounds__(NT_ROUTE) k_route_batch(
                                      c.pfree + (size_t)js * nb, nb, nabs, sc, &S.us, R.warp_tot,
                                      &R.scan_pos);
     else
-      cache_lookup_all<NT_ROUTE, false>(tv, hb, nb, sc, &S.us, &S.probes);
+      cache_lookup_all<NT_ROUTE>(tv, hb, nb, sc, &S.us, &S.probes);
     cache_apply<NT_ROUTE>(tv, &meta[js], g.K, hb, nb, sc, &S.us, R.warp_tot, &R.scan_pos, captured);
     if (tid == 0) {
       if (S.us.err) R.status = S.us.err;

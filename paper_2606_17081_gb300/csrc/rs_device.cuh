@@ -147,55 +147,15 @@ __device__ __forceinline__ float router_cost(float omega, int64_t bprefill, int6
   return __fadd_rn(__fmul_rn(omega, __int2float_rn((int)bprefill)), __int2float_rn((int)active));
 }
 
-// Lowest-index argmin over c[0..W) (one thread).
-__device__ __forceinline__ int argmin_lowest(const float* c, int W) {
-  int b = 0;
-  for (int j = 1; j < W; j++)
-    if (c[j] < c[b]) b = j;
-  return b;
-}
-
-// Eq. (2): tau == 0 -> argmin; tau > 0 -> the first j whose cumulative weight
-// (sequential fp32 sum in worker order) exceeds u * S.  One thread.
-// ds (nullable) receives the draw's position for the near-boundary
+// Eq. (2) by a whole warp (W <= 64; every lane returns the same worker): tau == 0
+// -> the lowest-index argmin b of c; tau > 0 -> the first j whose cumulative
+// weight (sequential fp32 sum in worker order) exceeds u * S.  Lane l computes
+// the weights of workers l and l + 32, each once; every lane then sums them in
+// worker order from shuffles and keeps the sum at its own workers, so one pass
+// gives S, the worker where the draw falls and the sums around it.  ds (nullable;
+// written by lane 0) receives the draw's position for the near-boundary
 // statistic: {u S, S, largest cumulative weight <= u S (or NaN), smallest
 // cumulative weight > u S (or NaN)}.
-__device__ __forceinline__ int select_worker(const float* c, int W, float tau, uint32_t u24,
-                                             float* ds) {
-  const int b = argmin_lowest(c, W);
-  if (tau == 0.0f) return b;
-  const float cmin = c[b];
-  float S = 0.0f;
-  for (int j = 0; j < W; j++) S = __fadd_rn(S, exp_sm(-__fdiv_rn(__fsub_rn(c[j], cmin), tau)));
-  const float target = __fmul_rn(__fmul_rn((float)u24, 0x1p-24f), S);
-  const float qnan = __int_as_float(0x7FC00000);
-  float cum = 0.0f, lo = qnan, hi = qnan;
-  int pick = -1, last = b;
-  for (int j = 0; j < W; j++) {
-    const float e = exp_sm(-__fdiv_rn(__fsub_rn(c[j], cmin), tau));
-    cum = __fadd_rn(cum, e);
-    if (e > 0.0f) last = j;
-    if (pick < 0 && target < cum) {
-      pick = j;
-      hi = cum;
-    }
-    if (!(target < cum)) lo = cum;
-  }
-  if (ds) {
-    ds[0] = target;
-    ds[1] = S;
-    ds[2] = lo;
-    ds[3] = hi;
-  }
-  return pick >= 0 ? pick : last;
-}
-
-// select_worker computed by a whole warp (W <= 64; every lane returns the
-// same worker): lane l computes the weights of workers l and l + 32, each
-// once; every lane then sums them in worker order from shuffles and keeps the
-// sum at its own workers, so one pass gives S, the worker where the draw falls
-// and the sums around it, those of select_worker bit for bit.  b: the
-// lowest-index argmin of c.  ds (nullable) is written by lane 0.
 __device__ __forceinline__ int select_worker_warp(const float* c, int W, float tau, uint32_t u24,
                                                   int b, float* ds, int lane) {
   if (tau == 0.0f) return b;
@@ -414,11 +374,6 @@ __device__ __forceinline__ uint32_t table_find_free(const TableView& t, uint64_t
   return table_find_free_from(t, h, home_bucket(h, t.bmask), err, free_slot);
 }
 
-__device__ __forceinline__ uint32_t table_find(const TableView& t, uint64_t h, int* err) {
-  uint32_t fr;
-  return table_find_free(t, h, err, &fr);
-}
-
 // Claims the first EMPTY or TOMB slot of h's probe sequence (h known absent;
 // other threads of the CTA may insert concurrently).  *was_tomb reports a
 // reclaimed tombstone.
@@ -465,7 +420,8 @@ struct UpdateScratch {
 };
 
 struct UpdateShared {   // small shared scalars of the update
-  int n_absent, n_ins, reclaimed, n_victims, n_tomb, slow, err, dup;
+  int n_absent, n_ins, reclaimed, n_victims, n_tomb, slow, err;
+  int changed;   // of lru_exact
   uint32_t pmin, gathered;
 };
 
@@ -569,7 +525,6 @@ __device__ __forceinline__ void update_reset(UpdateShared* us) {
   us->n_victims = 0;
   us->n_tomb = 0;
   us->slow = 0;
-  us->dup = 0;
   us->pmin = STAMP_NONE;
   us->gathered = 0;
 }
@@ -582,14 +537,12 @@ __device__ __forceinline__ void freq_reset(FreqShared* fs) {
 }
 
 // Looks up every block of a request in one worker's cache (CTA-wide);
-// fills slot[] and pst[]; counts absent blocks; detects duplicate hashes
-// within the request (a shared-memory open-addressing set; each thread clears
-// the slot it claimed).  us must be reset before the call.
-template <int NT, bool DETECT_DUP = true>
+// fills slot[] and pst[]; counts absent blocks.  us must be reset before the call.
+template <int NT>
 __device__ __forceinline__ void cache_lookup_all(const TableView& t, const uint64_t* hbuf, int nb,
                                  UpdateScratch& sc, UpdateShared* us,
                                  unsigned long long* probes) {
-  int nabs = 0, err = 0, dup = 0;
+  int nabs = 0, err = 0;
   uint32_t pmin = STAMP_NONE;
   for (int k = threadIdx.x; k < nb; k += NT) {
     const uint64_t h = hbuf[k];
@@ -606,7 +559,6 @@ __device__ __forceinline__ void cache_lookup_all(const TableView& t, const uint6
     }
     sc.pst[k] = st;
     sc.evk[k] = 0;
-    if (DETECT_DUP) sc.owner[k] = dup_claim(sc, h, &dup);
   }
   nabs = __reduce_add_sync(FULL_MASK, (unsigned)nabs);
   pmin = __reduce_min_sync(FULL_MASK, pmin);
@@ -615,12 +567,8 @@ __device__ __forceinline__ void cache_lookup_all(const TableView& t, const uint6
     if (pmin != STAMP_NONE) atomicMin(&us->pmin, pmin);
   }
   if (err) us->err = RS_ERR_TIMEOUT;
-  if (dup) us->dup = 1;
   if (threadIdx.x == 0) atomicAdd(probes, (unsigned long long)nb);
   grp_bar<NT>();
-  if (DETECT_DUP)
-    for (int k = threadIdx.x; k < nb; k += NT)
-      if (sc.owner[k] >= 0) sc.dupset[sc.owner[k]] = 0ull;
 }
 
 // Claims table slot x for one insert of this update in the shared-memory set
@@ -637,37 +585,6 @@ __device__ __forceinline__ int32_t slot_claim(UpdateScratch& sc, uint32_t x) {
     d = (d + 1) & sc.dupmask;
   }
   return -1;
-}
-
-// The chosen worker's lookup from slots captured by the probe (no table
-// reads): stamps of present blocks, absent count, insert positions.
-template <int NT>
-__device__ __forceinline__ void cache_lookup_captured(const TableView& t, const uint32_t* pslot,
-                                                      const uint32_t* pfree, int nb,
-                                                      UpdateScratch& sc, UpdateShared* us) {
-  int nabs = 0;
-  uint32_t pmin = STAMP_NONE;
-  for (int k = threadIdx.x; k < nb; k += NT) {
-    const uint32_t sl = pslot[k];
-    sc.slot[k] = sl;
-    sc.fslot[k] = pfree[k];
-    sc.evk[k] = 0;
-    uint32_t st = STAMP_NONE;
-    if (sl != SLOT_NONE) {
-      st = __ldcg(t.stamp + sl);
-      pmin = min(pmin, st);
-    } else {
-      nabs++;
-    }
-    sc.pst[k] = st;
-  }
-  nabs = __reduce_add_sync(FULL_MASK, (unsigned)nabs);
-  pmin = __reduce_min_sync(FULL_MASK, pmin);
-  if ((threadIdx.x & 31) == 0) {
-    if (nabs) atomicAdd(&us->n_absent, nabs);
-    if (pmin != STAMP_NONE) atomicMin(&us->pmin, pmin);
-  }
-  grp_bar<NT>();
 }
 
 // Gathers live log entries starting at meta->head until `want` are held
@@ -885,7 +802,7 @@ __device__ __forceinline__ void cache_apply(const TableView& t, CacheMeta* meta,
       }
       w[k] = v;
     }
-    lru_exact<NT>(w, nb, (int)free_slots, &us->dup);   // (dup: free at this point)
+    lru_exact<NT>(w, nb, (int)free_slots, &us->changed);
     int ni = 0;
     for (int k = threadIdx.x; k < nb; k += NT) {
       const int v = w[k];
@@ -912,8 +829,7 @@ __device__ __forceinline__ void cache_apply(const TableView& t, CacheMeta* meta,
       if (have < E1) us->err = RS_ERR_TIMEOUT;
       us->n_victims = have < E1 ? 0 : E1;
       us->slow = 1;
-      us->dup = 0;
-    }
+        }
     grp_bar<NT>();
   }
   const int E = us->n_victims;

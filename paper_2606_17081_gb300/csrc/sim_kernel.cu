@@ -402,7 +402,7 @@ __device__ __forceinline__ void update_chosen(SimCtx& c, const uint64_t* hbuf, i
                                           c.pfree + (size_t)j * nb, nb, nabs, D, c.sc, &S.us,
                                           &S.fs, S.warp_tot, &S.scan_pos);
     } else {
-      cache_lookup_all<NT_UPD, false>(tv, hbuf, nb, c.sc, &S.us, &S.probes);
+      cache_lookup_all<NT_UPD>(tv, hbuf, nb, c.sc, &S.us, &S.probes);
       freq_present<NT_UPD>(tv, meta, fm, nb, D, c.sc, &S.us, &S.fs, &S.scan_pos);
     }
     cache_apply_freq<NT_UPD>(tv, meta, fm, g.K, hbuf, nb, D, (uint32_t)c.d->freq_max, c.sc, &S.us,
@@ -413,7 +413,7 @@ __device__ __forceinline__ void update_chosen(SimCtx& c, const uint64_t* hbuf, i
                                      c.pfree + (size_t)j * nb, nb, nabs, c.sc, &S.us,
                                      S.warp_tot, &S.scan_pos);
     else
-      cache_lookup_all<NT_UPD, false>(tv, hbuf, nb, c.sc, &S.us, &S.probes);
+      cache_lookup_all<NT_UPD>(tv, hbuf, nb, c.sc, &S.us, &S.probes);
     cache_apply<NT_UPD>(tv, meta, g.K, hbuf, nb, c.sc, &S.us, S.warp_tot, &S.scan_pos, captured);
     if (TIER) {
       grp_bar<NT_UPD>();   // the meta update of cache_apply
