@@ -387,7 +387,7 @@ __device__ __forceinline__ int ids_prefix(const uint32_t* st, const uint32_t* cd
       in[r] = kk < nz;
       const uint32_t c = in[r] ? cd[kk] : CODE_FRESH;
       v[r] = STAMP_NONE;
-      if (!(c >> 31)) {
+      if (!(c >> 31)) {   // (without the branch, as in ids_prefix4: 760 -> 980 cycles at W = 3)
         v[r] = st[c];
         cnt++;
       }
@@ -402,37 +402,36 @@ __device__ __forceinline__ int ids_prefix(const uint32_t* st, const uint32_t* cd
 }
 
 // The same for the workers j[q] of the set bits of `open`, four at a time, 64
-// blocks of each in flight, until each has its first miss.
+// blocks of each in flight, until each has its first miss.  Straight-line loads:
+// with a branch around each, and the window's in ids_update, the grid (648
+// replicas x 10 000 requests, W = 6) took 60.9 ms, 52.8 so.
 __device__ __forceinline__ void ids_prefix4(const uint32_t* stamps, size_t nre, const int (&j)[4],
                                             unsigned open, const uint32_t* cd, int k0, int nz,
                                             int (&m)[4], unsigned& cnt) {
   const int lane = (int)(threadIdx.x & 31);
+  const uint32_t* st[4];
 #pragma unroll
-  for (int q = 0; q < 4; q++) m[q] = nz;
+  for (int q = 0; q < 4; q++) {
+    m[q] = nz;
+    st[q] = stamps + (size_t)((open >> q) & 1u ? j[q] : j[0]) * nre;   // (bit 0 of open is set)
+  }
 #pragma unroll 1
   for (int k = k0; k < nz && open; k += 64) {
     const int ka = k + lane, kb = ka + 32;
-    const uint32_t ca = ka < nz ? cd[ka] : CODE_FRESH, cb = kb < nz ? cd[kb] : CODE_FRESH;
+    const uint32_t ca = cd[min(ka, nz - 1)], cb = cd[min(kb, nz - 1)];
+    const bool ia = ka < nz, ib = kb < nz, oa = ia && !(ca >> 31), ob = ib && !(cb >> 31);
+    const uint32_t xa = ca >> 31 ? 0u : ca, xb = cb >> 31 ? 0u : cb;
     uint32_t va[4], vb[4];
 #pragma unroll
-    for (int q = 0; q < 4; q++) {
-      const uint32_t* st = stamps + (size_t)j[q] * nre;
-      va[q] = vb[q] = STAMP_NONE;
-      if ((open >> q) & 1u) {
-        if (!(ca >> 31)) {
-          va[q] = st[ca];
-          cnt++;
-        }
-        if (!(cb >> 31)) {
-          vb[q] = st[cb];
-          cnt++;
-        }
-      }
+    for (int q = 0; q < 4; q++) {   // (no branch per load: what is not looked up reads a stamp not used)
+      va[q] = st[q][xa];
+      vb[q] = st[q][xb];
     }
+    cnt += (unsigned)__popc(open) * ((unsigned)oa + (unsigned)ob);
 #pragma unroll
     for (int q = 0; q < 4; q++) {
-      const unsigned ma = __ballot_sync(FULL_MASK, ka < nz && va[q] == STAMP_NONE);
-      const unsigned mb = __ballot_sync(FULL_MASK, kb < nz && vb[q] == STAMP_NONE);
+      const unsigned ma = __ballot_sync(FULL_MASK, ia && !(oa && va[q] != STAMP_NONE));
+      const unsigned mb = __ballot_sync(FULL_MASK, ib && !(ob && vb[q] != STAMP_NONE));
       if (((open >> q) & 1u) && (ma | mb)) {
         m[q] = ma ? k + __ffs(ma) - 1 : k + 32 + __ffs(mb) - 1;
         open &= ~(1u << q);
@@ -940,33 +939,38 @@ __device__ __forceinline__ void ids_update(SimScalars& A, IdsShared& S, uint32_t
   uint32_t pmin = STAMP_NONE;
 #pragma unroll 1
   for (int k = tid; k < nz; k += NT) {
-    const uint32_t x = cd[k];
-    const uint32_t st = x >> 31 ? STAMP_NONE : t.st[x];
+    const uint32_t x = cd[k], v = t.st[x >> 31 ? 0u : x];
+    const uint32_t st = x >> 31 ? STAMP_NONE : v;
     nabs += st == STAMP_NONE;
     pmin = min(pmin, st);
   }
   uint32_t x[R];
   bool live[R];
-  const uint32_t have_win = WINDOW && *whead == m.head ? *wlen : 0u;
+  if (full) {
+    const uint32_t have_win = WINDOW && *whead == m.head ? *wlen : 0u;
+    uint32_t v[R];
 #pragma unroll
-  for (int r = 0; r < R; r++) {
-    const uint32_t w = (uint32_t)(r * NT + tid), p = m.head + w;
-    live[r] = full && p < m.T;
-    x[r] = 0;
-    if (live[r]) x[r] = w < have_win ? win[w] : t.log[p & t.rmask];
+    for (int r = 0; r < R; r++) x[r] = WINDOW ? win[r * NT + tid] : LOG_DEAD;
+    if (have_win < (uint32_t)IDS_WIN) {
+#pragma unroll
+      for (int r = 0; r < R; r++) {
+        const uint32_t w = (uint32_t)(r * NT + tid), p = m.head + w;
+        if (w >= have_win) x[r] = p < m.T ? t.log[p & t.rmask] : LOG_DEAD;
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < R; r++) v[r] = t.st[x[r] >= LOG_DEAD ? 0u : x[r]];
+#pragma unroll
+    for (int r = 0; r < R; r++) {
+      live[r] = x[r] >= SINGLE_FLAG || (x[r] != LOG_DEAD && v[r] == m.head + (uint32_t)(r * NT + tid));
+      const unsigned lv = __ballot_sync(FULL_MASK, live[r]);
+      if (lane == 0) S.livew[r * (NT / 32) + (tid >> 5)] = lv;
+    }
   }
-#pragma unroll
-  for (int r = 0; r < R; r++)
-    if (live[r]) live[r] = ids_live(t, x[r], m.head + (uint32_t)(r * NT + tid));
   {
     const int a = (int)__reduce_add_sync(FULL_MASK, (unsigned)nabs);
     const uint32_t pm = __reduce_min_sync(FULL_MASK, pmin);
     if (lane == 0) S.red[tid >> 5] = make_uint2((unsigned)a, pm);
-#pragma unroll
-    for (int r = 0; r < R; r++) {
-      const unsigned lv = __ballot_sync(FULL_MASK, live[r]);
-      if (lane == 0) S.livew[r * (NT / 32) + (tid >> 5)] = lv;
-    }
   }
   grp_bar<NT>();
   nabs = nb - nz;   // past nz every block is fresh
@@ -1295,29 +1299,41 @@ __device__ __forceinline__ void ids_update_freq(SimScalars& A, IdsShared& S, uin
   uint32_t pmin = STAMP_NONE;   // least stamp of a present cold block
 #pragma unroll 1
   for (int k = tid; k < nz; k += NT) {
-    const uint32_t x = cd[k];
-    const uint32_t st = x >> 31 ? STAMP_NONE : t.st[x];
+    const uint32_t x = cd[k], id = x >> 31 ? 0u : x;
+    const uint32_t v = t.st[id], e = t.fe[id];
+    const uint32_t st = x >> 31 ? STAMP_NONE : v;
     nabs += st == STAMP_NONE;
-    if (st != STAMP_NONE && t.fe[x] <= D) pmin = min(pmin, st);
+    if (e <= D) pmin = min(pmin, st);   // (an absent block's is STAMP_NONE)
   }
   uint32_t x[R], he = 0xFFFFFFFFu, hp = 0xFFFFFFFFu;
   bool cold[R];
-  const uint32_t have_win = *whead == start ? *wlen : 0u;
 #pragma unroll
-  for (int r = 0; r < R; r++) {
-    const uint32_t w = (uint32_t)(r * NT + tid), p = start + w;
-    x[r] = LOG_DEAD;
-    if (full && p < m.T) x[r] = w < have_win ? win[w] : t.log[p & t.rmask];
-  }
+  for (int r = 0; r < R; r++) cold[r] = false;
+  if (full) {
+    const uint32_t have_win = *whead == start ? *wlen : 0u;
+    uint32_t v[R], e[R];
 #pragma unroll
-  for (int r = 0; r < R; r++) {
-    const uint32_t p = start + (uint32_t)(r * NT + tid);
-    cold[r] = ids_live(t, x[r], p);
-    if (cold[r] && !(x[r] & SINGLE_FLAG)) {
-      const uint32_t e = t.fe[x[r]];
-      if (e > D) {
-        cold[r] = false;
-        he = min(he, e);
+    for (int r = 0; r < R; r++) x[r] = win[r * NT + tid];
+    if (have_win < (uint32_t)IDS_WIN) {
+#pragma unroll
+      for (int r = 0; r < R; r++) {
+        const uint32_t w = (uint32_t)(r * NT + tid), p = start + w;
+        if (w >= have_win) x[r] = p < m.T ? t.log[p & t.rmask] : LOG_DEAD;
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < R; r++) {
+      const uint32_t id = x[r] >= LOG_DEAD ? 0u : x[r];
+      v[r] = t.st[id];
+      e[r] = t.fe[id];
+    }
+#pragma unroll
+    for (int r = 0; r < R; r++) {
+      const uint32_t p = start + (uint32_t)(r * NT + tid);
+      const bool held = x[r] < LOG_DEAD && v[r] == p;
+      cold[r] = x[r] >= SINGLE_FLAG || (held && e[r] <= D);
+      if (held && e[r] > D) {
+        he = min(he, e[r]);
         hp = min(hp, p);
       }
     }
