@@ -31,14 +31,16 @@
 // What the groups hand one another at the join is double-buffered by the
 // request's parity.  Between 5 and 7 cycles pass per instruction of a warp
 // that has its SM sub-partition to itself, and with four replicas per SM the
-// wait for instructions is the longest (7 of 17 cycles): the loop's code and
-// its instruction count are what to keep small.
+// wait for instructions is the longest after the barriers (3 of 16 cycles): the
+// loop's code and its instruction count are what to keep small.
 //
 // Calls before (hash tables) and now: 64 replicas x 10 000 requests at W = 3
-// 53.5 and 21.2 ms, 648 x 10 000 at W = 6 246 and 62.8 ms, 256 x 6 000 at
-// W = 6 with controller and sampling 62.5 and 18.7 ms, 16 x 5 000 at W = 64
-// 206 and 38.3 ms, 512 requests at W = 3 2.33 and 1.04 ms.
+// 53.5 and 19.9 ms, 648 x 10 000 at W = 6 246 and 52.1 ms, 256 x 6 000 at
+// W = 6 with controller and sampling 62.5 and 18.1 ms, 16 x 5 000 at W = 64
+// 206 and 31.3 ms, 512 requests at W = 3 2.33 and 0.96 ms; under frequency
+// eviction 64 x 10 000 at W = 3 59.8 and 22.8 ms.
 #include <algorithm>
+#include <type_traits>
 
 #include "sim_common.cuh"
 
@@ -387,7 +389,7 @@ __device__ __forceinline__ int ids_prefix(const uint32_t* st, const uint32_t* cd
       in[r] = kk < nz;
       const uint32_t c = in[r] ? cd[kk] : CODE_FRESH;
       v[r] = STAMP_NONE;
-      if (!(c >> 31)) {   // (without the branch, as in ids_prefix4: 760 -> 980 cycles at W = 3)
+      if (!(c >> 31)) {   // (without the branch, as in ids_prefixes: 760 -> 980 cycles at W = 3)
         v[r] = st[c];
         cnt++;
       }
@@ -401,17 +403,19 @@ __device__ __forceinline__ int ids_prefix(const uint32_t* st, const uint32_t* cd
   return nz;
 }
 
-// The same for the workers j[q] of the set bits of `open`, four at a time, 64
+// The same for the workers j[q] of the set bits of `open`, Q at a time, 64
 // blocks of each in flight, until each has its first miss.  Straight-line loads:
 // with a branch around each, and the window's in ids_update, the grid (648
-// replicas x 10 000 requests, W = 6) took 60.9 ms, 52.8 so.
-__device__ __forceinline__ void ids_prefix4(const uint32_t* stamps, size_t nre, const int (&j)[4],
+// replicas x 10 000 requests, W = 6) took 60.9 ms, 52.8 so, 51.3 with three workers
+// a walk where a warp has three.
+template <int Q>
+__device__ __forceinline__ void ids_prefixes(const uint32_t* stamps, size_t nre, const int (&j)[Q],
                                             unsigned open, const uint32_t* cd, int k0, int nz,
-                                            int (&m)[4], unsigned& cnt) {
+                                            int (&m)[Q], unsigned& cnt) {
   const int lane = (int)(threadIdx.x & 31);
-  const uint32_t* st[4];
+  const uint32_t* st[Q];
 #pragma unroll
-  for (int q = 0; q < 4; q++) {
+  for (int q = 0; q < Q; q++) {
     m[q] = nz;
     st[q] = stamps + (size_t)((open >> q) & 1u ? j[q] : j[0]) * nre;   // (bit 0 of open is set)
   }
@@ -421,15 +425,15 @@ __device__ __forceinline__ void ids_prefix4(const uint32_t* stamps, size_t nre, 
     const uint32_t ca = cd[min(ka, nz - 1)], cb = cd[min(kb, nz - 1)];
     const bool ia = ka < nz, ib = kb < nz, oa = ia && !(ca >> 31), ob = ib && !(cb >> 31);
     const uint32_t xa = ca >> 31 ? 0u : ca, xb = cb >> 31 ? 0u : cb;
-    uint32_t va[4], vb[4];
+    uint32_t va[Q], vb[Q];
 #pragma unroll
-    for (int q = 0; q < 4; q++) {   // (no branch per load: what is not looked up reads a stamp not used)
+    for (int q = 0; q < Q; q++) {   // (no branch per load: what is not looked up reads a stamp not used)
       va[q] = st[q][xa];
       vb[q] = st[q][xb];
     }
     cnt += (unsigned)__popc(open) * ((unsigned)oa + (unsigned)ob);
 #pragma unroll
-    for (int q = 0; q < 4; q++) {
+    for (int q = 0; q < Q; q++) {
       const unsigned ma = __ballot_sync(FULL_MASK, ia && !(oa && va[q] != STAMP_NONE));
       const unsigned mb = __ballot_sync(FULL_MASK, ib && !(ob && vb[q] != STAMP_NONE));
       if (((open >> q) & 1u) && (ma | mb)) {
@@ -459,19 +463,23 @@ __device__ __forceinline__ void ids_probe(const uint32_t* stamps, size_t nre, co
     }
     return;
   }
-  int j[4], m[4];
-  if (W <= 4 * NU) {
+  auto together = [&](auto n) {   // n workers per warp
+    constexpr int Q = decltype(n)::value;
+    int j[Q], m[Q];
     unsigned open = 0;
 #pragma unroll
-    for (int q = 0; q < 4; q++) {
+    for (int q = 0; q < Q; q++) {
       j[q] = warp + q * NU;
       open |= (unsigned)(j[q] < W) << q;
     }
-    ids_prefix4(stamps, nre, j, open, cd, 0, nz, m, cnt);
-    if (lane < 4 && warp + lane * NU < W)
-      wm[warp + lane * NU] = lane == 0 ? m[0] : (lane == 1 ? m[1] : (lane == 2 ? m[2] : m[3]));
-    return;
-  }
+    ids_prefixes<Q>(stamps, nre, j, open, cd, 0, nz, m, cnt);
+#pragma unroll
+    for (int q = 0; q < Q; q++)
+      if (lane == q && j[q] < W) wm[j[q]] = m[q];
+  };
+  if (W <= 3 * NU) return together(std::integral_constant<int, 3>());
+  if (W <= 4 * NU) return together(std::integral_constant<int, 4>());
+  int j[4], m[4];
   const uint32_t c = lane < nz ? cd[lane] : CODE_FRESH;
   const bool old = !(c >> 31);
   const uint32_t x = old ? c : 0u;
@@ -502,7 +510,7 @@ __device__ __forceinline__ void ids_probe(const uint32_t* stamps, size_t nre, co
         open &= open - 1u;
         j[q] = j0 + w[q] * NU;
       }
-      ids_prefix4(stamps, nre, j, some, cd, 32, nz, m, cnt);
+      ids_prefixes<4>(stamps, nre, j, some, cd, 32, nz, m, cnt);
 #pragma unroll
       for (int q = 0; q < 4; q++)
         if (((some >> q) & 1u) && lane == w[q]) mine = m[q];
