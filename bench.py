@@ -199,8 +199,8 @@ def _table_bytes(K: int) -> int:
 # workload (dram__bytes_read.sum + dram__bytes_write.sum), with the SHA-256 of
 # the simulation kernel's sources it was taken with.  The capture ran on 760 of
 # its 8192 simulations (one resident wave, five per SM) and is scaled.
-SIM_TRAFFIC = {"bytes": (3742924544 + 4207784448) * 8192 / 760,
-               "sources_sha256": "2277c66bc86672f04db7f8c64cb98e8dff21747e4cbdfb214705b18b3621d74d",
+SIM_TRAFFIC = {"bytes": (3756686848 + 4197738496) * 8192 / 760,
+               "sources_sha256": "4f1da12673921cc8eff74c06593bb58fefafa9e6720a89f69d5da4e9f3961846",
                "summary": "profiles/k_sim_ids.md",
                "scaled_from": "760 simulations x 10 000 requests, times 8192 / 760"}
 

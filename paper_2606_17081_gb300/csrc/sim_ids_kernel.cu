@@ -30,15 +30,15 @@
 //            request i+1's update would do to each).
 // What the groups hand one another at the join is double-buffered by the
 // request's parity.  Between 5 and 7 cycles pass per instruction of a warp
-// that has its SM sub-partition to itself, and with four replicas per SM the
-// wait for instructions is the longest after the barriers (3 of 16 cycles): the
-// loop's code and its instruction count are what to keep small.
+// that has its SM sub-partition to itself, and with four replicas per SM
+// they are 13, 1.7 of them waits for instruction fetch: the loop's code and its
+// instruction count are what to keep small.
 //
 // Calls before (hash tables) and now: 64 replicas x 10 000 requests at W = 3
-// 53.5 and 19.9 ms, 648 x 10 000 at W = 6 246 and 52.1 ms, 256 x 6 000 at
-// W = 6 with controller and sampling 62.5 and 18.1 ms, 16 x 5 000 at W = 64
-// 206 and 31.3 ms, 512 requests at W = 3 2.33 and 0.96 ms; under frequency
-// eviction 64 x 10 000 at W = 3 59.8 and 22.8 ms.
+// 53.5 and 19.9 ms, 648 x 10 000 at W = 6 246 and 51.7 ms, 256 x 6 000 at
+// W = 6 with controller and sampling 62.5 and 18.3 ms, 16 x 5 000 at W = 64
+// 206 and 32.9 ms, 512 requests at W = 3 2.33 and 0.96 ms; under frequency
+// eviction 64 x 10 000 at W = 3 59.8 and 22.7 ms.
 #include <algorithm>
 #include <type_traits>
 
@@ -405,9 +405,9 @@ __device__ __forceinline__ int ids_prefix(const uint32_t* st, const uint32_t* cd
 
 // The same for the workers j[q] of the set bits of `open`, Q at a time, 64
 // blocks of each in flight, until each has its first miss.  Straight-line loads:
-// with a branch around each, and the window's in ids_update, the grid (648
-// replicas x 10 000 requests, W = 6) took 60.9 ms, 52.8 so, 51.3 with three workers
-// a walk where a warp has three.
+// with a branch around each, and the window's in ids_update, a call on the grid
+// (648 replicas x 10 000 requests, W = 6, three workers a warp) took 61.4 ms,
+// 54.3 so, and 52.1 with Q = 3 there instead of 4.
 template <int Q>
 __device__ __forceinline__ void ids_prefixes(const uint32_t* stamps, size_t nre, const int (&j)[Q],
                                             unsigned open, const uint32_t* cd, int k0, int nz,
