@@ -350,7 +350,8 @@ rs_status poa_estimate(rs_ctx* ctx, const rs_records* records, int64_t n, double
 
 /* Cache contents of one worker, least- to most-recently used, into keys_host
  * (capacity entries); *size = entries held.  source 0: live router instance
- * `index`; source 1: replica `index` of the last simulate_replicas call.
+ * `index`; source 1: replica `index` of the last simulate_replicas call (after
+ * one that failed for want of memory there is none: RS_ERR_INVALID).
  * Synchronises. */
 rs_status route_cache_dump(rs_ctx* ctx, int32_t source, int32_t index, int32_t worker,
                            uint64_t* keys_host, int64_t capacity, int64_t* size);

@@ -973,9 +973,11 @@ rs_status simulate_replicas(rs_ctx* ctx, const rs_trace* traces, int32_t n_trace
     // (a device trace's own hashes are copied when the caches will refer to them)
     if (used[t] && (!dhash[t] || (use_ids && !host))) hash_total += (size_t)(tot[t] / 16 + 1);
   }
-  if ((r = ensure(ctx, ctx->hashes, hash_total * 8, "block hashes")) != RS_OK) return r;
-  ctx->last_nsim = 0;   // the last call's caches are overwritten from here on
+  // the last call's caches are overwritten from here on (its hashes may be freed
+  // by a growth that then fails)
+  ctx->last_nsim = 0;
   ctx->last_ids.clear();
+  if ((r = ensure(ctx, ctx->hashes, hash_total * 8, "block hashes")) != RS_OK) return r;
   // ---- K1: block hashes of every trace in use that comes as tokens.  The
   // hash jobs number their requests among themselves; the per-request flags
   // number the requests of every trace in use (rbase).

@@ -1,0 +1,51 @@
+"""simulate_replicas calls that are refused or run out of device memory: what
+they leave of the call before."""
+import numpy as np
+import pytest
+
+from paper_2606_17081_gb300 import routesim as rs
+from paper_2606_17081_gb300 import workloads as wk
+
+from gpu_helpers import gpu_run
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("needs a CUDA device", allow_module_level=True)
+
+
+def _trace(n, seed, hi=600):
+    return wk.make_trace(wk.TraceSpec(n_req=n, len_kind="uniform", len_min=16, len_max=hi, n_groups=4, prefix_min=32,
+                                      prefix_max=200, zipf_s=None, out_kind="uniform", out_min=1, out_max=100), seed)
+
+
+def _rep(n, trace=0):
+    return wk.Replica(trace, 8, wk.POLICY_DYNAMO, 0, 1.0, 0.0, 0, n)
+
+
+def _claims(length, hashes=None):
+    """A device trace of one prompt of `length` tokens whose tokens (or hashes) are not there: for calls that end before
+    any of them is read."""
+    t = rs.TraceBuffers(None if hashes is not None else torch.zeros(16, dtype=torch.int32, device="cuda"),
+                        torch.tensor([0, length], dtype=torch.int64, device="cuda"),
+                        torch.zeros(1, dtype=torch.float64, device="cuda"),
+                        torch.ones(1, dtype=torch.int32, device="cuda"), 1, hashes)
+    return t
+
+
+def test_no_caches_after_a_call_without_memory():
+    # the hashes of 2^45 tokens (2^44 bytes) cannot be had; the old buffer that the caches' hashes lay in is gone
+    ctx = rs.Context(W=3, K=100)
+    tr = _trace(80, 1)
+    st, _ = gpu_run(ctx, [tr], [_rep(80)])
+    assert st == rs.RS_OK and rs.route_cache_dump(ctx.h, 1, 0, 0, 100).size
+    big = _claims(1 << 45)
+    with pytest.raises(rs.RoutesimError) as e:
+        rs.simulate_replicas(ctx.h, [big.desc()], rs.RS_MEM_DEVICE, [rs.replica_params(_rep(1))], None)
+    assert e.value.status == rs.RS_ERR_OOM
+    with pytest.raises(rs.RoutesimError) as e:
+        rs.route_cache_dump(ctx.h, 1, 0, 0, 100)
+    assert e.value.status == rs.RS_ERR_INVALID
+    st, _ = gpu_run(ctx, [tr], [_rep(80)])   # the context stays usable
+    assert st == rs.RS_OK and rs.route_cache_dump(ctx.h, 1, 0, 0, 100).size
