@@ -932,6 +932,7 @@ __device__ __forceinline__ void ids_update(SimScalars& A, IdsShared& S, uint32_t
   if (WINDOW) cp_async_wait_all();   // this thread's window entries
   if ((uint64_t)meta->T - meta->head + (uint64_t)nb > (uint64_t)t.rmask + 1 ||
       (uint64_t)meta->T + nb > STAMP_LIMIT) {
+    if (!WINDOW) cp_async_wait_all();   // this thread's copies of the log into the rings
     grp_bar<NT>();
     ids_compact<NT>(t, meta, S.warp_tot, &S.err);
     if (tid == 0) {
@@ -2101,7 +2102,12 @@ __global__ void __launch_bounds__((NU + 2) * 32, MINB)
       const uint32_t* cd = codes + (size_t)ek * nbcap;
       if constexpr (PLAN) {
         // the rings' next entries, once a victim may be needed soon; those
-        // copied before the last time have landed
+        // copied the last time have landed before others are sent to their
+        // places (copies in flight keep no order: after a compaction, or when
+        // two updates together pass more entries than the ring holds, the same
+        // place is written again)
+        cp_async_wait_all();
+        __syncwarp();
         uint32_t safe[PW];
 #pragma unroll
         for (int w = 0; w < PW; w++) {
@@ -2120,7 +2126,6 @@ __global__ void __launch_bounds__((NU + 2) * 32, MINB)
           }
           if (lane == 0) wlen[j] = wend;
         }
-        asm volatile("cp.async.commit_group;\ncp.async.wait_group 1;" ::: "memory");
         __syncwarp();
 #pragma unroll 1
         for (int w = 0; w < PW; w++) {

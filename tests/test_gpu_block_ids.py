@@ -59,6 +59,8 @@ def _both(ctx, traces, reps, caches=()):
     (3, 190, 40, 0.7, wk.POLICY_DYNAMO, 3000),       # ring of 2 K: every update evicts
     (6, 511, 33, 0.0, wk.POLICY_LOADBAL, 7000),      # more victims than the window
     (6, 512, 33, 0.0, wk.POLICY_DYNAMO, 7000),       # ring of 4 K
+    (2, 700, 20, 0.0, wk.POLICY_RANDOM, 11000),      # two updates pass more entries than the plans' ring holds
+    (4, 60, 20, 0.0, wk.POLICY_DYNAMO, 950),         # compactions while the rings are being filled
     (7, 900, 64, 0.5, wk.POLICY_DYNAMO, 1040),      # past one worker per warp
     (24, 300, 200, 0.0, wk.POLICY_DYNAMO, 3000),
     (25, 300, 200, 1.0, wk.POLICY_P2C, 3000),
@@ -70,6 +72,8 @@ def test_ids_equal_tables(W, K, C, tau, policy, hi):
     rep = wk.Replica(0, C, policy, int(tau > 0), 1.0, tau, 5, tr.n_req)
     st, g = _both(rs.Context(W=W, K=K), [tr], [rep], [(0, j) for j in range(0, W, 5)])
     assert st == rs.RS_OK and g[0]["result"]["evicted_blocks"] > 0
+    if K < 100 and C < 4096:
+        assert g[0]["result"]["rebuilds"] > 0
 
 
 def test_ids_equal_tables_many_replicas():
