@@ -219,7 +219,8 @@ struct IdsShared {
   alignas(16) IdsPlan plan[8];
 
   IdsArrival pub[2];
-  int stat[2];                 // by parity: an error seen before that join
+  int2 stat[2];                // by parity: errors seen before that join, of the events (x) and of
+                               // the update (y: of the request before, so it comes first)
   alignas(16) uint2 red[8];    // per update warp: absent blocks, least stamp
   unsigned livew[IDS_WIN / 32];   // live entries of the window (frequency eviction: cold ones)
   uint2 hot[8];                // per update warp: least e and position of the hot entries passed
@@ -357,6 +358,12 @@ __device__ __forceinline__ void cp_async4(void* dst, const void* src) {
 template <int NT>
 __device__ __forceinline__ void join_cta() {
   asm volatile("barrier.sync 0, %0;" ::"n"(NT) : "memory");
+}
+
+// Whether an error before the join of parity p stops the replica.
+__device__ __forceinline__ bool ids_stopped(const IdsShared& Sh, int p) {
+  const int2 s = Sh.stat[p];
+  return (s.x | s.y) != RS_OK;
 }
 
 // The choice of request i: made by the staging warp (Sh.js written), waited
@@ -1586,15 +1593,16 @@ __device__ __noinline__ void ids_tick_empty(SimScalars& S, const SimLaunch& L, i
   __syncwarp();
 }
 
-// Request i's arrival: every event before it, then what its choice needs (one
-// thread and a heap: for concurrencies whose slots are in global memory).
-__device__ __forceinline__ void ids_arrive(SimCtx& c, IdsShared& Sh, int64_t i, float* act,
+// Request i's arrival: every event before it, then what its choice needs (dup as
+// in ev_arrive; one thread and a heap: for concurrencies whose slots are in global memory).
+__device__ __forceinline__ void ids_arrive(SimCtx& c, IdsShared& Sh, int64_t i, bool dup, float* act,
                                            int* nfz, int lane) {
   SimScalars& S = *c.S;
   IdsReq& q = Sh.q[i & (IDS_RING - 1)];
   const int p = (int)(i & 1), W = c.L->mc.W;
-  if (q.nb > (int)c.L->g.K) {
-    if (lane == 0) Sh.stat[p] = S.status = RS_ERR_CAPACITY;
+  if (dup || q.nb > (int)c.L->g.K) {
+    if (lane == 0) Sh.stat[p].x = S.status = dup ? RS_ERR_COLLISION : RS_ERR_CAPACITY;
+    __syncwarp();
     return;
   }
   for (;;) {
@@ -1608,7 +1616,7 @@ __device__ __forceinline__ void ids_arrive(SimCtx& c, IdsShared& Sh, int64_t i, 
     Sh.pub[p].a = q.a;
     Sh.pub[p].tau = q.tau;
     Sh.pub[p].omega = q.omega;
-    if (S.status != RS_OK) Sh.stat[p] = S.status;
+    if (S.status != RS_OK) Sh.stat[p].x = S.status;
   }
   __syncwarp();
   for (int j = lane; j < W; j += 32) {
@@ -1829,15 +1837,17 @@ __device__ __forceinline__ void ev_sample(SimCtx& c, IdsEvents<WIDE>& E, int lan
 // Request i's arrival: every event before it in time order (completions,
 // controller samples, steps of the load-spike schedule; ties in that order),
 // then what its choice needs.  drain: past the last request, the completions
-// that remain (they start the queued requests).
+// that remain (they start the queued requests).  dup: two blocks of the request
+// before have one chained hash (a 64-bit collision): that request is routed,
+// its update cannot be made, and nothing after its arrival takes place.
 template <bool WIDE, bool FREQ>
 __device__ __forceinline__ void ev_arrive(SimCtx& c, IdsShared& Sh, IdsEvents<WIDE>& E, int64_t i,
-                                          bool drain, float* act, int* nfz, int lane) {
+                                          bool drain, bool dup, float* act, int* nfz, int lane) {
   SimScalars& S = *c.S;
   const IdsReq& q = Sh.q[i & (IDS_RING - 1)];
   const int p = (int)(i & 1), W = c.L->mc.W;
-  if (!drain && q.nb > (int)c.L->g.K) {
-    if (lane == 0) Sh.stat[p] = S.status = RS_ERR_CAPACITY;
+  if (dup || (!drain && q.nb > (int)c.L->g.K)) {
+    if (lane == 0) Sh.stat[p].x = S.status = dup ? RS_ERR_COLLISION : RS_ERR_CAPACITY;
     return;
   }
   const uint64_t krel = tkey(q.rel);
@@ -1924,7 +1934,7 @@ __device__ __forceinline__ void ev_arrive(SimCtx& c, IdsShared& Sh, IdsEvents<WI
       ar.tau = shift ? c.L->mc.regime_tau[S.regime] : E.tau;
       ar.omega = shift ? c.L->mc.regime_omega[S.regime] : E.omega;
     }
-    if (!ok) Sh.stat[p] = S.status;
+    if (!ok) Sh.stat[p].x = S.status;
   }
 }
 
@@ -2076,7 +2086,7 @@ __global__ void __launch_bounds__((NU + 2) * 32, MINB)
       S.nfree = cslots;
       S.first_switch_t = -1.0;
       S.first_evict_i = -1;
-      Sh.stat[0] = Sh.stat[1] = RS_OK;
+      Sh.stat[0] = Sh.stat[1] = make_int2(RS_OK, RS_OK);
       Sh.err = 0;
     }
   }
@@ -2149,14 +2159,11 @@ __global__ void __launch_bounds__((NU + 2) * 32, MINB)
       const int p = (int)(i & 1), e = (int)(i & (IDS_RING - 1));
       if (i >= 0) {
         join_cta<NT>();
-        if (Sh.stat[p] != RS_OK) break;
+        if (ids_stopped(Sh, p)) break;
         const IdsReq& q = Sh.q[e];
         choice_wait<NT>();
         const int js = Sh.js;
-        if (q.dup) {
-          // two blocks of the prompt with one chained hash (a 64-bit collision)
-          if (threadIdx.x == 0) Sh.stat[p ^ 1] = RS_ERR_COLLISION;
-        } else {
+        if (!q.dup) {   // (else the replica stops here: see ev_arrive)
           const IdsTable t = table(js);
           const uint32_t* cd = codes + (size_t)e * nbcap;
           if (PLAN && Sh.plan[js].step != IDS_GENERAL) {
@@ -2171,7 +2178,7 @@ __global__ void __launch_bounds__((NU + 2) * 32, MINB)
             else
               ids_update<NTU, true>(S, Sh, L.g.K, L.nbmax, t, c.wmeta + js, cd, q, scratch,
                                     win + (size_t)js * IDS_WIN, whead + js, wlen + js, i);
-            if (threadIdx.x == 0 && Sh.err) Sh.stat[p ^ 1] = Sh.err;
+            if (threadIdx.x == 0 && Sh.err) Sh.stat[p ^ 1].y = Sh.err;
           }
         }
         grp_bar<NTU>();   // the update's stamps, before the next probe
@@ -2258,9 +2265,10 @@ __global__ void __launch_bounds__((NU + 2) * 32, MINB)
 #pragma unroll 1
     for (int64_t i = -1; i < n; i++) {
       const int p = (int)(i & 1), e = (int)(i & (IDS_RING - 1));
+      bool dup = false;
       if (i >= 0) {
         join_cta<NT>();
-        if (Sh.stat[p] != RS_OK) break;
+        if (ids_stopped(Sh, p)) break;
         const IdsReq& q = Sh.q[e];
         // w_c o_ij of workers lane, lane + 32: from the table of every (nbt, m),
         // or m / nbt correctly rounded from the rounded reciprocal (one exact
@@ -2294,6 +2302,7 @@ __global__ void __launch_bounds__((NU + 2) * 32, MINB)
           }
         }
         const int blk = (int)q.blk;
+        dup = q.dup != 0;
         choice_wait<NT>();
         const int js = Sh.js;
         auto of = [&](const double (&v)[H]) {
@@ -2354,13 +2363,13 @@ __global__ void __launch_bounds__((NU + 2) * 32, MINB)
         }
       }
       if constexpr (!SG)
-        ev_arrive<WIDE, FREQ>(c, Sh, E, i + 1, i + 1 == n, act, nfz, lane);
-      else if (i + 1 < n)
-        ids_arrive(c, Sh, i + 1, act, nfz, lane);
+        ev_arrive<WIDE, FREQ>(c, Sh, E, i + 1, i + 1 == n, dup, act, nfz, lane);
+      else if (i + 1 < n || dup)
+        ids_arrive(c, Sh, i + 1, dup, act, nfz, lane);
     }
     if constexpr (SG) {
       // drain: remaining completions start the queued requests
-      if (lane == 0 && S.status == RS_OK && Sh.stat[0] == RS_OK && Sh.stat[1] == RS_OK)
+      if (lane == 0 && S.status == RS_OK)
         while (S.nheap > 0) {
           uint64_t k;
           int f;
@@ -2382,7 +2391,7 @@ __global__ void __launch_bounds__((NU + 2) * 32, MINB)
       IdsChoice ch;
       if (i >= 0) {
         join_cta<NT>();
-        if (Sh.stat[p] != RS_OK) break;
+        if (ids_stopped(Sh, p)) break;
         ch = ids_choice<WIDE>(policy, q, Sh.pub[p], wm + p * W, act + p * W, W, i, lane);
         if (lane == 0) Sh.js = ch.js;
         choice_made<NT>();
@@ -2447,8 +2456,8 @@ __global__ void __launch_bounds__((NU + 2) * 32, MINB)
     }
   }
   __syncthreads();
-  if (threadIdx.x == 0 && S.status == RS_OK)
-    S.status = Sh.stat[0] != RS_OK ? Sh.stat[0] : Sh.stat[1];
+  if (threadIdx.x == 0 && (Sh.stat[0].y | Sh.stat[1].y) != RS_OK)   // (at most one: the loop has ended there)
+    S.status = Sh.stat[0].y | Sh.stat[1].y;
   __syncthreads();
   {
     double st = 0.0, se = 0.0, mk = 0.0;

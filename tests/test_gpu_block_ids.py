@@ -123,6 +123,31 @@ def test_ids_from_given_hashes_repeated_block_and_long_prompt():
     assert st == rs.RS_ERR_CAPACITY
 
 
+@pytest.mark.parametrize("W,C", [(3, 8), (7, 8), (3, 5000)])   # planned updates, not planned, slot arrays in global memory
+def test_first_error_in_request_order(W, C):
+    # a prompt that repeats a block, right before one longer than the cache: the replica stops at the former
+    K, i = 200, 50
+    lens = np.array([320] * i + [100, 16 * K + 16, 320])
+    rng = np.random.default_rng(3)
+    off = np.concatenate([[0], np.cumsum(lens)]).astype(np.int64)
+    tr = wk.Trace(rng.integers(0, 32000, int(off[-1]) + 3).astype(np.int32), off, np.zeros(lens.size),
+                  np.full(lens.size, 20, np.int32), np.zeros(lens.size, np.int32))
+    ctx = rs.Context(W=W, K=K)
+    d = rs.device_trace(tr)
+    h = torch.zeros(int(off[-1]) // 16 + 1, dtype=torch.int64, device="cuda")
+    rs.route_hash_blocks(ctx.h, d.tokens, d.offsets, tr.n_req, h)
+    b = int(off[i]) // 16
+    h[b + 3] = h[b + 1]
+    t = d.desc()
+    t.tokens, t.hashes = None, h.data_ptr()
+    p = [rs.replica_params(wk.Replica(0, C, wk.POLICY_DYNAMO, 0, 1.0, 0.0, 0, tr.n_req))]
+    for f in (0, rs.RS_SIM_TABLES):
+        with pytest.raises(rs.RoutesimError) as e:
+            rs.simulate_replicas(ctx.h, [t], rs.RS_MEM_DEVICE, p, None, f)
+        r = e.value.results[0].as_dict()
+        assert (r["status"], r["n_routed"]) == (rs.RS_ERR_COLLISION, i + 1), f
+
+
 @pytest.mark.parametrize("W,K,nrep,hi,decay,fmax", [
     (3, 190, 4, 3000, 0.5, 64),       # ring of 2 K, frequencies that decay between requests
     (6, 900, 5, 7000, 50.0, 1 << 20),  # mostly hot: the sequence is replayed, hot victims
