@@ -298,8 +298,7 @@ typedef struct {
   double kv_cost;
 } rs_replica_result;
 
-/* Per-request records, device memory, each pointer may be NULL (of a replica that
- * stops with an error, ttft is not filled).  Replica r's
+/* Per-request records, device memory, each pointer may be NULL.  Replica r's
  * requests start at row R_r = sum of n_req of replicas before r; per-worker
  * arrays hold W entries per row. */
 typedef struct {

@@ -2367,6 +2367,14 @@ __global__ void __launch_bounds__((NU + 2) * 32, MINB)
       else if (i + 1 < n || dup)
         ids_arrive(c, Sh, i + 1, dup, act, nfz, lane);
     }
+    if constexpr (!SG) {
+      // each worker's first request still queued (none: past every request): a
+      // queue is in request order, and nobody overtakes it
+#pragma unroll
+      for (int h = 0; h < IdsEvents<WIDE>::H; h++)
+        if (lane + 32 * h < W)
+          c.wqh[lane + 32 * h] = E.qh[h] >= 0 ? E.srec[E.qh[h]].w : 0x7FFFFFFF;
+    }
     if constexpr (SG) {
       // drain: remaining completions start the queued requests
       if (lane == 0 && S.status == RS_OK)
@@ -2470,6 +2478,12 @@ __global__ void __launch_bounds__((NU + 2) * 32, MINB)
         st = __dadd_rn(st, tt);
         se = __dadd_rn(se, __dsub_rn(ct, a));
         mk = fmax(mk, ct);
+      }
+    else if constexpr (!SG)   // (else written at the service starts)
+      for (int64_t q = threadIdx.x; q < S.n_routed; q += NT) {
+        const int64_t row = d.rec_base + q;
+        if (q < c.wqh[b.rec.worker[row]])   // service has started
+          b.rec.ttft[row] = __dsub_rn(b.rec.first_token[row], b.rec.arrival[row]);
       }
     for (int o = 16; o > 0; o >>= 1) {
       st = __dadd_rn(st, __shfl_xor_sync(FULL_MASK, st, o));
