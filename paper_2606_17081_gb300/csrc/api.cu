@@ -827,8 +827,6 @@ rs_status simulate_replicas(rs_ctx* ctx, const rs_trace* traces, int32_t n_trace
   auto prehashed = [&](int t) { return traces[t].tokens == nullptr; };
   std::vector<const uint64_t*> dhash(n_traces, nullptr);
   if (host) {
-    ctx->last_nsim = 0;   // the last call's caches may refer to its staged hashes
-    ctx->last_ids.clear();
     size_t tb = 0, ob = 0, nb = 0, hb = 0;
     for (int t = 0; t < n_traces; t++) {
       if (!used[t] || traces[t].n_req == 0) continue;
@@ -841,6 +839,10 @@ rs_status simulate_replicas(rs_ctx* ctx, const rs_trace* traces, int32_t n_trace
         tb += ((size_t)(tot[t] + 3) / 4 * 4) * 4 + 16;
       ob += (size_t)(n + 1) * 8;
       nb += (size_t)n;
+    }
+    if (hb > 0) {   // the last call's caches may refer to its staged hashes
+      ctx->last_nsim = 0;
+      ctx->last_ids.clear();
     }
     if ((r = ensure(ctx, ctx->h_tokens, tb, "staged tokens")) ||
         (r = ensure(ctx, ctx->h_hashes, hb, "staged block hashes")) ||

@@ -49,3 +49,20 @@ def test_no_caches_after_a_call_without_memory():
     assert e.value.status == rs.RS_ERR_INVALID
     st, _ = gpu_run(ctx, [tr], [_rep(80)])   # the context stays usable
     assert st == rs.RS_OK and rs.route_cache_dump(ctx.h, 1, 0, 0, 100).size
+
+
+def test_caches_stay_after_a_refused_host_call():
+    # refused before anything of the last call is overwritten: a prompt too long for the kernels' shared memory
+    ctx = rs.Context(W=3, K=20000)
+    tr = _trace(60, 2)
+    st, _ = gpu_run(ctx, [tr], [_rep(60)], trace_mem=rs.RS_MEM_HOST)
+    assert st == rs.RS_OK
+    before = [rs.route_cache_dump(ctx.h, 1, 0, j, 20000) for j in range(3)]
+    n = 16 * 16000
+    long = rs.TraceBuffers(torch.zeros(n, dtype=torch.int32), torch.tensor([0, n]), torch.zeros(1, dtype=torch.float64),
+                           torch.ones(1, dtype=torch.int32), 1)
+    with pytest.raises(rs.RoutesimError) as e:
+        rs.simulate_replicas(ctx.h, [long.desc()], rs.RS_MEM_HOST, [rs.replica_params(_rep(1))], None)
+    assert e.value.status == rs.RS_ERR_CAPACITY
+    for j in range(3):
+        assert np.array_equal(rs.route_cache_dump(ctx.h, 1, 0, j, 20000), before[j])
