@@ -969,17 +969,26 @@ rs_status simulate_replicas(rs_ctx* ctx, const rs_trace* traces, int32_t n_trace
       if (any_freq || sim_ids_smem_bytes(W, (int)nbmax, cmax, ctx->cfg.cap, ntu, true) > smem_room) use_ids = false;
     }
   }
-  size_t hash_total = 0;
-  for (int t = 0; t < n_traces; t++) {
-    hoff[t] = (int64_t)hash_total;
-    // (a device trace's own hashes are copied when the caches will refer to them)
-    if (used[t] && (!dhash[t] || (use_ids && !host))) hash_total += (size_t)(tot[t] / 16 + 1);
-  }
+  auto hash_room = [&] {
+    size_t total = 0;
+    for (int t = 0; t < n_traces; t++) {
+      hoff[t] = (int64_t)total;
+      // (a device trace's own hashes are copied when the caches will refer to them)
+      if (used[t] && (!dhash[t] || (use_ids && !host))) total += (size_t)(tot[t] / 16 + 1);
+    }
+    return total * 8;
+  };
   // the last call's caches are overwritten from here on (its hashes may be freed
   // by a growth that then fails)
   ctx->last_nsim = 0;
   ctx->last_ids.clear();
-  if ((r = ensure(ctx, ctx->hashes, hash_total * 8, "block hashes")) != RS_OK) return r;
+  r = ensure(ctx, ctx->hashes, hash_room(), "block hashes");
+  if (r == RS_ERR_OOM && use_ids) {   // no room for the copies: the tables, which need none
+    use_ids = false;
+    ctx->err.clear();
+    r = ensure(ctx, ctx->hashes, hash_room(), "block hashes");
+  }
+  if (r != RS_OK) return r;
   // ---- K1: block hashes of every trace in use that comes as tokens.  The
   // hash jobs number their requests among themselves; the per-request flags
   // number the requests of every trace in use (rbase).
@@ -1030,9 +1039,12 @@ rs_status simulate_replicas(rs_ctx* ctx, const rs_trace* traces, int32_t n_trace
     if (r == RS_OK) r = ensure(ctx, ctx->i_stamps, stamp_words * 4 * (any_freq ? 2 : 1), "block stamps");
     if (r == RS_OK)
       r = ensure(ctx, ctx->i_scratch, nsim * sim_ids_scratch_bytes((int)nbmax), "update scratch");
-    if (r == RS_ERR_OOM) {   // no room for the ids: the tables
+    if (r == RS_ERR_OOM) {   // no room for the ids: the tables, which get back what the ids took
       use_ids = false;
       ctx->err.clear();
+      for (DevBuf* b : {&ctx->i_keys, &ctx->i_first, &ctx->i_num, &ctx->i_ids, &ctx->i_nz, &ctx->i_stamps,
+                        &ctx->i_scratch})
+        release(*b);
     } else if (r != RS_OK) {
       return r;
     }

@@ -66,3 +66,15 @@ def test_caches_stay_after_a_refused_host_call():
     assert e.value.status == rs.RS_ERR_CAPACITY
     for j in range(3):
         assert np.array_equal(rs.route_cache_dump(ctx.h, 1, 0, j, 20000), before[j])
+
+
+def test_device_hashes_that_cannot_be_copied():
+    # forty traces whose hashes take 8.6 GB each: no room for copies of them beside what the hash tables need (of each,
+    # one prompt of 16 blocks is routed; the second, longer than the cache, is not and its hashes are not there)
+    ctx = rs.Context(W=2, K=64)
+    h = torch.arange(2, 34, dtype=torch.int64, device="cuda")
+    t = rs.TraceBuffers(None, torch.tensor([0, 256, (1 << 34) - 256], dtype=torch.int64, device="cuda"),
+                        torch.zeros(2, dtype=torch.float64, device="cuda"), torch.ones(2, dtype=torch.int32, device="cuda"), 2, h)
+    res = rs.simulate_replicas(ctx.h, [t.desc()] * 40, rs.RS_MEM_DEVICE, [rs.replica_params(_rep(1, k)) for k in range(40)], None)
+    assert all(r.status == rs.RS_OK and r.n_routed == 1 and r.inserted_blocks == 16 for r in res)
+    assert np.array_equal(rs.route_cache_dump(ctx.h, 1, 39, 0, 64), np.arange(2, 18))
