@@ -448,12 +448,11 @@ rs_status route_batch(rs_ctx* ctx, int32_t instance, const int32_t* tokens_dev,
   int64_t nbmax = 0;
   if ((r = hash_batch(ctx, tokens_dev, offsets_dev, n_req, &nbmax)) != RS_OK) return r;
   if (nbmax > (int64_t)ctx->g.K) nbmax = ctx->g.K;   // longer prompts stop with RS_ERR_CAPACITY
-  // (4 KB beside the arrays for the kernel's own variables)
   int maxsmem = 0;
   cudaDeviceGetAttribute(&maxsmem, cudaDevAttrMaxSharedMemoryPerBlockOptin, ctx->device);
   const int nbl = (int)std::max<int64_t>(nbmax, 1);
-  const bool lean = router_smem(ctx->cfg.W, nbl, false) + 4096 > (size_t)maxsmem;
-  if (lean && router_smem(ctx->cfg.W, nbl, true) + 3584 > (size_t)maxsmem)
+  const bool lean = router_smem(ctx->cfg.W, nbl, false) + ROUTE_OWN_SMEM > (size_t)maxsmem;
+  if (lean && router_smem(ctx->cfg.W, nbl, true) + ROUTE_OWN_SMEM > (size_t)maxsmem)
     return fail(ctx, RS_ERR_CAPACITY, "a prompt of %lld blocks needs too much shared memory",
                 (long long)nbmax);
   ModelConsts mc = ctx->mc;

@@ -33,6 +33,8 @@ struct RouterShared {
   uint64_t ordinal;
 };
 
+static_assert(sizeof(RouterShared) + sizeof(SimScalars) + 64 <= ROUTE_OWN_SMEM, "the host's margin");
+
 struct RouteLayout {
   size_t hbuf, dupset, pslot, pfree, A, meta, slot, pst, fslot, vslot, vt, owner, victim, wm, wabs,
       wcost, wopen, kind, evk, touched, total;

@@ -259,6 +259,10 @@ cudaError_t launch_route_batch(const RouterState& s, int32_t instance, const int
                                int nbmax, const TableGeom& g, const ModelConsts& mc, float omega,
                                float tau, uint64_t seed, bool lean, cudaStream_t st);
 size_t router_smem(int W, int nbmax, bool lean);
+// What the routing kernel's own variables may take beside those arrays: 3 KB, so
+// that at 227 KB prompts of up to 2 904 (W = 1), 2 902 (W = 6) and 2 864 blocks
+// (W = 64) are routed.
+constexpr size_t ROUTE_OWN_SMEM = 3072;
 // host: pinned, receives the instance's sticky status and whether entries were
 // skipped (then the flag stays set on the device).
 cudaError_t launch_route_release(const RouterState& s, const int32_t* worker, const int32_t* blocks,

@@ -46,3 +46,30 @@ def test_route_batch_forms(W, K, n, hi, pre, tau):
         assert np.array_equal(rs.route_active(ctx.h, 0, W), ref.active(0))
     for j in range(W):
         assert np.array_equal(rs.route_cache_dump(ctx.h, 0, 0, j, K), ref.cache(0, j))
+
+
+# the longest prompts that 227 KB of shared memory hold, and one block more (refused, the state as it was)
+@pytest.mark.parametrize("W,nb", [(1, 2904), (3, 2904), (6, 2902), (64, 2864)])
+def test_route_batch_longest_prompt(W, nb):
+    K = 3000
+    ctx = rs.Context(W=W, K=K, n_instances=1, tau=0.0, omega=1.0, seed=5)
+    ref = O.Router(O.OracleConfig(W=W, K=K), 1.0, 0.0, 5, n_instances=1)
+    rng = np.random.default_rng(nb)
+    long = rng.integers(0, 32000, 16 * (nb + 1)).astype(np.int32)
+    for parts in ([long[:16 * nb + 15], long[:160], long[:16 * nb], long[16 * 50:]], [long]):
+        off = np.concatenate([[0], np.cumsum([p.size for p in parts])]).astype(np.int64)
+        tok = np.concatenate(parts + [np.zeros(-int(off[-1]) % 4, np.int32)])
+        tr = wk.Trace(tok, off, np.zeros(len(parts)), np.full(len(parts), 7, np.int32), np.zeros(len(parts), np.int32))
+        d = rs.device_trace(tr)
+        wo = torch.zeros(tr.n_req, dtype=torch.int32, device="cuda")
+        if len(parts) == 1:
+            with pytest.raises(rs.RoutesimError) as e:
+                rs.route_batch(ctx.h, 0, d.tokens, d.offsets, 1, d.out_len, wo)
+            assert e.value.status == rs.RS_ERR_CAPACITY
+        else:
+            rs.route_batch(ctx.h, 0, d.tokens, d.offsets, tr.n_req, d.out_len, wo)
+            st, rw, _, _ = ref.route(0, tr.tokens, tr.offsets, tr.out_len)
+            assert st == 0 and np.array_equal(wo.cpu().numpy(), rw)
+        assert np.array_equal(rs.route_active(ctx.h, 0, W), ref.active(0))
+        for j in range(min(W, 4)):
+            assert np.array_equal(rs.route_cache_dump(ctx.h, 0, 0, j, K), ref.cache(0, j))
