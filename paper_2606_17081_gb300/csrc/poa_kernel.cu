@@ -32,11 +32,12 @@
 // only the weights whose minimum moved out are looked up again.
 //
 // The paths run on integers: a window's costs become multiples of 2^-s (s from
-// the window's largest cost: 53 significant bits of it at W <= 16, 51 above),
+// the window's largest cost: 55 significant bits of it at W <= 16, 53 above),
 // so sums and comparisons are exact, no cycle is negative by rounding, and the
 // integer units carry the serial chain (a dependent FP64 add costs 64 cycles).
-// The rounding, at most 2^-52 of the window's largest cost per request, is far
-// below the 1e-12 below which a search on doubles must ignore gains.
+// The assignment found is optimal for costs that differ from the window's by at
+// most 2^-56 (2^-54) of its largest each.  OPT is the sum of that assignment's
+// own costs, taken in two integer parts and rounded once (opt_add).
 // Measured: poa_estimate on 20 000 records, W = 6 (81 windows): 4.22 -> 0.61 ms
 // a call (keys 97 -> 5 us, sort and costs 1480 -> 17 us, solver 2941 -> 578 us,
 // total 19 -> 6 us) with one warp per window, 0.43 ms with a CTA; the estimate
@@ -297,24 +298,23 @@ __global__ void __launch_bounds__(POA_SORT_NT) k_poa_sort(const PoaProblem* __re
 }
 
 // Fixed-point costs of one window: value = cost * 2^s.  With BITS bits for the
-// largest cost, |value| < 2^BITS, an edge weight is below 2^(BITS + 1) and the
-// sum of a path's weights (at most W of them) below 2^59 < FX_INF / 4.
+// largest cost, |value| <= 2^BITS, an edge weight is at most 2^(BITS + 1), and a
+// path's weights (at most 15, or 63, of them) sum to less than FX_REAL.
 constexpr long long FX_INF = 1ll << 61;    // no path / no row
 constexpr long long FX_REAL = 1ll << 60;   // every finite distance is below
-constexpr int FX_BITS = 53;                // W <= 16
-constexpr int FX_BITS_WIDE = 51;           // W <= 64
+constexpr int FX_BITS = 55;                // W <= 16: 15 2^56 < 2^60
+constexpr int FX_BITS_WIDE = 53;           // W <= 64: 63 2^54 < 2^60
 
 // Biased exponent of a finite cost (0 for one that is not finite).
 __device__ __forceinline__ int cost_exp(double c) {
   const int e = (int)((uint64_t)__double_as_longlong(c) >> 52) & 0x7FF;
   return e < 0x7FF ? e : 0;
 }
-// The scale 2^s that puts costs of biased exponent emax below 2^bits, and
-// 2^-s (s within the normal range: smaller costs than it covers round to 0).
-__device__ __forceinline__ double fx_scale(int emax, int bits, double* inv) {
+// The scale 2^s that puts costs of biased exponent emax below 2^bits (s within
+// the normal range: smaller costs than it covers round to 0).
+__device__ __forceinline__ double fx_scale(int emax, int bits) {
   int s = bits - (emax - 1022);
   s = s > 1000 ? 1000 : (s < -1000 ? -1000 : s);
-  *inv = __longlong_as_double((long long)(1023 - s) << 52);
   return __longlong_as_double((long long)(1023 + s) << 52);
 }
 // A cost that is not finite counts as the largest magnitude.
@@ -335,6 +335,34 @@ __device__ __forceinline__ int warp_argmin(long long v, bool in, long long* best
   const unsigned who = __ballot_sync(FULL_MASK, c1 && lo == ml);
   *best = (long long)(((unsigned long long)(mh ^ 0x80000000u) << 32) | ml);
   return who ? __ffs(who) - 1 : -1;
+}
+
+// A row's cost at its worker in units of 2^(emax - 1084) (62 bits: emax is the
+// largest biased exponent of the costs summed, all finite), rounded, in two
+// parts of 31 bits: sums of either over a window's rows are exact.
+__device__ __forceinline__ void opt_add(double c, int emax, long long& hi, long long& lo) {
+  const unsigned long long u = (unsigned long long)__double_as_longlong(c);
+  const int e = (int)(u >> 52) & 0x7FF, sh = emax - (e ? e : 1);
+  unsigned long long v = ((u & 0xFFFFFFFFFFFFFull) | (e ? 1ull << 52 : 0ull)) << 9;
+  v = sh < 63 ? (v + (sh ? 1ull << (sh - 1) : 0ull)) >> sh : 0ull;
+  const long long h = (long long)(v >> 31), l = (long long)(v & 0x7FFFFFFFull);
+  hi += u >> 63 ? -h : h;
+  lo += u >> 63 ? -l : l;
+}
+
+// The cost whose parts these are, with one rounding.
+__device__ __forceinline__ double opt_value(long long hi, long long lo, int emax) {
+  hi += lo >> 31;
+  lo &= 0x7FFFFFFFll;
+  const double d = (double)hi;
+  const double r = d + ((double)(hi - (long long)d) + (double)lo * 0x1p-31);
+  return scalbn(r, emax - 1084 + 31);
+}
+
+__device__ __forceinline__ long long warp_sum_int(long long v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(FULL_MASK, v, o);
+  return v;
 }
 
 constexpr int NT_SOLVE = 128;   // threads of a narrow solver CTA at one warp per window
@@ -426,6 +454,65 @@ __device__ __forceinline__ bool poa_next(const PoaProblem* __restrict__ probs, c
     *w = ww;
     return true;
   }
+}
+
+// OPT of a solved window (a warp's or a CTA's): the sum of its rows' costs at their
+// workers asg[r].  kept: those costs are still in b.cost; else they are computed
+// again where the fixed point took their place.
+template <int NWP>
+__device__ __forceinline__ double narrow_opt(PoaWinShared& S, const PoaBuffers& b, const ModelConsts& mc,
+                                          const double* ftab, bool wc_finite, double (*red)[NWP],
+                                          int64_t rec_base, int64_t base, int m, const uint8_t* asg,
+                                          bool kept) {
+  constexpr int NT = 32 * NWP;
+  const int lane = threadIdx.x & 31, ww = NWP == 1 ? 0 : (int)threadIdx.x >> 5, tid = 32 * ww + lane;
+  const int W = mc.W, nft = mc.cap < POA_FTAB ? mc.cap : POA_FTAB;
+  double* cost = b.cost + base * W;   // [W][m]
+  int ex = 1;
+  for (int r = tid; r < m; r += NT) {
+    const int j = asg[r];
+    double* at = cost + (int64_t)j * m + r;
+    if (!kept) {
+      const int64_t q = rec_base + b.order[base + r];
+      *at = frozen_cost(mc, ftab, nft, wc_finite, b.rec.n_frozen[q * W + j], b.rec.prefix[q * W + j],
+                        b.rec.nbt[q]);
+    }
+    ex = max(ex, (int)(__double_as_longlong(*at) >> 52) & 0x7FF);
+  }
+  ex = __reduce_max_sync(FULL_MASK, ex);
+  if (NWP > 1) {
+    if (tid == 0) S.emax = 0;
+    __syncthreads();
+    if (lane == 0) atomicMax(&S.emax, ex);
+    __syncthreads();
+    ex = S.emax;
+  }
+  long long hi = 0, lo = 0;
+  double opt = 0.0;
+  for (int r = tid; r < m; r += NT) {
+    const double c = cost[(int64_t)asg[r] * m + r];
+    if (ex < 0x7FF) opt_add(c, ex, hi, lo); else opt += c;
+  }
+  hi = warp_sum_int(hi);
+  lo = warp_sum_int(lo);
+  if (ex == 0x7FF) opt = warp_sum(opt);
+  if (NWP > 1) {
+    if (lane == 0) {
+      red[0][ww] = __longlong_as_double(hi);
+      red[1][ww] = __longlong_as_double(lo);
+      red[2][ww] = opt;
+    }
+    __syncthreads();
+    hi = lo = 0;
+    opt = 0.0;
+    for (int q = 0; q < NWP; q++) {
+      hi += __double_as_longlong(red[0][q]);
+      lo += __double_as_longlong(red[1][q]);
+      opt += red[2][q];
+    }
+    __syncthreads();
+  }
+  return ex < 0x7FF ? opt_value(hi, lo, ex) : opt;
 }
 
 // WT: a compile-time bound on W (the exact W for the common 3 and 6, else
@@ -544,8 +631,7 @@ __global__ void __launch_bounds__(NWP == 1 ? NT_SOLVE : 32 * NWP)
     sum3(num, nst, opt);
     int count = lane < W ? S.counts[lane] : 0;   // lane j of warp 0 keeps worker j's load
     if (__any_sync(FULL_MASK, lane < W && count > capw)) {   // (every warp alike)
-      double inv;
-      const double scale = fx_scale(S.emax, FX_BITS, &inv);
+      const double scale = fx_scale(S.emax, FX_BITS);
       long long* fx = NWP > 1 && (int64_t)m * W <= SOLVE_SCOST ? s_fx
                                                                 : reinterpret_cast<long long*>(cost);
       for (int64_t e = tid; e < (int64_t)m * W; e += NT) fx[e] = to_fx(cost[e], scale, FX_BITS);
@@ -632,27 +718,7 @@ __global__ void __launch_bounds__(NWP == 1 ? NT_SOLVE : 32 * NWP)
       }
       // (a load past its capacity cannot be left: W capw >= m)
       const bool bad = ww == 0 && __any_sync(FULL_MASK, lane < W && count > capw);
-      opt = 0.0;
-      if (m <= 1 << (62 - FX_BITS)) {
-        // the integers' sum is exact: one rounding
-        long long si = 0;
-        for (int r = tid; r < m; r += NT) si += fx[(int64_t)asg[r] * m + r];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) si += __shfl_xor_sync(FULL_MASK, si, o);
-        if (NWP > 1) {
-          if (lane == 0) red[0][ww] = __longlong_as_double(si);
-          __syncthreads();
-          si = __double_as_longlong(red[0][lane & (NWP - 1)]);
-#pragma unroll
-          for (int o = NWP / 2; o > 0; o >>= 1) si += __shfl_xor_sync(FULL_MASK, si, o);
-          __syncthreads();
-        }
-        opt = (double)si * inv;
-      } else {
-        for (int r = tid; r < m; r += NT) opt += (double)fx[(int64_t)asg[r] * m + r] * inv;
-        double z0 = 0.0, z1 = 0.0;
-        sum3(opt, z0, z1);
-      }
+      opt = narrow_opt<NWP>(S, b, mc, ftab, wc_finite, red, pr.rec_base, base, m, asg, fx == s_fx);
       if (bad) opt = __longlong_as_double(0x7FF8000000000000ll);
     }
     if (tid == 0) {
@@ -701,7 +767,7 @@ struct PoaWideShared {
   int pred[POA_WMAX_WIDE], counts[POA_WMAX_WIDE], fill[POA_WMAX_WIDE];
   int path[POA_WMAX_WIDE + 1];           // workers from the target back to the source
   int mv_r[POA_WMAX_WIDE];               // the request moved from path[t + 1] to path[t]
-  int nmv, nitems, emax, pi_next;
+  int nmv, nitems, emax, pi_next, q_first, q_last;
   int64_t w_next;
 };
 
@@ -749,6 +815,75 @@ __device__ __forceinline__ void wide_weight(const int32_t* rows, const int32_t* 
   const bool mine = row >= 0 && best == *least;
   *lrow = (int)__reduce_min_sync(FULL_MASK, mine ? (unsigned)row : 0xFFFFFFFFu);
   if (*lrow < 0) *least = FX_INF;
+}
+
+// OPT of a solved window: the sum of its rows' costs at their workers pos[r].  The
+// costs are computed again where the fixed point took their place.  Out of line:
+// with this in the kernel's body its loops took 5% more time.
+// Where the lists took the place of the window's rows in order[], S.q_first ..
+// S.q_last are the rows between its first and its last (else none).
+__device__ __noinline__ double wide_opt(PoaWideShared& S, const PoaProblem* __restrict__ probs,
+                                        const PoaBuffers& b, const ModelConsts& mc, int m,
+                                        const int32_t* pos) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, W = mc.W;
+  const int nft = mc.cap < POA_FTAB ? mc.cap : POA_FTAB;
+  const bool wc_finite = __dmul_rn(mc.w_c, 0.0) == 0.0;
+  const int64_t rec_base = probs[S.pi_next].rec_base, w = S.w_next;
+  const int64_t base = probs[S.pi_next].scratch_base + b.wstart[probs[S.pi_next].win_base + S.pi_next + w];
+  double* cost = b.cost + base * W;   // [m][W]
+  const int q_first = S.q_first, q_last = S.q_last;
+  // those of them that complete in the window, in order
+  int have = 0;
+  for (int q0 = q_first; q0 <= q_last; q0 += NT_WIDE) {
+    const int q = q0 + (int)threadIdx.x;
+    bool in = q <= q_last;
+    if (in) {
+      const int64_t r = rec_base + q;
+      in = b.rec.worker[r] >= 0 &&
+           floor(__ddiv_rn(b.rec.completion[r], mc.poa_window)) == (double)w;
+    }
+    const unsigned mk = __ballot_sync(FULL_MASK, in);
+    if (lane == 0) S.part_r[warp] = __popc(mk);
+    __syncthreads();
+    const int n = S.part_r[lane];
+    const int below = (int)__reduce_add_sync(FULL_MASK, (unsigned)(lane < warp ? n : 0));
+    if (in) b.order[base + have + below + __popc(mk & ((1u << lane) - 1u))] = q;
+    have += (int)__reduce_add_sync(FULL_MASK, (unsigned)n);
+    __syncthreads();
+  }
+  int ex = 1;
+  for (int r = threadIdx.x; r < m; r += NT_WIDE) {
+    const int64_t q = rec_base + b.order[base + r];
+    const int j = pos[r];
+    const double c = frozen_cost(mc, S.ftab, nft, wc_finite, b.rec.n_frozen[q * W + j],
+                                 b.rec.prefix[q * W + j], b.rec.nbt[q]);
+    cost[(int64_t)r * W + j] = c;
+    ex = max(ex, (int)(__double_as_longlong(c) >> 52) & 0x7FF);
+  }
+  ex = __reduce_max_sync(FULL_MASK, ex);
+  if (threadIdx.x == 0) S.emax = 0;
+  __syncthreads();
+  if (lane == 0) atomicMax(&S.emax, ex);
+  __syncthreads();
+  ex = S.emax;
+  long long hi = 0, lo = 0;
+  double opt = 0.0;
+  for (int r = threadIdx.x; r < m; r += NT_WIDE) {
+    const double c = cost[(int64_t)r * W + pos[r]];
+    if (ex < 0x7FF) opt_add(c, ex, hi, lo); else opt += c;
+  }
+  hi = warp_sum_int(hi);
+  lo = warp_sum_int(lo);
+  opt = warp_sum(opt);
+  if (lane == 0) {
+    S.red[0][warp] = __longlong_as_double(hi);
+    S.red[1][warp] = __longlong_as_double(lo);
+    S.red[2][warp] = opt;
+  }
+  __syncthreads();
+  hi = warp_sum_int(__double_as_longlong(S.red[0][lane]));
+  lo = warp_sum_int(__double_as_longlong(S.red[1][lane]));
+  return ex < 0x7FF ? opt_value(hi, lo, ex) : warp_sum(S.red[2][lane]);
 }
 
 __global__ void __launch_bounds__(NT_WIDE) k_poa_solve_wide(const PoaProblem* __restrict__ probs,
@@ -849,9 +984,12 @@ __global__ void __launch_bounds__(NT_WIDE) k_poa_solve_wide(const PoaProblem* __
     nst = warp_sum(S.red[1][lane]);
     opt = warp_sum(S.red[2][lane]);
     if (__syncthreads_or(threadIdx.x < W && S.counts[threadIdx.x] > capw)) {
-      double inv;
-      const double scale = fx_scale(S.emax, FX_BITS_WIDE, &inv);
+      const double scale = fx_scale(S.emax, FX_BITS_WIDE);
       long long* fx = reinterpret_cast<long long*>(cost);   // in place
+      if (threadIdx.x == 0) {
+        S.q_first = listed && !in_smem ? b.order[base] : 0;
+        S.q_last = listed && !in_smem ? b.order[base + m - 1] : -1;
+      }
       for (int64_t e = threadIdx.x; e < (int64_t)m * W; e += NT_WIDE)
         fx[e] = to_fx(cost[e], scale, FX_BITS_WIDE);
       // room for a worker's first load or, below it, its capacity
@@ -1132,16 +1270,11 @@ __global__ void __launch_bounds__(NT_WIDE) k_poa_solve_wide(const PoaProblem* __
         __syncthreads();
       }
       const bool bad = __syncthreads_or(threadIdx.x < W && S.counts[threadIdx.x] > capw);
-      // each row's worker again, then the sum in row order
+      // each row's worker again
       for (int j = warp; listed && j < W; j += NW_WIDE)
         for (int t = lane; t < S.counts[j]; t += 32) pos[S.list[j][t]] = j;
       __syncthreads();
-      opt = 0.0;
-      for (int r = threadIdx.x; r < m; r += NT_WIDE) opt += (double)fx[(int64_t)r * W + pos[r]] * inv;
-      opt = warp_sum(opt);
-      if (lane == 0) S.red[0][warp] = opt;
-      __syncthreads();
-      opt = warp_sum(S.red[0][lane]);
+      opt = wide_opt(S, probs, b, mc, m, pos);
       if (bad) opt = __longlong_as_double(0x7FF8000000000000ll);
     }
     if (threadIdx.x == 0) {

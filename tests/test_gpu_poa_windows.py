@@ -3,6 +3,8 @@ than they have rows (a slow Poisson client, long outputs), so every window the
 records reach must get a slot.  The estimate of simulate_replicas, of
 poa_estimate and of poa_estimate_noalloc must all equal the oracle's per
 window (numerator, count, OPT) and in total."""
+import math
+
 import numpy as np
 import pytest
 
@@ -130,7 +132,36 @@ def test_sort_and_solvers_at_their_edges(W, n, windows, tied, cap):
     rec, keep = _to_device(o, n, W)
     gn, go, gc, gt, nw = rs.poa_estimate(ctx.h, rec, n, windows)
     assert nw == windows and np.array_equal(gc, cnt)
-    # sums of at most 1400 rows of one sign: n 2^-53 relative (1.6e-13); OPT's costs also carry
-    # 2^-52 of the window's largest cost each
+    # sums of at most 4500 rows of one sign: n 2^-53 relative (5e-13)
     assert np.allclose(gn, num, rtol=1e-12, atol=0) and np.allclose(go, opt, rtol=1e-12, atol=0)
     assert abs(gt - tot) <= 1e-12 * tot
+
+
+# a few costs of 1000 among many below 0.1 (on workers that no optimum takes), past a capacity: narrow
+# solver with a CTA and with a warp per window, costs in shared memory and in place; wide solver with its
+# lists in shared memory, in the window's rows' place, and without lists
+@pytest.mark.parametrize("W,n,windows,cap", [(6, 600, 2, 128), (6, 900, 1, 128), (3, 150 * 400, 400, 80), (16, 500, 1, 128),
+                                             (17, 800, 1, 200), (33, 700, 2, 100), (17, 9000, 2, 64), (20, 900, 1, 512)])
+def test_opt_keeps_the_costs_bits(W, n, windows, cap):
+    d = 1000.0
+    ctx = rs.Context(W=W, K=64, cap=cap, lat_d=d)
+    rng = np.random.default_rng(W + n)
+    o = _random_records(rng, n, W, 5.0 * windows, False, cap)
+    o["n_frozen"][:, 1:][rng.random((n, W - 1)) < 0.05] = cap - 1
+    rec, keep = _to_device(o, n, W)
+    _, go, gc, _, nw = rs.poa_estimate(ctx.h, rec, n, windows)
+    assert nw == windows
+    nf, pre = o["n_frozen"].astype(np.float64), o["prefix"].astype(np.float64)
+    cost = ((0.005 * nf + 0.020) + d / ((cap - nf) * (cap - nf))) - 0.015 * (pre / o["nbt"][:, None])
+    win = np.floor(o["completion"] / 5.0).astype(int)
+    bound = 0
+    for w in list(range(windows))[:4]:
+        c = cost[(win == w) & (o["worker"] >= 0)]
+        m = c.shape[0]
+        capw = max(cap, -(-m // W))
+        bound += np.bincount(c.argmin(1)).max() > capw
+        _, at = O.assign(c, capw, 0)
+        mine = c[np.arange(m), at]
+        # equal costs may differ by their own rounding: one of the largest cost's, per row
+        assert abs(go[w] - math.fsum(mine)) <= m * 2.0 ** -53 * mine.max(), (w, go[w], math.fsum(mine))
+    assert bound
