@@ -77,11 +77,12 @@ __device__ __forceinline__ double frozen_cost(const ModelConsts& mc, const doubl
   return __dsub_rn(f, __dmul_rn(mc.w_c, __ddiv_rn((double)m, (double)nbt)));
 }
 
-// Order-preserving map of a double onto int64 (not NaN; -0 below +0): the
+// Order-preserving map of a double onto int64 (NaN above all, -0 below +0): the
 // comparisons run on the integer units.
 __device__ __forceinline__ long long okey(double x) {
   const long long u = __double_as_longlong(x);
-  return u ^ ((u >> 63) & 0x7FFFFFFFFFFFFFFFll);
+  return (u & 0x7FFFFFFFFFFFFFFFll) > 0x7FF0000000000000ll ? 0x7FFFFFFFFFFFFFFFll
+                                                            : u ^ ((u >> 63) & 0x7FFFFFFFFFFFFFFFll);
 }
 
 // Window of each row into wkey: -1 for a row that was not routed, KEY_BAD for
@@ -317,10 +318,16 @@ __device__ __forceinline__ double fx_scale(int emax, int bits) {
   s = s > 1000 ? 1000 : (s < -1000 ? -1000 : s);
   return __longlong_as_double((long long)(1023 + s) << 52);
 }
-// A cost that is not finite counts as the largest magnitude.
-__device__ __forceinline__ long long to_fx(double c, double scale, int bits) {
-  const long long lim = 1ll << bits;
-  if (!(fabs(c) < __longlong_as_double(0x7FF0000000000000ll))) return c < 0.0 ? -lim : lim;
+// A cost that is not finite: +infinity (a load at the pole of Eq. (9)) or NaN is
+// FX_NONE, -infinity FX_NEG.  A row sits at its least cost first, so it is at an
+// FX_NONE only if all its costs are, and has an FX_NEG only where it is at one; a
+// move from a finite cost to an FX_NONE, or away from an FX_NEG, weighs more than
+// FX_INF, that is, there is no such edge, and from like to like weighs 0.
+constexpr long long FX_NONE = 1ll << 62;
+constexpr long long FX_NEG = -(3ll << 60);
+
+__device__ __forceinline__ long long to_fx(double c, double scale) {
+  if (!(fabs(c) < __longlong_as_double(0x7FF0000000000000ll))) return c < 0.0 ? FX_NEG : FX_NONE;
   return __double2ll_rn(__dmul_rn(c, scale));
 }
 
@@ -634,7 +641,7 @@ __global__ void __launch_bounds__(NWP == 1 ? NT_SOLVE : 32 * NWP)
       const double scale = fx_scale(S.emax, FX_BITS);
       long long* fx = NWP > 1 && (int64_t)m * W <= SOLVE_SCOST ? s_fx
                                                                 : reinterpret_cast<long long*>(cost);
-      for (int64_t e = tid; e < (int64_t)m * W; e += NT) fx[e] = to_fx(cost[e], scale, FX_BITS);
+      for (int64_t e = tid; e < (int64_t)m * W; e += NT) fx[e] = to_fx(cost[e], scale);
       if (tid < W) {
         S.wmin[tid][tid] = FX_INF;
         S.wrow[tid][tid] = -1;
@@ -716,10 +723,11 @@ __global__ void __launch_bounds__(NWP == 1 ? NT_SOLVE : 32 * NWP)
           __syncwarp();
         }
       }
-      // (a load past its capacity cannot be left: W capw >= m)
+      // (W capw >= m: a load past its capacity is left only where every way out
+      // costs infinity)
       const bool bad = ww == 0 && __any_sync(FULL_MASK, lane < W && count > capw);
       opt = narrow_opt<NWP>(S, b, mc, ftab, wc_finite, red, pr.rec_base, base, m, asg, fx == s_fx);
-      if (bad) opt = __longlong_as_double(0x7FF8000000000000ll);
+      if (bad) opt = __longlong_as_double(0x7FF0000000000000ll);
     }
     if (tid == 0) {
       b.wnum[slot] = num;
@@ -991,7 +999,7 @@ __global__ void __launch_bounds__(NT_WIDE) k_poa_solve_wide(const PoaProblem* __
         S.q_last = listed && !in_smem ? b.order[base + m - 1] : -1;
       }
       for (int64_t e = threadIdx.x; e < (int64_t)m * W; e += NT_WIDE)
-        fx[e] = to_fx(cost[e], scale, FX_BITS_WIDE);
+        fx[e] = to_fx(cost[e], scale);
       // room for a worker's first load or, below it, its capacity
       if (threadIdx.x == 0) {
         int32_t *over = in_smem ? s_list : b.order + base, *under = b.wkey + base;
@@ -1183,7 +1191,7 @@ __global__ void __launch_bounds__(NT_WIDE) k_poa_solve_wide(const PoaProblem* __
         }
         __syncthreads();
         const int nmv = S.nmv;
-        if (nmv == 0) break;   // (cannot happen: W capw >= m)
+        if (nmv == 0) break;   // every way out costs infinity (W capw >= m)
         // warp t (and t + 32 on a longer path): the weights out of path[t + 1]
         // whose minimum moved away are listed; the moved request's costs beside
         // the one at its new worker are loaded for the end of the step
@@ -1275,7 +1283,7 @@ __global__ void __launch_bounds__(NT_WIDE) k_poa_solve_wide(const PoaProblem* __
         for (int t = lane; t < S.counts[j]; t += 32) pos[S.list[j][t]] = j;
       __syncthreads();
       opt = wide_opt(S, probs, b, mc, m, pos);
-      if (bad) opt = __longlong_as_double(0x7FF8000000000000ll);
+      if (bad) opt = __longlong_as_double(0x7FF0000000000000ll);
     }
     if (threadIdx.x == 0) {
       b.wnum[slot] = num;

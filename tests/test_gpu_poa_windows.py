@@ -165,3 +165,29 @@ def test_opt_keeps_the_costs_bits(W, n, windows, cap):
         # equal costs may differ by their own rounding: one of the largest cost's, per row
         assert abs(go[w] - math.fsum(mine)) <= m * 2.0 ** -53 * mine.max(), (w, go[w], math.fsum(mine))
     assert bound
+
+
+@pytest.mark.parametrize("W,n", [(3, 180), (6, 380), (17, 1080), (20, 9000)])
+def test_no_assignment_at_the_pole(W, n):
+    # loads at the pole of Eq. (9) (n_frozen = cap: infinite cost).  Worker 0 is cheap for all; at worker 1 two rows of
+    # three cannot be, and a third can only at nearly the largest cost, which the optimum must take: the capacities
+    # leave little room.  A penalty for the pole in its place would be the better bargain.
+    cap = 64
+    ctx = rs.Context(W=W, K=64)
+    rng = np.random.default_rng(W)
+    nf = rng.integers(45, 55, (n, W))
+    nf[:, 0] = rng.integers(1, 4, n)
+    other = np.arange(n) % 3 == 0
+    nf[other, 1:] = rng.integers(1, 4, (int(other.sum()), W - 1))
+    nf[:, 1] = np.where(other, cap - 1, cap)
+    o = {"worker": np.zeros(n, np.int32), "completion": rng.uniform(0.0, 5.0, n), "ttft": np.ones(n),
+         "nbt": np.ones(n, np.int32), "n_frozen": nf.astype(np.uint16), "prefix": np.zeros((n, W), np.uint16)}
+    _, opt, _, tot = O.poa(oracle_cfg(ctx), o)
+    assert opt.size == 1 and np.isfinite(opt[0])
+    rec, keep = _to_device(o, n, W)
+    _, go, _, gt, _ = rs.poa_estimate(ctx.h, rec, n, 1)
+    assert np.allclose(go, opt, rtol=1e-12, atol=0) and abs(gt - tot) <= 1e-12 * tot
+    o["n_frozen"][:, 1:] = cap   # no way out of worker 0
+    rec, keep = _to_device(o, n, W)
+    _, go, _, gt, _ = rs.poa_estimate(ctx.h, rec, n, 1)
+    assert go[0] == np.inf and gt == 0.0
