@@ -421,7 +421,6 @@ struct UpdateScratch {
 
 struct UpdateShared {   // small shared scalars of the update
   int n_absent, n_ins, reclaimed, n_victims, n_tomb, slow, err;
-  int changed;   // of lru_exact
   uint32_t pmin, gathered;
 };
 
@@ -696,47 +695,80 @@ __device__ __forceinline__ void cache_prepare_captured(const TableView& t, const
 
 // Exact LRU where blocks of a prompt lie among the least recent entries: which
 // of them are evicted before their turn.  w[k] = LRU_ABSENT, LRU_FAR (present,
-// past the entries gathered) or the place o of block k's entry in recency
+// past the G entries gathered) or the place o < G of block k's entry in recency
 // order; on return LRU_EVICTED is set in those evicted before block k comes.
 // Touching blocks 0 .. nb-1 in order, block k finds
 //   ins = absent or evicted blocks before k, E = max(0, ins - free) evictions,
 //   T = blocks before k that were touched and lie below o;
 // the entries below o that can be victims are o - T, so block k is gone iff
-// E > o - T.  Every block depends on earlier ones only: the blocks are evaluated
-// together until none changes (at least one more is final after each turn, in
-// practice all after two to four).  One thread replaying the sequence took
-// about 300 cycles a block.
+// E > o - T.  One warp takes the blocks 32 at a time, a lane per block.  Places
+// touched by earlier chunks are a bitmap with the count below each of its words
+// (bits: shared, 2 ceil(G / 32) words, 0 before and after).  Within the chunk
+// every block depends on lower lanes only, so it is evaluated until no verdict
+// changes, in practice two or three times.  Bound by the latency of that chain,
+// linear in the prompt.  (8 replicas x 300 requests of 1 250 to 2 000 blocks at
+// W = 7, a fifth of them exact: one thread replaying the sequence on hash tables
+// 36.8 ms, a thread per block counting T and ins over all blocks before it 37.4,
+// so 7.5; 250 to 500 blocks 24.3, 9.6 and 4.4.)
 constexpr int LRU_ABSENT = -1, LRU_FAR = -2, LRU_EVICTED = 0x40000000;
 
 template <int NT>
-__device__ __forceinline__ void lru_exact(volatile int32_t* w, int nb, int free_slots, int* changed) {
-  for (;;) {
-    grp_bar<NT>();   // (w is written; *changed has been read)
-    if (threadIdx.x == 0) *changed = 0;
-    grp_bar<NT>();
-    bool ch = false;
-    for (int k = threadIdx.x; k < nb; k += NT) {
-      const int x = w[k];
-      if (x < 0) continue;
-      const int o = x & ~LRU_EVICTED;
-      int ins = 0, touched = 0;
-#pragma unroll 4
-      for (int q = 0; q < k; q++) {
-        const int y = w[q];
-        ins += y == LRU_ABSENT || y >= LRU_EVICTED;
-        touched += y >= 0 && y < o;
+__device__ __forceinline__ void lru_exact(int32_t* w, int nb, int free_slots, int G, uint32_t* bits) {
+  grp_bar<NT>();   // (w is written)
+  if (threadIdx.x < 32) {
+    const int lane = (int)threadIdx.x, nw = (G + 31) >> 5;
+    const unsigned before = (1u << lane) - 1u;
+    uint32_t* below = bits + nw;
+    int ins = 0;
+#pragma unroll 1
+    for (int k0 = 0; k0 < nb; k0 += 32) {
+      const int o = k0 + lane < nb ? w[k0 + lane] : LRU_FAR;
+      const unsigned absent = __ballot_sync(FULL_MASK, o == LRU_ABSENT);
+      unsigned gone = 0u;
+      if (__any_sync(FULL_MASK, o >= 0)) {
+        unsigned lower = 0u;   // lanes before this one at lower places
+#pragma unroll
+        for (int q = 0; q < 31; q++) {
+          const int y = __shfl_sync(FULL_MASK, o, q);
+          lower |= (unsigned)(y >= 0 && y < o) << q;
+        }
+        lower &= before;
+        int room = 0x7FFFFFFF;   // places below o not touched by earlier chunks
+        if (o >= 0)
+          room = o - (int)(below[o >> 5] + __popc(bits[o >> 5] & ((1u << (o & 31)) - 1u)));
+        for (;;) {
+          const int E = max(0, ins + __popc((absent | gone) & before) - free_slots);
+          const unsigned g = __ballot_sync(FULL_MASK, o >= 0 && E > room - __popc(lower & ~gone));
+          if (g == gone) break;
+          gone = g;
+        }
+        __syncwarp();   // (the bitmap has been read)
+        if ((gone >> lane) & 1u)
+          w[k0 + lane] = o | LRU_EVICTED;
+        else if (o >= 0)
+          atomicOr(bits + (o >> 5), 1u << (o & 31));
+        __syncwarp();
+        uint32_t run = 0;
+#pragma unroll 1
+        for (int q0 = 0; q0 < nw; q0 += 32) {
+          const int q = q0 + lane;
+          const uint32_t c = q < nw ? (uint32_t)__popc(bits[q]) : 0u;
+          uint32_t x = c;
+#pragma unroll
+          for (int s = 1; s < 32; s <<= 1) {
+            const uint32_t y = __shfl_up_sync(FULL_MASK, x, s);
+            if (lane >= s) x += y;
+          }
+          if (q < nw) below[q] = run + x - c;
+          run += __shfl_sync(FULL_MASK, x, 31);
+        }
+        __syncwarp();
       }
-      const int E = ins > free_slots ? ins - free_slots : 0;
-      const int v = E > o - touched ? o | LRU_EVICTED : o;
-      if (v != x) {
-        w[k] = v;
-        ch = true;
-      }
+      ins += __popc(absent | gone);
     }
-    if (ch) *changed = 1;
-    grp_bar<NT>();
-    if (!*changed) break;
+    for (int q = lane; q < 2 * nw; q += 32) bits[q] = 0u;
   }
+  grp_bar<NT>();
 }
 
 // Applies one request's block list to the chosen worker's cache: exact LRU
@@ -802,7 +834,7 @@ __device__ __forceinline__ void cache_apply(const TableView& t, CacheMeta* meta,
       }
       w[k] = v;
     }
-    lru_exact<NT>(w, nb, (int)free_slots, &us->changed);
+    lru_exact<NT>(w, nb, (int)free_slots, (int)G, reinterpret_cast<uint32_t*>(sc.dupset));   // (empty until the claims below)
     int ni = 0;
     for (int k = threadIdx.x; k < nb; k += NT) {
       const int v = w[k];
@@ -829,7 +861,7 @@ __device__ __forceinline__ void cache_apply(const TableView& t, CacheMeta* meta,
       if (have < E1) us->err = RS_ERR_TIMEOUT;
       us->n_victims = have < E1 ? 0 : E1;
       us->slow = 1;
-        }
+    }
     grp_bar<NT>();
   }
   const int E = us->n_victims;

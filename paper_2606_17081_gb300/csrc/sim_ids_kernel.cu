@@ -231,6 +231,7 @@ struct IdsShared {
   int nvic, nins, changed;
   uint32_t nh;
   int js;                      // the chosen worker
+  uint32_t* lru_bits;          // of lru_exact
 };
 
 // Workers per update warp up to which updates are planned before the choice.
@@ -238,7 +239,7 @@ __host__ __device__ constexpr int ids_plan_workers(int) { return 1; }
 
 struct IdsLayout {
   size_t ftab, f_oitl, f_a, f_o, h_k, srec, gk, gf, wA, codes, meta, f_req, f_worker, f_blk, f_next, h_f,
-      freestk, winserv, wqh, wqt, wm, act, nfz, whead, wlen, win, wfreq;
+      freestk, winserv, wqh, wqt, wm, act, nfz, whead, wlen, win, wfreq, lru;
   size_t total, slot_bytes;
 };
 
@@ -296,6 +297,7 @@ __host__ __device__ inline IdsLayout make_ids_layout(int W, int nbmax, int cmax,
   const int nu = ntu / 32;
   L.win = take(4 * (size_t)W * (!freq && W <= nu * ids_plan_workers(nu) ? IDS_WRING : IDS_WIN));
   L.wfreq = take(freq ? sizeof(FreqMeta) * (size_t)W : 0);
+  L.lru = take(8 * ((2 * nb + 31) / 32));
   L.total = o;
   L.slot_bytes = (og + 255) & ~(size_t)255;
   return L;
@@ -764,7 +766,7 @@ __device__ __noinline__ uint32_t ids_evict_general(IdsTable t, CacheMeta m, uint
     sc.w[k] = v;
   }
   if (threadIdx.x == 0) S.nins = 0;
-  lru_exact<NT>(sc.w, nb, freeb, &S.changed);
+  lru_exact<NT>(sc.w, nb, freeb, (int)G, S.lru_bits);
   int ni = 0;
   for (int k = threadIdx.x; k < nb; k += NT) ni += sc.w[k] == LRU_ABSENT || sc.w[k] >= LRU_EVICTED;
   ni = (int)__reduce_add_sync(FULL_MASK, (unsigned)ni);
@@ -2066,6 +2068,8 @@ __global__ void __launch_bounds__((NU + 2) * 32, MINB)
     for (size_t s = threadIdx.x; s < nst / 4; s += NT)
       reinterpret_cast<uint4*>(stamps)[s] = make_uint4(STAMP_NONE, STAMP_NONE, STAMP_NONE, STAMP_NONE);
     for (int q = 1 + threadIdx.x; q < nft; q += NT) c.ftab[q] = latency_f(mc, q);
+    for (int q = threadIdx.x; q < 2 * ((2 * nbcap + 31) / 32); q += NT)
+      reinterpret_cast<uint32_t*>(smem + lay.lru)[q] = 0u;
     const int cslots = max(d.C, max(d.c_mid, d.c_end));
     for (int p = threadIdx.x; p < cslots; p += NT) c.freestk[p] = cslots - 1 - p;
     for (int j = threadIdx.x; j < W; j += NT) {
@@ -2088,6 +2092,7 @@ __global__ void __launch_bounds__((NU + 2) * 32, MINB)
       S.first_evict_i = -1;
       Sh.stat[0] = Sh.stat[1] = make_int2(RS_OK, RS_OK);
       Sh.err = 0;
+      Sh.lru_bits = reinterpret_cast<uint32_t*>(smem + lay.lru);
     }
   }
   __syncthreads();

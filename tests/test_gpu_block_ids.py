@@ -13,7 +13,7 @@ import pytest
 from paper_2606_17081_gb300 import routesim as rs
 from paper_2606_17081_gb300 import workloads as wk
 
-from gpu_helpers import gpu_run
+from gpu_helpers import assert_replica_equal, gpu_run, oracle_cfg, oracle_run
 
 pytestmark = pytest.mark.gpu
 
@@ -142,6 +142,24 @@ def test_records_of_stopped_replicas(W, C):
     assert started.sum() > 100 and (W != 2 or started.sum() < n)
     assert np.array_equal(g[0]["ttft"][:n][started], (g[0]["first_token"] - g[0]["arrival"])[:n][started])
     assert not g[0]["ttft"][n:].any()
+
+
+# exact sequences of one chunk of 32 blocks, of whole chunks and of one block more, up to the longest prompts: blocks of
+# a prompt among the least recent entries, evicted before their turn
+@pytest.mark.parametrize("W,K,n,nrep", [(2, 31, 400, 1), (3, 64, 300, 1), (8, 65, 300, 1), (2, 700, 150, 1), (7, 2100, 60, 1),
+                                        (4, 129, 120, 306)])   # (two update warps)
+def test_exact_sequences_against_the_oracle(W, K, n, nrep):
+    tr = _trace(n, K, groups=3, lo=0, hi=16 * K + 15, pre=(8 * K, 16 * K))
+    reps = [wk.Replica(0, 6, wk.POLICY_RANDOM, 0, 1.0, 0.0, r, n) for r in range(nrep)]
+    ctx = rs.Context(W=W, K=K)
+    ref = {r: oracle_run(oracle_cfg(ctx), tr, reps[r], want_cache=True) for r in {0, nrep - 1}}
+    for flags in (0, rs.RS_SIM_TABLES):
+        st, g = gpu_run(ctx, [tr], reps, flags=flags)
+        assert st == rs.RS_OK and g[0]["result"]["slow_path"] > 0
+        for r, o in ref.items():
+            assert_replica_equal(g[r], o, W)
+            for j in range(W):
+                assert np.array_equal(rs.route_cache_dump(ctx.h, 1, r, j, K), o["cache"][j])
 
 
 @pytest.mark.parametrize("W,C", [(3, 8), (7, 8), (3, 5000)])   # planned updates, not planned, slot arrays in global memory
