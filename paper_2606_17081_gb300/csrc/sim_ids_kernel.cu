@@ -234,9 +234,6 @@ struct IdsShared {
   uint32_t* lru_bits;          // of lru_exact
 };
 
-// Workers per update warp up to which updates are planned before the choice.
-__host__ __device__ constexpr int ids_plan_workers(int) { return 1; }
-
 struct IdsLayout {
   size_t ftab, f_oitl, f_a, f_o, h_k, srec, gk, gf, wA, codes, meta, f_req, f_worker, f_blk, f_next, h_f,
       freestk, winserv, wqh, wqt, wm, act, nfz, whead, wlen, win, wfreq, lru;
@@ -295,7 +292,7 @@ __host__ __device__ inline IdsLayout make_ids_layout(int W, int nbmax, int cmax,
   L.whead = take(4 * (size_t)W);
   L.wlen = take(4 * (size_t)W);
   const int nu = ntu / 32;
-  L.win = take(4 * (size_t)W * (!freq && W <= nu * ids_plan_workers(nu) ? IDS_WRING : IDS_WIN));
+  L.win = take(4 * (size_t)W * (!freq && W <= nu ? IDS_WRING : IDS_WIN));
   L.wfreq = take(freq ? sizeof(FreqMeta) * (size_t)W : 0);
   L.lru = take(8 * ((2 * nb + 31) / 32));
   L.total = o;
@@ -2002,7 +1999,6 @@ __global__ void __launch_bounds__((NU + 2) * 32, MINB)
               const __grid_constant__ SimLaunch L) {
   constexpr int NT = (NU + 2) * 32, NTU = NU * 32;
   constexpr bool WIDE = VAR == 2, PLAN = VAR == 0;
-  constexpr int PW = ids_plan_workers(NU);   // workers per update warp with planned updates
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ SimScalars S;
   __shared__ IdsShared Sh;
@@ -2116,43 +2112,29 @@ __global__ void __launch_bounds__((NU + 2) * 32, MINB)
       if (qk.nb > (int)L.g.K) return;
       const uint32_t* cd = codes + (size_t)ek * nbcap;
       if constexpr (PLAN) {
-        // the rings' next entries, once a victim may be needed soon; those
+        // the ring's next entries, once a victim may be needed soon; those
         // copied the last time have landed before others are sent to their
         // places (copies in flight keep no order: after a compaction, or when
         // two updates together pass more entries than the ring holds, the same
         // place is written again)
         cp_async_wait_all();
         __syncwarp();
-        uint32_t safe[PW];
-#pragma unroll
-        for (int w = 0; w < PW; w++) {
-          const int j = warp + w * NU;
-          if (j >= W) break;
-          const CacheMeta m = c.wmeta[j];
-          uint32_t wend = max(wlen[j], m.head);   // (a compaction sets it to 0)
-          safe[w] = wend;
+        if (warp < W) {
+          const IdsTable t = table(warp);
+          const CacheMeta m = c.wmeta[warp];
+          uint32_t* ring = win + warp * IDS_WRING;
+          const uint32_t safe = max(wlen[warp], m.head);   // (a compaction sets it to 0)
           const uint32_t to = min(m.T, m.head + IDS_WRING);
-          if (m.size + 2 * (uint32_t)L.nbmax > L.g.K && wend < to) {
-            const uint32_t* lg = table(j).log;
+          const bool more = m.size + 2 * (uint32_t)L.nbmax > L.g.K && safe < to;
+          __syncwarp();   // (every lane has read the last end)
+          if (more) {
 #pragma unroll 1
-            for (uint32_t p = wend + lane; p < to; p += 32)
-              cp_async4(win + j * IDS_WRING + (p & (IDS_WRING - 1)), lg + (p & L.ids_rmask));
-            wend = to;
+            for (uint32_t p = safe + lane; p < to; p += 32)
+              cp_async4(ring + (p & (IDS_WRING - 1)), t.log + (p & L.ids_rmask));
           }
-          if (lane == 0) wlen[j] = wend;
-        }
-        __syncwarp();
-#pragma unroll 1
-        for (int w = 0; w < PW; w++) {
-          const int j = warp + w * NU;
-          if (j >= W) break;
-          uint32_t sf = safe[0];
-#pragma unroll
-          for (int v = 1; v < PW; v++)
-            if (w == v) sf = safe[v];
-          const int mj = ids_plan(table(j), c.wmeta[j], L.g.K, cd, qk.nb, qk.nz, win + j * IDS_WRING, sf,
-                                  Sh.plan[j], cnt);
-          if (lane == 0) wm[pk * W + j] = mj;
+          if (lane == 0) wlen[warp] = more ? to : safe;
+          const int mj = ids_plan(t, m, L.g.K, cd, qk.nb, qk.nz, ring, safe, Sh.plan[warp], cnt);
+          if (lane == 0) wm[pk * W + warp] = mj;
         }
       } else {
         ids_probe<NU>(stamps, nre, cd, qk.nz, W, wm + pk * W, cnt);
@@ -2537,7 +2519,7 @@ cudaError_t launch_sim_ids(const SimDesc* d_desc, const SimBuffers& b, const Sim
   if (freq && sg) return cudaErrorInvalidValue;   // (such launches use the tables)
   const size_t smem = sim_ids_smem_bytes(L.mc.W, L.nbmax, L.cmax, L.mc.cap, 32 * nu, sg, freq);
   void (*kern)(const SimDesc*, const SimBuffers, const SimLaunch);
-  const int var = L.mc.W <= nu * ids_plan_workers(nu) ? 0 : (L.mc.W <= 32 ? 1 : 2);
+  const int var = L.mc.W <= nu ? 0 : (L.mc.W <= 32 ? 1 : 2);
   if (freq)
     kern = nu == 6 ? (var == 2 ? k_sim_ids<6, 2, false, 2, true> : k_sim_ids<6, 2, false, 1, true>)
                    : (var == 2 ? k_sim_ids<2, 5, false, 2, true> : k_sim_ids<2, 5, false, 1, true>);
