@@ -276,7 +276,8 @@ typedef struct {
   int32_t max_regime, reserved0;
   int64_t ticks_in_regime[3];
   double final_ewma;        /* -1 if no sample */
-  int64_t probes;           /* hash-table lookups issued (work counter) */
+  int64_t probes;           /* lookups issued in the workers' caches (work counter: hash-table
+                               lookups, or block stamps read on block ids) */
   int64_t probe_blocks;     /* sum over decisions and workers of min(m_ij + 1, nb_i):
                                the lookups a first-miss probe needs */
   int64_t hashed_blocks;    /* sum of nb_i (full blocks) over routed requests */

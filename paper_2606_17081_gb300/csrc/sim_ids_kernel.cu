@@ -2194,8 +2194,9 @@ __global__ void __launch_bounds__((NU + 2) * 32, MINB)
       if (i + 1 < n) probe(i + 1, p ^ 1);
     }
     cp_async_wait_all();
-    cnt = __reduce_add_sync(FULL_MASK, cnt);
-    if (lane == 0) atomicAdd(&S.probes, (unsigned long long)cnt);
+    // (each lane its own: a lane makes one lookup per worker and 32 blocks, so
+    // its 32 bits last for 10^8 requests; their sum over the warp would not)
+    if (cnt) atomicAdd(&S.probes, (unsigned long long)cnt);
   } else if (warp == NU) {
     // ================ control warp
     IdsEvents<WIDE> E;
