@@ -1226,18 +1226,21 @@ rs_status poa_estimate(rs_ctx* ctx, const rs_records* records, int64_t n, double
   rs_status r = run_poa(ctx, u, probs, std::max<int64_t>(n, 1), nullptr);
   if (r != RS_OK) return r;
   // the windows are known (run_poa has read the last one): every output in one
-  // set of copies through pinned memory
+  // set of copies through pinned memory, up to POA_PINNED windows (50 MB that
+  // the context keeps); more are copied once the totals are there
+  constexpr int64_t POA_PINNED = 1 << 21;
   const int64_t cap = *n_windows_inout;
-  const int64_t k = std::max<int64_t>(0, std::min(cap, probs[0].win_cap - 1));
+  const int64_t most = std::max<int64_t>(0, std::min(cap, probs[0].win_cap - 1));
+  const int64_t k = most <= POA_PINNED ? most : 0;
   if ((r = ensure_pinned(ctx, 2 + 3 * (size_t)k)) != RS_OK) return r;
   int64_t* p = ctx->pinned;
   CK(cudaMemcpyAsync(p, ctx->p_nwin.p, 8, cudaMemcpyDeviceToHost, ctx->st), "read");
   CK(cudaMemcpyAsync(p + 1, ctx->p_total.p, 8, cudaMemcpyDeviceToHost, ctx->st), "read");
-  if (k > 0) {
-    if (numer_host) CK(cudaMemcpyAsync(p + 2, ctx->p_wnum.p, k * 8, cudaMemcpyDeviceToHost, ctx->st), "read");
-    if (opt_host) CK(cudaMemcpyAsync(p + 2 + k, ctx->p_wopt.p, k * 8, cudaMemcpyDeviceToHost, ctx->st), "read");
-    if (count_host) CK(cudaMemcpyAsync(p + 2 + 2 * k, ctx->p_wcnt.p, k * 8, cudaMemcpyDeviceToHost, ctx->st), "read");
-  }
+  void* const host[3] = {numer_host, opt_host, count_host};
+  const void* const dev[3] = {ctx->p_wnum.p, ctx->p_wopt.p, ctx->p_wcnt.p};
+  for (int q = 0; q < 3; q++)
+    if (k > 0 && host[q])
+      CK(cudaMemcpyAsync(p + 2 + q * k, dev[q], k * 8, cudaMemcpyDeviceToHost, ctx->st), "read");
   CK(cudaStreamSynchronize(ctx->st), "sync");
   const int64_t nw = p[0];
   double tot;
@@ -1246,12 +1249,15 @@ rs_status poa_estimate(rs_ctx* ctx, const rs_records* records, int64_t n, double
     return fail(ctx, RS_ERR_INVALID, "a routed row has a negative or non-finite completion time");
   *n_windows_inout = nw;
   *poa_total_host = tot;
-  const int64_t got = std::min(k, nw);
-  if (got > 0) {
-    if (numer_host) memcpy(numer_host, p + 2, got * 8);
-    if (opt_host) memcpy(opt_host, p + 2 + k, got * 8);
-    if (count_host) memcpy(count_host, p + 2 + 2 * k, got * 8);
+  const int64_t got = std::min(most, nw);
+  for (int q = 0; q < 3; q++) {
+    if (got <= 0 || !host[q]) continue;
+    if (k > 0)
+      memcpy(host[q], p + 2 + q * k, got * 8);
+    else
+      CK(cudaMemcpyAsync(host[q], dev[q], got * 8, cudaMemcpyDeviceToHost, ctx->st), "read");
   }
+  if (k == 0) CK(cudaStreamSynchronize(ctx->st), "sync");
   return RS_OK;
 }
 

@@ -191,3 +191,19 @@ def test_no_assignment_at_the_pole(W, n):
     rec, keep = _to_device(o, n, W)
     _, go, _, gt, _ = rs.poa_estimate(ctx.h, rec, n, 1)
     assert go[0] == np.inf and gt == 0.0
+
+
+def test_more_windows_than_are_staged():
+    W, last = 2, 11_500_000.0   # 2.3 M windows (2^21 go through pinned memory)
+    ctx = rs.Context(W=W, K=16)
+    o = {"worker": np.array([1, 0, 0], np.int32), "completion": np.array([2.0, 10_600_001.0, last]),
+         "ttft": np.array([0.5, 0.25, 0.125]), "nbt": np.array([4, 8, 2], np.int32),
+         "n_frozen": np.array([[1, 2], [5, 6], [7, 8]], np.uint16), "prefix": np.array([[0, 1], [8, 2], [1, 1]], np.uint16)}
+    num, opt, cnt, tot = O.poa(oracle_cfg(ctx), o)
+    rec, keep = _to_device(o, 3, W)
+    gn, go, gc, gt, nw = rs.poa_estimate(ctx.h, rec, 3, num.size)
+    assert nw == num.size == 2_300_001 and np.array_equal(gc, cnt)
+    assert np.allclose(gn, num, rtol=1e-12, atol=0) and np.allclose(go, opt, rtol=1e-12, atol=0)
+    assert abs(gt - tot) <= 1e-12 * tot
+    gn2, _, _, _, nw2 = rs.poa_estimate(ctx.h, rec, 3, 10)   # fewer entries than windows
+    assert nw2 == nw and np.array_equal(gn2[:10], gn[:10])
