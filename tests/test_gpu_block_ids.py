@@ -75,6 +75,23 @@ def test_ids_equal_tables(W, K, C, tau, policy, hi):
         assert g[0]["result"]["rebuilds"] > 0
 
 
+# more than 1024 in flight with the request slots in shared memory: completion times in more groups than lanes; requests
+# queued behind full workers, and workers enough for all
+@pytest.mark.parametrize("W,C,tau,nrep", [(3, 1100, 0.5, 1), (24, 1500, 0.0, 1), (40, 2300, 0.0, 1), (20, 1300, 0.3, 306)])
+def test_ids_equal_tables_thousands_in_flight(W, C, tau, nrep):
+    tr = _trace(2 * C, W, hi=400, pre=(64, 300))
+    tr.out_len[:] = np.random.default_rng(C).integers(0, 3000, tr.n_req)
+    reps = [wk.Replica(0, C - r % 7, wk.POLICY_DYNAMO, r % 2, 1.0, tau, r, tr.n_req) for r in range(nrep)]
+    reps.append(wk.Replica(0, 64, wk.POLICY_LOADBAL, 1, 0.0, 0.0, 3, tr.n_req))   # a spike to C and back
+    reps[-1].c_t1, reps[-1].c_t2, reps[-1].c_mid, reps[-1].c_end = 2.0, 30.0, C, 40
+    st, g = _both(rs.Context(W=W, K=2000), [tr], reps, [(0, 0), (nrep, W - 1)])
+    assert st == rs.RS_OK
+    a, e = g[0]["arrival"], g[0]["completion"]
+    assert max(int(((a <= t) & (e > t)).sum()) for t in a[::50]) > 1024
+    o = oracle_run(oracle_cfg(W, 2000), tr, reps[0])
+    assert_replica_equal(g[0], o, W)
+
+
 def test_ids_equal_tables_many_replicas():
     # two update warps per replica, traces of unequal length, truncated replicas, an idle one
     trs = [_trace(150, 1), _trace(90, 2, groups=3, hi=900), _trace(40, 3, lo=0, hi=40)]
