@@ -1322,41 +1322,37 @@ rs_status sweep_knee(rs_ctx* ctx, const rs_records* records, const int64_t* row_
   return RS_OK;
 }
 
-// The cache of a replica that ran on block ids: its live log entries' hashes.
+// The cache of a replica that ran on block ids: its live log entries' hashes,
+// found on the device (the trace's ids and hashes may be gigabytes).
 static rs_status dump_ids(rs_ctx* ctx, int32_t index, int32_t worker, uint64_t* keys_host,
                           int64_t capacity, int64_t* size) {
   const rs_ctx::IdCache& ic = ctx->last_ids[index];
   const size_t wi = (size_t)index * ctx->cfg.W + worker;
-  std::vector<uint32_t> stamps(ic.nre), log((size_t)ctx->last_ids_rmask + 1);
-  std::vector<uint32_t> ids(ic.blocks);
-  std::vector<uint64_t> hashes(ic.blocks);
   CacheMeta m;
-  CK(cudaMemcpyAsync(stamps.data(), ic.stamps + (size_t)worker * ic.nre, (size_t)ic.nre * 4,
-                     cudaMemcpyDeviceToHost, ctx->st), "read");
-  CK(cudaMemcpyAsync(log.data(), P<uint32_t>(ctx->log) + wi * ctx->gs.R, log.size() * 4,
-                     cudaMemcpyDeviceToHost, ctx->st), "read");
   CK(cudaMemcpyAsync(&m, P<CacheMeta>(ctx->meta_out) + wi, sizeof m, cudaMemcpyDeviceToHost, ctx->st),
      "read");
-  if (ic.blocks > 1) {   // (the last position is never a full block's)
-    CK(cudaMemcpyAsync(ids.data(), ic.ids, (size_t)(ic.blocks - 1) * 4, cudaMemcpyDeviceToHost, ctx->st),
-       "read");
-    CK(cudaMemcpyAsync(hashes.data(), ic.hashes, (size_t)(ic.blocks - 1) * 8, cudaMemcpyDeviceToHost,
-                       ctx->st), "read");
-  }
   CK(cudaStreamSynchronize(ctx->st), "sync");
-  std::vector<uint64_t> of(ic.nre, 0);   // a numbered block's hash: that of its first occurrence
-  for (size_t q = 0; q < ids.size(); q++)
-    if ((ids[q] >> 31) && (ids[q] & 0x7FFFFFFFu) < (uint32_t)ic.nre) of[ids[q] & 0x7FFFFFFFu] = hashes[q];
+  std::vector<uint64_t> entry(m.T - m.head);   // by log entry, 0: dead
+  if (!entry.empty()) {
+    // (the last position of a trace is never a full block's)
+    DevBuf tmp;   // hash of every numbered block, then of every entry
+    const size_t nre = (size_t)ic.nre;
+    rs_status r = ensure(ctx, tmp, (nre + entry.size()) * 8, "cache dump");
+    if (r != RS_OK) return r;
+    uint64_t* out = P<uint64_t>(tmp) + nre;
+    cudaError_t e = launch_ids_dump(ic.ids, ic.hashes, ic.blocks - 1, P<uint64_t>(tmp), ic.nre,
+                                    ic.stamps + (size_t)worker * ic.nre,
+                                    P<uint32_t>(ctx->log) + wi * ctx->gs.R, ctx->last_ids_rmask, m.head,
+                                    m.T, out, ctx->st);
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(entry.data(), out, entry.size() * 8, cudaMemcpyDeviceToHost, ctx->st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->st);
+    release(tmp);
+    CK(e, "cache dump");
+  }
   int64_t k = 0;
-  for (uint32_t t = m.head; t < m.T; t++) {
-    const uint32_t x = log[t & ctx->last_ids_rmask];
-    uint64_t h;
-    if (x >> 31)
-      h = hashes[x & 0x7FFFFFFFu];
-    else if ((int64_t)x < ic.nre && stamps[x] == t)   // (else dead)
-      h = of[x];
-    else
-      continue;
+  for (const uint64_t h : entry) {
+    if (h == 0) continue;
     if (k < capacity) keys_host[k] = h;
     k++;
   }

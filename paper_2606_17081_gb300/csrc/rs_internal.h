@@ -173,6 +173,11 @@ struct IdJob {
 };
 constexpr int IDS_MAX_JOBS = 64;
 cudaError_t launch_block_ids(const IdJob* jobs_dev, int njobs, int64_t total_req, cudaStream_t st);
+// out[t - head] = the hash of the block that log entry t of a worker holds, 0
+// where it is dead.  of: [nre], becomes the hash of each numbered block.
+cudaError_t launch_ids_dump(const uint32_t* ids, const uint64_t* hashes, int64_t blocks, uint64_t* of,
+                            int64_t nre, const uint32_t* stamps, const uint32_t* log, uint32_t rmask,
+                            uint32_t head, uint32_t T, uint64_t* out, cudaStream_t st);
 // The simulation on block ids (exact LRU; frequency eviction when b.fexp is set,
 // then with the request slots in shared memory only).
 cudaError_t launch_sim_ids(const SimDesc* d_desc, const SimBuffers& b, const SimLaunch& L,
