@@ -578,9 +578,6 @@ static rs_status records_effective(rs_ctx* ctx, const rs_records* user, int64_t 
   return RS_OK;
 }
 
-// Eq. (12) for every problem in probs (rec_base, n, scratch_base set; the
-// window slots are sized here): the last window of each problem is found on
-// the device first, so that every window its records span gets a slot.
 // Block ids of one trace of a call.
 struct TraceIds {
   const uint32_t* ids = nullptr;
@@ -588,6 +585,9 @@ struct TraceIds {
   int64_t nre = 8;   // numbered blocks, rounded up to whole sectors
 };
 
+// Eq. (12) for every problem in probs (rec_base, n, scratch_base set; the
+// window slots are sized here): the last window of each problem is found on
+// the device first, so that every window its records span gets a slot.
 static rs_status run_poa(rs_ctx* ctx, const rs_records& rec, std::vector<PoaProblem>& probs,
                          int64_t rows, rs_replica_result* res_dev) {
   const int W = ctx->cfg.W;

@@ -18,8 +18,9 @@
 // four unrolled reads.  Loads straight from global memory touch 16 lines per
 // instruction.  Bound by instruction issue (about 300 per 32 blocks, ragged
 // ends included) and by the latency of short prompts.  60 000 requests of median
-// 1 024 tokens (366 MB) 103 -> 92 us, 5 000 of 256 17.4 -> 12.3, 40 000 of 100
-// 27.6 -> 23.0; three chunks in flight leave fewer warps: 107 us.
+// 1 024 tokens (325 MB) 101 -> 82 us a call (105 -> 92 with a cold L2), 5 000 of
+// 256 12.3 -> 8.3 (19.1 -> 10.9), 40 000 of 100 22.6 -> 18.6 (29.3 -> 23.2);
+// three chunks in flight leave fewer warps: 96 us at best on the first.
 #include <algorithm>
 #include <climits>
 
@@ -157,7 +158,7 @@ static cudaError_t hash_launch(const HashJob* jobs_dev, const HashJob& one, int 
   // one warp per request, up to 48 CTAs per SM: prompt lengths vary, and short
   // CTAs leave a shorter tail than one wave with the tokens shared out (which
   // also spends a third more instructions on finding its work: 106 us against
-  // 92 on 60 000 requests)
+  // 82 on 60 000 requests)
   int64_t nblk = (total_req + HASH_NT / 32 - 1) / (HASH_NT / 32);
   if (nblk > (int64_t)sms * 48) nblk = (int64_t)sms * 48;
   k_block_hash<<<(unsigned)nblk, HASH_NT, 0, st>>>(jobs_dev, one, njobs, total_req, seed);

@@ -12,8 +12,9 @@
 // bins at once, and once a bin holds at most PCT_LAST keys their ranks are
 // counted directly: two or three passes in place of eight 8-bit digits from the
 // top byte, each with a serial scan of its 256 bins (54 replicas x 6 000 rows:
-// 152 -> 91 us a call with its copies).  Bound by the latency of its barriers.
-// The result is an element of the input, so it is bit-exact.
+// 152 -> 91 us a call with its eight copies, 55 with one in and one out).  Bound
+// by the latency of its barriers.  The result is an element of the input, so it
+// is bit-exact.
 //
 // k_sweep_knee (one warp per sweep; a sweep is a handful of levels): the
 // neighbour difference quotients, the three-point second divided difference

@@ -40,8 +40,8 @@
 // own costs, taken in two integer parts and rounded once (opt_add).
 // Measured: poa_estimate on 20 000 records, W = 6 (81 windows): 4.22 -> 0.61 ms
 // a call (keys 97 -> 5 us, sort and costs 1480 -> 17 us, solver 2941 -> 578 us,
-// total 19 -> 6 us) with one warp per window, 0.43 ms with a CTA; the estimate
-// of 16 replicas x 5000 requests at W = 64, 126 -> 7 ms.
+// total 19 -> 6 us) with one warp per window, 0.42 ms with a CTA; the estimate
+// of 16 replicas x 5000 requests at W = 64, 126 -> 10.7 ms.
 //
 // k_poa_total (one warp per replica): the whole-run PoA, sum of observed
 // latency over sum of OPT across the replica's windows; and the static

@@ -9,7 +9,7 @@
 
 namespace rs {
 
-// Per request (256 threads):
+// Per request (512 threads):
 //   probe    every (worker, block) pair at once while W nb <= PROBE_CAP, its
 //            slot kept for the update, else in rounds to each worker's first
 //            miss; beside it the request's hashes go through the repeat
@@ -21,7 +21,7 @@ namespace rs {
 // (W = 6, tau = 0.5) the probe takes 4 600, the choice 3 000, the update's reads
 // 2 600 and its writes 3 700.  With two lookups of every block of the chosen
 // worker, the choice on one thread and each request's hashes loaded on arrival
-// a call of 256 requests took 2.39 ms, now 1.76; 256 threads with two lookups
+// a call of 256 requests took 2.39 ms, now 1.81; 256 threads with two lookups
 // each in flight take the same.
 constexpr int NT_ROUTE = 512;
 
@@ -346,9 +346,10 @@ cudaError_t launch_clear_tables(uint64_t* keys, uint32_t* stamp, size_t nslots, 
 // same home bucket in every worker's table, and two workers' buckets are
 // requested before any is scanned.  A worker closes at its first absent block.
 // Bound by the latency of the bucket loads and by issue.  20 000 requests at
-// W = 64 (a call with its hashing): 437 us with a warp's 64 pairs walked together
-// in steps of shared lookup slots (5 460 instructions per 64 pairs), 294 us so;
-// with three or four workers' buckets in flight 297 and 310 us (registers).
+// W = 64 (a call with its hashing): 443 us with a warp's 64 pairs walked together
+// in steps of shared lookup slots (5 460 instructions per 64 pairs), 257 us so
+// (294 before the hashing staged its chunks; then three or four workers' buckets
+// in flight took 297 and 310 us: registers).
 constexpr int PROBE_NT = 128;
 constexpr int PROBE_ILP = 2;
 
