@@ -199,8 +199,8 @@ def _table_bytes(K: int) -> int:
 # workload (dram__bytes_read.sum + dram__bytes_write.sum), with the SHA-256 of
 # the simulation kernel's sources it was taken with.  The capture ran on 760 of
 # its 8192 simulations (one resident wave, five per SM) and is scaled.
-SIM_TRAFFIC = {"bytes": (3756686848 + 4197738496) * 8192 / 760,
-               "sources_sha256": "4f1da12673921cc8eff74c06593bb58fefafa9e6720a89f69d5da4e9f3961846",
+SIM_TRAFFIC = {"bytes": (3777521152 + 4198919936) * 8192 / 760,
+               "sources_sha256": "86847055f3850f869dd1c1a183d4a98f6308b5d53dba6bca842a8dd7fd0f6ae9",
                "summary": "profiles/k_sim_ids.md",
                "scaled_from": "760 simulations x 10 000 requests, times 8192 / 760"}
 

@@ -749,9 +749,9 @@ __global__ void __launch_bounds__(NWP == 1 ? NT_SOLVE : 32 * NWP)
 // its requests between the workers' lists; the weights that lost their minimum
 // are listed, and a warp looks up one of them, or a part of one while there
 // are fewer than warps, lanes over its worker's requests.  (16 replicas x 5000
-// requests, 48 windows of 950 to 1450 rows with 450 to 1070 rows to move: 18 ms
-// with 8 warps and a quarter of the sources per thread, 7 ms so; a round costs
-// about 500 cycles, of 6 per augmentation.)
+// requests with 1024 in flight, windows of 950 to 1450 rows with 450 to 1070 to
+// move: 10.6 ms; with 8 warps and a quarter of the sources per thread it took 2.6
+// times as long.  A round costs about 500 cycles, of 6 per augmentation.)
 constexpr int NT_WIDE = 1024;
 constexpr int NW_WIDE = NT_WIDE / 32;
 constexpr int WIDE_G = NT_WIDE / POA_WMAX_WIDE;            // source groups of a round
