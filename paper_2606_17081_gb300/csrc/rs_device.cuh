@@ -702,14 +702,15 @@ __device__ __forceinline__ void cache_prepare_captured(const TableView& t, const
 //   T = blocks before k that were touched and lie below o;
 // the entries below o that can be victims are o - T, so block k is gone iff
 // E > o - T.  One warp takes the blocks 32 at a time, a lane per block.  Places
-// touched by earlier chunks are a bitmap with the count below each of its words
-// (bits: shared, 2 ceil(G / 32) words, 0 before and after).  Within the chunk
-// every block depends on lower lanes only, so it is evaluated until no verdict
-// changes, in practice two or three times.  Bound by the latency of that chain,
-// linear in the prompt.  (8 replicas x 300 requests of 1 250 to 2 000 blocks at
-// W = 7, a fifth of them exact: one thread replaying the sequence on hash tables
-// 36.8 ms, a thread per block counting T and ins over all blocks before it 37.4,
-// so 7.5; 250 to 500 blocks 24.3, 9.6 and 4.4.)
+// touched by earlier chunks are a bitmap, and a count below each of its words is
+// taken when a later chunk has blocks among the entries (bits: shared, 2 ceil(G
+// / 32) words, 0 before and after).  Within the chunk every block depends on
+// lower lanes only, so it is evaluated until no verdict changes, in practice two
+// or three times.  Bound by the latency of that chain, linear in the prompt.  (8
+// replicas x 300 requests of 1 250 to 2 000 blocks at W = 7, a fifth of them
+// exact: one thread replaying the sequence on hash tables 36.8 ms, a thread per
+// block counting T and ins over all blocks before it 37.4, so 6.6; 250 to 500
+// blocks 24.3, 9.6 and 4.1; at most 56 blocks 8.0, 3.2 and 2.7.)
 constexpr int LRU_ABSENT = -1, LRU_FAR = -2, LRU_EVICTED = 0x40000000;
 
 template <int NT>
@@ -720,22 +721,50 @@ __device__ __forceinline__ void lru_exact(int32_t* w, int nb, int free_slots, in
     const unsigned before = (1u << lane) - 1u;
     uint32_t* below = bits + nw;
     int ins = 0;
+    bool any = false, counted = false;   // places in the bitmap, counts up to date
 #pragma unroll 1
     for (int k0 = 0; k0 < nb; k0 += 32) {
       const int o = k0 + lane < nb ? w[k0 + lane] : LRU_FAR;
       const unsigned absent = __ballot_sync(FULL_MASK, o == LRU_ABSENT);
+      const unsigned here = __ballot_sync(FULL_MASK, o >= 0);
       unsigned gone = 0u;
-      if (__any_sync(FULL_MASK, o >= 0)) {
-        unsigned lower = 0u;   // lanes before this one at lower places
+      if (here) {
+        // lanes before this one at lower places: all, for a run of blocks that
+        // were touched together (their places increase)
+        unsigned lower = here & before;
+        const unsigned run = here >> (__ffs(here) - 1);
+        const int prev = __shfl_up_sync(FULL_MASK, o, 1);
+        if ((run & (run + 1u)) || __any_sync(FULL_MASK, (lower >> ((lane + 31) & 31) & 1u) && o >= 0 && prev > o)) {
+          lower = 0u;
 #pragma unroll
-        for (int q = 0; q < 31; q++) {
-          const int y = __shfl_sync(FULL_MASK, o, q);
-          lower |= (unsigned)(y >= 0 && y < o) << q;
+          for (int q = 0; q < 31; q++) {
+            const int y = __shfl_sync(FULL_MASK, o, q);
+            lower |= (unsigned)(y < o) << q;
+          }
+          lower &= here & before;
         }
-        lower &= before;
-        int room = 0x7FFFFFFF;   // places below o not touched by earlier chunks
-        if (o >= 0)
-          room = o - (int)(below[o >> 5] + __popc(bits[o >> 5] & ((1u << (o & 31)) - 1u)));
+        int room = o;   // places below o not touched by earlier chunks
+        if (any) {
+          if (!counted) {
+            uint32_t sum = 0;
+#pragma unroll 1
+            for (int q0 = 0; q0 < nw; q0 += 32) {
+              const int q = q0 + lane;
+              const uint32_t c = q < nw ? (uint32_t)__popc(bits[q]) : 0u;
+              uint32_t x = c;
+#pragma unroll
+              for (int s = 1; s < 32; s <<= 1) {
+                const uint32_t y = __shfl_up_sync(FULL_MASK, x, s);
+                if (lane >= s) x += y;
+              }
+              if (q < nw) below[q] = sum + x - c;
+              sum += __shfl_sync(FULL_MASK, x, 31);
+            }
+            __syncwarp();
+            counted = true;
+          }
+          if (o >= 0) room -= (int)(below[o >> 5] + __popc(bits[o >> 5] & ((1u << (o & 31)) - 1u)));
+        }
         for (;;) {
           const int E = max(0, ins + __popc((absent | gone) & before) - free_slots);
           const unsigned g = __ballot_sync(FULL_MASK, o >= 0 && E > room - __popc(lower & ~gone));
@@ -748,24 +777,14 @@ __device__ __forceinline__ void lru_exact(int32_t* w, int nb, int free_slots, in
         else if (o >= 0)
           atomicOr(bits + (o >> 5), 1u << (o & 31));
         __syncwarp();
-        uint32_t run = 0;
-#pragma unroll 1
-        for (int q0 = 0; q0 < nw; q0 += 32) {
-          const int q = q0 + lane;
-          const uint32_t c = q < nw ? (uint32_t)__popc(bits[q]) : 0u;
-          uint32_t x = c;
-#pragma unroll
-          for (int s = 1; s < 32; s <<= 1) {
-            const uint32_t y = __shfl_up_sync(FULL_MASK, x, s);
-            if (lane >= s) x += y;
-          }
-          if (q < nw) below[q] = run + x - c;
-          run += __shfl_sync(FULL_MASK, x, 31);
+        if (here != gone) {
+          any = true;
+          counted = false;
         }
-        __syncwarp();
       }
       ins += __popc(absent | gone);
     }
+    __syncwarp();
     for (int q = lane; q < 2 * nw; q += 32) bits[q] = 0u;
   }
   grp_bar<NT>();
