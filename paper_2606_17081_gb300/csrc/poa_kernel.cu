@@ -522,6 +522,19 @@ __device__ __forceinline__ double narrow_opt(PoaWinShared& S, const PoaBuffers& 
   return ex < 0x7FF ? opt_value(hi, lo, ex) : opt;
 }
 
+// The same out of line, for a window per CTA: with it in the kernel's body the
+// augmentations took 2% more time.
+template <int NWP>
+__device__ __noinline__ double narrow_opt_out(PoaWinShared& S, const PoaProblem* __restrict__ probs,
+                                              const PoaBuffers& b, const ModelConsts& mc,
+                                              const double* ftab, double (*red)[NWP], int pi, int64_t w,
+                                              int m, const uint8_t* asg, bool kept) {
+  const PoaProblem pr = probs[pi];
+  const int64_t base = pr.scratch_base + b.wstart[pr.win_base + pi + w];
+  return narrow_opt<NWP>(S, b, mc, ftab, __dmul_rn(mc.w_c, 0.0) == 0.0, red, pr.rec_base, base, m, asg,
+                         kept);
+}
+
 // WT: a compile-time bound on W (the exact W for the common 3 and 6, else
 // POA_WMAX), so that the unrolled per-worker loops hold no dead iterations:
 // the solver's warps run different phases at once and its code must stay
@@ -726,7 +739,10 @@ __global__ void __launch_bounds__(NWP == 1 ? NT_SOLVE : 32 * NWP)
       // (W capw >= m: a load past its capacity is left only where every way out
       // costs infinity)
       const bool bad = ww == 0 && __any_sync(FULL_MASK, lane < W && count > capw);
-      opt = narrow_opt<NWP>(S, b, mc, ftab, wc_finite, red, pr.rec_base, base, m, asg, fx == s_fx);
+      if constexpr (NWP > 1)
+        opt = narrow_opt_out<NWP>(S, probs, b, mc, ftab, red, pi, w, m, asg, fx == s_fx);
+      else
+        opt = narrow_opt<NWP>(S, b, mc, ftab, wc_finite, red, pr.rec_base, base, m, asg, false);
       if (bad) opt = __longlong_as_double(0x7FF0000000000000ll);
     }
     if (tid == 0) {
