@@ -199,8 +199,8 @@ def _table_bytes(K: int) -> int:
 # workload (dram__bytes_read.sum + dram__bytes_write.sum), with the SHA-256 of
 # the simulation kernel's sources it was taken with.  The capture ran on 760 of
 # its 8192 simulations (one resident wave, five per SM) and is scaled.
-SIM_TRAFFIC = {"bytes": (3777521152 + 4198919936) * 8192 / 760,
-               "sources_sha256": "86847055f3850f869dd1c1a183d4a98f6308b5d53dba6bca842a8dd7fd0f6ae9",
+SIM_TRAFFIC = {"bytes": (3792514560 + 4200633856) * 8192 / 760,
+               "sources_sha256": "281c1b3318eb493f726f0d233b595b4d6e35464a409d7588e58a91e32f1ade50",
                "summary": "profiles/k_sim_ids.md",
                "scaled_from": "760 simulations x 10 000 requests, times 8192 / 760"}
 

@@ -35,7 +35,7 @@
 // instruction count are what to keep small.
 //
 // Calls before (hash tables) and now: 64 replicas x 10 000 requests at W = 3
-// 53.5 and 19.8 ms, 648 x 10 000 at W = 6 246 and 51.2 ms, 256 x 6 000 at
+// 53.5 and 19.8 ms, 648 x 10 000 at W = 6 246 and 50.7 ms, 256 x 6 000 at
 // W = 6 with controller and sampling 62.5 and 18.4 ms, 16 x 5 000 at W = 64
 // 206 and 32.8 ms, 512 requests at W = 3 2.33 and 0.97 ms; under frequency
 // eviction 64 x 10 000 at W = 3 59.8 and 22.8 ms.
